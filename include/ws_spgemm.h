@@ -287,7 +287,7 @@ ws_status_t ws_csr_nnz(ws_csr_t handle, int64_t* nnz_out);
  * info[6] total products (sum over rows of the product count),
  * info[7] number of kernel launches queued by the last symbolic pass,
  * info[8] number queued by the last numeric pass, info[9] bitmap rows,
- * info[10] heavy rows on the dense column-slice path, info[11] heavy rows
+ * info[10] heavy rows on the dense path (value windows), info[11] heavy rows
  * on the wide-bitmap path.
  * `n` is the length of `info` (at most 12 values are written).
  */
@@ -309,7 +309,7 @@ ws_status_t ws_spgemm_plan_info(ws_csr_t C, int64_t* info, int n);
  *   key 5: most stored A entries of a row that uses the one-warp register
  *          bitmap path (default and maximum 16; 0 disables that path)
  *   key 6: most stored A entries of a heavy row that uses the dense
- *          column-slice path (default and maximum 8192; 0 disables it)
+ *          path (value windows) (default and maximum 8192; 0 disables it)
  *   key 7: widest column range of a heavy row that uses the wide-bitmap path
  *          (default and maximum 1048576; 0 disables it)
  *   key 8: elementwise operations, lanes per row chunk: -1 (default:

@@ -1,25 +1,21 @@
 // Heavy rows: rows with too many products for the one-warp workspaces.  One
-// CTA owns one row, or one (row, column slice) item of a row with many
-// stored entries (the shard pattern of Sec. 4), so every output segment is
-// written by one CTA and no CTA waits on another.
+// CTA owns one row, or one window of a row's output (the shard pattern of
+// Sec. 4), so every output segment is written by one CTA and no CTA waits on
+// another.
 //
 // Dense rows (kClsRcd): the row's column range is at most 65,536 columns and
 // it has at most kRcdMaxA stored A entries (typically hub rows: few stored A
-// entries whose B rows are long).  This is the dense workspace of Gustavson's
-// algorithm (Sec. 5.1) -- a value per column plus a flag per column, the
-// sparse byte-map workspace -- over column slices:
+// entries whose B rows are long).
 //   symbolic: every product stores 1 into the flag byte of its column (plain
-//             byte stores, no atomics: the store is idempotent); nnz of the
-//             row is the number of set flags.
-//   numeric:  for each slice of `width` columns, groups of lanes walk the B
-//             rows of the stored A entries from their cursors (where the
-//             previous slice stopped) and add a * b into the dense value
-//             window with shared-memory atomics (the atomic level of Sec. 4).
-//             The flags of the slice are then scanned in column order, so the
-//             slice's entries are written sorted.  A row whose output fits
-//             one or two windows indexes the window by output rank instead
-//             (a bitmap of its columns and word ranks; rcd_compact_row) and
-//             needs no slices.
+//             byte stores, no atomics: the store is idempotent, the sparse
+//             byte-map workspace); the flags are then packed into a bitmap that
+//             stays in the plan, and nnz of the row is its population count.
+//   numeric:  the row's output is cut into windows of consecutive entries
+//             (ranks), each an item of its own; a CTA reads the row's bitmap
+//             back, ranks its words, writes the window's columns from it and
+//             adds a * b at the rank of every product that falls into the
+//             window.  The CTA takes one long B row at a time: its columns are
+//             distinct, so the adds need no atomics.
 //
 // Wide rows (kClsWb): column range up to 2^20 columns.  A bitmap over the
 // whole range (one bit per column) is the workspace:
@@ -29,6 +25,7 @@
 //             values, and let every product add its value at the rank of its
 //             column in C (global atomic add; the row's segment is private).
 #include <climits>
+#include <cstddef>
 
 #include "ws_internal.cuh"
 
@@ -36,695 +33,475 @@ namespace wsk {
 
 namespace {
 
-constexpr unsigned kFull = 0xffffffffu;
 constexpr int kRcdThreads = 512;
-constexpr int kRcdNumThreads = 512;
 constexpr int kWbThreads = 1024;  // one CTA per SM (its 128 KB bitmap), so 32 warps hide the gathers
 constexpr int kWbBatch = 4;  // stored A entries a lane group has in flight in the wide-bitmap kernel
 
 // ---------------------------------------------------------------- dense rows
 
-constexpr int kRcdCacheA = 1024;  // stored A entries of a row kept in shared memory (and of a batch)
-// Rows with more stored A entries are split into (row, slice) items (256 was
-// faster than 64 or 1024 on the R-MAT inputs; splitting every row was 1.8x slower).
-constexpr int kRcdMegaA = 256;
-static_assert(kRcdMegaA <= kRcdCacheA, "rows done whole keep all entries in shared memory");
+constexpr int kRcdCacheA = 1024;  // stored A entries handled at a time
+constexpr int kRcdWords = kMaxBitmapSpan / 32;
+constexpr long long kRcdBigProducts = 32768;  // rows with more products are taken first
+static_assert(kRcdWords == 4 * kRcdThreads, "four bitmap words per thread");
+static_assert(kRcdCacheA == 2 * kRcdThreads, "two cached entries per thread");
 
-// Counts the non-zero bytes of 16 bytes.
-__device__ __forceinline__ int nonzero_bytes(const uint4 v) {
-  return __popc(__vcmpne4(v.x, 0u) & 0x01010101u) + __popc(__vcmpne4(v.y, 0u) & 0x01010101u) +
-         __popc(__vcmpne4(v.z, 0u) & 0x01010101u) + __popc(__vcmpne4(v.w, 0u) & 0x01010101u);
+// The parts of B rows a CTA walks next: those of up to kRcdCacheA stored A
+// entries.  Parts of more than SHORT entries are cut into pieces of PIECE;
+// first[j] counts the pieces before entry j.
+struct RcdParts {
+  long long b0[kRcdCacheA];   // first position of the part in B
+  int len[kRcdCacheA];
+  int first[kRcdCacheA + 2];
+};
+
+// Exclusive scan of the piece counts of the cached entries 0..n-1 (two
+// consecutive ones per thread).  Every thread calls it; returns the total.
+template <int PIECE, int SHORT>
+__device__ __forceinline__ int rcd_scan_pieces(RcdParts& e, int n, int* s_scan) {
+  const int j = threadIdx.x * 2;
+  auto pieces = [&](int i) { return i < n && e.len[i] > SHORT ? (e.len[i] + PIECE - 1) / PIECE : 0; };
+  const int p0 = pieces(j), p1 = pieces(j + 1);
+  int total;
+  const int before = block_exclusive_scan(p0 + p1, s_scan, &total);
+  e.first[j] = before;
+  e.first[j + 1] = before + p0;
+  if (threadIdx.x == 0) e.first[kRcdCacheA] = total;
+  __syncthreads();
+  return total;
 }
 
+// Symbolic pass.  The warps share the row's B rows in pieces of kSymPiece
+// entries, so a row of a few long B rows keeps every warp busy: 610 us on
+// R-MAT 2^16 squared, a warp per B row 906 us.  Bound by the shared-memory
+// pipe (60% of its peak) and the barriers of a row.
+constexpr int kSymPiece = 256;
+constexpr int kSymShort = 32;  // B rows up to this length: a group of kSymLanes lanes, one round of loads
+constexpr int kSymLanes = 8;
+static_assert(kSymLanes * 4 >= kSymShort, "a short B row takes one round of loads");
+
+struct RcdSymbolic {
+  alignas(16) uint8_t flags[kMaxBitmapSpan];  // read in 16-byte words
+  RcdParts e;
+};
+
 template <typename T>
-__global__ void __launch_bounds__(kRcdThreads, 3) rcd_symbolic_kernel(const RowPlan<T> p) {
+__global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowPlan<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint8_t* flags = smem_raw;  // kMaxBitmapSpan bytes
-  uint4* flags4 = reinterpret_cast<uint4*>(smem_raw);
-  __shared__ long long s_scan[32];
+  RcdSymbolic& s = *reinterpret_cast<RcdSymbolic*>(smem_raw);
+  RcdParts& e = s.e;
+  __shared__ int s_scan[32];
+  __shared__ long long s_sums[32];
+  __shared__ int s_row;
   constexpr int kS = rcd_slices<T>();
-  __shared__ int s_slice[kS];  // entries per dense-window slice of the row
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kWidth = kRcdWidthBytes / static_cast<int>(sizeof(T));
   constexpr int kWarps = kRcdThreads / 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  uint4* flags4 = reinterpret_cast<uint4*>(s.flags);
   for (int i = threadIdx.x; i < kMaxBitmapSpan / 16; i += kRcdThreads) flags4[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (threadIdx.x < kS) s_slice[threadIdx.x] = 0;
-  __syncthreads();
-  for (int64_t r = blockIdx.x; r < p.seg_len; r += gridDim.x) {
+  for (int64_t guard = 0; guard <= p.seg_len; ++guard) {
+    if (threadIdx.x == 0) s_row = atomicAdd(&p.rcd_ctr[kRcdNextRow], 1);
+    __syncthreads();
+    const int r = s_row;
+    if (r >= p.seg_len) break;
     const int32_t row = p.perm[p.seg_begin + r];
     const int lo = p.lo[row];
     const int span = p.hi[row] - lo + 1;
     const int64_t ra = p.A.rowptr[row], re = p.A.rowptr[row + 1];
-    // A warp takes four stored A entries per round, one per group of 8
-    // lanes: a B row of at most 32 entries is flagged by its group in one
-    // round of loads (four per lane), longer ones by the whole warp after.
-    for (int64_t pa0 = ra + static_cast<int64_t>(warp) * 4; pa0 < re; pa0 += kWarps * 4) {
-      const int64_t pa = pa0 + (lane >> 3);
-      int64_t qb = 0, qe = 0;
-      if (pa < re) {
-        const int k = p.A.colidx[pa];
-        qb = p.B.rowptr[k];
-        qe = p.B.rowptr[k + 1];
+    long long products = 0;
+    for (int64_t e0 = ra; e0 < re; e0 += kRcdCacheA) {
+      const int n = static_cast<int>(min(static_cast<int64_t>(kRcdCacheA), re - e0));
+      for (int j = threadIdx.x; j < n; j += kRcdThreads) {
+        const int k = p.A.colidx[e0 + j];
+        const int64_t b0 = p.B.rowptr[k];
+        e.b0[j] = b0;
+        e.len[j] = static_cast<int>(p.B.rowptr[k + 1] - b0);
+        products += e.len[j];
       }
-      const bool lng = qe - qb > 32;
-      const unsigned longs = __ballot_sync(kFull, lng && (lane & 7) == 0);
-      if (!lng) {
-        int c[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int64_t t = qb + (lane & 7) + 8 * u;
-          c[u] = t < qe ? p.B.colidx[t] : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (c[u] >= 0) flags[c[u] - lo] = 1;
-        }
-      }
-      for (unsigned m = longs; m; m &= m - 1u) {
-        const int src = __ffs(m) - 1;
-        const int64_t be = __shfl_sync(kFull, qe, src);
-        int64_t q = __shfl_sync(kFull, qb, src) + lane;
-        for (; q + 96 < be; q += 128) {  // four loads in flight per lane
-          const int c0 = p.B.colidx[q], c1 = p.B.colidx[q + 32], c2 = p.B.colidx[q + 64], c3 = p.B.colidx[q + 96];
-          flags[c0 - lo] = 1;
-          flags[c1 - lo] = 1;
-          flags[c2 - lo] = 1;
-          flags[c3 - lo] = 1;
-        }
-        for (; q < be; q += 32) flags[p.B.colidx[q] - lo] = 1;
-      }
-    }
-    __syncthreads();
-    long long cnt = 0;
-    const int n16 = (span + 15) >> 4;
-    constexpr int kChunksPerSlice = kRcdWidthBytes / static_cast<int>(sizeof(T)) / 16;
-    static_assert(kChunksPerSlice % 32 == 0, "a warp's 32 chunks lie in one slice");
-    // Lane l of warp w reads chunk i0 + l; the warp's chunks share one slice,
-    // so their counts are summed in the warp and added with one atomic.
-    for (int i0 = threadIdx.x & ~31; i0 < n16; i0 += kRcdThreads) {
-      const int i = i0 + (threadIdx.x & 31);
-      const int n = i < n16 ? nonzero_bytes(flags4[i]) : 0;
-      cnt += n;
-      const int wsum = __reduce_add_sync(kFull, n);
-      if ((threadIdx.x & 31) == 0 && wsum) atomicAdd(&s_slice[i0 / kChunksPerSlice], wsum);
-      if (i < n16) flags4[i] = make_uint4(0u, 0u, 0u, 0u);
-    }
-    long long total;
-    block_exclusive_scan(cnt, s_scan, &total);
-    if (threadIdx.x == 0) {
-      p.c_rowptr[row + 1] = total;
-      if (re - ra > kRcdMegaA) {
-        const int idx = atomicAdd(p.rcd_nmega, 1);
-        p.rcd_mega[idx] = static_cast<int32_t>(r);
-        p.rcd_mna[idx] = static_cast<int32_t>(re - ra);
-        p.rcd_moff[idx] = static_cast<int64_t>(
-            atomicAdd(reinterpret_cast<unsigned long long*>(&p.sum->rcd_mega_entries), static_cast<unsigned long long>(re - ra)));
-      }
-    }
-    if (threadIdx.x < kS) {
-      p.rcd_scnt[r * kS + threadIdx.x] = s_slice[threadIdx.x];
-      s_slice[threadIdx.x] = 0;
-    }
-    __syncthreads();
-  }
-}
-
-// Slice starts of the mega rows' B rows, found once per stored A entry
-// instead of once per (row, slice) item.  Blocks (b, y) take mega rows b,
-// b + gridDim.x, ...; thread t of block (b, y) the row's entries
-// y * blockDim.x + t, stepping by gridDim.y * blockDim.x (the gridDim.y blocks
-// of a row share its entries, so one long row is no tail): for
-// every slice start lo + s * width (s = 1 .. ns - 1) the first position of the
-// sorted B row at or past it, the ns - 1 binary searches run in lockstep so
-// their loads are in flight together.  Row idx's table holds (kS - 1) arrays
-// of its na entries, slice by slice, from rcd_moff[idx] * (kS - 1).
-template <typename T>
-__global__ void __launch_bounds__(kRcdNumThreads) rcd_bounds_kernel(const RowPlan<T> p, int width) {
-  constexpr int kS = rcd_slices<T>();
-  const int n_mega = *p.rcd_nmega;
-  for (int idx = blockIdx.x; idx < n_mega; idx += gridDim.x) {
-    const int32_t row = p.perm[p.seg_begin + p.rcd_mega[idx]];
-    const long long lo = p.lo[row], hi = p.hi[row];
-    const int ns = static_cast<int>((hi - lo + width) / width);
-    const int64_t ra = p.A.rowptr[row];
-    const int na = p.rcd_mna[idx];
-    if (p.A.rowptr[row + 1] - ra != na) continue;  // the input changed: the numeric item reports it
-    int32_t* tab = p.rcd_bnd + p.rcd_moff[idx] * (kS - 1);
-    for (int j = blockIdx.y * blockDim.x + threadIdx.x; j < na; j += gridDim.y * blockDim.x) {
-      const int k = p.A.colidx[ra + j];
-      const int64_t b0 = p.B.rowptr[k];
-      const int len = static_cast<int>(p.B.rowptr[k + 1] - b0);
-      const int32_t* cols = p.B.colidx + b0;
-      int slo[kS], shi[kS];
-#pragma unroll
-      for (int q = 1; q < kS; ++q) {
-        slo[q] = 0;
-        shi[q] = q < ns ? len : 0;
-      }
-      for (int round = 0; round < 64; ++round) {  // each search halves its interval: <= 32 rounds
-        int v[kS];
-        bool open = false;
-#pragma unroll
-        for (int q = 1; q < kS; ++q) {
-          v[q] = 0;
-          if (slo[q] < shi[q]) {
-            open = true;
-            v[q] = cols[(slo[q] + shi[q]) >> 1];
-          }
-        }
-        if (!open) break;
-#pragma unroll
-        for (int q = 1; q < kS; ++q) {
-          if (slo[q] < shi[q]) {
-            const int mid = (slo[q] + shi[q]) >> 1;
-            if (v[q] < lo + static_cast<long long>(q) * width) {
-              slo[q] = mid + 1;
-            } else {
-              shi[q] = mid;
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int q = 1; q < kS; ++q) {
-        if (q < ns) tab[static_cast<int64_t>(q - 1) * na + j] = slo[q];
-      }
-    }
-  }
-}
-
-// Numeric pass of the dense heavy rows.  Two kinds of work, taken from two
-// counters so CTAs balance themselves:
-//   1. mega rows (more than kRcdMegaA stored A entries, typically the hub
-//      rows of a power-law matrix): every (row, slice) pair is a separate
-//      item, so one row's slices run on several CTAs at once.  An item reads
-//      the part of each entry's B row inside its slice from the table of
-//      slice starts (rcd_bounds_kernel), walks the long parts with a warp
-//      each and the short ones with a group of lanes each, and emits the
-//      slice from the offset the symbolic pass's per-slice counts give.
-//   2. the other rows, one CTA per row.  A row whose output fits one or two
-//      value windows takes the compact window (rcd_compact_row: no column
-//      slices); the others go slice by slice, each entry's B-row position,
-//      end and A value staying in shared memory for the whole row and every
-//      slice continuing where the last one stopped.
-constexpr int kRcdShort = 32;  // parts of B rows walked by one group of kShortLanes lanes
-constexpr int kShortLanes = 8;  // lanes walking one short part, four entries each
-static_assert(kShortLanes * 4 >= kRcdShort, "a short part takes one round of loads");
-
-// Emits one slice of the dense window in column order: thread t owns the
-// contiguous 16-byte flag chunks [t * cpt, (t + 1) * cpt); it counts their set
-// flags, the CTA scans the counts, and every thread writes its entries in
-// order from `pos0` and clears its chunks and values.  Returns the count.
-template <typename T>
-__device__ long long rcd_emit(const RowPlan<T>& p, T* dense, uint8_t* flags, int w, long long c0, int64_t pos0,
-                              int64_t cend, long long* s_scan, bool* bad) {
-  const int nq = (w + 15) >> 4;
-  const int cpt = (nq + kRcdNumThreads - 1) / kRcdNumThreads;
-  const int q0 = threadIdx.x * cpt;
-  const int q1 = min(q0 + cpt, nq);
-  uint4* f4 = reinterpret_cast<uint4*>(flags);
-  long long mine = 0;
-  for (int q = q0; q < q1; ++q) mine += nonzero_bytes(f4[q]);
-  long long total;
-  const long long before = block_exclusive_scan(mine, s_scan, &total);
-  int64_t pos = pos0 + before;
-  for (int q = q0; q < q1; ++q) {
-    const uint4 v = f4[q];
-    const uint32_t words[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int h = 0; h < 4; ++h) {
-      // bytes of this word that are set, lowest column first
-      for (uint32_t m = __vcmpne4(words[h], 0u) & 0x01010101u; m; m &= m - 1u) {
-        const int i = (q << 4) + (h << 2) + ((__ffs(m) - 1) >> 3);
-        if (pos < cend) {
-          p.c_colidx[pos] = static_cast<int32_t>(c0 + i);
-          p.c_vals[pos] = dense[i];
-        } else {
-          *bad = true;
-        }
-        dense[i] = T(0);
-        ++pos;
-      }
-    }
-    f4[q] = make_uint4(0u, 0u, 0u, 0u);
-  }
-  return total;
-}
-
-// Adds a * B[., c] for the B entries [b, b + n) (all inside [c0, c1)) into the
-// window, a warp at a time, four loads in flight per lane.
-template <typename T>
-__device__ __forceinline__ void rcd_warp_add(const RowPlan<T>& p, T* dense, uint8_t* flags, long long b, long long n,
-                                             T av, long long c0, int lane) {
-  for (long long t0 = 0; t0 < n; t0 += 128) {
-    int cc[4];
-    T bv[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const long long t = t0 + u * 32 + lane;
-      cc[u] = t < n ? p.B.colidx[b + t] : -1;
-      bv[u] = t < n ? p.B.vals[b + t] : T(0);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (cc[u] >= 0) {
-        const int off = static_cast<int>(cc[u] - c0);
-        atomicAdd(dense + off, av * bv[u]);
-        flags[off] = 1;
-      }
-    }
-  }
-}
-
-// Compact window for a dense heavy row whose output fits a few value windows
-// (nnz(row) <= kCompactPasses * width): the window is indexed by output
-// position instead of column, so the row needs no column slices; a row with
-// more entries than one window takes one pass of step 4-5 per window of
-// positions.  The flag bytes serve as a bitmap over the row's range
-// (8 * width bits >= 65,536 columns).
-//   1. warp 0 lists the stored A entries and cuts their whole B rows into
-//      pieces of kRcdPiece entries (scan of the piece counts into e_pp);
-//   2. the warps share the pieces and set the bit of every product column;
-//   3. each thread ranks four consecutive bitmap words (one barrier for
-//      the CTA scan) and keeps the rank of every word (uint16);
-//   4. the warps take the pieces again and add a * b at the rank of each
-//      column (shared-memory atomics); the product that set a column's bit
-//      in step 2 (its flag is kept per piece and lane) writes the column
-//      index of C there (rows with too many pieces for the flags write the
-//      column indices from the bitmap in step 3 instead);
-//   5. the window is copied to C's values with coalesced stores and cleared;
-//      after the last pass every thread clears its bitmap words.
-// All threads of the CTA call it; the caller's barrier follows.  Returns
-// false, having written only the entry cache, when the extra walks of a
-// multi-pass row would cost more than column slices.
-constexpr int kRcdPiece = 256;  // B entries of one warp-sized piece
-constexpr int kCompactPre = 6400;  // byte offset of the word ranks in the entry cache
-constexpr int kCompactFresh = kCompactPre + kMaxBitmapSpan / 32 * 2;  // byte offset of the fresh flags
-constexpr int kCompactPasses = 2;  // value windows a compact row may take
-constexpr long long kCompactExtraProducts = 65536;  // products re-walked by the extra passes, at most
-
-template <typename T>
-__device__ bool rcd_compact_row(const RowPlan<T>& p, T* dense, uint8_t* flags, unsigned char* cache, int width,
-                                int64_t ra, int na, long long lo, long long hi, int64_t cbase, int64_t cend,
-                                long long* s_cnt, int* s_work, bool* bad) {
-  constexpr int kWarps = kRcdNumThreads / 32;
-  constexpr int kPerLane = kRcdMegaA / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  long long* e_b0 = reinterpret_cast<long long*>(cache);              // kRcdMegaA B row starts
-  T* e_av = reinterpret_cast<T*>(cache + kRcdMegaA * 8);              // kRcdMegaA A values
-  int* e_pp = reinterpret_cast<int*>(cache + kRcdMegaA * 16);         // first piece of every entry
-  int* e_len = e_pp + kRcdMegaA + 1;                                  // B row lengths
-  uint16_t* pre = reinterpret_cast<uint16_t*>(cache + kCompactPre);  // rank of every bitmap word
-  // Per piece and lane, which of the lane's products set its column's bit
-  // first (one byte: bit u for the product at u * 32 + lane of the piece).
-  // That product writes the column index of C in step 4; a row with more
-  // pieces than the array holds writes them from the bitmap in step 3.
-  uint8_t* fresh = cache + kCompactFresh;
-  const int cache_bytes = kRcdCacheA * static_cast<int>(2 * sizeof(long long) + sizeof(T) + sizeof(int));
-  uint32_t* bm = reinterpret_cast<uint32_t*>(flags);
-  const int nnz = static_cast<int>(cend - cbase);
-  // 1. entries and pieces
-  if (warp == 0) {
-    int np[kPerLane];
-    int run = 0;
-#pragma unroll
-    for (int u = 0; u < kPerLane; ++u) {
-      const int j = lane * kPerLane + u;
-      np[u] = 0;
-      if (j < na) {
-        const int k = p.A.colidx[ra + j];
-        const long long b0 = p.B.rowptr[k];
-        const int len = static_cast<int>(p.B.rowptr[k + 1] - b0);
-        e_b0[j] = b0;
-        e_av[j] = p.A.vals[ra + j];
-        e_len[j] = len;
-        np[u] = (len + kRcdPiece - 1) / kRcdPiece;
-      }
-      run += np[u];
-    }
-    int incl = run;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(kFull, incl, o);
-      if (lane >= o) incl += y;
-    }
-    int at = incl - run;
-#pragma unroll
-    for (int u = 0; u < kPerLane; ++u) {
-      const int j = lane * kPerLane + u;
-      if (j < na) e_pp[j] = at;
-      at += np[u];
-    }
-    if (lane == 31) s_work[0] = incl;
-    long long prod = 0;  // the row's products
-#pragma unroll
-    for (int u = 0; u < kPerLane; ++u) {
-      const int j = lane * kPerLane + u;
-      if (j < na) prod += e_len[j];
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) prod += __shfl_xor_sync(kFull, prod, o);
-    if (lane == 0) s_work[1] = static_cast<int>(min(prod, static_cast<long long>(INT_MAX)));
-  }
-  __syncthreads();
-  const int npieces = s_work[0];
-  const bool by_fresh = static_cast<long long>(npieces) * 32 <= cache_bytes - kCompactFresh;
-  // Every window pass after the first walks all products again; past the
-  // budget the column-sliced path (one walk) is cheaper.
-  const int passes = (nnz + width - 1) / width;
-  if (static_cast<long long>(passes - 1) * s_work[1] > kCompactExtraProducts) return false;
-  // 2. bitmap of the product columns
-  for (int pc = warp; pc < npieces; pc += kWarps) {
-    int jl = 0, jh = na - 1;  // the entry of the piece: last one whose first piece is <= pc
-    while (jl < jh) {         // O(log na) probes of shared memory
-      const int mid = (jl + jh + 1) >> 1;
-      if (e_pp[mid] <= pc) {
-        jl = mid;
-      } else {
-        jh = mid - 1;
-      }
-    }
-    const int t0 = (pc - e_pp[jl]) * kRcdPiece + lane;
-    const int e = min((pc - e_pp[jl] + 1) * kRcdPiece, e_len[jl]);
-    const long long b = e_b0[jl];
-    int cc[kRcdPiece / 32];
-#pragma unroll
-    for (int u = 0; u < kRcdPiece / 32; ++u) cc[u] = t0 + u * 32 < e ? p.B.colidx[b + t0 + u * 32] : -1;
-    uint32_t first = 0;
-#pragma unroll
-    for (int u = 0; u < kRcdPiece / 32; ++u) {
-      const long long off = cc[u] - lo;
-      if (cc[u] >= 0) {
-        if (off >= 0 && off <= hi - lo) {
-          const uint32_t bit = 1u << (off & 31);
-          if ((atomicOr(bm + (off >> 5), bit) & bit) == 0u) first |= 1u << u;
-        } else {
-          *bad = true;
-        }
-      }
-    }
-    if (by_fresh) fresh[pc * 32 + lane] = static_cast<uint8_t>(first);
-  }
-  __syncthreads();
-  // 3. word ranks and C's column indices; thread t owns the bitmap words
-  // [4 t, 4 t + 4) (the range has at most 4 * kRcdNumThreads words; words
-  // past it are zero)
-  const int w0 = threadIdx.x * 4;
-  const uint4 v4 = *reinterpret_cast<const uint4*>(bm + w0);
-  const uint32_t wv[4] = {v4.x, v4.y, v4.z, v4.w};
-  const int mine = __popc(wv[0]) + __popc(wv[1]) + __popc(wv[2]) + __popc(wv[3]);
-  int incl = mine;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(kFull, incl, o);
-    if (lane >= o) incl += y;
-  }
-  if (lane == 31) s_cnt[warp] = incl;
-  __syncthreads();
-  int run = incl - mine, total = 0;
-#pragma unroll
-  for (int v = 0; v < kWarps; ++v) {
-    const int n = static_cast<int>(s_cnt[v]);
-    run += v < warp ? n : 0;
-    total += n;
-  }
-  if (total != nnz) *bad = true;
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    pre[w0 + q] = static_cast<uint16_t>(run);
-    run += __popc(wv[q]);
-  }
-  __syncthreads();
-  // Rows with too many pieces for the fresh flags: column indices in order,
-  // thread t writing those of the words t, t + 512, t + 1024, t + 1536
-  // (strided, so a dense stretch of columns is shared out).
-#pragma unroll
-  for (int q = 0; q < 4 && !by_fresh; ++q) {
-    const int w = q * kRcdNumThreads + threadIdx.x;
-    const long long col0 = lo + (static_cast<long long>(w) << 5) - 1;
-    int at = pre[w];
-    for (uint32_t m = bm[w]; m; m &= m - 1u) {
-      if (at < nnz) p.c_colidx[cbase + at] = static_cast<int32_t>(col0 + __ffs(m));
-      ++at;
-    }
-  }
-  // 4. values at the ranks of their columns, one window of ranks per pass
-  for (int q0 = 0; q0 < nnz; q0 += width) {
-    for (int pc = warp; pc < npieces; pc += kWarps) {
-      int jl = 0, jh = na - 1;
-      while (jl < jh) {  // O(log na) probes of shared memory
+      __syncthreads();
+      const int npieces = rcd_scan_pieces<kSymPiece, kSymShort>(e, n, s_scan);
+      // Long B rows: the warp's pieces are consecutive, so it finds its first
+      // entry by a binary search and then only moves on.
+      const int pc1 = static_cast<int>(static_cast<long long>(npieces) * (warp + 1) / kWarps);
+      int pc = static_cast<int>(static_cast<long long>(npieces) * warp / kWarps);
+      int jl = 0, jh = n - 1;  // the last entry whose first piece is <= pc
+      while (pc < pc1 && jl < jh) {
         const int mid = (jl + jh + 1) >> 1;
-        if (e_pp[mid] <= pc) {
+        if (e.first[mid] <= pc) {
           jl = mid;
         } else {
           jh = mid - 1;
         }
       }
-      const int t0 = (pc - e_pp[jl]) * kRcdPiece + lane;
-      const int e = min((pc - e_pp[jl] + 1) * kRcdPiece, e_len[jl]);
-      const long long b = e_b0[jl];
-      const T av = e_av[jl];
-      int cc[kRcdPiece / 32];
-      T bv[kRcdPiece / 32];
+      for (; pc < pc1; ++pc) {
+        while (jl + 1 < n && e.first[jl + 1] <= pc) ++jl;
+        const int t0 = (pc - e.first[jl]) * kSymPiece + lane, end = e.len[jl];
+        const int32_t* cols = p.B.colidx + e.b0[jl];
+        int c[kSymPiece / 32];
 #pragma unroll
-      for (int u = 0; u < kRcdPiece / 32; ++u) {
-        const int t = t0 + u * 32;
-        cc[u] = t < e ? p.B.colidx[b + t] : -1;
-        bv[u] = t < e ? p.B.vals[b + t] : T(0);
-      }
-      const uint32_t first = by_fresh ? fresh[pc * 32 + lane] : 0u;
+        for (int u = 0; u < kSymPiece / 32; ++u) c[u] = t0 + u * 32 < end ? cols[t0 + u * 32] : -1;
 #pragma unroll
-      for (int u = 0; u < kRcdPiece / 32; ++u) {
-        const long long off = cc[u] - lo;
-        if (cc[u] >= 0 && off >= 0 && off <= hi - lo) {
-          const int w = static_cast<int>(off >> 5);
-          const int rank = pre[w] + __popc(bm[w] & ((1u << (off & 31)) - 1u)) - q0;
-          if (rank >= 0 && rank < width) {
-            atomicAdd(dense + rank, av * bv[u]);
-            if ((first >> u) & 1u) p.c_colidx[cbase + q0 + rank] = cc[u];
-          }
+        for (int u = 0; u < kSymPiece / 32; ++u) {
+          if (c[u] >= 0) s.flags[c[u] - lo] = 1;
         }
       }
+      for (int j = warp * (32 / kSymLanes) + lane / kSymLanes; j < n; j += kWarps * (32 / kSymLanes)) {
+        const int len = e.len[j];
+        if (len > kSymShort) continue;
+        const int32_t* cols = p.B.colidx + e.b0[j];
+        int c[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) c[u] = lane % kSymLanes + u * kSymLanes < len ? cols[lane % kSymLanes + u * kSymLanes] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (c[u] >= 0) s.flags[c[u] - lo] = 1;
+        }
+      }
+      __syncthreads();
     }
-    __syncthreads();
-    // 5. copy the window out and clear it
-    const int n = min(width, nnz - q0);
-    for (int i = threadIdx.x; i < n; i += kRcdNumThreads) {
-      p.c_vals[cbase + q0 + i] = dense[i];
-      dense[i] = T(0);
+    // Packs 16 flag bytes into 16 bits of the plan's bitmap, counts and clears them.
+    uint16_t* bits16 = reinterpret_cast<uint16_t*>(p.rcd_bits + static_cast<int64_t>(r) * p.rcd_words);
+    int cnt = 0;
+    for (int i = threadIdx.x; i < p.rcd_words * 2; i += kRcdThreads) {
+      uint32_t m = 0;
+      if (i * 16 < span) {
+        const uint4 v = flags4[i];
+        flags4[i] = make_uint4(0u, 0u, 0u, 0u);
+        // byte k of a word (0 or 1) to bit 24 + k of the product
+        m = ((v.x * 0x01020408u) >> 24 & 15u) | ((v.y * 0x01020408u) >> 24 & 15u) << 4 |
+            ((v.z * 0x01020408u) >> 24 & 15u) << 8 | ((v.w * 0x01020408u) >> 24 & 15u) << 12;
+      }
+      bits16[i] = static_cast<uint16_t>(m);
+      cnt += __popc(m);
     }
-    __syncthreads();
+    // products in the high half, entries in the low half of one sum
+    long long sums;
+    block_exclusive_scan((products << 32) | cnt, s_sums, &sums);
+    if (threadIdx.x == 0) {
+      const int total = static_cast<int>(sums & 0xffffffffll);
+      const bool big = (sums >> 32) > kRcdBigProducts;
+      p.c_rowptr[row + 1] = total;
+      const int nw = (total + kWidth - 1) / kWidth;
+      const long long cap = static_cast<long long>(p.seg_len) * kS;
+      if (big) {
+        const int at = atomicAdd(&p.rcd_ctr[kRcdBigItems], nw);
+        for (int w = 0; w < nw; ++w) p.rcd_items[at + w] = static_cast<long long>(r) * kS + w;
+      } else {
+        const int at = atomicAdd(&p.rcd_ctr[kRcdItems], nw);
+        for (int w = 0; w < nw; ++w) p.rcd_items[cap - 1 - at - w] = static_cast<long long>(r) * kS + w;
+      }
+    }
   }
-  *reinterpret_cast<uint4*>(bm + w0) = make_uint4(0u, 0u, 0u, 0u);
-  return true;
+}
+
+// Numeric pass: one item (row, window of kWidth output ranks) per CTA at a
+// time, the items of rows with many products first.
+//
+// A B row part of more than kNumShort entries is taken by the whole CTA, in
+// rounds of kNumPiece entries: its columns are distinct, so the window is
+// updated with a load, one multiply-add and a store, and a barrier separates
+// it from the next part.  Shared-memory fp64 adds by compare-and-swap were
+// what bound this pass: this GPU issues an fp64 instruction over about 16
+// cycles of the SM, a swap loop that loses its slot repeats it, and a multiply
+// followed by the built-in atomic add pays it twice.  Measured on R-MAT 2^16
+// (edge factor 16, fp64) squared, 372 million products in these rows: 2.6 ms;
+// the built-in adds over column slices 3.6 ms; pieces spread over the warps
+// with a fused multiply-add in a swap loop 9.2 ms.  The multiply-adds alone
+// keep the fp64 pipe busy for 0.8 ms; the rest is the latency of an item's
+// other steps, which three CTAs per SM overlap (windows of 64 KB with two CTAs
+// per SM: 3.9 ms against 3.3 ms).  Columns and values are loaded kAhead rounds
+// before they are added and ranked one round before.  Short parts go to groups
+// of lanes and are added atomically.
+constexpr int kNumThreads = 256;
+constexpr int kNumCacheA = kNumThreads;       // stored A entries handled at a time
+constexpr int kNumPer = 2;                    // entries per thread and round
+constexpr int kNumPiece = kNumThreads * kNumPer;
+constexpr int kNumDesc = 128;                 // rounds described at a time
+constexpr int kNumWords = kRcdWords / kNumThreads;  // bitmap words per thread
+constexpr int kNumShort = 64;
+constexpr int kNumLanes = 16;  // lanes of a group, four entries each
+constexpr int kAhead = 3;
+static_assert(kNumLanes * 4 >= kNumShort, "a short part takes one round of loads");
+static_assert(kNumWords == 8, "two 16-byte words of the bitmap per thread");
+
+// One round: entries [b, b + n) of B, times a stored A entry (cached entry j).
+struct alignas(16) RcdRound {
+  long long b;
+  int n;
+  int j;
+};
+
+template <typename T>
+struct RcdNumeric {
+  static constexpr int kWidth = kRcdWidthBytes / static_cast<int>(sizeof(T));
+  alignas(16) T win[kWidth];          // accessed in 16-byte words too
+  RcdRound round[kNumDesc];
+  alignas(16) uint2 rk[kRcdWords];    // bitmap word and the rank, in the window, of its first column
+  long long b0[kNumCacheA];           // parts of B rows: first position,
+  T a[kNumCacheA];                    //   the A value,
+  int len[kNumCacheA];                //   length,
+  int first[kNumCacheA];              //   rounds before the part
+};
+
+// Start and end of the part of the sorted cols[0..n) inside [c0, c1]: two
+// searches in 4-way steps whose six loads are in flight together.
+__device__ __forceinline__ void part_bounds(const int32_t* cols, int n, int c0, int c1, int* start, int* end) {
+  int l[2] = {0, 0}, h[2] = {n, n};
+  const int limit[2] = {c0, c1};  // first column >= c0, first column > c1
+  auto before = [&](int i, int v) { return i == 0 ? v < limit[0] : v <= limit[1]; };
+  while (h[0] - l[0] >= 4 || h[1] - l[1] >= 4) {
+    int v[2][3];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int q = (h[i] - l[i]) >> 2;
+#pragma unroll
+      for (int t = 0; t < 3; ++t) v[i][t] = h[i] - l[i] >= 4 ? cols[l[i] + (t + 1) * q] : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int q = (h[i] - l[i]) >> 2, m = l[i];
+      if (h[i] - m < 4) continue;
+      if (before(i, v[i][1])) {
+        l[i] = before(i, v[i][2]) ? m + 3 * q + 1 : m + 2 * q + 1;
+        h[i] = before(i, v[i][2]) ? h[i] : m + 3 * q;
+      } else {
+        l[i] = before(i, v[i][0]) ? m + q + 1 : m;
+        h[i] = before(i, v[i][0]) ? m + 2 * q : m + q;
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {  // at most three columns are left: their count before the limit
+    int below = 0;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) below += l[i] + t < h[i] && before(i, cols[l[i] + t]);
+    (i == 0 ? *start : *end) = l[i] + below;
+  }
 }
 
 template <typename T>
-__global__ void __launch_bounds__(kRcdNumThreads, 2) rcd_numeric_kernel(const RowPlan<T> p, int width) {
-  constexpr int kS = rcd_slices<T>();
-  static_assert(kRcdCacheA * (2 * sizeof(long long) + sizeof(T) + sizeof(int)) <= kRcdMaxA * sizeof(int),
-                "the entry cache fits the space after the window");
-  static_assert(kRcdMegaA * 16 + (2 * kRcdMegaA + 1) * static_cast<int>(sizeof(int)) <= kCompactPre &&
-                    kCompactPre + kMaxBitmapSpan / 32 * sizeof(uint16_t) <=
-                        kRcdCacheA * (2 * sizeof(long long) + sizeof(T) + sizeof(int)),
-                "the compact-window layout fits the entry cache");
-  static_assert(kMaxBitmapSpan <= 65536, "a row has at most 65,536 entries, so word ranks fit uint16");
-  static_assert(kRcdWidthBytes / static_cast<int>(sizeof(T)) * 8 >= kMaxBitmapSpan &&
-                    kMaxBitmapSpan / 32 == 4 * kRcdNumThreads,
-                "the flag bytes hold a bitmap of the range; four bitmap words per thread");
+__global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPlan<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* dense = reinterpret_cast<T*>(smem_raw);                           // width values
-  uint8_t* flags = smem_raw + static_cast<size_t>(width) * sizeof(T);  // width bytes
-  long long* c_pos = reinterpret_cast<long long*>(flags + width);      // per entry: position in B,
-  long long* c_end = c_pos + kRcdCacheA;                               //   end of the B row (or of the part),
-  T* c_av = reinterpret_cast<T*>(c_end + kRcdCacheA);                  //   the A value,
-  int* c_long = reinterpret_cast<int*>(c_av + kRcdCacheA);             //   and the list of long parts
-  __shared__ long long s_scan[32];
-  __shared__ int s_item, s_next, s_next2, s_nlong, s_work[2];
-  __shared__ long long s_out0;
-  const int lane = threadIdx.x & 31;
-  for (int i = threadIdx.x; i < width; i += kRcdNumThreads) {
-    dense[i] = T(0);
-    flags[i] = 0;
-  }
+  using S = RcdNumeric<T>;
+  S& s = *reinterpret_cast<S*>(smem_raw);
+  constexpr int kS = rcd_slices<T>();
+  constexpr int kWidth = S::kWidth;
+  constexpr int kWarps = kNumThreads / 32;
+  __shared__ int s_scan[32];
+  __shared__ int s_item, s_c0, s_c1;
+  const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
+  const int nbig = p.rcd_ctr[kRcdBigItems], nitems = nbig + p.rcd_ctr[kRcdItems];
+  const long long cap = static_cast<long long>(p.seg_len) * kS;
   bool bad = false;
-  const int n_mega = *p.rcd_nmega;
-
-  // 1. (mega row, slice) items
-  for (int guard = 0; guard <= n_mega * kS; ++guard) {
+  for (int guard = 0; guard <= nitems; ++guard) {
     __syncthreads();  // the previous item is done with the shared state
-    if (threadIdx.x == 0) {
-      s_item = atomicAdd(p.rcd_ctr, 1);
-      s_nlong = 0;
+    if (tid == 0) s_item = atomicAdd(&p.rcd_ctr[kRcdNextItem], 1);
+    __syncthreads();
+    const int it = s_item;
+    if (it >= nitems) break;
+    const long long item = it < nbig ? p.rcd_items[it] : p.rcd_items[cap - 1 - (it - nbig)];
+    const int64_t r = item / kS;
+    const int q0 = static_cast<int>(item % kS) * kWidth;  // first rank of the window
+    const int32_t row = p.perm[p.seg_begin + r];
+    const int lo = p.lo[row];
+    const int64_t cbase = p.c_rowptr[row] + q0;
+    const long long want = p.c_rowptr[row + 1] - cbase;  // entries of the row from this window on
+    // 1. the row's bitmap and the rank of every word
+    uint32_t wv[kNumWords];
+    int cnt = 0;
+#pragma unroll
+    for (int h = 0; h < kNumWords / 4; ++h) {
+      const int i = tid * (kNumWords / 4) + h;  // 16-byte word
+      uint4 v = make_uint4(0u, 0u, 0u, 0u);
+      if (i * 4 < p.rcd_words) v = reinterpret_cast<const uint4*>(p.rcd_bits + r * p.rcd_words)[i];
+      wv[4 * h] = v.x;
+      wv[4 * h + 1] = v.y;
+      wv[4 * h + 2] = v.z;
+      wv[4 * h + 3] = v.w;
+      cnt += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+    }
+    int total;
+    int run = block_exclusive_scan(cnt, s_scan, &total);
+#pragma unroll
+    for (int q = 0; q < kNumWords; ++q) {
+      s.rk[tid * kNumWords + q] = make_uint2(wv[q], static_cast<uint32_t>(run - q0));
+      run += __popc(wv[q]);
+    }
+    if (total - q0 != want) bad = true;
+    const int in_win = min(kWidth, total - q0);  // ranks in the window, at least 1
+    const int n_out = static_cast<int>(max(0ll, min(static_cast<long long>(in_win), want)));
+    __syncthreads();
+    // 2. the window's columns, placed in the (still unused) window memory:
+    // every thread takes as many consecutive ranks (an odd number, so the
+    // lanes' stores fall into different banks) and walks the set bits from the
+    // word that holds its first one.  With a thread or a warp per word the
+    // densest words set the time (2.0 of 8.0 million cycles per CTA on R-MAT
+    // 2^16 squared).
+    int* cols = reinterpret_cast<int*>(s.win);
+    const int per = ((in_win + kNumThreads - 1) / kNumThreads) | 1;
+    const int t0 = tid * per, t1 = min(t0 + per, in_win);
+    if (t0 < t1) {
+      int w = 0, wh = kRcdWords - 1;  // the last word whose first rank is <= t0
+      while (w < wh) {
+        const int mid = (w + wh + 1) >> 1;
+        if (static_cast<int>(s.rk[mid].y) <= t0) {
+          w = mid;
+        } else {
+          wh = mid - 1;
+        }
+      }
+      uint32_t m = s.rk[w].x;
+      for (int skip = t0 - static_cast<int>(s.rk[w].y); skip > 0; --skip) m &= m - 1u;
+      for (int at = t0; at < t1; ++at, m &= m - 1u) {
+        while (m == 0u && w + 1 < kRcdWords) m = s.rk[++w].x;
+        const int c = lo + (w << 5) + __ffs(m) - 1;
+        cols[at] = c;
+        if (at == 0) s_c0 = c;
+        if (at == in_win - 1) s_c1 = c;
+      }
     }
     __syncthreads();
-    const int item = s_item;
-    if (item >= n_mega * kS) break;
-    const int r = p.rcd_mega[item / kS], sl = item % kS;
-    const int32_t row = p.perm[p.seg_begin + r];
-    const long long lo = p.lo[row], hi = p.hi[row];
-    const long long c0 = lo + static_cast<long long>(sl) * width;
-    if (c0 > hi) continue;
-    const long long c1 = min(c0 + width, hi + 1);
-    if (threadIdx.x == 0) {
-      long long o = p.c_rowptr[row];
-      for (int t = 0; t < sl; ++t) o += p.rcd_scnt[static_cast<int64_t>(r) * kS + t];
-      s_out0 = o;
-    }
-    const int64_t ra = p.A.rowptr[row];
-    const int na = static_cast<int>(p.A.rowptr[row + 1] - ra);
-    const int ns = static_cast<int>((hi - lo + width) / width);
-    const int32_t* tab = p.rcd_bnd + p.rcd_moff[item / kS] * (kS - 1);
-    if (na != p.rcd_mna[item / kS]) {  // the input changed since the symbolic pass
-      bad = true;
-      continue;
-    }
-    for (int e0 = 0; e0 < na; e0 += kRcdCacheA) {
-      const int nb = min(kRcdCacheA, na - e0);
-      // the part of each entry's B row inside the slice, from the table of
-      // slice starts (rcd_bounds_kernel)
-      for (int j = threadIdx.x; j < nb; j += kRcdNumThreads) {
-        const int e = e0 + j;
-        const int k = p.A.colidx[ra + e];
-        const long long b0 = p.B.rowptr[k], len = p.B.rowptr[k + 1] - b0;
-        const long long st = sl == 0 ? 0 : tab[static_cast<int64_t>(sl - 1) * na + e];
-        const long long en = sl + 1 < ns ? tab[static_cast<int64_t>(sl) * na + e] : len;
-        c_pos[j] = b0 + st;
-        c_end[j] = b0 + en;
-        c_av[j] = p.A.vals[ra + e];
-        if (en - st > kRcdShort) c_long[atomicAdd(&s_nlong, 1)] = j;
+#pragma unroll 4
+    for (int i = tid; i < n_out; i += kNumThreads) p.c_colidx[cbase + i] = cols[i];
+    __syncthreads();
+    for (int i = tid; i < kWidth * static_cast<int>(sizeof(T)) / 16; i += kNumThreads)
+      reinterpret_cast<uint4*>(s.win)[i] = make_uint4(0u, 0u, 0u, 0u);
+    const int c0 = s_c0, c1 = s_c1;
+    const bool whole = total <= kWidth;
+    // Rank of column c in the window; kWidth (and an error) if it has none,
+    // which only an input changed since the symbolic pass can cause.
+    auto rank_of = [&](int c) {
+      const uint32_t off = static_cast<uint32_t>(c - lo);
+      const uint2 rk = s.rk[(off >> 5) & (kRcdWords - 1)];
+      const uint32_t at = rk.y + __popc(rk.x & ((1u << (off & 31u)) - 1u));
+      return at < static_cast<uint32_t>(kWidth) ? static_cast<int>(at) : kWidth;
+    };
+    const int64_t ra = p.A.rowptr[row], re = p.A.rowptr[row + 1];
+    for (int64_t e0 = ra; e0 < re; e0 += kNumCacheA) {
+      const int n = static_cast<int>(min(static_cast<int64_t>(kNumCacheA), re - e0));
+      // 3. the part of every entry's B row inside the window's columns, and the
+      // rounds of the long parts
+      int rounds = 0;
+      if (tid < n) {
+        const int k = p.A.colidx[e0 + tid];
+        s.a[tid] = p.A.vals[e0 + tid];
+        const long long b0 = p.B.rowptr[k];
+        int start = 0, end = static_cast<int>(p.B.rowptr[k + 1] - b0);
+        if (!whole) part_bounds(p.B.colidx + b0, end, c0, c1, &start, &end);
+        s.b0[tid] = b0 + start;
+        s.len[tid] = end - start;
+        rounds = end - start > kNumShort ? (end - start + kNumPiece - 1) / kNumPiece : 0;
       }
-      if (threadIdx.x == 0) {
-        s_next = 0;
-        s_next2 = 0;
-      }
+      int nrounds;
+      s.first[tid] = block_exclusive_scan(rounds, s_scan, &nrounds);
       __syncthreads();
-      const int nl = s_nlong;
-      for (int g2 = 0; g2 <= nl; ++g2) {  // long parts: a warp each
-        int t = 0;
-        if (lane == 0) t = atomicAdd(&s_next, 1);
-        t = __shfl_sync(kFull, t, 0);
-        if (t >= nl) break;
-        const int j = c_long[t];
-        rcd_warp_add(p, dense, flags, c_pos[j], c_end[j] - c_pos[j], c_av[j], c0, lane);
-      }
-      // short parts: a group of kShortLanes lanes each, every lane loading up
-      // to four of the part's entries at once (one round of loads per part)
-      constexpr int kGroupsPerWarp = 32 / kShortLanes;
-      for (int g2 = 0; g2 <= nb / kGroupsPerWarp + 1; ++g2) {
-        int base = 0;
-        if (lane == 0) base = atomicAdd(&s_next2, kGroupsPerWarp);
-        base = __shfl_sync(kFull, base, 0);
-        if (base >= nb) break;
-        const int j = base + lane / kShortLanes;
-        if (j < nb && c_end[j] - c_pos[j] <= kRcdShort) {
-          const T av = c_av[j];
-          const long long t0 = c_pos[j] + lane % kShortLanes, e = c_end[j];
-          int cc[4];
-          T bv[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const long long t = t0 + u * kShortLanes;
-            cc[u] = t < e ? p.B.colidx[t] : -1;
-            bv[u] = t < e ? p.B.vals[t] : T(0);
+      // 4a. long parts, round by round
+      for (int p0 = 0; p0 < nrounds; p0 += kNumDesc) {
+        const int np = min(kNumDesc, nrounds - p0);
+        if (tid < np) {
+          int jl = 0, jh = n - 1;  // the last entry whose first round is <= p0 + tid
+          while (jl < jh) {
+            const int mid = (jl + jh + 1) >> 1;
+            if (s.first[mid] <= p0 + tid) {
+              jl = mid;
+            } else {
+              jh = mid - 1;
+            }
           }
+          const int t0 = (p0 + tid - s.first[jl]) * kNumPiece;
+          s.round[tid] = RcdRound{s.b0[jl] + t0, min(kNumPiece, s.len[jl] - t0), jl};
+        }
+        __syncthreads();
+        // Round i sits in registers i % kAhead: its columns and values, and its
+        // stored A entry.  The loads of shared memory a round needs (window,
+        // A value, the next round's ranks, the descriptor of the round to load)
+        // are issued together, ahead of the multiply-adds.
+        int col[kAhead][kNumPer], ent[kAhead];
+        T val[kAhead][kNumPer];
+        int at[kNumPer];
+        auto load = [&](const RcdRound& d, int u) {
+          ent[u] = d.j;
+          const int32_t* bc = p.B.colidx + d.b + tid;
+          const T* bv = p.B.vals + d.b + tid;
 #pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            if (cc[u] >= 0) {
-              const int off = static_cast<int>(cc[u] - c0);
-              atomicAdd(dense + off, av * bv[u]);
-              flags[off] = 1;
+          for (int h = 0; h < kNumPer; ++h) {
+            col[u][h] = -1;
+            if (tid + h * kNumThreads < d.n) {
+              col[u][h] = bc[h * kNumThreads];
+              val[u][h] = bv[h * kNumThreads];
+            }
+          }
+        };
+        const RcdRound none{0, 0, -1};
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) load(u < np ? s.round[u] : none, u);
+#pragma unroll
+        for (int h = 0; h < kNumPer; ++h) at[h] = col[0][h] >= 0 ? rank_of(col[0][h]) : -1;
+        for (int i0 = 0; i0 < np; i0 += kAhead) {
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u) {
+            const int v = (u + 1) % kAhead;
+            if (i0 + u < np) {
+              const RcdRound d = i0 + u + kAhead < np ? s.round[i0 + u + kAhead] : none;
+              const int j = ent[u];
+              const T a = s.a[j];
+              T w[kNumPer], x[kNumPer];
+              int next[kNumPer];
+#pragma unroll
+              for (int h = 0; h < kNumPer; ++h) {
+                w[h] = at[h] >= 0 && at[h] < kWidth ? s.win[at[h]] : T(0);
+                x[h] = val[u][h];
+              }
+#pragma unroll
+              for (int h = 0; h < kNumPer; ++h) next[h] = col[v][h] >= 0 ? rank_of(col[v][h]) : -1;
+              load(d, u);
+#pragma unroll
+              for (int h = 0; h < kNumPer; ++h) {
+                if (at[h] >= 0) {
+                  if (at[h] < kWidth) {
+                    s.win[at[h]] = fma(a, x[h], w[h]);
+                  } else {
+                    bad = true;
+                  }
+                }
+                at[h] = next[h];
+              }
+              if (ent[v] != j) __syncthreads();  // the same in every thread
+            }
+          }
+        }
+        __syncthreads();
+      }
+      // 4b. short parts
+      for (int j = warp * (32 / kNumLanes) + lane / kNumLanes; j < n; j += kWarps * (32 / kNumLanes)) {
+        const int len = s.len[j];
+        if (len > kNumShort) continue;
+        const T a = s.a[j];
+        const long long b0 = s.b0[j];
+        int c[4];
+        T bv[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int t = lane % kNumLanes + u * kNumLanes;
+          c[u] = t < len ? p.B.colidx[b0 + t] : -1;
+          bv[u] = t < len ? p.B.vals[b0 + t] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if (c[u] >= 0) {
+            const int q = rank_of(c[u]);
+            if (q < kWidth) {
+              atomicAdd(s.win + q, a * bv[u]);
+            } else {
+              bad = true;
             }
           }
         }
       }
       __syncthreads();
-      if (threadIdx.x == 0) s_nlong = 0;
-      __syncthreads();
     }
-    const int64_t want = p.rcd_scnt[static_cast<int64_t>(r) * kS + sl];
-    const long long got = rcd_emit(p, dense, flags, static_cast<int>(c1 - c0), c0, s_out0, s_out0 + want, s_scan, &bad);
-    if (threadIdx.x == 0 && got != want) bad = true;
-  }
-
-  // 2. the other rows, one CTA each
-  for (int guard = 0; guard <= p.seg_len; ++guard) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      s_item = atomicAdd(p.rcd_ctr + 1, 1);
-      s_nlong = 0;
-      s_next = 0;
-      s_next2 = 0;
-    }
-    __syncthreads();
-    const int r = s_item;
-    if (r >= p.seg_len) break;
-    const int32_t row = p.perm[p.seg_begin + r];
-    const int64_t ra = p.A.rowptr[row];
-    const int na = static_cast<int>(p.A.rowptr[row + 1] - ra);
-    if (na > kRcdMegaA) continue;  // a mega row: done in part 1
-    const long long lo = p.lo[row], hi = p.hi[row];
-    const int64_t cbase = p.c_rowptr[row];
-    const int64_t cend = p.c_rowptr[row + 1];
-    if (cend - cbase <= static_cast<int64_t>(kCompactPasses) * width &&
-        rcd_compact_row(p, dense, flags, reinterpret_cast<unsigned char*>(c_pos), width, ra, na, lo, hi, cbase, cend,
-                        s_scan, s_work, &bad))
-      continue;  // done without column slices
-    for (int j = threadIdx.x; j < na; j += kRcdNumThreads) {
-      const int k = p.A.colidx[ra + j];
-      c_pos[j] = p.B.rowptr[k];
-      c_end[j] = p.B.rowptr[k + 1];
-      c_av[j] = p.A.vals[ra + j];
-    }
-    __syncthreads();
-    int64_t emitted = 0;
-    for (long long c0 = lo; c0 <= hi; c0 += width) {
-      const long long c1 = min(c0 + width, hi + 1);
-      // Warps take stored A entries one at a time from a shared counter and
-      // walk each B row from where the last slice stopped, four loads in
-      // flight per lane; the columns of one B row are distinct, entries of
-      // different warps meet in shared-memory atomics.
-      for (int g2 = 0; g2 <= na; ++g2) {
-        int j = 0;
-        if (lane == 0) j = atomicAdd(&s_next, 1);
-        j = __shfl_sync(kFull, j, 0);
-        if (j >= na) break;
-        const long long pos = c_pos[j], end = c_end[j];
-        const T av = c_av[j];
-        long long stop = end;
-        for (long long t0 = pos; t0 < end; t0 += 128) {
-          int cc[4];
-          T bv[4];
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const long long t = t0 + u * 32 + lane;
-            cc[u] = t < end ? p.B.colidx[t] : INT_MAX;
-            bv[u] = t < end ? p.B.vals[t] : T(0);
-          }
-          bool past = false;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {
-            const long long t = t0 + u * 32 + lane;
-            if (cc[u] < c1) {
-              const int off = static_cast<int>(cc[u] - c0);
-              atomicAdd(dense + off, av * bv[u]);
-              flags[off] = 1;
-            } else if (t < end) {
-              stop = min(stop, t);
-              past = true;
-            }
-          }
-          if (__any_sync(kFull, past)) break;  // the rest of this B row lies past the slice
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) stop = min(stop, __shfl_xor_sync(kFull, stop, o));
-        if (lane == 0) c_pos[j] = stop;
-      }
-      __syncthreads();
-      emitted += rcd_emit(p, dense, flags, static_cast<int>(c1 - c0), c0, cbase + emitted, cend, s_scan, &bad);
-      if (threadIdx.x == 0) s_next = 0;  // every warp has left this slice's entry loop
-      __syncthreads();
-    }
-    if (threadIdx.x == 0 && emitted != cend - cbase) bad = true;
+    // 5. the window's values
+#pragma unroll 4
+    for (int i = tid; i < n_out; i += kNumThreads) p.c_vals[cbase + i] = s.win[i];
   }
   if (bad) atomicOr(&p.sum->status, kErrCount);
 }
@@ -886,34 +663,19 @@ int grid_of(int64_t rows, int num_sms, int per_sm) {
 
 }  // namespace
 
-size_t rcd_numeric_smem(int width, size_t value_bytes) {
-  return static_cast<size_t>(width) * (value_bytes + 1) +
-         static_cast<size_t>(kRcdCacheA) * (2 * sizeof(long long) + value_bytes + sizeof(int));
-}
-
 template <typename T>
 void launch_rcd(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, int* launches) {
   if (!numeric) {
-    const size_t smem = kMaxBitmapSpan;
+    const size_t smem = sizeof(RcdSymbolic);
     static int per_sm = 0;
     if (per_sm == 0) per_sm = occupancy(rcd_symbolic_kernel<T>, kRcdThreads, smem);
     rcd_symbolic_kernel<T><<<grid_of(p.seg_len, num_sms, per_sm), kRcdThreads, smem, s>>>(p);
   } else {
-    const int width = kRcdWidthBytes / static_cast<int>(sizeof(T));
-    const size_t smem = rcd_numeric_smem(width, sizeof(T));
+    const size_t smem = sizeof(RcdNumeric<T>);
     static int per_sm = 0;
-    if (per_sm == 0) per_sm = occupancy(rcd_numeric_kernel<T>, kRcdNumThreads, smem);
-    rcd_numeric_kernel<T><<<grid_of(p.seg_len, num_sms, per_sm), kRcdNumThreads, smem, s>>>(p, width);
+    if (per_sm == 0) per_sm = occupancy(rcd_numeric_kernel<T>, kNumThreads, smem);
+    rcd_numeric_kernel<T><<<grid_of(p.seg_len * rcd_slices<T>(), num_sms, per_sm), kNumThreads, smem, s>>>(p);
   }
-  *launches += 1;
-}
-
-template <typename T>
-void launch_rcd_bounds(const RowPlan<T>& p, int num_sms, cudaStream_t s, int* launches) {
-  const int width = kRcdWidthBytes / static_cast<int>(sizeof(T));
-  constexpr int kBlocksPerRow = 8;
-  const dim3 grid(grid_of(p.seg_len, num_sms, 1), kBlocksPerRow);
-  rcd_bounds_kernel<T><<<grid, kRcdNumThreads, 0, s>>>(p, width);
   *launches += 1;
 }
 
@@ -929,8 +691,6 @@ void launch_wb(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, i
 
 template void launch_rcd<float>(const RowPlan<float>&, bool, int, cudaStream_t, int*);
 template void launch_rcd<double>(const RowPlan<double>&, bool, int, cudaStream_t, int*);
-template void launch_rcd_bounds<float>(const RowPlan<float>&, int, cudaStream_t, int*);
-template void launch_rcd_bounds<double>(const RowPlan<double>&, int, cudaStream_t, int*);
 template void launch_wb<float>(const RowPlan<float>&, bool, int, cudaStream_t, int*);
 template void launch_wb<double>(const RowPlan<double>&, bool, int, cudaStream_t, int*);
 

@@ -76,8 +76,11 @@ constexpr uint8_t kClsWb = kClsRcd + 1;         // heavy rows, wide bitmap works
 // Heavy-row limits.
 constexpr int kRcdMaxA = 8192;            // stored A entries a dense row may have (cursor slots)
 constexpr int kRcdDefaultMaxA = 8192;     // default limit used by the classification
-constexpr int kRcdWidthBytes = 65536;     // dense value window per slice
-// Dense-window slices of a dense heavy row (its span is at most kMaxBitmapSpan columns).
+constexpr int kRcdWidthBytes = 49152;     // value window of one item of a dense heavy row
+// Counters of the dense heavy rows: items of rows with many products, other
+// items, next row of the symbolic pass, next item of the numeric pass.
+constexpr int kRcdBigItems = 0, kRcdItems = 1, kRcdNextRow = 2, kRcdNextItem = 3, kRcdCounters = 4;
+// Value windows of a dense heavy row at most (it has at most kMaxBitmapSpan entries).
 template <typename T>
 constexpr int rcd_slices() {
   return (kMaxBitmapSpan + kRcdWidthBytes / static_cast<int>(sizeof(T)) - 1) / (kRcdWidthBytes / static_cast<int>(sizeof(T)));
@@ -111,7 +114,6 @@ struct DevSummary {
   long long products;  // sum of ub_i
   long long dense_slices;
   long long slice_cursor;
-  long long rcd_mega_entries;  // stored A entries of the dense heavy rows split into (row, slice) items
   int status;
   int n_sort;
   int n_long;   // rows analysed by a CTA each (queued from the back of the long-row list)
@@ -149,13 +151,11 @@ struct RowPlan {
   const int32_t* slice_first;
   int32_t* slice_cnt;          // entries per dense-window slice
   uint16_t* ranks;             // register bitmap rows: output position of every product, kBmrSlots per row
-  int32_t* rcd_scnt;           // dense heavy rows: entries per dense-window slice, rcd_slices<T>() per row
-  int32_t* rcd_mega;           // dense heavy rows with more than 256 stored A entries (segment positions)
-  int32_t* rcd_nmega;          // their number
-  int32_t* rcd_ctr;            // two work counters of the numeric kernel (zeroed before it)
-  int64_t* rcd_moff;           // per mega row: first of its entries in the slice-start table
-  int32_t* rcd_mna;            // per mega row: its stored A entries when the table was sized
-  int32_t* rcd_bnd;            // slice-start table of the mega rows' B rows (numeric only)
+  uint32_t* rcd_bits;          // dense heavy rows: bitmap of the row's columns from lo on, rcd_words words per row
+  int rcd_words;               // a multiple of 4, enough for min(columns of B, kMaxBitmapSpan)
+  long long* rcd_items;        // their numeric work items (row * rcd_slices<T>() + window): rows with many products
+                               // from the front, the others from the back of seg_len * rcd_slices<T>() places
+  int32_t* rcd_ctr;            // counters kRcdBigItems .. kRcdNextItem
   DevSummary* sum;
   int64_t seg_begin;   // first position in perm of the segment a kernel processes
   int64_t seg_len;     // rows in that segment
@@ -266,8 +266,6 @@ template <typename T>
 void launch_bitmap(const RowPlan<T>& p, int bin, bool numeric, int num_sms, cudaStream_t s, int* launches);
 template <typename T>
 void launch_rcd(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, int* launches);
-template <typename T>
-void launch_rcd_bounds(const RowPlan<T>& p, int num_sms, cudaStream_t s, int* launches);
 template <typename T>
 void launch_wb(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, int* launches);
 template <typename T>

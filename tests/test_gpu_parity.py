@@ -278,6 +278,47 @@ def test_dense_rows_many_products_few_columns(dtype):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+def test_dense_rows_windows_and_rounds(dtype):
+    """Dense heavy rows at the edges of their output windows (49,152 bytes of
+    values: one entry less than a window, exactly one, one more, exactly two)
+    and of the parts of B rows inside a window: around the short-part limit
+    (64), around one and two rounds (512, 1024), more rounds than are
+    described at a time (128), and 255, 256 and 257 stored entries (256 are
+    cached at a time; the symbolic pass caches 1024)."""
+    rng = np.random.default_rng(37)
+    n = 1 << 16
+    window = 49152 // np.dtype(dtype).itemsize
+    perm = rng.permutation(n)
+    blocks = [perm[:window - 1], perm[:window], perm[:window + 1], perm[:2 * window]]
+    rows = {i: c.tolist() for i, c in enumerate(blocks)}
+    lens = [1, 63, 64, 65, 511, 512, 513, 1023, 1024, 1025, 3000]
+    first_len = len(rows)
+    for L in lens:
+        rows[len(rows)] = rng.choice(n, size=L, replace=False).tolist()
+    inside = len(rows)                                    # subsets of the smallest block
+    for _ in range(20):
+        rows[len(rows)] = rng.choice(blocks[0], size=600, replace=False).tolist()
+    k = 1400
+    many = len(rows)
+    while len(rows) < k:
+        rows[len(rows)] = rng.choice(n, size=int(rng.integers(0, 120)), replace=False).tolist()
+    B = _csr(k, n, rows, dtype=dtype)
+    B.vals = (2 * rng.random(B.nnz) - 1).astype(dtype)
+    sub = list(range(inside, inside + 20))
+    arows = {i: [i] + sub for i in range(4)}              # windows
+    arows[4] = list(range(first_len, first_len + len(lens)))
+    arows[5] = list(range(k - 200, k)) + list(range(4)) + sub          # more than 128 rounds
+    for i, na in enumerate((255, 256, 257, 1030)):
+        arows[6 + i] = rng.choice(np.arange(many, k), size=na - 1, replace=False).tolist() + [0]
+    A = _csr(10, k, arows, dtype=dtype)
+    A.vals = (2 * rng.random(A.nnz) - 1).astype(dtype)
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["rcd_rows"] == 10
+    assert np.diff(rowptr)[:4].tolist() == [window - 1, window, window + 1, 2 * window]
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 def test_wide_heavy_rows(dtype):
     """Rows with thousands of stored A entries over short B rows spanning ~2^20 columns."""
     rng = np.random.default_rng(32)
