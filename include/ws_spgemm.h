@@ -282,8 +282,7 @@ ws_status_t ws_csr_nnz(ws_csr_t handle, int64_t* nnz_out);
 /*
  * ws_spgemm_plan_info -- counts from the last symbolic pass of C, for
  * diagnostics and tests: info[0] empty rows, info[1] single-entry (direct
- * copy) rows, info[2] hash rows, info[3] hash rows re-routed to the sorting
- * path, info[4] dense-window rows, info[5] dense-window slices,
+ * copy) rows, info[2] hash rows, info[3] hash rows ranked by a sort, info[4] dense-window rows, info[5] dense-window slices,
  * info[6] total products (sum over rows of the product count),
  * info[7] number of kernel launches queued by the last symbolic pass,
  * info[8] number queued by the last numeric pass, info[9] bitmap rows,
@@ -298,10 +297,9 @@ ws_status_t ws_spgemm_plan_info(ws_csr_t C, int64_t* info, int n);
  *   key 1: largest product count of a row that uses the shared-memory hash
  *          path (default 4096; smaller values send more rows to the
  *          dense-window path, 0 sends every multi-entry row there)
- *   key 2: longest run of occupied slots a row's hash table may hold
- *          (default 64; a row with a longer run, or whose probes wrap
- *          around the table, uses the sorting path; smaller values send
- *          more rows there)
+ *   key 2: most products a bucket of a hash row may hold (default 64; a row
+ *          with a fuller bucket is sorted; smaller values send more rows
+ *          there)
  *   key 3: dense-window slice width in columns (default 8192 for double,
  *          16384 for float; must be a multiple of 1024, 0 = default)
  *   key 4: widest column range of a row that uses the bitmap path

@@ -56,7 +56,7 @@ __device__ __forceinline__ uint8_t classify(long long nnza, long long ub, int lo
   if (bitmap_ok && span <= (32ll << bitmap_log_words(kNumBitmapBins - 1)) && est <= bitmap_cap(kNumBitmapBins - 1))
     return static_cast<uint8_t>(kClsBitmap0 + kNumBitmapBins - 1);
   if (ub <= ap.hash_max) {
-    int b = ceil_log2_ll(ub) - (kMinHashLog - 1);
+    int b = ceil_log2_ll(ub) - kMinHashLog;
     b = b < 0 ? 0 : b;
     return static_cast<uint8_t>(kClsHash0 + b);
   }

@@ -143,6 +143,7 @@ struct Plan {
   DevBuf ranks;   // register bitmap rows: kBmrSlots uint16 ranks per row of A
   DevBuf ew;      // elementwise operations: summary, chunk arrays, scan partials
   DevBuf sv;      // sparse matrix - sparse vector product (in A^T's handle): accumulator, byte-map, offsets
+  DevBuf hranks;  // hash rows: uint16 ranks of their products, one block per bin
   DevBuf rcd;     // dense heavy rows: work counters, numeric items, the rows' bitmaps
   int kind = kPlanNone;  // which symbolic pass filled this plan
   // elementwise plan (kPlanEwise)
@@ -168,7 +169,6 @@ struct Plan {
   int32_t* lo = nullptr;
   int32_t* hi = nullptr;
   int32_t* long_rows = nullptr;
-  int32_t* sort_list = nullptr;
   int32_t* pending = nullptr;
   int64_t* partials = nullptr;
   int32_t* slice_row = nullptr;
@@ -187,6 +187,7 @@ struct Plan {
   bool all_planned = false;  // the planning pass took every row: its segment is rows 0..m-1 in order
   int dense_width = 0;
   int run_limit = 64;
+  bool hash_ranked = false;  // hranks holds the hash rows' ranks
   int sym_launches = 0, num_launches = 0;
   struct OuterState* outer = nullptr;  // outer-product SpGEMM between its two passes
 };
@@ -233,9 +234,7 @@ ws_status_t read_summary(Plan* pl, cudaStream_t s) {
 
 ws_status_t device_status(const DevSummary& hs) {
   if (hs.status == 0) return WS_OK;
-  return fail(WS_ERR_DEVICE, "device status 0x%x (probe=%d rank=%d count=%d sortcap=%d)", hs.status,
-              !!(hs.status & kErrProbe), !!(hs.status & kErrRank), !!(hs.status & kErrCount),
-              !!(hs.status & kErrSortCap));
+  return fail(WS_ERR_DEVICE, "device status 0x%x (count=%d)", hs.status, !!(hs.status & kErrCount));
 }
 
 template <typename T>
@@ -250,7 +249,6 @@ RowPlan<T> make_rowplan(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan*
   p.cls = pl->cls;
   p.lo = pl->lo;
   p.hi = pl->hi;
-  p.sort_list = pl->sort_list;
   p.slice_row = pl->slice_row;
   p.slice_idx = pl->slice_idx;
   p.slice_first = pl->slice_first;
@@ -271,7 +269,6 @@ ws_status_t carve_rows(Plan* pl, int64_t m, cudaStream_t s) {
   const size_t o_lo = off; off = align_up(off + 4 * static_cast<size_t>(m), 256);
   const size_t o_hi = off; off = align_up(off + 4 * static_cast<size_t>(m), 256);
   const size_t o_long = off; off = align_up(off + 4 * static_cast<size_t>(m), 256);
-  const size_t o_sort = off; off = align_up(off + 4 * static_cast<size_t>(m), 256);
   const size_t o_pend = off; off = align_up(off + 4 * static_cast<size_t>(m), 256);
   const size_t o_part = off; off = align_up(off + 8 * static_cast<size_t>(nb + 1), 256);
   const size_t o_cls = off; off = align_up(off + static_cast<size_t>(m), 256);
@@ -283,7 +280,6 @@ ws_status_t carve_rows(Plan* pl, int64_t m, cudaStream_t s) {
   pl->lo = reinterpret_cast<int32_t*>(b + o_lo);
   pl->hi = reinterpret_cast<int32_t*>(b + o_hi);
   pl->long_rows = reinterpret_cast<int32_t*>(b + o_long);
-  pl->sort_list = reinterpret_cast<int32_t*>(b + o_sort);
   pl->pending = reinterpret_cast<int32_t*>(b + o_pend);
   pl->partials = reinterpret_cast<int64_t*>(b + o_part);
   pl->cls = reinterpret_cast<uint8_t*>(b + o_cls);
@@ -301,6 +297,26 @@ ws_status_t carve_slices(Plan* pl, int64_t nslices, cudaStream_t s) {
   pl->slice_first = reinterpret_cast<int32_t*>(b + 2 * each);
   pl->slice_cnt = reinterpret_cast<int32_t*>(b + 3 * each);
   return WS_OK;
+}
+
+// The ranks of hash bin b's products in the plan (nullptr if it has no room).
+uint16_t* hash_ranks_of(const Plan* pl, int b) {
+  if (!pl->hash_ranked) return nullptr;
+  size_t off = 0;
+  for (int i = 0; i < b; ++i) off += static_cast<size_t>(pl->seg_count[kSegHash0 + i]) << (kMinHashLog + i);
+  return static_cast<uint16_t*>(pl->hranks.ptr) + off;
+}
+
+// Room for the ranks of the hash rows.  They are an aid, not a need: if the
+// memory is not to be had the numeric pass works them out again.
+void reserve_hash_ranks(Plan* pl, cudaStream_t s) {
+  size_t n = 0;
+  for (int b = 0; b < kNumHashBins; ++b) n += static_cast<size_t>(pl->seg_count[kSegHash0 + b]) << (kMinHashLog + b);
+  pl->hash_ranked = n > 0 && pl->hranks.reserve(n * sizeof(uint16_t), s) == WS_OK;
+  if (n > 0 && !pl->hash_ranked) {
+    cudaGetLastError();  // the failed allocation is not an error of this call
+    g_last_error.clear();
+  }
 }
 
 // Second half of the symbolic pass when some rows were not ranked by the
@@ -369,11 +385,13 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     p.seg_len = pl->seg_count[g];
     launch_bitmap<T>(p, b, false, sms, s, &pl->sym_launches);
   }
+  reserve_hash_ranks(pl, s);
   for (int b = 0; b < kNumHashBins; ++b) {
     const int g = kSegHash0 + b;
     if (pl->seg_count[g] == 0) continue;
     p.seg_begin = pl->seg_offset[g];
     p.seg_len = pl->seg_count[g];
+    p.hash_ranks = hash_ranks_of(pl, b);
     launch_hash<T>(p, b, false, sms, s, &pl->sym_launches);
   }
   launch_scan(C->rowptr, m, pl->partials, pl->dsum, s, &pl->sym_launches);
@@ -507,9 +525,9 @@ ws_status_t numeric_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan
     if (pl->seg_count[g] == 0) continue;
     p.seg_begin = pl->seg_offset[g];
     p.seg_len = pl->seg_count[g];
+    p.hash_ranks = hash_ranks_of(pl, b);
     launch_hash<T>(p, b, true, sms, s, &pl->num_launches);
   }
-  if (pl->n_sort > 0) launch_sort<T>(p, pl->n_sort, sms, s, &pl->num_launches);
   if (pl->seg_count[kSegDense] > 0) {
     p.seg_begin = pl->seg_offset[kSegDense];
     p.seg_len = pl->seg_count[kSegDense];
@@ -771,7 +789,7 @@ void release_outer(Plan* pl, cudaStream_t s) {
 void release_plan_async(Plan* pl, cudaStream_t s) {
   if (!pl) return;
   release_outer(pl, s);
-  DevBuf* bufs[] = {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->rcd};
+  DevBuf* bufs[] = {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd};
   for (DevBuf* b : bufs) {
     if (b->ptr) cudaFreeAsync(b->ptr, s);
     b->ptr = nullptr;
@@ -1285,7 +1303,7 @@ ws_status_t ws_csr_destroy(ws_csr_t h) {
   if (!h) return WS_OK;
   if (h->plan) {
     if (h->plan->rows.ptr || h->plan->slices.ptr || h->plan->ranks.ptr || h->plan->ew.ptr || h->plan->sv.ptr ||
-        h->plan->rcd.ptr || h->plan->outer)
+        h->plan->hranks.ptr || h->plan->rcd.ptr || h->plan->outer)
       cudaDeviceSynchronize();
     release_outer(h->plan, nullptr);
     h->plan->rows.release();
@@ -1293,6 +1311,7 @@ ws_status_t ws_csr_destroy(ws_csr_t h) {
     h->plan->ranks.release();
     h->plan->ew.release();
     h->plan->sv.release();
+    h->plan->hranks.release();
     h->plan->rcd.release();
     release_host_sum(h->plan->host_sum);
     delete h->plan;

@@ -8,10 +8,8 @@
 //   direct        exactly one stored A[i,k]      -> C[i,:] = A[i,k] * B[k,:]
 //   bitmap bin b  column range of the row at most 32 << log_words(b) columns and
 //                 min(ub_i, range) <= cap(b)     -> bitmap + rank workspace
-//   hash bin b    ub_i <= 32 << b (b = 0..7)     -> shared-memory hash workspace of
-//                                                  64 << b slots, sort-free ranking
-//   sort          a hash row whose table showed a long run of occupied slots
-//                 (or wrapped) -> shared-memory hash + bitonic sort
+//   hash bin b    ub_i <= 32 << b (b = 0..7)     -> products in registers, ranked through
+//                                                  32 << b monotone-hash buckets
 //   dense window  ub_i above the hash limit      -> column slices of the row, each a
 //                                                  dense bitmap + value workspace
 // Each class is a different realisation of the per-row workspace w of
@@ -26,7 +24,7 @@
 namespace wsk {
 
 constexpr int kNumHashBins = 8;
-constexpr int kMinHashLog = 6;  // bin b uses a table of 1 << (kMinHashLog + b) slots
+constexpr int kMinHashLog = 5;  // bin b holds rows of at most 1 << (kMinHashLog + b) products
 constexpr int kMaxHashProducts = 32 << (kNumHashBins - 1);  // 4096
 
 // Bitmap bins: bitmap of 1 << log_words 32-bit words (the row's column range
@@ -68,8 +66,7 @@ constexpr uint8_t kClsBmr0 = 2;                            // .. + kNumBmrBins -
 constexpr uint8_t kClsBitmap0 = kClsBmr0 + kNumBmrBins;    // .. + kNumBitmapBins - 1
 constexpr uint8_t kClsHash0 = kClsBitmap0 + kNumBitmapBins;  // .. + kNumHashBins - 1
 constexpr uint8_t kClsDense = kClsHash0 + kNumHashBins;
-constexpr uint8_t kClsSort = kClsDense + 1;
-constexpr uint8_t kClsBmrWide = kClsSort + 1;  // register bitmap rows counted by the planning pass
+constexpr uint8_t kClsBmrWide = kClsDense + 1;  // register bitmap rows counted by the planning pass
 constexpr uint8_t kClsRcd = kClsBmrWide + 1;    // heavy rows, dense column-slice workspace, CTA per row
 constexpr uint8_t kClsWb = kClsRcd + 1;         // heavy rows, wide bitmap workspace, CTA per row
 
@@ -101,11 +98,8 @@ constexpr int kNumSegs = kSegWb + 1;
 
 // Device error flags (OR-ed into DevSummary::status).
 enum DevError : int {
-  kErrProbe = 1,       // a hash insert ran through a whole table (cannot happen at load <= 1/2)
-  kErrRank = 2,        // a run of occupied slots longer than the ranking limit in the numeric pass
   kErrCount = 4,       // the numeric pass found a different entry count than the symbolic pass
   kErrInvalidCsr = 8,  // validation found broken CSR invariants
-  kErrSortCap = 16,    // a sort-path row exceeded its workspace
 };
 
 // Counters shared between the kernels of one product and read back by the host.
@@ -115,7 +109,7 @@ struct DevSummary {
   long long dense_slices;
   long long slice_cursor;
   int status;
-  int n_sort;
+  int n_sort;  // hash rows ranked by a sort
   int n_long;   // rows analysed by a CTA each (queued from the back of the long-row list)
   int n_mid;    // rows analysed by a warp each (queued from the front)
   int n_empty;
@@ -145,12 +139,13 @@ struct RowPlan {
   uint8_t* cls;        // row class per row
   int32_t* lo;         // smallest column any product of the row can hit
   int32_t* hi;         // largest such column
-  int32_t* sort_list;  // rows rerouted to the sorting path
   const int32_t* slice_row;    // dense-window slices: row, slice index, first slice of the row
   const int32_t* slice_idx;
   const int32_t* slice_first;
   int32_t* slice_cnt;          // entries per dense-window slice
   uint16_t* ranks;             // register bitmap rows: output position of every product, kBmrSlots per row
+  uint16_t* hash_ranks;        // hash bin: output position of every product, 32 << bin per row of the segment
+                               // (nullptr: the plan has no room, the numeric pass ranks again)
   uint32_t* rcd_bits;          // dense heavy rows: bitmap of the row's columns from lo on, rcd_words words per row
   int rcd_words;               // a multiple of 4, enough for min(columns of B, kMaxBitmapSpan)
   long long* rcd_items;        // their numeric work items (row * rcd_slices<T>() + window): rows with many products
@@ -160,7 +155,7 @@ struct RowPlan {
   int64_t seg_begin;   // first position in perm of the segment a kernel processes
   int64_t seg_len;     // rows in that segment
   int log2_group;      // lanes per stored A entry when walking B rows (1 << log2_group)
-  int run_limit;       // longest occupied run a hash row may hold (longer: sorting path)
+  int run_limit;       // most products a bucket of a hash row may hold (more: the row is sorted)
   int dense_width;     // dense-window slice width in columns
 };
 
@@ -273,8 +268,6 @@ void launch_dense(const RowPlan<T>& p, int64_t nslices, bool numeric, int num_sm
                   int* launches);
 template <typename T>
 void launch_direct(const RowPlan<T>& p, int num_sms, cudaStream_t s, int* launches);
-template <typename T>
-void launch_sort(const RowPlan<T>& p, int64_t nrows, int num_sms, cudaStream_t s, int* launches);
 
 // skip != nullptr: the scan does nothing when *skip != 0 (read on the device).
 void launch_scan(int64_t* rowptr, int64_t m, int64_t* partials, DevSummary* sum, cudaStream_t s, int* launches,
@@ -284,10 +277,8 @@ int64_t scan_partials_needed(int64_t m);
 void launch_validate(const int64_t* rowptr, const int32_t* colidx, int64_t nrows, int64_t ncols, int64_t nnz,
                      DevSummary* sum, int num_sms, cudaStream_t s);
 
-// Dynamic shared memory needed by the dense-window kernel and the sort kernel.
+// Dynamic shared memory needed by the dense-window kernel.
 size_t dense_smem_bytes(int width, size_t value_bytes, bool numeric);
-size_t sort_smem_bytes(size_t value_bytes);
-constexpr int kSortTableLog = 13;  // sort path: 8192-slot table, up to 4096 entries
 
 // Exclusive prefix sum over the threads of a CTA of blockDim.x threads
 // (a multiple of 32, at most 1024).  `scratch` holds 32 values; returns this

@@ -318,6 +318,106 @@ def test_dense_rows_windows_and_rounds(dtype):
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+def _hash_edge_case(dtype):
+    """Rows of every hash bin at its edges (one product less, exactly, one more
+    than a power of two), over 3,000,000 columns: B rows of 0, 1 and 40
+    entries, rows of many one-entry B rows, repeated columns, and rows whose
+    columns crowd at one end."""
+    rng = np.random.default_rng(38)
+    n = 3_000_000
+    rows = {0: [0], 1: [n - 1]}
+    rows[2] = []                                                     # an empty B row
+    ones = list(range(3, 4500))                                      # one entry each
+    for r in ones:
+        rows[r] = [int(rng.integers(1, n - 1))]
+    forty = list(range(4500, 4650))
+    for r in forty:
+        rows[r] = rng.choice(n - 2, size=40, replace=False).tolist()
+    shared = list(range(4650, 4750))                                 # 40 of 100 columns: repeats
+    pool = rng.choice(n - 2, size=100, replace=False)
+    for r in shared:
+        rows[r] = rng.choice(pool, size=40, replace=False).tolist()
+    crowd = list(range(4750, 4850))                                  # 40 of the first 3000 columns
+    for r in crowd:
+        rows[r] = rng.choice(np.arange(1, 3000), size=40, replace=False).tolist()
+    B = _csr(4850, n, rows, dtype=dtype)
+    B.vals = (2 * rng.random(B.nnz) - 1).astype(dtype)
+    lens = np.diff(B.rowptr)
+    arows = {}
+    sizes = sorted({s + d for s in (32, 64, 128, 256, 512, 1024, 2048) for d in (-1, 0, 1)} | {2, 3, 4095, 4096})
+    for u in sizes:
+        for kind in range(4):
+            pick = [0, 1, 2]                                         # both ends, and the empty row
+            left = u - 2
+            group = (forty, shared, crowd, [])[kind]
+            for r in rng.permutation(group)[:left // 40]:
+                pick.append(int(r))
+                left -= int(lens[r])
+            pick += [int(r) for r in rng.choice(ones, size=left, replace=False)]
+            arows[len(arows)] = pick
+    A = _csr(len(arows), 4850, arows, dtype=dtype)
+    A.vals = (2 * rng.random(A.nnz) - 1).astype(dtype)
+    return A, B
+
+
+@pytest.mark.parametrize("run_limit", [64, 2])
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_hash_rows_bin_edges(dtype, run_limit):
+    """Every hash bin at its edges, with and without the sort of crowded rows."""
+    A, B = _hash_edge_case(dtype)
+    with tuning(run_limit=run_limit):
+        rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["hash_rows"] == A.nrows
+    assert 0 < info["sorted_rows"] < A.nrows
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
+def test_hash_rows_without_room_for_ranks():
+    """With almost all device memory taken the symbolic pass cannot keep the
+    ranks of the hash rows and the numeric pass works them out: the same C.
+    (A process of its own: an earlier test's freed scratch would serve.)"""
+    import subprocess
+    import sys
+    code = """
+import numpy as np, torch
+from tests.test_gpu_parity import _hash_edge_case
+from tests._gpu import assert_matches_oracle
+from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+from synth import HostCSR
+A, B = _hash_edge_case(np.float64)
+reps = 400  # 100 rows, 400 times: the ranks take about 88 MB
+rp = np.concatenate([[0], np.cumsum(np.tile(np.diff(A.rowptr), reps))]).astype(np.int64)
+A = HostCSR(A.nrows * reps, A.ncols, rp, np.tile(A.colidx, reps), np.tile(A.vals, reps))
+dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+def product(hog):
+    op = SpGEMM(dA, dB)
+    held = []
+    if hog:
+        size = 1 << 30
+        while size >= 1 << 24:  # leave less than 48 MB
+            if torch.cuda.mem_get_info()[0] - size > 40 << 20:
+                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            else:
+                size >>= 1
+    op.symbolic()
+    del held
+    torch.cuda.empty_cache()
+    C = op.numeric()
+    op.wait()
+    return op, C.to_host()
+op2, (rp2, ci2, v2) = product(False)  # kept: its scratch stays taken
+op1, (rp1, ci1, v1) = product(True)
+assert op1.plan_info()["hash_rows"] == A.nrows
+assert np.array_equal(rp1, rp2) and np.array_equal(ci1, ci2)
+assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.arange(100))
+assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.arange(A.nrows - 100, A.nrows))
+"""
+    import os
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-2000:]
+
+
 @pytest.mark.parametrize("dtype", DTYPES)
 def test_wide_heavy_rows(dtype):
     """Rows with thousands of stored A entries over short B rows spanning ~2^20 columns."""
