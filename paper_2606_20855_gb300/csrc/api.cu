@@ -10,6 +10,7 @@
 //   -- read nnz(C) and the status word back (one small copy + stream sync)
 // Numeric pass (ws_spgemm_numeric): one launch per non-empty class, no sync.
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -135,6 +136,135 @@ void keep_pool_memory(int dev) {
   done[dev] = true;
 }
 
+// Side streams for the independent row kernels of one pass: the classes of
+// rows touch different rows of C, so their kernels may overlap, and a class of
+// few long rows then does not leave the GPU to one CTA per row.  Sets are
+// checked out for the duration of one call, recycled across handles and
+// threads, and at most kMaxSets are kept.
+struct SideStreams {
+  static constexpr int kStreams = 3;
+  int device = 0;
+  cudaStream_t st[kStreams] = {};
+  cudaEvent_t fork = nullptr, join[kStreams] = {};
+};
+constexpr size_t kMaxSets = 8;
+std::mutex g_side_mutex;
+std::vector<SideStreams*> g_side_free;
+
+void destroy_side(SideStreams* x) {
+  for (int i = 0; i < SideStreams::kStreams; ++i) {
+    if (x->st[i]) cudaStreamDestroy(x->st[i]);
+    if (x->join[i]) cudaEventDestroy(x->join[i]);
+  }
+  if (x->fork) cudaEventDestroy(x->fork);
+  delete x;
+}
+
+SideStreams* acquire_side(int device) {
+  {
+    std::lock_guard<std::mutex> lock(g_side_mutex);
+    for (size_t i = 0; i < g_side_free.size(); ++i) {
+      if (g_side_free[i]->device == device) {
+        SideStreams* x = g_side_free[i];
+        g_side_free.erase(g_side_free.begin() + static_cast<std::ptrdiff_t>(i));
+        return x;
+      }
+    }
+  }
+  SideStreams* x = new (std::nothrow) SideStreams;
+  if (!x) return nullptr;
+  x->device = device;
+  bool ok = cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
+  for (int i = 0; i < SideStreams::kStreams && ok; ++i) {
+    ok = cudaStreamCreateWithFlags(&x->st[i], cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) == cudaSuccess;
+  }
+  if (!ok) {
+    cudaGetLastError();  // the caller goes on without side streams
+    destroy_side(x);
+    return nullptr;
+  }
+  return x;
+}
+
+void release_side(SideStreams* x) {
+  {
+    std::lock_guard<std::mutex> lock(g_side_mutex);
+    if (g_side_free.size() < kMaxSets) {
+      try {
+        g_side_free.push_back(x);
+        return;
+      } catch (...) {
+      }
+    }
+  }
+  destroy_side(x);  // pending work completes first
+}
+
+// Spreads `kernels` independent launches over the caller's stream and a set
+// of side streams, everything ordered after what the caller's stream holds;
+// join() orders the caller's stream after all of them, so outside the call
+// the work looks as if it had been queued on that stream alone.  Fewer than
+// kMinKernels launches, and streams that are being captured (a recycled stream
+// must not stay in a capture), use the caller's stream only.
+class Fork {
+ public:
+  static constexpr int kMinKernels = 3;
+  Fork(cudaStream_t main, int device, int kernels) : main_(main) {
+    if (kernels < kMinKernels) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(main, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+      cudaGetLastError();
+      return;
+    }
+    side_ = acquire_side(device);
+    if (side_ && cudaEventRecord(side_->fork, main_) != cudaSuccess) {
+      cudaGetLastError();
+      release_side(side_);
+      side_ = nullptr;
+    }
+  }
+  Fork(const Fork&) = delete;
+  Fork& operator=(const Fork&) = delete;
+  ~Fork() { join(); }
+  // Stream of the next launch.
+  cudaStream_t next() {
+    if (!side_) return main_;
+    const int i = turn_++ % (SideStreams::kStreams + 1) - 1;
+    if (i < 0) return main_;
+    if (!used_[i]) {
+      if (cudaStreamWaitEvent(side_->st[i], side_->fork, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return main_;
+      }
+      used_[i] = true;
+    }
+    return side_->st[i];
+  }
+  cudaError_t join() {
+    if (!side_) return cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < SideStreams::kStreams; ++i) {
+      if (!used_[i]) continue;
+      cudaError_t x = cudaEventRecord(side_->join[i], side_->st[i]);
+      if (x == cudaSuccess) x = cudaStreamWaitEvent(main_, side_->join[i], 0);
+      if (x != cudaSuccess) {
+        cudaStreamSynchronize(side_->st[i]);  // keeps the order all the same
+        e = x;
+      }
+    }
+    release_side(side_);
+    side_ = nullptr;
+    return e;
+  }
+
+ private:
+  cudaStream_t main_;
+  SideStreams* side_ = nullptr;
+  bool used_[SideStreams::kStreams] = {};
+  int turn_ = 0;
+};
+
 enum PlanKind { kPlanNone = 0, kPlanSpgemm = 1, kPlanEwise = 2, kPlanSub = 3 };
 
 struct Plan {
@@ -254,6 +384,10 @@ RowPlan<T> make_rowplan(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan*
   p.slice_first = pl->slice_first;
   p.slice_cnt = pl->slice_cnt;
   p.ranks = static_cast<uint16_t*>(pl->ranks.ptr);
+  p.rcd_ctr = pl->rcd_ctr;
+  p.rcd_items = pl->rcd_items;
+  p.rcd_bits = pl->rcd_bits;
+  p.rcd_words = pl->rcd_words;
   p.sum = pl->dsum;
   p.log2_group = pl->log2_group;
   p.run_limit = pl->run_limit;
@@ -319,6 +453,13 @@ void reserve_hash_ranks(Plan* pl, cudaStream_t s) {
   }
 }
 
+// Row kernels of a pass (the symbolic pass has none for direct and planned rows).
+int bin_launches(const Plan* pl, bool numeric) {
+  int n = 0;
+  for (int g = 0; g < kNumSegs; ++g) n += pl->seg_count[g] > 0 && (numeric || (g != kSegDirect && g != kSegBmrWide));
+  return n;
+}
+
 // Second half of the symbolic pass when some rows were not ranked by the
 // planning pass: group the rows by segment, run the per-bin symbolic kernels,
 // scan the counts into C's row pointer and read the summary back.
@@ -330,21 +471,16 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
   if (off > 0) {
     launch_scatter<T>(p, m, pl->seg_offset, sms, s, &pl->sym_launches);
   }
+  // All scratch and counters first, on the caller's stream.
   int64_t bmr_rows = 0;
   for (int b = 0; b < kNumBmrBins; ++b) bmr_rows += pl->seg_count[kSegBmr0 + b];
   if (bmr_rows > 0) {
     st = pl->ranks.reserve(static_cast<size_t>(m) * kBmrSlots * sizeof(uint16_t), s);
     if (st != WS_OK) return st;
-    p.ranks = static_cast<uint16_t*>(pl->ranks.ptr);
   }
   if (pl->seg_count[kSegDense] > 0) {
     st = carve_slices(pl, pl->dense_slices, s);
     if (st != WS_OK) return st;
-    p = make_rowplan<T>(A, B, C, pl);
-    p.seg_begin = pl->seg_offset[kSegDense];
-    p.seg_len = pl->seg_count[kSegDense];
-    launch_dense_slices<T>(p, pl->slice_row, pl->slice_idx, pl->slice_first, sms, s, &pl->sym_launches);
-    launch_dense<T>(p, pl->dense_slices, false, sms, s, &pl->sym_launches);
   }
   if (pl->seg_count[kSegRcd] > 0) {
     const int64_t nr = pl->seg_count[kSegRcd];
@@ -358,42 +494,33 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     pl->rcd_items = reinterpret_cast<long long*>(b + o_items);
     pl->rcd_bits = reinterpret_cast<uint32_t*>(b + o_bits);
     WS_CUDA(cudaMemsetAsync(pl->rcd_ctr, 0, kRcdCounters * sizeof(int32_t), s), "cudaMemsetAsync(rcd counters)");
-    p.rcd_ctr = pl->rcd_ctr;
-    p.rcd_items = pl->rcd_items;
-    p.rcd_bits = pl->rcd_bits;
-    p.rcd_words = pl->rcd_words;
-    p.seg_begin = pl->seg_offset[kSegRcd];
-    p.seg_len = nr;
-    launch_rcd<T>(p, false, sms, s, &pl->sym_launches);
-  }
-  if (pl->seg_count[kSegWb] > 0) {
-    p.seg_begin = pl->seg_offset[kSegWb];
-    p.seg_len = pl->seg_count[kSegWb];
-    launch_wb<T>(p, false, sms, s, &pl->sym_launches);
-  }
-  for (int b = 0; b < kNumBmrBins; ++b) {
-    const int g = kSegBmr0 + b;
-    if (pl->seg_count[g] == 0) continue;
-    p.seg_begin = pl->seg_offset[g];
-    p.seg_len = pl->seg_count[g];
-    launch_bmr<T>(p, b, false, sms, s, &pl->sym_launches);
-  }
-  for (int b = 0; b < kNumBitmapBins; ++b) {
-    const int g = kSegBitmap0 + b;
-    if (pl->seg_count[g] == 0) continue;
-    p.seg_begin = pl->seg_offset[g];
-    p.seg_len = pl->seg_count[g];
-    launch_bitmap<T>(p, b, false, sms, s, &pl->sym_launches);
   }
   reserve_hash_ranks(pl, s);
-  for (int b = 0; b < kNumHashBins; ++b) {
-    const int g = kSegHash0 + b;
-    if (pl->seg_count[g] == 0) continue;
+  p = make_rowplan<T>(A, B, C, pl);
+  Fork fork(s, C->device, bin_launches(pl, false));
+  auto segment = [&](int g) {
     p.seg_begin = pl->seg_offset[g];
     p.seg_len = pl->seg_count[g];
-    p.hash_ranks = hash_ranks_of(pl, b);
-    launch_hash<T>(p, b, false, sms, s, &pl->sym_launches);
+    return p.seg_len > 0;
+  };
+  if (segment(kSegRcd)) launch_rcd<T>(p, false, sms, fork.next(), &pl->sym_launches);
+  if (segment(kSegWb)) launch_wb<T>(p, false, sms, fork.next(), &pl->sym_launches);
+  if (segment(kSegDense)) {
+    const cudaStream_t q = fork.next();
+    launch_dense_slices<T>(p, pl->slice_row, pl->slice_idx, pl->slice_first, sms, q, &pl->sym_launches);
+    launch_dense<T>(p, pl->dense_slices, false, sms, q, &pl->sym_launches);
   }
+  for (int b = kNumHashBins - 1; b >= 0; --b) {
+    p.hash_ranks = hash_ranks_of(pl, b);
+    if (segment(kSegHash0 + b)) launch_hash<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
+  }
+  for (int b = kNumBitmapBins - 1; b >= 0; --b) {
+    if (segment(kSegBitmap0 + b)) launch_bitmap<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
+  }
+  for (int b = kNumBmrBins - 1; b >= 0; --b) {
+    if (segment(kSegBmr0 + b)) launch_bmr<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
+  }
+  WS_CUDA(fork.join(), "joining the side streams");
   launch_scan(C->rowptr, m, pl->partials, pl->dsum, s, &pl->sym_launches);
   WS_CUDA(cudaGetLastError(), "symbolic launches");
   st = read_summary(pl, s);
@@ -479,60 +606,34 @@ ws_status_t numeric_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan
   const int sms = num_sms_of(C->device);
   pl->num_launches = 0;
   RowPlan<T> p = make_rowplan<T>(A, B, C, pl);
-  if (pl->seg_count[kSegDirect] > 0) {
-    p.seg_begin = pl->seg_offset[kSegDirect];
-    p.seg_len = pl->seg_count[kSegDirect];
-    launch_direct<T>(p, sms, s, &pl->num_launches);
-  }
-  if (pl->seg_count[kSegBmrWide] > 0) {
-    p.seg_begin = pl->seg_offset[kSegBmrWide];
-    p.seg_len = pl->seg_count[kSegBmrWide];
+  if (pl->seg_count[kSegRcd] > 0)
+    WS_CUDA(cudaMemsetAsync(pl->rcd_ctr + kRcdNextItem, 0, sizeof(int32_t), s), "cudaMemsetAsync(rcd work counter)");
+  Fork fork(s, C->device, bin_launches(pl, true));
+  auto segment = [&](int g) {
+    p.seg_begin = pl->seg_offset[g];
+    p.seg_len = pl->seg_count[g];
+    return p.seg_len > 0;
+  };
+  if (segment(kSegRcd)) launch_rcd<T>(p, true, sms, fork.next(), &pl->num_launches);
+  if (segment(kSegWb)) launch_wb<T>(p, true, sms, fork.next(), &pl->num_launches);
+  if (segment(kSegDense)) launch_dense<T>(p, pl->dense_slices, true, sms, fork.next(), &pl->num_launches);
+  if (segment(kSegBmrWide)) {
     if (pl->all_planned) p.perm = nullptr;  // rows in order, no permutation was built
-    launch_bmr<T>(p, kBmrPlannedBin, true, sms, s, &pl->num_launches);
+    launch_bmr<T>(p, kBmrPlannedBin, true, sms, fork.next(), &pl->num_launches);
     p.perm = pl->perm;
   }
-  if (pl->seg_count[kSegRcd] > 0) {
-    WS_CUDA(cudaMemsetAsync(pl->rcd_ctr + kRcdNextItem, 0, sizeof(int32_t), s), "cudaMemsetAsync(rcd work counter)");
-    p.rcd_ctr = pl->rcd_ctr;
-    p.rcd_items = pl->rcd_items;
-    p.rcd_bits = pl->rcd_bits;
-    p.rcd_words = pl->rcd_words;
-    p.seg_begin = pl->seg_offset[kSegRcd];
-    p.seg_len = pl->seg_count[kSegRcd];
-    launch_rcd<T>(p, true, sms, s, &pl->num_launches);
-  }
-  if (pl->seg_count[kSegWb] > 0) {
-    p.seg_begin = pl->seg_offset[kSegWb];
-    p.seg_len = pl->seg_count[kSegWb];
-    launch_wb<T>(p, true, sms, s, &pl->num_launches);
-  }
-  for (int b = 0; b < kNumBmrBins; ++b) {
-    const int g = kSegBmr0 + b;
-    if (pl->seg_count[g] == 0) continue;
-    p.seg_begin = pl->seg_offset[g];
-    p.seg_len = pl->seg_count[g];
-    launch_bmr<T>(p, b, true, sms, s, &pl->num_launches);
-  }
-  for (int b = 0; b < kNumBitmapBins; ++b) {
-    const int g = kSegBitmap0 + b;
-    if (pl->seg_count[g] == 0) continue;
-    p.seg_begin = pl->seg_offset[g];
-    p.seg_len = pl->seg_count[g];
-    launch_bitmap<T>(p, b, true, sms, s, &pl->num_launches);
-  }
-  for (int b = 0; b < kNumHashBins; ++b) {
-    const int g = kSegHash0 + b;
-    if (pl->seg_count[g] == 0) continue;
-    p.seg_begin = pl->seg_offset[g];
-    p.seg_len = pl->seg_count[g];
+  for (int b = kNumHashBins - 1; b >= 0; --b) {
     p.hash_ranks = hash_ranks_of(pl, b);
-    launch_hash<T>(p, b, true, sms, s, &pl->num_launches);
+    if (segment(kSegHash0 + b)) launch_hash<T>(p, b, true, sms, fork.next(), &pl->num_launches);
   }
-  if (pl->seg_count[kSegDense] > 0) {
-    p.seg_begin = pl->seg_offset[kSegDense];
-    p.seg_len = pl->seg_count[kSegDense];
-    launch_dense<T>(p, pl->dense_slices, true, sms, s, &pl->num_launches);
+  for (int b = kNumBitmapBins - 1; b >= 0; --b) {
+    if (segment(kSegBitmap0 + b)) launch_bitmap<T>(p, b, true, sms, fork.next(), &pl->num_launches);
   }
+  for (int b = kNumBmrBins - 1; b >= 0; --b) {
+    if (segment(kSegBmr0 + b)) launch_bmr<T>(p, b, true, sms, fork.next(), &pl->num_launches);
+  }
+  if (segment(kSegDirect)) launch_direct<T>(p, sms, fork.next(), &pl->num_launches);
+  WS_CUDA(fork.join(), "joining the side streams");
   WS_CUDA(cudaGetLastError(), "numeric launches");
   return WS_OK;
 }

@@ -616,6 +616,74 @@ def test_many_live_handles():
             np.testing.assert_array_equal(a, b)
 
 
+def _mixed_rows(seed):
+    """A product with rows of many classes: several kernels per pass."""
+    rng = np.random.default_rng(seed)
+    k, n = 3000, 70_000
+    B = uniform_csr(k, n, 40, rng, np.float64, "sym")
+    lens = [0, 1, 2, 3, 5, 9, 17, 33, 65, 100, 150, 400, 1000, 2000]
+    rows = {i: rng.choice(k, size=L, replace=False).tolist() for i, L in enumerate(lens * 6)}
+    A = _csr(len(lens) * 6, k, rows)
+    A.vals = 2 * rng.random(A.nnz) - 1
+    return A, B
+
+
+def test_products_on_threads_and_streams():
+    """Four threads, each with its own stream, handles and inputs, twenty
+    products each: the kernels of a pass spread over recycled side streams and
+    every product still sees its own order of work."""
+    import threading
+    from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+    cases = [_mixed_rows(s) for s in range(4)]
+    results, errors = [None] * 4, []
+
+    def work(i):
+        try:
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                dA, dB = DeviceCSR.from_host(cases[i][0]), DeviceCSR.from_host(cases[i][1])
+                with SpGEMM(dA, dB) as op:
+                    for _ in range(20):
+                        op.symbolic()
+                        C = op.numeric()
+                        op.wait()
+                        results[i] = C.to_host()
+        except Exception as e:  # reported by the main thread
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(4)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for (A, B), (rowptr, colidx, vals) in zip(cases, results):
+        assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
+def test_numeric_pass_under_capture():
+    """The numeric pass of a product with several row classes captured in a
+    graph and replayed with other values (captured work stays on the caller's
+    stream)."""
+    from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+    A, B = _mixed_rows(9)
+    dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+    with SpGEMM(dA, dB) as op:
+        op.symbolic()
+        C = op.numeric()
+        op.wait()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            op.numeric(out=C)
+        A.vals *= -0.5
+        dA.vals.copy_(torch.from_numpy(A.vals))
+        C.vals.zero_()
+        graph.replay()
+        op.wait()
+        rowptr, colidx, vals = C.to_host()
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
 def test_device_count_check_reports_error():
     """A row pointer altered between the passes is caught by the numeric pass's count check."""
     from paper_2606_20855_gb300 import _abi
