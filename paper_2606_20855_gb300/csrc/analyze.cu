@@ -209,7 +209,8 @@ __global__ void __launch_bounds__(256) analyze_kernel(const RowPlan<T> p, const 
 // the CTA reduces the product count and column range.
 template <typename T>
 __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, const AnalyzeParams ap,
-                                                           const int32_t* long_rows) {
+                                                           const int32_t* long_rows, DevSummary* host) {
+  __shared__ int s_last;
   __shared__ int s_seg[kNumSegs];
   __shared__ long long s_prod, s_slices;
   __shared__ int s_empty;
@@ -289,6 +290,16 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
   }
   __syncthreads();
   flush_counts(p, s_seg, &s_prod, &s_slices, &s_empty);
+  if (host) {  // the last CTA to get here copies the summary for the host
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(&p.sum->n_done, 1) == static_cast<int>(gridDim.x) - 1;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      publish_summary(p.sum, host, false);
+    }
+  }
 }
 
 struct SegOffsets {
@@ -380,9 +391,11 @@ int grid_for(int64_t work, int per_block, int num_sms, int blocks_per_sm) {
 
 template <typename T>
 void launch_analyze(const RowPlan<T>& p, const AnalyzeParams& ap, int32_t* long_rows, const int32_t* rows,
-                    int num_sms, cudaStream_t s, int* launches) {
+                    DevSummary* host, int num_sms, cudaStream_t s, int* launches) {
   analyze_kernel<T><<<grid_for(ap.m, 256, num_sms, 8), 256, 0, s>>>(p, ap, long_rows, rows);
-  analyze_long_kernel<T><<<num_sms * 8, 256, 0, s>>>(p, ap, long_rows);
+  // a warp per long row: A's entries bound their number (a full grid of CTAs
+  // without work takes 7 us)
+  analyze_long_kernel<T><<<grid_for(ap.nnz / (ap.long_threshold + 1), 8, num_sms, 8), 256, 0, s>>>(p, ap, long_rows, host);
   *launches += 2;
 }
 
@@ -409,8 +422,8 @@ void launch_validate(const int64_t* rowptr, const int32_t* colidx, int64_t nrows
 }
 
 #define WS_INST(T)                                                                                          \
-  template void launch_analyze<T>(const RowPlan<T>&, const AnalyzeParams&, int32_t*, const int32_t*, int,      \
-                                  cudaStream_t, int*);                                                       \
+  template void launch_analyze<T>(const RowPlan<T>&, const AnalyzeParams&, int32_t*, const int32_t*,           \
+                                  DevSummary*, int, cudaStream_t, int*);                                                       \
   template void launch_scatter<T>(const RowPlan<T>&, int64_t, const int64_t*, int, cudaStream_t, int*);      \
   template void launch_dense_slices<T>(const RowPlan<T>&, int32_t*, int32_t*, int32_t*, int, cudaStream_t, int*);
 WS_INST(float)

@@ -2,11 +2,11 @@
 //
 // Symbolic pass (ws_spgemm_symbolic), all on the caller's stream:
 //   1. analyze   per-row product count, column range, class       (2 launches)
-//   -- read the class counts back (one small copy + stream sync)
+//   -- the class counts reach the host (written by the last kernel, stream sync)
 //   2. scatter   group rows by class                                (1 launch)
 //   3. dense     expand dense-window rows into column slices, count (2 launches)
 //   4. hash      count distinct columns per hash bin                (1 launch per non-empty bin)
-//   5. scan      counts -> C.rowptr                                 (3 launches)
+//   5. scan      counts -> C.rowptr                                 (1 or 2 launches)
 //   -- read nnz(C) and the status word back (one small copy + stream sync)
 // Numeric pass (ws_spgemm_numeric): one launch per non-empty class, no sync.
 #include <cstdarg>
@@ -66,6 +66,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 struct DevBuf {
   void* ptr = nullptr;
   size_t bytes = 0;
+  uint64_t gen = 0;  // changes with every allocation (0: none yet)
   ws_status_t reserve(size_t need, cudaStream_t s) {
     if (need <= bytes) return WS_OK;
     if (ptr) {
@@ -81,6 +82,7 @@ struct DevBuf {
       return fail(WS_ERR_ALLOC, "cudaMallocAsync(%zu bytes): %s", want, cudaGetErrorString(e));
     }
     bytes = want;
+    ++gen;
     return WS_OK;
   }
   // Returns the memory to the stream-ordered pool (callers synchronise the
@@ -97,23 +99,24 @@ struct DevBuf {
 // product.  Blocks are allocated 64 at a time and kept until the process
 // exits.
 std::mutex g_host_sum_mutex;
-std::vector<DevSummary*> g_host_sum_free;
+std::vector<HostSummary*> g_host_sum_free;
 
-DevSummary* acquire_host_sum() {
+HostSummary* acquire_host_sum() {
   std::lock_guard<std::mutex> lock(g_host_sum_mutex);
   if (g_host_sum_free.empty()) {
     constexpr int kBlocks = 64;
-    const size_t each = (sizeof(DevSummary) + 255) / 256 * 256;
+    const size_t each = (sizeof(HostSummary) + 255) / 256 * 256;
     char* base = nullptr;
     if (cudaMallocHost(reinterpret_cast<void**>(&base), each * kBlocks) != cudaSuccess) return nullptr;
-    for (int i = kBlocks - 1; i >= 0; --i) g_host_sum_free.push_back(reinterpret_cast<DevSummary*>(base + i * each));
+    for (int i = kBlocks - 1; i >= 0; --i) g_host_sum_free.push_back(reinterpret_cast<HostSummary*>(base + i * each));
   }
-  DevSummary* h = g_host_sum_free.back();
+  HostSummary* h = g_host_sum_free.back();
   g_host_sum_free.pop_back();
+  h->slot[0] = h->slot[1] = 0;
   return h;
 }
 
-void release_host_sum(DevSummary* h) {
+void release_host_sum(HostSummary* h) {
   if (!h) return;
   std::lock_guard<std::mutex> lock(g_host_sum_mutex);
   g_host_sum_free.push_back(h);
@@ -291,7 +294,10 @@ struct Plan {
   int rcd_words = 0;
   // submatrix plan (kPlanSub): the block the symbolic pass counted
   int64_t sub_r0 = 0, sub_r1 = 0, sub_c0 = 0, sub_c1 = 0;
-  DevSummary* host_sum = nullptr;  // pinned
+  HostSummary* host_sum = nullptr;  // pinned
+  int slot = 0;                     // status word of the current pass in it
+  const DevBuf* clean_buf = nullptr;  // buffer whose summary block the last pass left cleared,
+  uint64_t clean_gen = 0;             // in this allocation of it
   // carved pointers
   DevSummary* dsum = nullptr;
   int32_t* perm = nullptr;
@@ -355,16 +361,36 @@ int log2_group_for(const ws_csr_s* B) {
   return 5;
 }
 
-ws_status_t read_summary(Plan* pl, cudaStream_t s) {
-  WS_CUDA(cudaMemcpyAsync(pl->host_sum, pl->dsum, sizeof(DevSummary), cudaMemcpyDeviceToHost, s),
-          "cudaMemcpyAsync(summary)");
+// Start of a symbolic pass whose summary block heads `buf`: a fresh status
+// word, and the block cleared unless the last pass left it so.
+ws_status_t begin_pass(Plan* pl, const DevBuf& buf, cudaStream_t s) {
+  pl->slot ^= 1;
+  pl->host_sum->slot[pl->slot] = 0;
+  const bool clean = pl->clean_buf == &buf && pl->clean_gen == buf.gen;
+  pl->clean_buf = nullptr;
+  if (!clean) WS_CUDA(cudaMemsetAsync(pl->dsum, 0, sizeof(DevSummary), s), "cudaMemsetAsync(summary)");
+  return WS_OK;
+}
+
+// The pass ended with a scan that cleared the block.
+void end_pass(Plan* pl, const DevBuf& buf) {
+  pl->clean_buf = &buf;
+  pl->clean_gen = buf.gen;
+}
+
+int* status_word(const Plan* pl) { return &pl->host_sum->slot[pl->slot]; }
+
+// Waits for a summary that the stream's last kernels publish.
+ws_status_t wait_summary(cudaStream_t s) {
   WS_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
   return WS_OK;
 }
 
-ws_status_t device_status(const DevSummary& hs) {
-  if (hs.status == 0) return WS_OK;
-  return fail(WS_ERR_DEVICE, "device status 0x%x (count=%d)", hs.status, !!(hs.status & kErrCount));
+// Status of the plan's current pass, whose queued work has completed.
+ws_status_t device_status(const Plan* pl) {
+  const int st = *static_cast<volatile const int*>(status_word(pl));
+  if (st == 0) return WS_OK;
+  return fail(WS_ERR_DEVICE, "device status 0x%x (count=%d)", st, !!(st & kErrCount));
 }
 
 template <typename T>
@@ -389,6 +415,7 @@ RowPlan<T> make_rowplan(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan*
   p.rcd_bits = pl->rcd_bits;
   p.rcd_words = pl->rcd_words;
   p.sum = pl->dsum;
+  p.status = status_word(pl);
   p.log2_group = pl->log2_group;
   p.run_limit = pl->run_limit;
   p.dense_width = pl->dense_width;
@@ -521,11 +548,9 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     if (segment(kSegBmr0 + b)) launch_bmr<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
   }
   WS_CUDA(fork.join(), "joining the side streams");
-  launch_scan(C->rowptr, m, pl->partials, pl->dsum, s, &pl->sym_launches);
+  launch_scan(C->rowptr, m, pl->partials, pl->dsum, s, &pl->sym_launches, nullptr, pl->host_sum);
   WS_CUDA(cudaGetLastError(), "symbolic launches");
-  st = read_summary(pl, s);
-  if (st != WS_OK) return st;
-  return WS_OK;
+  return wait_summary(s);
 }
 
 template <typename T>
@@ -544,13 +569,16 @@ ws_status_t symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
 
   ws_status_t st = carve_rows(pl, m, s);
   if (st != WS_OK) return st;
-  WS_CUDA(cudaMemsetAsync(pl->dsum, 0, sizeof(DevSummary), s), "cudaMemsetAsync(summary)");
-  WS_CUDA(cudaMemsetAsync(C->rowptr, 0, sizeof(int64_t), s), "cudaMemsetAsync(rowptr[0])");
+  st = begin_pass(pl, pl->rows, s);
+  if (st != WS_OK) return st;
 
   RowPlan<T> p = make_rowplan<T>(A, B, C, pl);
-  if (m > 0) {
+  if (m == 0) {
+    WS_CUDA(cudaMemsetAsync(C->rowptr, 0, sizeof(int64_t), s), "cudaMemsetAsync(rowptr[0])");
+    static_cast<DevSummary&>(*pl->host_sum) = DevSummary{};
+  } else {
     AnalyzeParams ap{m,           g_hash_max, g_bitmap_span,   1 << pl->log2_group, g_bmr_max_a,
-                     g_rcd_max_a, g_wb_span,  pl->dense_width, kLongRowThreshold};
+                     g_rcd_max_a, g_wb_span,  pl->dense_width, kLongRowThreshold,   A->nnz};
     // When every row of C fits the widest register bitmap (B has at most
     // 65,536 columns), the planning pass counts the eligible rows in its first
     // read of A and only the remaining rows go through the analysis kernel.
@@ -560,16 +588,16 @@ ws_status_t symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
       if (st != WS_OK) return st;
       p.ranks = static_cast<uint16_t*>(pl->ranks.ptr);
       launch_bmr_plan<T>(p, ap, B->ncols, pl->pending, sms, s, &pl->sym_launches);
-      launch_analyze<T>(p, ap, pl->long_rows, pl->pending, sms, s, &pl->sym_launches);
+      launch_analyze<T>(p, ap, pl->long_rows, pl->pending, nullptr, sms, s, &pl->sym_launches);
       // If the planning pass took every row, all counts are in place now: a
       // scan queued here (a no-op otherwise) saves the second read-back.
-      launch_scan(C->rowptr, m, pl->partials, pl->dsum, s, &pl->sym_launches, &pl->dsum->n_pending);
+      launch_scan(C->rowptr, m, pl->partials, pl->dsum, s, &pl->sym_launches, &pl->dsum->n_pending, pl->host_sum);
     } else {
-      launch_analyze<T>(p, ap, pl->long_rows, nullptr, sms, s, &pl->sym_launches);
+      launch_analyze<T>(p, ap, pl->long_rows, nullptr, pl->host_sum, sms, s, &pl->sym_launches);
     }
     WS_CUDA(cudaGetLastError(), "analyze launch");
   }
-  st = read_summary(pl, s);
+  st = wait_summary(s);
   if (st != WS_OK) return st;
   const DevSummary& hs = *pl->host_sum;
   int64_t off = 0;
@@ -584,11 +612,12 @@ ws_status_t symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
   pl->dense_slices = hs.dense_slices;
   if (pl->dense_slices > INT32_MAX) return fail(WS_ERR_OVERFLOW, "too many dense-window slices (%lld)", (long long)pl->dense_slices);
   pl->all_planned = m > 0 && hs.n_pending == 0 && pl->seg_count[kSegBmrWide] == m;
-  if (!pl->all_planned) {
+  if (m > 0 && !pl->all_planned) {
     st = symbolic_bins<T>(A, B, C, pl, p, off, sms, s);
     if (st != WS_OK) return st;
   }
-  st = device_status(*pl->host_sum);
+  if (m > 0) end_pass(pl, pl->rows);
+  st = device_status(pl);
   if (st != WS_OK) return st;
   pl->n_sort = pl->host_sum->n_sort;
   C->nnz = m > 0 ? pl->host_sum->nnz : 0;
@@ -689,6 +718,8 @@ EwisePlan<T> make_ewise(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, const
   p.nc_max = pl->ew_nc_max;
   p.partials = pl->ew_partials;
   p.sum = pl->dsum;
+  p.status = status_word(pl);
+  p.host = pl->host_sum;
   p.diag = pl->ew_diag;
   p.group = pl->ew_group;
   p.op = pl->ew_op;
@@ -717,17 +748,18 @@ ws_status_t ewise_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
   pl->ew_nc_max = m + merged / pl->ew_diag + 1;  // row i has at most 1 + len_i / diag chunks
   ws_status_t st = carve_ewise(pl, m, pl->ew_nc_max, s);
   if (st != WS_OK) return st;
-  WS_CUDA(cudaMemsetAsync(pl->dsum, 0, sizeof(DevSummary), s), "cudaMemsetAsync(summary)");
-  WS_CUDA(cudaMemsetAsync(C->rowptr, 0, sizeof(int64_t), s), "cudaMemsetAsync(rowptr[0])");
-  WS_CUDA(cudaMemsetAsync(pl->ew_chunk_begin, 0, sizeof(int64_t), s), "cudaMemsetAsync(chunk_begin[0])");
-  WS_CUDA(cudaMemsetAsync(pl->ew_chunk_off, 0, sizeof(int64_t), s), "cudaMemsetAsync(chunk_off[0])");
+  st = begin_pass(pl, pl->ew, s);
+  if (st != WS_OK) return st;
   if (m > 0) {
     launch_ewise_symbolic<T>(make_ewise<T>(A, B, C, pl), num_sms_of(C->device), s, &pl->sym_launches);
     WS_CUDA(cudaGetLastError(), "elementwise symbolic launches");
+  } else {
+    WS_CUDA(cudaMemsetAsync(C->rowptr, 0, sizeof(int64_t), s), "cudaMemsetAsync(rowptr[0])");
   }
-  st = read_summary(pl, s);
+  st = wait_summary(s);
   if (st != WS_OK) return st;
-  st = device_status(*pl->host_sum);
+  if (m > 0) end_pass(pl, pl->ew);
+  st = device_status(pl);
   if (st != WS_OK) return st;
   C->nnz = m > 0 ? pl->host_sum->nnz : 0;
   pl->products = merged;
@@ -794,19 +826,21 @@ ws_status_t spmspv_impl(ws_csr_s* At, int64_t nx, const int32_t* x_idx, const vo
   p.y_vals = static_cast<T*>(y_vals);
   p.cap = m;
   pl->dsum = p.sum;
+  pl->slot ^= 1;
+  pl->host_sum->slot[pl->slot] = 0;
+  p.status = status_word(pl);
+  p.host = pl->host_sum;
   pl->sym_launches = 0;
   pl->num_launches = 0;
-  // zero the summary, the accumulator and the byte-map (contiguous), and the scan heads
+  // zero the summary, the accumulator and the byte-map (contiguous)
   WS_CUDA(cudaMemsetAsync(b, 0, o_off, s), "cudaMemsetAsync(spmspv scratch)");
-  WS_CUDA(cudaMemsetAsync(p.off, 0, sizeof(int64_t), s), "cudaMemsetAsync(off[0])");
-  WS_CUDA(cudaMemsetAsync(p.cnt, 0, sizeof(int64_t), s), "cudaMemsetAsync(cnt[0])");
   if (m > 0) {
     launch_spmspv<T>(p, num_sms_of(At->device), s, &pl->num_launches);
     WS_CUDA(cudaGetLastError(), "spmspv launches");
   }
-  st = read_summary(pl, s);
+  st = wait_summary(s);
   if (st != WS_OK) return st;
-  st = device_status(*pl->host_sum);
+  st = device_status(pl);
   if (st != WS_OK) return st;
   *nnz_y = m > 0 ? pl->host_sum->nnz : 0;
   return WS_OK;
@@ -936,10 +970,9 @@ ws_status_t owned_entries(Owned* o, int64_t cap, cudaStream_t s) {
   return WS_OK;
 }
 
-// Device status word of a plan whose queued work has completed.
+// Status of a partial product or merge whose queued work has completed.
 ws_status_t plan_status(const Plan* pl) {
-  int st = 0;
-  WS_CUDA(cudaMemcpy(&st, &pl->dsum->status, sizeof(int), cudaMemcpyDeviceToHost), "cudaMemcpy(status)");
+  const int st = *static_cast<volatile const int*>(status_word(pl));
   if (st != 0) return fail(WS_ERR_DEVICE, "device status 0x%x in an outer-product step", st);
   return WS_OK;
 }
@@ -988,17 +1021,16 @@ ws_status_t outer_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
   }
   DevSummary* ex_sum = static_cast<DevSummary*>(ex_mem);
   int64_t* ex_part = reinterpret_cast<int64_t*>(static_cast<char*>(ex_mem) + o_part);
-  if (cudaMemsetAsync(ex_sum, 0, sizeof(DevSummary), s) != cudaSuccess ||
-      (st = new_owned(m, 1, A->dtype, C->device, s, &ab)) != WS_OK || (st = owned_entries(ab, A->nnz, s)) != WS_OK) {
+  if ((st = new_owned(m, 1, A->dtype, C->device, s, &ab)) != WS_OK || (st = owned_entries(ab, A->nnz, s)) != WS_OK) {
     cleanup();
-    return st != WS_OK ? st : fail(WS_ERR_CUDA, "cudaMemsetAsync(extraction summary)");
+    return st;
   }
   ab->h.nnz = A->nnz;  // capacity: the block's own count stays on the device
   for (int p = 0; p < P && st == WS_OK; ++p) {
     const int64_t k0 = K * p / P, k1 = K * (p + 1) / P;
     // A[:, k0:k1], columns shifted by -k0
     ab->h.ncols = k1 - k0;
-    if (cudaMemsetAsync(ab->h.rowptr, 0, sizeof(int64_t), s) != cudaSuccess) {
+    if (m == 0 && cudaMemsetAsync(ab->h.rowptr, 0, sizeof(int64_t), s) != cudaSuccess) {
       st = fail(WS_ERR_CUDA, "cudaMemsetAsync(block row pointer)");
       break;
     }
@@ -1006,7 +1038,7 @@ ws_status_t outer_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
       launch_submatrix_count(A->rowptr, A->colidx, 0, m, k0, k1, ab->h.rowptr, sms, s, &launches);
       launch_scan(ab->h.rowptr, m, ex_part, ex_sum, s, &launches);
       launch_submatrix_copy<T>(A->rowptr, A->colidx, static_cast<const T*>(A->vals), 0, m, k0, ab->h.rowptr,
-                               ab->h.colidx, static_cast<T*>(ab->h.vals), ex_sum, sms, s, &launches);
+                               ab->h.colidx, static_cast<T*>(ab->h.vals), status_word(ab->h.plan), sms, s, &launches);
     }
     // B[k0:k1, :]: a view of B's rows (positions stay absolute in B's arrays)
     ws_csr_s bp = *B;
@@ -1025,13 +1057,8 @@ ws_status_t outer_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
     if ((st = numeric_impl<T>(&ab->h, &bp, &cp->h, cp->h.plan, s)) != WS_OK) break;
     launches += cp->h.plan->sym_launches + cp->h.plan->num_launches;
   }
-  if (st == WS_OK) {  // every extraction has completed (each block's structure pass synchronised)
-    int ex_status = 0;
-    if (cudaMemcpy(&ex_status, &ex_sum->status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess)
-      st = fail(WS_ERR_CUDA, "cudaMemcpy(extraction status)");
-    else if (ex_status != 0)
-      st = fail(WS_ERR_DEVICE, "device status 0x%x in a column-block extraction", ex_status);
-  }
+  // every extraction has completed (each block's structure pass synchronised)
+  if (st == WS_OK) st = plan_status(ab->h.plan);
   release_owned(ab, s);
   ab = nullptr;
   // merge levels: pairwise sparse additions until two copies are left
@@ -1333,16 +1360,17 @@ ws_status_t ws_csr_submatrix_symbolic(ws_csr_t A, int64_t r0, int64_t r1, int64_
   pl->sym_launches = 0;
   pl->num_launches = 0;
   S->nnz = -1;
-  WS_CUDA(cudaMemsetAsync(pl->dsum, 0, sizeof(DevSummary), s), "cudaMemsetAsync(summary)");
-  WS_CUDA(cudaMemsetAsync(S->rowptr, 0, sizeof(int64_t), s), "cudaMemsetAsync(rowptr[0])");
-  if (rows > 0) {
+  if ((st = begin_pass(pl, pl->ew, s)) != WS_OK) return st;
+  if (rows == 0) {
+    WS_CUDA(cudaMemsetAsync(S->rowptr, 0, sizeof(int64_t), s), "cudaMemsetAsync(rowptr[0])");
+  } else {
     const int sms = num_sms_of(S->device);
     launch_submatrix_count(A->rowptr, A->colidx, r0, rows, c0, c1, S->rowptr, sms, s, &pl->sym_launches);
-    launch_scan(S->rowptr, rows, partials, pl->dsum, s, &pl->sym_launches);
+    launch_scan(S->rowptr, rows, partials, pl->dsum, s, &pl->sym_launches, nullptr, pl->host_sum);
     WS_CUDA(cudaGetLastError(), "submatrix symbolic launches");
   }
-  st = read_summary(pl, s);
-  if (st != WS_OK) return st;
+  if ((st = wait_summary(s)) != WS_OK) return st;
+  if (rows > 0) end_pass(pl, pl->ew);
   S->nnz = rows > 0 ? pl->host_sum->nnz : 0;
   pl->A = A;
   pl->B = nullptr;
@@ -1375,11 +1403,11 @@ ws_status_t ws_csr_submatrix_numeric(ws_csr_t A, ws_csr_t S, int32_t* s_colidx, 
   const int64_t rows = pl->sub_r1 - pl->sub_r0;
   if (A->dtype == WS_F64) {
     launch_submatrix_copy<double>(A->rowptr, A->colidx, static_cast<const double*>(A->vals), pl->sub_r0, rows,
-                                  pl->sub_c0, S->rowptr, s_colidx, static_cast<double*>(s_vals), pl->dsum, sms, s,
+                                  pl->sub_c0, S->rowptr, s_colidx, static_cast<double*>(s_vals), status_word(pl), sms, s,
                                   &pl->num_launches);
   } else {
     launch_submatrix_copy<float>(A->rowptr, A->colidx, static_cast<const float*>(A->vals), pl->sub_r0, rows,
-                                 pl->sub_c0, S->rowptr, s_colidx, static_cast<float*>(s_vals), pl->dsum, sms, s,
+                                 pl->sub_c0, S->rowptr, s_colidx, static_cast<float*>(s_vals), status_word(pl), sms, s,
                                  &pl->num_launches);
   }
   WS_CUDA(cudaGetLastError(), "submatrix numeric launch");
@@ -1391,13 +1419,9 @@ ws_status_t ws_spgemm_wait(ws_csr_t C, ws_stream_t stream) {
   if (!C) return fail(WS_ERR_INVALID_ARG, "C is NULL");
   Plan* pl = C->plan;
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-  if (!pl || !pl->host_sum || !pl->dsum) {
-    WS_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
-    return WS_OK;
-  }
-  ws_status_t st = read_summary(pl, s);
-  if (st != WS_OK) return st;
-  return device_status(*pl->host_sum);
+  WS_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
+  if (!pl || !pl->host_sum || !pl->dsum) return WS_OK;
+  return device_status(pl);
 }
 
 ws_status_t ws_csr_destroy(ws_csr_t h) {

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(32 * WPR * RPC, 1024 / (32 * WPR * RPC))
       cbase = p.c_rowptr[row];
       const int64_t want = p.c_rowptr[row + 1] - cbase;
       cnt = want < CAP ? want : CAP;  // the staging array bounds every access
-      if (t == 0 && want > CAP) atomicOr(&p.sum->status, kErrCount);
+      if (t == 0 && want > CAP) atomicOr(p.status, kErrCount);
     }
     // Clear the workspace.
     for (int s = t; s < S::kPhysChunks; s += kNT) bm4[s] = make_uint4(0u, 0u, 0u, 0u);
@@ -145,7 +145,7 @@ __global__ void __launch_bounds__(32 * WPR * RPC, 1024 / (32 * WPR * RPC))
           base[t] = static_cast<int>(block_exclusive_scan(static_cast<long long>(run), s_scan, &tot));
           total = static_cast<int>(tot);
         }
-        if (t == 0 && total != cnt) atomicOr(&p.sum->status, kErrCount);
+        if (t == 0 && total != cnt) atomicOr(p.status, kErrCount);
       }
       team_sync<WPR>();
       for (int64_t cb = ra; cb < re; cb += kNT) {

@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, sizeof(T) == 8 ? 5 : 7) bmr_
       const long long cbase = h_cbase[i];
       const long long want = h_cnt[i];
       const int cnt = static_cast<int>(want < kCap ? want : kCap);  // staging bounds every access
-      if (lane == 0 && want > kCap) atomicOr(&p.sum->status, kErrCount);
+      if (lane == 0 && want > kCap) atomicOr(p.status, kErrCount);
       int* out_key = p.c_colidx + cbase;
       T* out_val = p.c_vals + cbase;
       const int pk = static_cast<int>((reinterpret_cast<uintptr_t>(out_key) >> 2) & 3);
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, sizeof(T) == 8 ? 5 : 7) bmr_
               }
             }
           }
-          if (__any_sync(kFull, bad) && lane == 0) atomicOr(&p.sum->status, kErrCount);
+          if (__any_sync(kFull, bad) && lane == 0) atomicOr(p.status, kErrCount);
         }
       };
       if (h_full[i]) {
@@ -777,7 +777,7 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, 6) bmr_group_numeric_kernel(
         }
       }
     }
-    if (__any_sync(kFull, bad) && lane == 0) atomicOr(&p.sum->status, kErrCount);
+    if (__any_sync(kFull, bad) && lane == 0) atomicOr(p.status, kErrCount);
     __syncwarp();
     for (int s2 = gl; s2 < cnt; s2 += G) {
       p.c_colidx[cbase + s2] = st_key[s2];
@@ -974,7 +974,7 @@ __global__ void __launch_bounds__(kPlanThreads, 16) bmr_plan_kernel(const RowPla
           col[st] = (kFullRow || gl < static_cast<int>(h >> kLenShift)) ? p.B.colidx[(h & kPosMask) + gl] : -1;
         }
         if (clr_pending) {  // the previous row's clear is complete
-        if (!mbar_wait(&s_mbar, mphase) && t == 0) atomicOr(&p.sum->status, kErrCount);
+        if (!mbar_wait(&s_mbar, mphase) && t == 0) atomicOr(p.status, kErrCount);
         mphase ^= 1u;
         clr_pending = false;
       }
@@ -1075,7 +1075,7 @@ __global__ void __launch_bounds__(kPlanThreads, 16) bmr_plan_kernel(const RowPla
       prod += static_cast<unsigned long long>(hr.y);
     }
   }
-  if (clr_pending && !mbar_wait(&s_mbar, mphase) && t == 0) atomicOr(&p.sum->status, kErrCount);
+  if (clr_pending && !mbar_wait(&s_mbar, mphase) && t == 0) atomicOr(p.status, kErrCount);
   if (t == 0) {
     if (taken) atomicAdd(&p.sum->seg_count[kSegBmrWide], taken);
     if (prod) atomicAdd(reinterpret_cast<unsigned long long*>(&p.sum->products), prod);

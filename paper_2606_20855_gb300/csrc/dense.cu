@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(kDenseThreads) dense_rows_kernel(const RowPlan
         emitted_total += round_total;
       }
       if (emitted_total != expect) bad = true;
-      if (bad) atomicOr(&p.sum->status, kErrCount);
+      if (bad) atomicOr(p.status, kErrCount);
     }
     __syncthreads();
   }

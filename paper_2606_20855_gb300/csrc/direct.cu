@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(256) direct_rows_kernel(const RowPlan<T> p) {
       len = p.B.rowptr[k + 1] - qb;
       base = p.c_rowptr[row];
       if (len != p.c_rowptr[row + 1] - base) {
-        if (gl == 0) atomicOr(&p.sum->status, kErrCount);
+        if (gl == 0) atomicOr(p.status, kErrCount);
         len = 0;
       }
     }

@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kEwThreads, FILL ? 4 : 6) ew_merge_seq_kernel(
       p.chunk_off[c + 1] = merge_seq<T, OP, false>(a + i0, nullptr, i1 - i0, b + j0, nullptr, j1 - j0, nullptr, &bad);
     }
   }
-  if (bad) atomicOr(&p.sum->status, kErrCount);
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 // Warp-staged tiles: a warp takes 32 consecutive chunks, one per lane.  The
@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(32 * kTileWarps) ew_tile_kernel(const EwisePla
     }
     __syncwarp();  // the next tile rewrites the staging
   }
-  if (bad) atomicOr(&p.sum->status, kErrCount);
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 __global__ void __launch_bounds__(kEwThreads) ew_chunks_per_row_kernel(int64_t m, const int64_t* arp,
@@ -581,7 +581,7 @@ __global__ void __launch_bounds__(kEwThreads, FILL ? 4 : 6) ew_merge_kernel(cons
       if (gl == 0) p.chunk_off[c + 1] = n;
     }
   }
-  if (bad) atomicOr(&p.sum->status, kErrCount);
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 // A warp per chunk, chunks taken 32 at a time (kEwiseRankChunk merged
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(kEwThreads) ew_rank_kernel(const EwisePlan<T> 
       __syncwarp();  // the staged parts are overwritten by the next chunk
     }
   }
-  if (bad) atomicOr(&p.sum->status, kErrCount);
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 // C.rowptr[i] = output offset of the first chunk of row i (i = 0..m; the
@@ -849,7 +849,7 @@ void launch_ewise_symbolic(const EwisePlan<T>& p, int num_sms, cudaStream_t s, i
   } else {
     launch_merge_g<T, kEwiseMul, false>(p, num_sms, s);
   }
-  launch_scan(p.chunk_off, p.nc_max, p.partials, p.sum, s, launches);
+  launch_scan(p.chunk_off, p.nc_max, p.partials, p.sum, s, launches, nullptr, p.host);
   ew_rowptr_kernel<<<grid_for(p.m + 1, kEwThreads, num_sms, 8), kEwThreads, 0, s>>>(p.m, p.chunk_begin, p.chunk_off,
                                                                                     p.c_rowptr);
   *launches += 4;

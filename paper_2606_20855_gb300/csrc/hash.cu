@@ -570,7 +570,7 @@ __global__ void __launch_bounds__(32 * W * RPC, NUMERIC ? (sizeof(T) == 8 ? 640 
       }
     }
   }
-  if (bad) atomicOr(&p.sum->status, kErrCount);
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 template <typename T, int LOGC, int W, int RPC, bool NUMERIC, bool RANKED>

@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
 #pragma unroll 4
     for (int i = tid; i < n_out; i += kNumThreads) p.c_vals[cbase + i] = s.win[i];
   }
-  if (bad) atomicOr(&p.sum->status, kErrCount);
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 // ----------------------------------------------------------------- wide rows
@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(kWbThreads, 1) wb_kernel(const RowPlan<T> p) {
         }
         }
       }
-      if (bad) atomicOr(&p.sum->status, kErrCount);
+      if (bad) atomicOr(p.status, kErrCount);
       __syncthreads();
       for (int i = threadIdx.x; i < nchunks; i += kWbThreads) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
       __syncthreads();

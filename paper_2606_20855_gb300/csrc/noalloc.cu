@@ -75,7 +75,7 @@ ws_status_t ws_rowptr_scan_static(int64_t* rowptr, int64_t nrows, ws_stream_t st
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   // Nothing in the scratch has to start at zero: the scan writes every tile
   // partial it reads, and the summary block is written, never read.
-  if (cudaMemsetAsync(rowptr, 0, sizeof(int64_t), s) != cudaSuccess) return WS_ERR_CUDA;
+  if (nrows == 0 && cudaMemsetAsync(rowptr, 0, sizeof(int64_t), s) != cudaSuccess) return WS_ERR_CUDA;
   int launches = 0;
   DevSummary* sum = reinterpret_cast<DevSummary*>(scratch + kStaticScanTiles);
   launch_scan(rowptr, nrows, scratch, sum, s, &launches);

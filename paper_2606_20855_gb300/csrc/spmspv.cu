@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_offsets_kernel(const SpmspvPlan
       first = p.At.rowptr[j];
       len = p.At.rowptr[j + 1] - first;
     } else {
-      atomicOr(&p.sum->status, kErrCount);  // index outside A's columns: skipped
+      atomicOr(p.status, kErrCount);  // index outside A's columns: skipped
     }
     p.off[k + 1] = len;
     p.first[k] = first;
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_scatter_kernel(const SpmspvPlan
       p.mark[i] = 1;
     }
   }
-  if (bad) atomicOr(&p.sum->status, kErrCount);
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 // Marked positions of every compaction tile: cnt[t + 1].  One thread reads 16
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_write_kernel(const SpmspvPlan<T
           p.y_idx[at] = static_cast<int32_t>(i);
           p.y_vals[at] = p.acc[i];
         } else {
-          atomicOr(&p.sum->status, kErrCount);
+          atomicOr(p.status, kErrCount);
         }
       }
       pos += __popc(bal);
@@ -271,7 +271,7 @@ void launch_spmspv(const SpmspvPlan<T>& p, int num_sms, cudaStream_t s, int* lau
   }
   const int64_t tiles = spmspv_tiles(p.m);
   sv_tile_count_kernel<<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p.mark, p.m, p.cnt);
-  launch_scan(p.cnt, tiles, p.partials, p.sum, s, launches);
+  launch_scan(p.cnt, tiles, p.partials, p.sum, s, launches, nullptr, p.host);
   sv_write_kernel<T><<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p);
   *launches += 2;
 }

@@ -45,7 +45,7 @@ template <typename T>
 __global__ void __launch_bounds__(kSubThreads) sub_copy_kernel(const int64_t* rowptr, const int32_t* colidx,
                                                                const T* vals, int64_t r0, int64_t rows, int64_t c0,
                                                                const int64_t* s_rowptr, int32_t* s_colidx, T* s_vals,
-                                                               DevSummary* sum) {
+                                                               int* status) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(kSubThreads) sub_copy_kernel(const int64_t* ro
     }
     const int64_t o0 = s_rowptr[r], len = s_rowptr[r + 1] - o0;
     if (lo + len > n) {  // inconsistent with the count pass (input changed in between)
-      if (lane == 0) atomicOr(&sum->status, kErrCount);
+      if (lane == 0) atomicOr(status, kErrCount);
       continue;
     }
     for (int64_t e = lane; e < len; e += 32) {
@@ -91,16 +91,16 @@ void launch_submatrix_count(const int64_t* rowptr, const int32_t* colidx, int64_
 
 template <typename T>
 void launch_submatrix_copy(const int64_t* rowptr, const int32_t* colidx, const T* vals, int64_t r0, int64_t rows,
-                           int64_t c0, const int64_t* s_rowptr, int32_t* s_colidx, T* s_vals, DevSummary* sum,
+                           int64_t c0, const int64_t* s_rowptr, int32_t* s_colidx, T* s_vals, int* status,
                            int num_sms, cudaStream_t s, int* launches) {
   sub_copy_kernel<T><<<grid_for(rows * 32, kSubThreads, num_sms, 8), kSubThreads, 0, s>>>(
-      rowptr, colidx, vals, r0, rows, c0, s_rowptr, s_colidx, s_vals, sum);
+      rowptr, colidx, vals, r0, rows, c0, s_rowptr, s_colidx, s_vals, status);
   *launches += 1;
 }
 
 template void launch_submatrix_copy<float>(const int64_t*, const int32_t*, const float*, int64_t, int64_t, int64_t,
-                                           const int64_t*, int32_t*, float*, DevSummary*, int, cudaStream_t, int*);
+                                           const int64_t*, int32_t*, float*, int*, int, cudaStream_t, int*);
 template void launch_submatrix_copy<double>(const int64_t*, const int32_t*, const double*, int64_t, int64_t, int64_t,
-                                            const int64_t*, int32_t*, double*, DevSummary*, int, cudaStream_t, int*);
+                                            const int64_t*, int32_t*, double*, int*, int, cudaStream_t, int*);
 
 }  // namespace wsk

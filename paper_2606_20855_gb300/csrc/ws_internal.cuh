@@ -108,7 +108,8 @@ struct DevSummary {
   long long products;  // sum of ub_i
   long long dense_slices;
   long long slice_cursor;
-  int status;
+  int status;   // validation only; the passes use the status word of their plan
+  int n_done;   // CTAs of analyze_long_kernel that have added their counts
   int n_sort;  // hash rows ranked by a sort
   int n_long;   // rows analysed by a CTA each (queued from the back of the long-row list)
   int n_mid;    // rows analysed by a warp each (queued from the front)
@@ -118,6 +119,25 @@ struct DevSummary {
   int seg_count[kNumSegs];
   int seg_cursor[kNumSegs];
 };
+
+// Pinned host side of a plan: the copy of the summary, and two status words
+// that kernels write errors to directly.  Passes of one handle alternate
+// between the words, so a late error of an earlier pass cannot mark the next.
+struct HostSummary : DevSummary {
+  int slot[2];
+};
+
+// Copies the summary to its host copy and, with `reset`, clears it.  Called by
+// a whole CTA after a barrier that follows the last change of the summary.
+__device__ __forceinline__ void publish_summary(DevSummary* sum, DevSummary* host, bool reset) {
+  static_assert(sizeof(DevSummary) % sizeof(int) == 0, "copied as ints");
+  volatile int* d = reinterpret_cast<volatile int*>(sum);
+  volatile int* h = reinterpret_cast<volatile int*>(host);
+  for (int w = threadIdx.x; w < static_cast<int>(sizeof(DevSummary) / sizeof(int)); w += blockDim.x) {
+    h[w] = d[w];
+    if (reset) d[w] = 0;
+  }
+}
 
 // Read-only view of an input CSR matrix.
 template <typename T>
@@ -152,6 +172,7 @@ struct RowPlan {
                                // from the front, the others from the back of seg_len * rcd_slices<T>() places
   int32_t* rcd_ctr;            // counters kRcdBigItems .. kRcdNextItem
   DevSummary* sum;
+  int* status;         // error flags (pinned host memory)
   int64_t seg_begin;   // first position in perm of the segment a kernel processes
   int64_t seg_len;     // rows in that segment
   int log2_group;      // lanes per stored A entry when walking B rows (1 << log2_group)
@@ -184,6 +205,8 @@ struct EwisePlan {
   int64_t nc_max;        // bound on the number of chunks: m + (nnz(A) + nnz(B)) / diag + 1
   int64_t* partials;     // scan scratch for max(m, nc_max) entries
   DevSummary* sum;
+  int* status;           // error flags (pinned host memory)
+  DevSummary* host;      // host copy of the summary
   int64_t diag;          // merged positions per chunk
   int group;             // lanes per chunk (1: one thread merges entry by entry; kEwiseTileGroup: the same
                          // from shared-memory copies of a warp's 32 chunks; 4, 8, 16, 32: windows;
@@ -212,6 +235,8 @@ struct SpmspvPlan {
   int64_t* cnt;          // [tiles + 1]: set bits per compaction tile, then scanned in place
   int64_t* partials;     // scan scratch for max(nx, tiles) entries
   DevSummary* sum;
+  int* status;           // error flags (pinned host memory)
+  DevSummary* host;      // host copy of the summary
   int32_t* y_idx;        // [cap]
   T* y_vals;             // [cap]
   int64_t cap;           // capacity of y (m)
@@ -225,7 +250,7 @@ void launch_submatrix_count(const int64_t* rowptr, const int32_t* colidx, int64_
                             int64_t c1, int64_t* s_rowptr, int num_sms, cudaStream_t s, int* launches);
 template <typename T>
 void launch_submatrix_copy(const int64_t* rowptr, const int32_t* colidx, const T* vals, int64_t r0, int64_t rows,
-                           int64_t c0, const int64_t* s_rowptr, int32_t* s_colidx, T* s_vals, DevSummary* sum,
+                           int64_t c0, const int64_t* s_rowptr, int32_t* s_colidx, T* s_vals, int* status,
                            int num_sms, cudaStream_t s, int* launches);
 
 // Host-side launchers (one translation unit each).
@@ -239,11 +264,13 @@ struct AnalyzeParams {
   int64_t wb_span;     // widest column range of a wide-bitmap heavy row (0: none)
   int dense_width;
   int long_threshold;
+  int64_t nnz;         // stored entries of A, at most
 };
 // rows == nullptr: every row of A; otherwise the first sum->n_pending entries of rows.
+// host != nullptr: the summary is copied there at the end.
 template <typename T>
 void launch_analyze(const RowPlan<T>& p, const AnalyzeParams& ap, int32_t* long_rows, const int32_t* rows,
-                    int num_sms, cudaStream_t s, int* launches);
+                    DevSummary* host, int num_sms, cudaStream_t s, int* launches);
 template <typename T>
 void launch_bmr_plan(const RowPlan<T>& p, const AnalyzeParams& ap, int64_t ncols, int32_t* pending, int num_sms,
                      cudaStream_t s, int* launches);
@@ -269,9 +296,12 @@ void launch_dense(const RowPlan<T>& p, int64_t nslices, bool numeric, int num_sm
 template <typename T>
 void launch_direct(const RowPlan<T>& p, int num_sms, cudaStream_t s, int* launches);
 
+// Writes rowptr[0] = 0 too (not when m = 0: nothing is launched then).
 // skip != nullptr: the scan does nothing when *skip != 0 (read on the device).
+// host != nullptr: the summary block is copied there at the end, and cleared
+// on the device unless the scan was skipped.
 void launch_scan(int64_t* rowptr, int64_t m, int64_t* partials, DevSummary* sum, cudaStream_t s, int* launches,
-                 const int* skip = nullptr);
+                 const int* skip = nullptr, DevSummary* host = nullptr);
 int64_t scan_partials_needed(int64_t m);
 
 void launch_validate(const int64_t* rowptr, const int32_t* colidx, int64_t nrows, int64_t ncols, int64_t nnz,
