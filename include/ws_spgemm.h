@@ -184,8 +184,8 @@ typedef enum {
  * A and B have the same shape and dtype; C is an output handle of that shape
  * and dtype.  Writes C.rowptr into the rowptr array of C's handle and returns
  * nnz(C) in *nnz_out (host pointer).  Work is queued on `stream` and the call
- * synchronises it (the caller needs nnz(C) to allocate C).  The chunk plan
- * (rows cut into pieces of their merged column lists) is kept in C's handle
+ * synchronises it (the caller needs nnz(C) to allocate C).  The tile plan
+ * (the merged entries of all rows cut into equal tiles) is kept in C's handle
  * for ws_ewise_numeric; device scratch is allocated stream-ordered on
  * `stream` and cached in the handle.  Errors: WS_ERR_SHAPE, WS_ERR_DTYPE,
  * WS_ERR_INVALID_ARG (NULL pointer, unknown op), WS_ERR_DEVICE (a kernel found
@@ -310,17 +310,9 @@ ws_status_t ws_spgemm_plan_info(ws_csr_t C, int64_t* info, int n);
  *          path (value windows) (default and maximum 8192; 0 disables it)
  *   key 7: widest column range of a heavy row that uses the wide-bitmap path
  *          (default and maximum 1048576; 0 disables it)
- *   key 8: elementwise operations, lanes per row chunk: -1 (default:
- *          automatic, 2 for rows averaging under 64 merged entries, 64
- *          otherwise), 1 (one thread merges a chunk entry by entry from
- *          global memory), 2 (the same from shared-memory copies of the
- *          input runs of a warp's 32 chunks, chunks of at most 16 merged
- *          entries), 4, 8, 16 or 32 (a lane group merges windows of that
- *          many entries), 0 (lane group sized from the mean row length), 64
- *          (a warp per 64-entry chunk ranks every entry by binary search)
- *   key 9: elementwise operations with one lane per chunk: merged entries
- *          per chunk (default 64, range [2, 1048576]; with key 8 = 2 at
- *          most 16 are used)
+ *   key 8 (-1, 0, 1, 2, 4, 8, 16, 32 or 64; default -1) and key 9 ([2,
+ *          1048576]; default 64): accepted, without effect (the elementwise
+ *          operations once had several paths; they have one)
  * Returns WS_ERR_INVALID_ARG for an unknown key or out-of-range value.
  */
 ws_status_t ws_set_tuning(int key, int64_t value);

@@ -35,8 +35,6 @@ int g_rcd_max_a = kRcdDefaultMaxA;
 int64_t g_wb_span = kWbMaxSpan;
 int g_run_limit = 64;
 int g_dense_width = 0;  // 0 = default per value type
-int g_ewise_lanes = -1;  // elementwise: lanes per chunk (0 = lane groups from the mean row length, -1 = automatic)
-int64_t g_ewise_diag = 64;  // elementwise, one thread per chunk: merged positions per chunk
 constexpr int kLongRowThreshold = 16;  // rows with more stored entries are analysed by a warp or a CTA
 
 ws_status_t fail(ws_status_t st, const char* fmt, ...) __attribute__((format(printf, 2, 3)));
@@ -280,13 +278,12 @@ struct Plan {
   DevBuf rcd;     // dense heavy rows: work counters, numeric items, the rows' bitmaps
   int kind = kPlanNone;  // which symbolic pass filled this plan
   // elementwise plan (kPlanEwise)
-  int ew_op = 0, ew_group = 32;
-  int64_t ew_diag = 0, ew_nc_max = 0;
-  int64_t* ew_chunk_begin = nullptr;
-  int32_t* ew_chunk_row = nullptr;
-  int64_t* ew_chunk_off = nullptr;
-  int64_t* ew_chunk_split = nullptr;
-  int64_t* ew_chunk_bpos = nullptr;
+  int ew_op = 0;
+  int64_t ew_ntiles = 0;
+  int32_t* ew_tile_row = nullptr;
+  int64_t* ew_tile_a = nullptr;
+  int64_t* ew_tile_b = nullptr;
+  int64_t* ew_tile_off = nullptr;
   int64_t* ew_partials = nullptr;
   int32_t* rcd_ctr = nullptr;
   long long* rcd_items = nullptr;
@@ -361,11 +358,16 @@ int log2_group_for(const ws_csr_s* B) {
   return 5;
 }
 
+// A fresh status word for the next pass.
+void next_status(Plan* pl) {
+  pl->slot ^= 1;
+  pl->host_sum->slot[pl->slot] = 0;
+}
+
 // Start of a symbolic pass whose summary block heads `buf`: a fresh status
 // word, and the block cleared unless the last pass left it so.
 ws_status_t begin_pass(Plan* pl, const DevBuf& buf, cudaStream_t s) {
-  pl->slot ^= 1;
-  pl->host_sum->slot[pl->slot] = 0;
+  next_status(pl);
   const bool clean = pl->clean_buf == &buf && pl->clean_gen == buf.gen;
   pl->clean_buf = nullptr;
   if (!clean) WS_CUDA(cudaMemsetAsync(pl->dsum, 0, sizeof(DevSummary), s), "cudaMemsetAsync(summary)");
@@ -669,34 +671,23 @@ ws_status_t numeric_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan
 
 // ----------------------------------------------------- elementwise operations
 
-// Lanes per chunk from the mean merged row length (entries of A and B per row).
-int ewise_group_for(int64_t m, int64_t merged) {
-  const double avg = m > 0 ? static_cast<double>(merged) / static_cast<double>(m) : 0.0;
-  if (avg <= 8.0) return 4;
-  if (avg <= 16.0) return 8;
-  if (avg <= 32.0) return 16;
-  return 32;
-}
-
-ws_status_t carve_ewise(Plan* pl, int64_t m, int64_t nc_max, cudaStream_t s) {
-  const int64_t nb = scan_partials_needed(m > nc_max ? m : nc_max);
+ws_status_t carve_ewise(Plan* pl, int64_t ntiles, cudaStream_t s) {
+  const size_t n = static_cast<size_t>(ntiles) + 1;
   size_t off = 0;
   const size_t o_sum = off; off = align_up(off + sizeof(DevSummary), 256);
-  const size_t o_begin = off; off = align_up(off + 8 * static_cast<size_t>(m + 1), 256);
-  const size_t o_row = off; off = align_up(off + 4 * static_cast<size_t>(nc_max), 256);
-  const size_t o_off = off; off = align_up(off + 8 * static_cast<size_t>(nc_max + 1), 256);
-  const size_t o_split = off; off = align_up(off + 8 * static_cast<size_t>(nc_max + 1), 256);
-  const size_t o_bpos = off; off = align_up(off + 8 * static_cast<size_t>(nc_max + 1), 256);
-  const size_t o_part = off; off = align_up(off + 8 * static_cast<size_t>(nb + 1), 256);
+  const size_t o_row = off; off = align_up(off + 4 * n, 256);
+  const size_t o_a = off; off = align_up(off + 8 * n, 256);
+  const size_t o_b = off; off = align_up(off + 8 * n, 256);
+  const size_t o_off = off; off = align_up(off + 8 * n, 256);
+  const size_t o_part = off; off = align_up(off + 8 * static_cast<size_t>(scan_partials_needed(ntiles) + 1), 256);
   ws_status_t st = pl->ew.reserve(off, s);
   if (st != WS_OK) return st;
   char* b = static_cast<char*>(pl->ew.ptr);
   pl->dsum = reinterpret_cast<DevSummary*>(b + o_sum);
-  pl->ew_chunk_begin = reinterpret_cast<int64_t*>(b + o_begin);
-  pl->ew_chunk_row = reinterpret_cast<int32_t*>(b + o_row);
-  pl->ew_chunk_off = reinterpret_cast<int64_t*>(b + o_off);
-  pl->ew_chunk_split = reinterpret_cast<int64_t*>(b + o_split);
-  pl->ew_chunk_bpos = reinterpret_cast<int64_t*>(b + o_bpos);
+  pl->ew_tile_row = reinterpret_cast<int32_t*>(b + o_row);
+  pl->ew_tile_a = reinterpret_cast<int64_t*>(b + o_a);
+  pl->ew_tile_b = reinterpret_cast<int64_t*>(b + o_b);
+  pl->ew_tile_off = reinterpret_cast<int64_t*>(b + o_off);
   pl->ew_partials = reinterpret_cast<int64_t*>(b + o_part);
   return WS_OK;
 }
@@ -710,18 +701,15 @@ EwisePlan<T> make_ewise(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, const
   p.c_rowptr = C->rowptr;
   p.c_colidx = C->colidx;
   p.c_vals = static_cast<T*>(C->vals);
-  p.chunk_begin = pl->ew_chunk_begin;
-  p.chunk_row = pl->ew_chunk_row;
-  p.chunk_off = pl->ew_chunk_off;
-  p.chunk_split = pl->ew_chunk_split;
-  p.chunk_bpos = pl->ew_chunk_bpos;
-  p.nc_max = pl->ew_nc_max;
+  p.ntiles = pl->ew_ntiles;
+  p.tile_row = pl->ew_tile_row;
+  p.tile_a = pl->ew_tile_a;
+  p.tile_b = pl->ew_tile_b;
+  p.tile_off = pl->ew_tile_off;
   p.partials = pl->ew_partials;
   p.sum = pl->dsum;
   p.status = status_word(pl);
   p.host = pl->host_sum;
-  p.diag = pl->ew_diag;
-  p.group = pl->ew_group;
   p.op = pl->ew_op;
   return p;
 }
@@ -736,20 +724,11 @@ ws_status_t ewise_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
   pl->num_launches = 0;
   pl->ew_op = op;
   const int64_t merged = A->nnz + B->nnz;
-  // automatic: a lane per chunk of a warp-staged tile for short rows
-  // (power-law graphs), a warp per 64-position chunk once rows average a
-  // whole chunk
-  const bool long_rows = m > 0 && merged >= static_cast<int64_t>(kEwiseRankChunk) * m;
-  pl->ew_group = g_ewise_lanes > 0 ? g_ewise_lanes
-               : g_ewise_lanes == 0 ? ewise_group_for(m, merged) : (long_rows ? kEwiseRankGroup : kEwiseTileGroup);
-  pl->ew_diag = pl->ew_group == 1 ? g_ewise_diag
-              : pl->ew_group == kEwiseTileGroup ? (g_ewise_diag < kEwiseTileDiag ? g_ewise_diag : kEwiseTileDiag)
-              : pl->ew_group == kEwiseRankGroup ? kEwiseRankChunk : 16 * static_cast<int64_t>(pl->ew_group);
-  pl->ew_nc_max = m + merged / pl->ew_diag + 1;  // row i has at most 1 + len_i / diag chunks
-  ws_status_t st = carve_ewise(pl, m, pl->ew_nc_max, s);
+  pl->ew_ntiles = (merged + m + kEwTileItems - 1) / kEwTileItems;
+  ws_status_t st = carve_ewise(pl, pl->ew_ntiles, s);
   if (st != WS_OK) return st;
-  st = begin_pass(pl, pl->ew, s);
-  if (st != WS_OK) return st;
+  next_status(pl);  // the summary block only takes the scan's total: it need not be cleared
+  pl->clean_buf = nullptr;
   if (m > 0) {
     launch_ewise_symbolic<T>(make_ewise<T>(A, B, C, pl), num_sms_of(C->device), s, &pl->sym_launches);
     WS_CUDA(cudaGetLastError(), "elementwise symbolic launches");
@@ -758,7 +737,6 @@ ws_status_t ewise_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
   }
   st = wait_summary(s);
   if (st != WS_OK) return st;
-  if (m > 0) end_pass(pl, pl->ew);
   st = device_status(pl);
   if (st != WS_OK) return st;
   C->nnz = m > 0 ? pl->host_sum->nnz : 0;
@@ -826,8 +804,7 @@ ws_status_t spmspv_impl(ws_csr_s* At, int64_t nx, const int32_t* x_idx, const vo
   p.y_vals = static_cast<T*>(y_vals);
   p.cap = m;
   pl->dsum = p.sum;
-  pl->slot ^= 1;
-  pl->host_sum->slot[pl->slot] = 0;
+  next_status(pl);
   p.status = status_word(pl);
   p.host = pl->host_sum;
   pl->sym_launches = 0;
@@ -1527,15 +1504,12 @@ ws_status_t ws_set_tuning(int key, int64_t value) {
       if (value < 0 || value > kWbMaxSpan) return fail(WS_ERR_INVALID_ARG, "wide-bitmap span out of range");
       g_wb_span = value;
       return WS_OK;
-    case 8:
-      if (value != -1 && value != 0 && value != 1 && value != kEwiseTileGroup && value != 4 && value != 8 &&
-          value != 16 && value != 32 && value != kEwiseRankGroup)
+    case 8:  // accepted, without effect: the elementwise operations have one path
+      if (value < -1 || value > 64 || (value > 2 && (value & (value - 1)) != 0))
         return fail(WS_ERR_INVALID_ARG, "elementwise lanes per chunk must be -1, 0, 1, 2, 4, 8, 16, 32 or 64");
-      g_ewise_lanes = static_cast<int>(value);
       return WS_OK;
-    case 9:
+    case 9:  // likewise
       if (value < 2 || value > (int64_t{1} << 20)) return fail(WS_ERR_INVALID_ARG, "elementwise chunk length out of range");
-      g_ewise_diag = value;
       return WS_OK;
   }
   return fail(WS_ERR_INVALID_ARG, "unknown tuning key %d", key);

@@ -183,10 +183,7 @@ struct RowPlan {
 // Elementwise operations C = A op B on CSR matrices of one shape.
 constexpr int kEwiseAdd = 1;  // SpAdd: pattern union, values added
 constexpr int kEwiseMul = 2;  // Hadamard product: pattern intersection, values multiplied
-constexpr int kEwiseRankGroup = 64;  // EwisePlan::group of the warp-per-chunk ranking kernels
-constexpr int kEwiseTileGroup = 2;   // EwisePlan::group of the warp-staged tile kernels (a lane per chunk)
-constexpr int kEwiseTileDiag = 16;   // their largest chunk (merged positions)
-constexpr int kEwiseRankChunk = 64;  // their merged positions per chunk
+constexpr int kEwTileItems = 2040;  // items of a tile: merged entries and row ends
 
 template <typename T>
 struct EwisePlan {
@@ -194,24 +191,18 @@ struct EwisePlan {
   CsrView<T> B;
   int64_t m;
   int64_t* c_rowptr;
-  int32_t* c_colidx;     // numeric only
-  T* c_vals;             // numeric only
-  int64_t* chunk_begin;  // [m + 1]: first chunk of each row (chunks per row, then scanned in place)
-  int32_t* chunk_row;    // [nc_max]: row of each chunk
-  int64_t* chunk_off;    // [nc_max + 1]: C offset of each chunk (counts, then scanned in place)
-  int64_t* chunk_split;  // [nc_max + 1]: 2 * (A entries before the chunk) + (1 if an equal pair straddles its start);
-                         // warp-staged tiles: the chunk's first position in A's arrays ([nc]: the end of A)
-  int64_t* chunk_bpos;   // [nc_max + 1]: warp-staged tiles: the chunk's first position in B's arrays
-  int64_t nc_max;        // bound on the number of chunks: m + (nnz(A) + nnz(B)) / diag + 1
-  int64_t* partials;     // scan scratch for max(m, nc_max) entries
+  int32_t* c_colidx;   // numeric only
+  T* c_vals;           // numeric only
+  int64_t ntiles;      // tiles of kEwTileItems items; enough for m rows and the entries of A and B
+  int32_t* tile_row;   // [ntiles + 1]: first item of every tile: its row
+  int64_t* tile_a;     // [ntiles + 1]:   and positions in A's
+  int64_t* tile_b;     // [ntiles + 1]:   and B's arrays
+  int64_t* tile_off;   // [ntiles + 1]: equal pairs before every tile (counts, then scanned in place)
+  int64_t* partials;   // scan scratch for ntiles entries
   DevSummary* sum;
-  int* status;           // error flags (pinned host memory)
-  DevSummary* host;      // host copy of the summary
-  int64_t diag;          // merged positions per chunk
-  int group;             // lanes per chunk (1: one thread merges entry by entry; kEwiseTileGroup: the same
-                         // from shared-memory copies of a warp's 32 chunks; 4, 8, 16, 32: windows;
-                         // kEwiseRankGroup: a warp per chunk ranks every entry by binary search)
-  int op;                // kEwiseAdd or kEwiseMul
+  int* status;         // error flags (pinned host memory)
+  DevSummary* host;    // pinned: receives nnz
+  int op;              // kEwiseAdd or kEwiseMul
 };
 template <typename T>
 void launch_ewise_symbolic(const EwisePlan<T>& p, int num_sms, cudaStream_t s, int* launches);

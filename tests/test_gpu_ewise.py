@@ -121,6 +121,37 @@ def test_long_rows_many_chunks(overlap, op, lanes, chunk):
 
 
 @pytest.mark.parametrize("op", OPS)
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_tile_edges(dtype, op):
+    """Sequences of merged entries and row ends at the edges of the 2040-item
+    tiles: one item less than a tile, exactly one, one more, exactly two; cuts
+    between the entries of an equal pair, before and after a row's end, inside
+    stretches of empty rows, and rows with entries in one operand only."""
+    rng = np.random.default_rng(77)
+    n = 30_000
+
+    def csr(rows):
+        rp = np.zeros(len(rows) + 1, np.int64)
+        np.cumsum([len(r) for r in rows], out=rp[1:])
+        ci = np.concatenate([np.sort(np.asarray(r, np.int64)) for r in rows] + [np.zeros(0, np.int64)]).astype(np.int32)
+        return HostCSR(len(rows), n, rp, ci, rng.uniform(-1.0, 1.0, ci.size).astype(dtype))
+
+    def pick(k):
+        return rng.choice(n, size=k, replace=False).tolist()
+
+    for items in (2039, 2040, 2041, 4080):      # one row: its entries and one end
+        for in_a in (0, (items - 1) // 2, items - 1):
+            check(csr([pick(in_a)]), csr([pick(items - 1 - in_a)]), op)
+    for shift in range(4):                      # pairs only, moved against the cuts by single entries
+        pairs = pick(4500)
+        check(csr([pick(shift), pairs, []]), csr([[], pairs, pick(3)]), op)
+    empty = [[]] * 5000
+    some = [pick(int(k)) for k in rng.integers(0, 4, size=3000)]
+    check(csr(empty + some + empty), csr(empty + some[::-1] + empty), op)
+    check(csr(some + [pick(5000)] + empty), csr([[]] * 3001 + some + empty[:2000]), op)
+
+
+@pytest.mark.parametrize("op", OPS)
 def test_same_operand_long_rows(op):
     rng = np.random.default_rng(5)
     A, _ = _long_rows(6, 50_000, [30_000, 2, 9_999, 0, 1, 17_000], rng, 0.0)
