@@ -354,9 +354,11 @@ __global__ void __launch_bounds__(256) dense_slices_kernel(const RowPlan<T> p, i
   }
 }
 
-// Checks the CSR invariants of one matrix; records the smallest offending row.
+// Checks the CSR invariants of one matrix; records the smallest offending row
+// in `sum` (pinned host memory, written only for a broken matrix).
 __global__ void __launch_bounds__(256) validate_kernel(const int64_t* rowptr, const int32_t* colidx, int64_t nrows,
                                                        int64_t ncols, int64_t nnz, DevSummary* sum) {
+  int worst = INT_MAX;  // first bad row this thread saw
   for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nrows;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
     const int64_t s = rowptr[i], e = rowptr[i + 1];
@@ -372,10 +374,12 @@ __global__ void __launch_bounds__(256) validate_kernel(const int64_t* rowptr, co
         prev = c;
       }
     }
-    if (bad) {
-      atomicOr(&sum->status, kErrInvalidCsr);
-      atomicMin(&sum->bad_row, static_cast<int>(i < INT_MAX ? i : INT_MAX));
-    }
+    if (bad) worst = min(worst, static_cast<int>(i < INT_MAX ? i : INT_MAX - 1));
+  }
+  worst = __reduce_min_sync(0xffffffffu, worst);
+  if ((threadIdx.x & 31) == 0 && worst < INT_MAX) {
+    atomicOr(&sum->status, kErrInvalidCsr);
+    atomicMin(&sum->bad_row, worst);
   }
 }
 

@@ -323,7 +323,67 @@ struct Plan {
   bool hash_ranked = false;  // hranks holds the hash rows' ranks
   int sym_launches = 0, num_launches = 0;
   struct OuterState* outer = nullptr;  // outer-product SpGEMM between its two passes
+  int device = 0;
+
+  size_t scratch_bytes() const {
+    size_t n = 0;
+    for (const DevBuf* b : {&rows, &slices, &ranks, &ew, &sv, &hranks, &rcd}) n += b->bytes;
+    return n;
+  }
+  // Back to a new plan that owns the same scratch and pinned block.
+  void recycle() {
+    Plan fresh;
+    fresh.rows = rows;
+    fresh.slices = slices;
+    fresh.ranks = ranks;
+    fresh.ew = ew;
+    fresh.sv = sv;
+    fresh.hranks = hranks;
+    fresh.rcd = rcd;
+    fresh.host_sum = host_sum;
+    fresh.slot = slot;
+    fresh.clean_buf = clean_buf;  // points into this object, whose address stays
+    fresh.clean_gen = clean_gen;
+    fresh.device = device;
+    *this = fresh;
+  }
 };
+
+// Plans of destroyed handles, for the next handles of their device: a one-shot
+// call otherwise spends as long on allocating and freeing its scratch as on a
+// small product.  A plan gets here after its device has finished all work, so
+// it may serve any stream.  At most kMaxPlans of at most kMaxPlanBytes scratch
+// each are kept; larger scratch goes back to the stream-ordered pool.
+constexpr size_t kMaxPlans = 8;
+constexpr size_t kMaxPlanBytes = size_t{32} << 20;
+std::mutex g_plan_mutex;
+std::vector<Plan*> g_plan_free;
+
+Plan* recycled_plan(int device) {
+  std::lock_guard<std::mutex> lock(g_plan_mutex);
+  for (size_t i = g_plan_free.size(); i-- > 0;) {
+    if (g_plan_free[i]->device == device) {
+      Plan* pl = g_plan_free[i];
+      g_plan_free.erase(g_plan_free.begin() + static_cast<std::ptrdiff_t>(i));
+      return pl;
+    }
+  }
+  return nullptr;
+}
+
+bool keep_plan(Plan* pl) {
+  if (!pl->host_sum || pl->scratch_bytes() > kMaxPlanBytes) return false;
+  std::lock_guard<std::mutex> lock(g_plan_mutex);
+  if (g_plan_free.size() >= kMaxPlans) return false;
+  try {
+    g_plan_free.reserve(kMaxPlans);
+  } catch (...) {
+    return false;
+  }
+  pl->recycle();
+  g_plan_free.push_back(pl);
+  return true;
+}
 
 }  // namespace
 
@@ -754,9 +814,11 @@ ws_status_t ewise_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
 
 // Creates a handle's plan and its pinned summary if missing.
 ws_status_t ensure_plan(ws_csr_s* h) {
+  if (!h->plan) h->plan = recycled_plan(h->device);
   if (!h->plan) {
     h->plan = new (std::nothrow) Plan;
     if (!h->plan) return fail(WS_ERR_ALLOC, "host allocation failed");
+    h->plan->device = h->device;
   }
   if (!h->plan->host_sum) {
     keep_pool_memory(h->device);
@@ -827,17 +889,7 @@ ws_status_t spmspv_impl(ws_csr_s* At, int64_t nx, const int32_t* x_idx, const vo
 ws_status_t prepare_output(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C) {
   if (C == A || C == B) return fail(WS_ERR_INVALID_ARG, "C must be a separate output handle");
   if (A->dtype != B->dtype || C->dtype != A->dtype) return fail(WS_ERR_DTYPE, "A, B and C dtypes differ");
-  if (!C->plan) {
-    C->plan = new (std::nothrow) Plan;
-    if (!C->plan) return fail(WS_ERR_ALLOC, "host allocation failed");
-  }
-  Plan* pl = C->plan;
-  if (!pl->host_sum) {
-    keep_pool_memory(C->device);
-    pl->host_sum = acquire_host_sum();
-    if (!pl->host_sum) return fail(WS_ERR_ALLOC, "cudaMallocHost failed");
-  }
-  return WS_OK;
+  return ensure_plan(C);
 }
 
 ws_status_t check_handle(const ws_csr_s* h, const char* name) {
@@ -1115,27 +1167,27 @@ ws_status_t ws_csr_create(ws_csr_t* out, int64_t nrows, int64_t ncols, int64_t n
   int dev = 0;
   WS_CUDA(cudaGetDevice(&dev), "cudaGetDevice");
   if (validate) {
-    DevSummary* d = nullptr;
-    DevSummary h{};
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    WS_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&d), sizeof(DevSummary), s), "cudaMallocAsync(validate)");
-    h.bad_row = INT32_MAX;
-    cudaError_t e = cudaMemcpyAsync(d, &h, sizeof(h), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess && nrows > 0) {
-      launch_validate(rowptr, colidx, nrows, ncols, nnz, d, num_sms_of(dev), s);
-      e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, s);
-    cudaFreeAsync(d, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return cuda_fail(e, "validation");
     if (nrows == 0) {
       int64_t r0 = -1;
-      WS_CUDA(cudaMemcpy(&r0, rowptr, sizeof(r0), cudaMemcpyDeviceToHost), "cudaMemcpy(rowptr[0])");
+      WS_CUDA(cudaMemcpyAsync(&r0, rowptr, sizeof(r0), cudaMemcpyDeviceToHost, s), "cudaMemcpyAsync(rowptr[0])");
+      WS_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
       if (r0 != 0 || nnz != 0) return fail(WS_ERR_INVALID_CSR, "empty matrix needs rowptr[0] = 0 and nnz = 0");
+    } else {
+      // the kernel writes what it finds to a pinned block: nothing for a valid matrix
+      HostSummary* h = acquire_host_sum();
+      if (!h) return fail(WS_ERR_ALLOC, "cudaMallocHost failed");
+      h->status = 0;
+      h->bad_row = INT32_MAX;
+      launch_validate(rowptr, colidx, nrows, ncols, nnz, h, num_sms_of(dev), s);
+      cudaError_t e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      const volatile HostSummary* v = h;
+      const int status = v->status, bad_row = v->bad_row;
+      if (e != cudaSuccess) return cuda_fail(e, "validation");  // the block is not reused: the kernel may still run
+      release_host_sum(h);
+      if (status & kErrInvalidCsr) return fail(WS_ERR_INVALID_CSR, "CSR invariants violated (first bad row %d)", bad_row);
     }
-    if (h.status & kErrInvalidCsr)
-      return fail(WS_ERR_INVALID_CSR, "CSR invariants violated (first bad row %d)", h.bad_row);
   }
   ws_csr_s* hnd = new (std::nothrow) ws_csr_s;
   if (!hnd) return fail(WS_ERR_ALLOC, "host allocation failed");
@@ -1403,20 +1455,15 @@ ws_status_t ws_spgemm_wait(ws_csr_t C, ws_stream_t stream) {
 
 ws_status_t ws_csr_destroy(ws_csr_t h) {
   if (!h) return WS_OK;
-  if (h->plan) {
-    if (h->plan->rows.ptr || h->plan->slices.ptr || h->plan->ranks.ptr || h->plan->ew.ptr || h->plan->sv.ptr ||
-        h->plan->hranks.ptr || h->plan->rcd.ptr || h->plan->outer)
-      cudaDeviceSynchronize();
-    release_outer(h->plan, nullptr);
-    h->plan->rows.release();
-    h->plan->slices.release();
-    h->plan->ranks.release();
-    h->plan->ew.release();
-    h->plan->sv.release();
-    h->plan->hranks.release();
-    h->plan->rcd.release();
-    release_host_sum(h->plan->host_sum);
-    delete h->plan;
+  if (Plan* pl = h->plan) {
+    bool idle = true;
+    if (pl->scratch_bytes() > 0 || pl->outer) idle = cudaDeviceSynchronize() == cudaSuccess;
+    release_outer(pl, nullptr);
+    if (!idle || !keep_plan(pl)) {
+      for (DevBuf* b : {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd}) b->release();
+      release_host_sum(pl->host_sum);
+      delete pl;
+    }
   }
   delete h;
   return WS_OK;

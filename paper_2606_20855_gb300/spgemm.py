@@ -23,8 +23,8 @@ _DTYPES = {torch.float32: _abi.WS_F32, torch.float64: _abi.WS_F64}
 
 
 def _stream_handle(stream) -> int:
-    if stream is None:
-        stream = torch.cuda.current_stream()
+    if stream is None:  # the raw handle of torch.cuda.current_stream(), without building the object
+        return int(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
     return int(stream.cuda_stream)
 
 

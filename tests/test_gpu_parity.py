@@ -684,6 +684,50 @@ def test_numeric_pass_under_capture():
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+def test_one_shot_calls_reuse_scratch_of_any_kind():
+    """One-shot products, elementwise operations, extractions and SpMSpV in
+    turn, on two streams: the scratch of a destroyed handle serves the next
+    handle, whatever its operation, and leaves no trace in results or counts."""
+    from oracle import oracle_ewise, oracle_spmspv
+    from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM, ewise, spgemm, spmspv, submatrix
+    from synth import sparse_vector, transpose_csr
+    rng = np.random.default_rng(51)
+    M, N = _mixed_rows(3)
+    A = random_csr(300, 280, 0.05, rng, np.float64, "sym")
+    B = random_csr(300, 280, 0.06, rng, np.float64, "sym")
+    S = uniform_csr(200, 280, 6, rng)
+    xi, xv = sparse_vector(280, 0.2, rng, np.float64, "sym")
+    ref_y, ref_add = oracle_spmspv(A, xi, xv), oracle_ewise(A, B, "add")
+    put = DeviceCSR.from_host
+    dM, dN, dA, dB, dS, dT = put(M), put(N), put(A), put(B), put(S), put(transpose_csr(S))
+    dAt = put(transpose_csr(A))
+    dxi, dxv = torch.from_numpy(xi).cuda(), torch.from_numpy(xv).cuda()
+    for stream in [torch.cuda.current_stream(), torch.cuda.Stream()] * 2:
+        torch.cuda.synchronize()
+        with torch.cuda.stream(stream):
+            C = spgemm(dM, dN)
+            y, yv = spmspv(dAt, dxi, dxv)
+            D = ewise(dA, dB, "add")
+            E = submatrix(dA, 10, 200, 5, 250)
+            F = spgemm(dS, dT, validate=True)
+            with SpGEMM(dS, dT) as op:
+                op.symbolic()
+                info = op.plan_info()
+            stream.synchronize()
+        assert_matches_oracle(M, N, *C.to_host())
+        assert_matches_oracle(S, transpose_csr(S), *F.to_host())
+        np.testing.assert_array_equal(y.cpu().numpy(), ref_y.idx)
+        np.testing.assert_allclose(yv.cpu().numpy(), ref_y.vals, rtol=0, atol=1e-12)
+        for got, want in zip(D.to_host(), (ref_add.rowptr, ref_add.colidx, ref_add.vals)):
+            np.testing.assert_array_equal(got, want)
+        lens = np.diff(A.rowptr)
+        keep = (A.colidx >= 5) & (A.colidx < 250) & (np.repeat(np.arange(300), lens) >= 10) & (np.repeat(np.arange(300), lens) < 200)
+        np.testing.assert_array_equal(E.to_host()[1], A.colidx[keep] - 5)
+        np.testing.assert_array_equal(E.to_host()[2], A.vals[keep])
+        assert info["bitmap_rows"] + info["hash_rows"] + info["direct_rows"] + info["empty_rows"] == 200
+        assert info["rcd_rows"] == info["wb_rows"] == info["dense_rows"] == 0
+
+
 def test_device_count_check_reports_error():
     """A row pointer altered between the passes is caught by the numeric pass's count check."""
     from paper_2606_20855_gb300 import _abi
