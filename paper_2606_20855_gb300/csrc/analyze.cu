@@ -24,14 +24,27 @@ __device__ __forceinline__ int ceil_log2_ll(long long x) {  // x >= 1
 }
 
 // Class of a row from its stored-entry count, product count and column range.
-// Bitmap bins take rows whose range fits a bitmap that is not much larger
-// than the row's products (at most 8 words per product plus 64).
-// Rows with at most bmr_max_a entries whose B rows fit one lane group take the
-// register bitmap bins; other narrow rows with at most 1024 entries the
-// bitmap bins.  Heavy rows (more entries than those) go to the dense rows
-// (narrow range, few stored A entries: long B rows), the 8192-entry bitmap
-// bin, the hash bins, the wide bitmap (range up to 2^20) and finally the
+// Regular rows (at most kBmrMaxA entries whose B rows fit one lane group) with
+// a range that fits a bitmap not much larger than their products (at most 8
+// words per product plus 64) take the register bitmap bins (the bitmap bins
+// if those are disabled).  The other rows of at most hash_max products take the
+// hash bins unless
+// - their products crowd a range of less than kCrowded columns per product:
+//   most products repeat a column there, and the hash buckets fill up; or
+// - one of their B rows is longer than kShortB: such rows (hub rows of a
+//   power-law matrix) tend to be dense at one end, which fills some buckets.
+// Those take the bitmap bins, and the dense rows above them.  Measured (100,000
+// rows, fp32, bitmap bins against hash bins): rows of 0-48 entries and B rows of
+// 0-24 over 1000 to 32,000 columns 0.97-1.69 against 0.69-0.72 ms; 20 entries
+// of 6 over 4000 columns 0.42 against 0.31, 24 of 12 0.62 against 0.72; 60 of
+// 60 inside 800 columns 5.3 against 10.4, 40 of 20 inside 80 0.65 against 1.45;
+// R-MAT 2^16 squared without the second exception 3.6 against 4.5.
+// Rows with more products go to the dense rows (range up to 65,536 columns), the
+// 8192-entry bitmap bin, the wide bitmap (range up to 2^20) and finally the
 // column-sliced dense window.
+constexpr long long kCrowded = 2;
+constexpr int kShortB = 64;
+
 __device__ __forceinline__ uint8_t classify(long long nnza, long long ub, int lo, int hi, int maxlen,
                                             const AnalyzeParams& ap) {
   if (ub == 0) return kClsEmpty;
@@ -39,8 +52,10 @@ __device__ __forceinline__ uint8_t classify(long long nnza, long long ub, int lo
   const long long span = static_cast<long long>(hi) - lo + 1;
   const long long est = ub < span ? ub : span;  // entries of the row are at most this
   const bool bitmap_ok = span <= ap.bitmap_span && ((span + 31) >> 5) <= 8 * ub + 64;
-  if (bitmap_ok) {
-    if (nnza <= ap.bmr_max_a && maxlen <= ap.group) {
+  const bool regular = nnza <= kBmrMaxA && maxlen <= ap.group;
+  const bool hashed = ub <= ap.hash_max && (!bitmap_ok || (!regular && maxlen <= kShortB && span >= kCrowded * ub));
+  if (bitmap_ok && !hashed) {
+    if (regular && nnza <= ap.bmr_max_a) {
 #pragma unroll
       for (int b = 0; b < kNumBmrBins; ++b) {
         if (span <= (32ll << bmr_log_words(b))) return static_cast<uint8_t>(kClsBmr0 + b);
@@ -51,9 +66,9 @@ __device__ __forceinline__ uint8_t classify(long long nnza, long long ub, int lo
       if (span <= (32ll << bitmap_log_words(b)) && est <= bitmap_cap(b)) return static_cast<uint8_t>(kClsBitmap0 + b);
     }
   }
-  const bool heavy = ub > 4096 || (bitmap_ok && est > bitmap_cap(kNumBitmapBins - 2));
+  const bool heavy = !hashed && (ub > 4096 || (bitmap_ok && est > bitmap_cap(kNumBitmapBins - 2)));
   if (heavy && span <= kMaxBitmapSpan && nnza <= ap.rcd_max_a) return kClsRcd;
-  if (bitmap_ok && span <= (32ll << bitmap_log_words(kNumBitmapBins - 1)) && est <= bitmap_cap(kNumBitmapBins - 1))
+  if (bitmap_ok && !hashed && span <= (32ll << bitmap_log_words(kNumBitmapBins - 1)) && est <= bitmap_cap(kNumBitmapBins - 1))
     return static_cast<uint8_t>(kClsBitmap0 + kNumBitmapBins - 1);
   if (ub <= ap.hash_max) {
     int b = ceil_log2_ll(ub) - kMinHashLog;
@@ -215,7 +230,7 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
   __shared__ long long s_prod, s_slices;
   __shared__ int s_empty;
   __shared__ long long s_ub[8];
-  __shared__ int s_lo[8], s_hi[8];
+  __shared__ int s_lo[8], s_hi[8], s_maxlen[8];
   if (threadIdx.x < kNumSegs) s_seg[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     s_prod = 0;
@@ -229,13 +244,14 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
     const int64_t i = long_rows[ap.m - 1 - w];  // long rows fill the list from the back
     const int64_t s = p.A.rowptr[i], e = p.A.rowptr[i + 1];
     long long ub = 0;
-    int lo = INT_MAX, hi = -1;
+    int lo = INT_MAX, hi = -1, maxlen = 0;
 #pragma unroll 8
     for (int64_t q = s + threadIdx.x; q < e; q += blockDim.x) {
       const int k = p.A.colidx[q];
       const int64_t bs = p.B.rowptr[k], be = p.B.rowptr[k + 1];
       if (be > bs) {
         ub += be - bs;
+        maxlen = max(maxlen, static_cast<int>(min(be - bs, static_cast<int64_t>(INT_MAX))));
         lo = min(lo, p.B.colidx[bs]);
         hi = max(hi, p.B.colidx[be - 1]);
       }
@@ -245,11 +261,13 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
       ub += __shfl_xor_sync(0xffffffffu, ub, o);
       lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
       hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      maxlen = max(maxlen, __shfl_xor_sync(0xffffffffu, maxlen, o));
     }
     if (lane == 0) {
       s_ub[warp] = ub;
       s_lo[warp] = lo;
       s_hi[warp] = hi;
+      s_maxlen[warp] = maxlen;
     }
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -257,8 +275,9 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
         ub += s_ub[w2];
         lo = min(lo, s_lo[w2]);
         hi = max(hi, s_hi[w2]);
+        maxlen = max(maxlen, s_maxlen[w2]);
       }
-      record_row(p, ap, i, e - s, ub, lo, hi, INT_MAX, s_seg, &s_prod, &s_slices, &s_empty);
+      record_row(p, ap, i, e - s, ub, lo, hi, maxlen, s_seg, &s_prod, &s_slices, &s_empty);
     }
     __syncthreads();  // s_ub/s_lo/s_hi are reused by the next row
   }
@@ -269,13 +288,14 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
     const int64_t i = long_rows[w];
     const int64_t s = p.A.rowptr[i], e = p.A.rowptr[i + 1];
     long long ub = 0;
-    int lo = INT_MAX, hi = -1;
+    int lo = INT_MAX, hi = -1, maxlen = 0;
 #pragma unroll 8
     for (int64_t q = s + lane; q < e; q += 32) {
       const int k = p.A.colidx[q];
       const int64_t bs = p.B.rowptr[k], be = p.B.rowptr[k + 1];
       if (be > bs) {
         ub += be - bs;
+        maxlen = max(maxlen, static_cast<int>(min(be - bs, static_cast<int64_t>(INT_MAX))));
         lo = min(lo, p.B.colidx[bs]);
         hi = max(hi, p.B.colidx[be - 1]);
       }
@@ -285,8 +305,9 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
       ub += __shfl_xor_sync(0xffffffffu, ub, o);
       lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
       hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+      maxlen = max(maxlen, __shfl_xor_sync(0xffffffffu, maxlen, o));
     }
-    if (lane == 0) record_row(p, ap, i, e - s, ub, lo, hi, INT_MAX, s_seg, &s_prod, &s_slices, &s_empty);
+    if (lane == 0) record_row(p, ap, i, e - s, ub, lo, hi, maxlen, s_seg, &s_prod, &s_slices, &s_empty);
   }
   __syncthreads();
   flush_counts(p, s_seg, &s_prod, &s_slices, &s_empty);
