@@ -54,6 +54,11 @@ constexpr int kBmrMaxA = 16;
 constexpr int kBmrCap = 512;  // >= kBmrMaxA * 32 products
 constexpr int kBmrSlots = 512;  // rank slots per register bitmap row (one per possible product)
 __host__ __device__ constexpr int bmr_log_words(int b) { return b == 0 ? 7 : b == 1 ? 9 : 11; }
+// Sparsest row the planning pass takes: its sweep and clear cost the same for
+// every row of a launch (the whole bitmap), so rows with fewer products go to
+// the hash bins, whose cost follows the product count.  At 16 words per
+// product a 65,536-column bitmap takes rows of 124 products and more.
+constexpr long long kPlanWordsPerProduct = 16;
 // Smallest register bitmap bin whose bitmap covers `span` columns (span <= kMaxBitmapSpan).
 __host__ __device__ constexpr int bmr_bin_for_span(long long span) {
   return span <= (32ll << bmr_log_words(0)) ? 0 : span <= (32ll << bmr_log_words(1)) ? 1 : 2;
