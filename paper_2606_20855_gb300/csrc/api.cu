@@ -846,7 +846,7 @@ ws_status_t spmspv_impl(ws_csr_s* At, int64_t nx, const int32_t* x_idx, const vo
   const int64_t nb = scan_partials_needed(nx > tiles ? nx : tiles);
   size_t off = 0;
   const size_t o_sum = off; off = align_up(off + sizeof(DevSummary), 256);
-  const size_t o_acc = off; off = align_up(off + sizeof(T) * static_cast<size_t>(m), 256);
+  const size_t o_acc = off; off = align_up(off + sizeof(T) * static_cast<size_t>(m), 256);  // whole 16-byte words
   const size_t o_mark = off; off = align_up(off + static_cast<size_t>(mark_bytes), 256);
   const size_t o_off = off; off = align_up(off + 8 * static_cast<size_t>(nx + 1), 256);
   const size_t o_first = off; off = align_up(off + 8 * static_cast<size_t>(nx), 256);
@@ -879,8 +879,7 @@ ws_status_t spmspv_impl(ws_csr_s* At, int64_t nx, const int32_t* x_idx, const vo
   p.host = pl->host_sum;
   pl->sym_launches = 0;
   pl->num_launches = 0;
-  // zero the summary, the accumulator and the byte-map (contiguous)
-  WS_CUDA(cudaMemsetAsync(b, 0, o_off, s), "cudaMemsetAsync(spmspv scratch)");
+  // the summary block only takes the scans' totals: it need not be cleared
   if (m > 0) {
     launch_spmspv<T>(p, num_sms_of(At->device), s, &pl->num_launches);
     WS_CUDA(cudaGetLastError(), "spmspv launches");

@@ -4,17 +4,21 @@
 // wrapped in a merge level because different columns hit the same positions
 // of y.  Here A is given by columns (the CSR of A^T), and the merge level is
 // the L2: every product is added into one dense accumulator of length m with
-// a global atomic add, and its position is marked in a byte-map (a plain
-// store of 1: idempotent, so positions that many columns hit need no atomic).
+// a global atomic add, and the first add to a position marks it in a byte-map.
 // The coalesce step is a compaction of the byte-map in index order.
 //
-//   1. product offsets: off[k + 1] = length of column x_idx[k] of A, and the
-//      column's first entry; scan -> off[k] = first product of x entry k
+//   1. clear, and product offsets: off[k + 1] = length of column x_idx[k] of A,
+//      and the column's first entry; scan -> off[k] = first product of x entry k
 //   2. scatter: tiles of consecutive products (balanced over the GPU) find
 //      the x entries they span, and every product finds its entry by binary
-//      search in those offsets, then acc[i] += A[i,j] x[j] and mark[i] = 1
-//   3. compaction: marks per tile of 4096 positions -> scan -> every tile
-//      writes its positions (ascending) and accumulated values to y
+//      search in those offsets, then acc[i] += A[i,j] x[j]
+//   3. compaction: marks per tile of 4096 positions, then every tile writes its
+//      positions (ascending) and accumulated values to y
+//
+// The scatter is bound by its scattered L2 transactions, one per product and
+// one more per position of y.  Marking after every add doubled them: 57 us
+// against 37 for 1.6 million products of an R-MAT 2^20 matrix (and as much in
+// fp32 as in fp64).
 #include "ws_internal.cuh"
 
 namespace wsk {
@@ -23,6 +27,7 @@ namespace {
 
 constexpr int kSvThreads = 256;
 constexpr int kSvTile = 4096;  // positions of y per compaction tile (4 KB of the byte-map)
+constexpr int64_t kDirectTiles = 2048;
 
 // Counts the non-zero bytes of 16 bytes.
 __device__ __forceinline__ int marked(const uint4 v) {
@@ -30,20 +35,43 @@ __device__ __forceinline__ int marked(const uint4 v) {
          __popc(__vcmpne4(v.z, 0u) & 0x01010101u) + __popc(__vcmpne4(v.w, 0u) & 0x01010101u);
 }
 
+// The accumulator starts at -0.0.  Adding to a position that still holds it
+// returns it, so whoever adds first marks the position, and only the first
+// adds cost a second scattered store (adds whose results are -0.0 again only
+// mark once more).
+__device__ __forceinline__ bool is_untouched(float old) { return __float_as_uint(old) == 0x80000000u; }
+__device__ __forceinline__ bool is_untouched(double old) {
+  return static_cast<unsigned long long>(__double_as_longlong(old)) == 0x8000000000000000ull;
+}
+
+// The accumulator to -0.0, the byte-map to 0 (n4 and m4 16-byte words), and
+// the length and first entry of the column of every x entry.
 template <typename T>
-__global__ void __launch_bounds__(kSvThreads) sv_offsets_kernel(const SpmspvPlan<T> p) {
-  for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < p.nx;
-       k += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+__global__ void __launch_bounds__(kSvThreads) sv_start_kernel(const SpmspvPlan<T> p, int64_t n4, int64_t m4) {
+  const int64_t first = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  const int64_t step = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  for (int64_t k = first; k < p.nx; k += step) {
     const int64_t j = p.x_idx[k];
-    int64_t len = 0, first = 0;
+    int64_t len = 0, at = 0;
     if (j >= 0 && j < p.n) {
-      first = p.At.rowptr[j];
-      len = p.At.rowptr[j + 1] - first;
+      at = p.At.rowptr[j];
+      len = p.At.rowptr[j + 1] - at;
     } else {
       atomicOr(p.status, kErrCount);  // index outside A's columns: skipped
     }
     p.off[k + 1] = len;
-    p.first[k] = first;
+    p.first[k] = at;
+  }
+  const uint4 none = sizeof(T) == 8 ? make_uint4(0u, 0x80000000u, 0u, 0x80000000u)
+                                    : make_uint4(0x80000000u, 0x80000000u, 0x80000000u, 0x80000000u);
+  uint4* acc = reinterpret_cast<uint4*>(p.acc);
+  uint4* mark = reinterpret_cast<uint4*>(p.mark);
+  for (int64_t i = first; i < n4 + m4; i += step) {
+    if (i < n4) {
+      acc[i] = none;
+    } else {
+      mark[i - n4] = make_uint4(0u, 0u, 0u, 0u);
+    }
   }
 }
 
@@ -70,20 +98,28 @@ __device__ __forceinline__ int64_t warp_last_le(const int64_t* off, int64_t lo, 
 // serialise in L2, and a power-law matrix concentrates its products on a few
 // rows (an R-MAT matrix without vertex permutation on its first rows).  The
 // result is the same for any input; only the speed depends on where the
-// heavy rows lie.
-constexpr int kPerThread = 8;
+// heavy rows lie.  Three CTAs per SM, each over several tiles, and 2048 positions
+// take 92 us for the whole call (R-MAT 2^20, 1.6 million products); 1024
+// positions and a CTA per tile 86 us, but there the sums of the heavy rows are
+// cut into more parts and end further from the exact ones (relative error
+// 1.41e-15 against 1.05e-15 on R-MAT 2^18 with half of x stored; 1.10e-15 with
+// the 4096 positions and tiles of 2048 products used before).
+constexpr int kPerThread = 4;
 constexpr int kScatterTile = kSvThreads * kPerThread;
 constexpr int kScatterSpan = 2048;  // x entries of one tile kept in shared memory
-constexpr int kPrivRows = 4096;     // positions of y summed per CTA in shared memory first
+constexpr int kPrivRows = 2048;     // positions of y summed per CTA in shared memory first
+constexpr int kScatterCtas = 5;     // resident per SM
+constexpr int kScatterGrid = 3;     // launched per SM
 
 template <typename T>
-__global__ void __launch_bounds__(kSvThreads) sv_scatter_kernel(const SpmspvPlan<T> p) {
+__global__ void __launch_bounds__(kSvThreads, kScatterCtas) sv_scatter_kernel(const SpmspvPlan<T> p) {
   __shared__ long long s_off[kScatterSpan + 1];
   __shared__ long long s_k[2];
   __shared__ T s_acc[kPrivRows];
   __shared__ uint8_t s_hit[kPrivRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t total = p.off[p.nx];
+  if (static_cast<int64_t>(blockIdx.x) * kScatterTile >= total) return;
   const int priv = static_cast<int>(p.m < kPrivRows ? p.m : kPrivRows);
   for (int i = threadIdx.x; i < kPrivRows; i += blockDim.x) {
     s_acc[i] = T(0);
@@ -171,8 +207,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_scatter_kernel(const SpmspvPlan
         atomicAdd(s_acc + i, vv[r]);
         s_hit[i] = 1;
       } else {
-        atomicAdd(p.acc + i, vv[r]);
-        p.mark[i] = 1;
+        if (is_untouched(atomicAdd(p.acc + i, vv[r]))) p.mark[i] = 1;
       }
     }
     __syncthreads();  // s_off and s_k are reused by the next tile
@@ -180,8 +215,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_scatter_kernel(const SpmspvPlan
   // The CTA's private sums: one add per position it hit.
   for (int i = threadIdx.x; i < priv; i += blockDim.x) {
     if (s_hit[i]) {
-      atomicAdd(p.acc + i, s_acc[i]);
-      p.mark[i] = 1;
+      if (is_untouched(atomicAdd(p.acc + i, s_acc[i]))) p.mark[i] = 1;
     }
   }
   if (bad) atomicOr(p.status, kErrCount);
@@ -209,44 +243,57 @@ __global__ void __launch_bounds__(kSvThreads) sv_tile_count_kernel(const uint8_t
 }
 
 // Tile t writes its marked positions in ascending order from y offset
-// cnt[t]: warp w takes the tile's positions [512 w, 512 w + 512) in 16 rounds
-// of 32, and ballots give the order.
+// cnt[t]: thread k takes the 16 positions from 16 k on, so a tile costs one
+// round of loads (rounds of 32 positions per warp were a chain of sixteen: 15
+// us for 2^20 positions).
 template <typename T>
-__global__ void __launch_bounds__(kSvThreads) sv_write_kernel(const SpmspvPlan<T> p) {
-  constexpr int kPerWarp = kSvTile / (kSvThreads / 32);  // 512
-  __shared__ long long s_base[kSvThreads / 32 + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__global__ void __launch_bounds__(kSvThreads) sv_write_kernel(const SpmspvPlan<T> p, bool scanned) {
+  __shared__ int scratch[32];
+  __shared__ long long sums[32];
   const int64_t tiles = (p.m + kSvTile - 1) / kSvTile;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    const int64_t i0 = t * kSvTile + static_cast<int64_t>(warp) * kPerWarp;
-    int c = marked(reinterpret_cast<const uint4*>(p.mark + i0)[lane]);
+    const int64_t i0 = t * kSvTile + static_cast<int64_t>(threadIdx.x) * 16;
+    const uint4 v = *reinterpret_cast<const uint4*>(p.mark + i0);
+    const uint32_t word[4] = {v.x, v.y, v.z, v.w};
+    uint32_t set = 0;  // bit b: position i0 + b is marked
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if (lane == 0) s_base[warp + 1] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      s_base[0] = p.cnt[t];
-      for (int w = 0; w < kSvThreads / 32; ++w) s_base[w + 1] += s_base[w];
+    for (int h = 0; h < 4; ++h) {
+      const uint32_t m = __vcmpne4(word[h], 0u) & 0x01010101u;
+      set |= ((m * 0x01020408u) >> 24 & 15u) << (4 * h);  // byte k of the word to bit k
     }
-    __syncthreads();
-    long long pos = s_base[warp];
-    const long long end = p.cnt[t + 1];
-    for (int q = 0; q < kPerWarp / 32; ++q) {
-      const int64_t i = i0 + q * 32 + lane;
-      const bool set = p.mark[i] != 0;
-      const unsigned bal = __ballot_sync(0xffffffffu, set);
-      if (set) {
-        const long long at = pos + __popc(bal & ((1u << lane) - 1u));
-        if (at < end && at < p.cap && i < p.m) {
-          p.y_idx[at] = static_cast<int32_t>(i);
-          p.y_vals[at] = p.acc[i];
+    T acc[16];
+#pragma unroll
+    for (int b = 0; b < 16; ++b) acc[b] = (set >> b) & 1u ? p.acc[i0 + b] + T(0) : T(0);  // + 0: no -0.0 from the start value
+    int total;
+    const int before = block_exclusive_scan(__popc(set), scratch, &total);
+    long long base = 0;  // marked positions of the tiles before
+    if (scanned) {
+      base = p.cnt[t];
+    } else {
+      long long x = 0;
+      for (int64_t q = threadIdx.x; q < t; q += kSvThreads) x += p.cnt[q + 1];
+      block_exclusive_scan(x, sums, &base);
+    }
+    bool bad = false;
+    int k = 0;
+#pragma unroll
+    for (int b = 0; b < 16; ++b) {
+      if ((set >> b) & 1u) {
+        const long long at = base + before + k;
+        if (at < p.cap && i0 + b < p.m) {
+          p.y_idx[at] = static_cast<int32_t>(i0 + b);
+          p.y_vals[at] = acc[b];
         } else {
-          atomicOr(p.status, kErrCount);
+          bad = true;
         }
+        ++k;
       }
-      pos += __popc(bal);
     }
-    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (total != p.cnt[t + 1] - (scanned ? base : 0)) bad = true;
+      if (t == tiles - 1) *const_cast<volatile long long*>(&p.host->nnz) = base + total;
+    }
+    if (bad) atomicOr(p.status, kErrCount);
   }
 }
 
@@ -262,18 +309,22 @@ int64_t spmspv_tiles(int64_t m) { return (m + kSvTile - 1) / kSvTile; }
 
 template <typename T>
 void launch_spmspv(const SpmspvPlan<T>& p, int num_sms, cudaStream_t s, int* launches) {
+  const int64_t tiles = spmspv_tiles(p.m);
+  const int64_t n4 = (p.m * static_cast<int64_t>(sizeof(T)) + 15) / 16, m4 = tiles * kSvTile / 16;
+  sv_start_kernel<T><<<grid_for(n4 + m4 > p.nx ? n4 + m4 : p.nx, kSvThreads, num_sms, 8), kSvThreads, 0, s>>>(p, n4, m4);
   if (p.nx > 0) {
-    sv_offsets_kernel<T><<<grid_for(p.nx, kSvThreads, num_sms, 8), kSvThreads, 0, s>>>(p);
     launch_scan(p.off, p.nx, p.partials, p.sum, s, launches);
     // products are at most nnz(A); the kernel stops at the scanned total
-    sv_scatter_kernel<T><<<grid_for(p.nnz_a, kScatterTile, num_sms, 8), kSvThreads, 0, s>>>(p);
-    *launches += 2;
+    sv_scatter_kernel<T><<<grid_for(p.nnz_a, kScatterTile, num_sms, kScatterGrid), kSvThreads, 0, s>>>(p);
+    *launches += 1;
   }
-  const int64_t tiles = spmspv_tiles(p.m);
+  // Every tile of the last kernel adds up the counts before it; past
+  // kDirectTiles tiles a scan does that once.
+  const bool scanned = tiles > kDirectTiles;
   sv_tile_count_kernel<<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p.mark, p.m, p.cnt);
-  launch_scan(p.cnt, tiles, p.partials, p.sum, s, launches, nullptr, p.host);
-  sv_write_kernel<T><<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p);
-  *launches += 2;
+  if (scanned) launch_scan(p.cnt, tiles, p.partials, p.sum, s, launches);
+  sv_write_kernel<T><<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p, scanned);
+  *launches += 3;
 }
 
 template void launch_spmspv<float>(const SpmspvPlan<float>&, int, cudaStream_t, int*);

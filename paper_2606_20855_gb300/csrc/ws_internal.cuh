@@ -226,8 +226,8 @@ struct SpmspvPlan {
   const T* x_vals;
   int64_t* off;          // [nx + 1]: products per x entry, then scanned in place
   int64_t* first;        // [nx]: first entry of each x entry's column in At
-  T* acc;                // [m]: dense accumulator (zeroed by the host)
-  uint8_t* mark;         // [tiles * 4096]: 1 at the positions of y hit (zeroed by the host)
+  T* acc;                // [m]: dense accumulator
+  uint8_t* mark;         // [tiles * 4096]: 1 at the positions of y hit
   int64_t* cnt;          // [tiles + 1]: set bits per compaction tile, then scanned in place
   int64_t* partials;     // scan scratch for max(nx, tiles) entries
   DevSummary* sum;

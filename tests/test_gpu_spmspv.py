@@ -119,3 +119,30 @@ def test_index_out_of_range_is_reported():
 def test_full_size_workload():
     A, xi, xv = spmspv_workload("spmspv_rmat20")
     check(A, xi, xv)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("m", [1, 15, 4095, 4096, 4097, 70_000])
+def test_signed_zeros_and_tiny_products(dtype, m):
+    """Positions whose products are -0.0, +0.0, subnormal of either sign or
+    cancel exactly stay in y's pattern, for lengths around the compaction tile
+    (4096) and the positions summed in shared memory (1024), more than once on
+    one handle; y holds no -0.0."""
+    rng = np.random.default_rng(m)
+    tiny = np.finfo(dtype).tiny
+    n = 40
+    pool = np.array([-0.0, 0.0, tiny / 4, -tiny / 4, 1.0, -1.0], dtype=dtype)
+    rows, cols = np.nonzero(rng.random((m, n)) < 0.2)
+    rowptr = np.zeros(m + 1, np.int64)
+    np.cumsum(np.bincount(rows, minlength=m), out=rowptr[1:])
+    A = HostCSR(m, n, rowptr, cols.astype(np.int32), rng.choice(pool, size=rows.size))
+    xi = np.arange(0, n, 3, dtype=np.int32)
+    xv = rng.choice(np.array([1.0, -1.0], dtype=dtype), size=xi.size)
+    ref = oracle_spmspv(A, xi, xv)
+    with SpMSpV(DeviceCSR.from_host(transpose_csr(A), torch.device("cuda:0"))) as op:
+        for _ in range(2):
+            yi, yv = run(A, xi, xv, op)
+            np.testing.assert_array_equal(yi, ref.idx)
+            # sums of +-1 and values below the smallest normal number: exact but for the latter
+            assert np.max(np.abs(yv.astype(np.float64) - ref.vals), initial=0.0) <= 40 * tiny
+            assert not np.any(np.signbit(yv) & (yv == 0))
