@@ -225,6 +225,12 @@ __global__ void __launch_bounds__(256) analyze_kernel(const RowPlan<T> p, const 
 template <typename T>
 __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, const AnalyzeParams ap,
                                                            const int32_t* long_rows, DevSummary* host) {
+  const int nlong = *reinterpret_cast<volatile int*>(&p.sum->n_long);
+  const int nmid = *reinterpret_cast<volatile int*>(&p.sum->n_mid);
+  if (nlong == 0 && nmid == 0) {  // no long rows: nothing changes the summary any more
+    if (host && blockIdx.x == 0) publish_summary(p.sum, host, false);
+    return;
+  }
   __shared__ int s_last;
   __shared__ int s_seg[kNumSegs];
   __shared__ long long s_prod, s_slices;
@@ -239,7 +245,6 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int nlong = *reinterpret_cast<volatile int*>(&p.sum->n_long);
   for (int64_t w = blockIdx.x; w < nlong; w += gridDim.x) {
     const int64_t i = long_rows[ap.m - 1 - w];  // long rows fill the list from the back
     const int64_t s = p.A.rowptr[i], e = p.A.rowptr[i + 1];
@@ -281,7 +286,6 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
     }
     __syncthreads();  // s_ub/s_lo/s_hi are reused by the next row
   }
-  const int nmid = *reinterpret_cast<volatile int*>(&p.sum->n_mid);
   const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   for (int64_t w = gw; w < nmid; w += nw) {

@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, sizeof(T) == 8 ? 5 : 7) bmr_
 // a row are stored as uint16 at slot st * G + gl.
 constexpr int kGrpLogW = 7;
 constexpr int kGrpWords = 1 << kGrpLogW;
-constexpr int kGrpChunk = 4;  // steps per warp-uniform branch
+constexpr int kGrpChunk = 8;  // steps per warp-uniform branch (a 2-D or 3-D stencil row takes one round of loads)
 static_assert(32 << kGrpLogW == 32 << bmr_log_words(0), "grouped rows are the rows of bin 0");
 
 // The per-group arrays (entry headers, staging) are padded so that the same
@@ -560,19 +560,26 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, 8) bmr_group_symbolic_kernel
   sm[lane] = 0u;
   __syncwarp();
 
-  const int64_t warps = static_cast<int64_t>(gridDim.x) * kRowsPerCta;
-  for (int64_t r0 = (static_cast<int64_t>(blockIdx.x) * kRowsPerCta + sub) * S::kRows; r0 < p.seg_len;
-       r0 += warps * S::kRows) {
-    const int64_t r = r0 + g;
-    int row = -1, na = 0, lo = 0;
-    long long ra = 0;
-    if (r < p.seg_len) {
-      row = p.perm[p.seg_begin + r];
-      ra = p.A.rowptr[row];
-      const long long n = p.A.rowptr[row + 1] - ra;
-      na = static_cast<int>(n < kBmrMaxA ? n : kBmrMaxA);
-      lo = p.lo[row];
+  // The next rows' numbers and extents are fetched while the current rows are
+  // worked on (two of the five dependent loads a row starts with).
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kRowsPerCta * S::kRows;
+  const int64_t r_first = (static_cast<int64_t>(blockIdx.x) * kRowsPerCta + sub) * S::kRows;
+  auto row_at = [&](int64_t r) { return r < p.seg_len ? p.perm[p.seg_begin + r] : -1; };
+  int row_n = row_at(r_first + g), lo_n = 0;
+  long long ra_n = 0, re_n = 0;
+  auto fetch_extent = [&]() {
+    if (row_n >= 0) {
+      ra_n = p.A.rowptr[row_n];
+      re_n = p.A.rowptr[row_n + 1];
+      lo_n = p.lo[row_n];
     }
+  };
+  fetch_extent();
+  for (int64_t r0 = r_first; r0 < p.seg_len; r0 += stride) {
+    const int row = row_n, lo = lo_n;
+    const long long ra = ra_n, n = row >= 0 ? re_n - ra_n : 0;
+    const int na = static_cast<int>(n < kBmrMaxA ? n : kBmrMaxA);
+    row_n = row_at(r0 + stride + g);
 #pragma unroll
     for (int jj = 0; jj < kBmrMaxA / G; ++jj) {
       const int j = jj * G + gl;
@@ -588,9 +595,10 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, 8) bmr_group_symbolic_kernel
     int nmax = na;
 #pragma unroll
     for (int o = 16; o >= G; o >>= 1) nmax = max(nmax, __shfl_xor_sync(kFull, nmax, o));
+    fetch_extent();
     __syncwarp();
     // Steps in chunks of kGrpChunk behind warp-uniform branches: a stencil
-    // row has 5 stored entries, so most of the 16 steps are skipped.
+    // row has 5 or 7 stored entries, so half of the 16 steps are skipped.
     int col[kBmrMaxA];
 #pragma unroll
     for (int st = 0; st < kBmrMaxA; ++st) col[st] = -1;
@@ -711,20 +719,25 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, 6) bmr_group_numeric_kernel(
   T* h_a = reinterpret_cast<T*>(ws + L::kAOff) + g * S::kHdr;
   int* h_len = reinterpret_cast<int*>(ws + L::kLenOff) + g * S::kHdr;
 
-  const int64_t warps = static_cast<int64_t>(gridDim.x) * kRowsPerCta;
-  for (int64_t r0 = (static_cast<int64_t>(blockIdx.x) * kRowsPerCta + sub) * S::kRows; r0 < p.seg_len;
-       r0 += warps * S::kRows) {
-    const int64_t r = r0 + g;
-    int row = -1, na = 0;
-    long long ra = 0, cbase = 0, want = 0;
-    if (r < p.seg_len) {
-      row = p.perm[p.seg_begin + r];
-      ra = p.A.rowptr[row];
-      const long long n = p.A.rowptr[row + 1] - ra;
-      na = static_cast<int>(n < kBmrMaxA ? n : kBmrMaxA);
-      cbase = p.c_rowptr[row];
-      want = p.c_rowptr[row + 1] - cbase;
+  const int64_t stride = static_cast<int64_t>(gridDim.x) * kRowsPerCta * S::kRows;
+  const int64_t r_first = (static_cast<int64_t>(blockIdx.x) * kRowsPerCta + sub) * S::kRows;
+  auto row_at = [&](int64_t r) { return r < p.seg_len ? p.perm[p.seg_begin + r] : -1; };
+  int row_n = row_at(r_first + g);
+  long long ra_n = 0, re_n = 0, cb_n = 0, ce_n = 0;
+  auto fetch_extent = [&]() {
+    if (row_n >= 0) {
+      ra_n = p.A.rowptr[row_n];
+      re_n = p.A.rowptr[row_n + 1];
+      cb_n = p.c_rowptr[row_n];
+      ce_n = p.c_rowptr[row_n + 1];
     }
+  };
+  fetch_extent();
+  for (int64_t r0 = r_first; r0 < p.seg_len; r0 += stride) {
+    const int row = row_n;
+    const long long ra = ra_n, n = row >= 0 ? re_n - ra_n : 0, cbase = cb_n, want = row >= 0 ? ce_n - cb_n : 0;
+    const int na = static_cast<int>(n < kBmrMaxA ? n : kBmrMaxA);
+    row_n = row_at(r0 + stride + g);
     const int cnt = static_cast<int>(want < kCap ? want : kCap);  // staging bounds every access
     bool bad = want > kCap;
 #pragma unroll
@@ -743,6 +756,7 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, 6) bmr_group_numeric_kernel(
     int nmax = na;
 #pragma unroll
     for (int o = 16; o >= G; o >>= 1) nmax = max(nmax, __shfl_xor_sync(kFull, nmax, o));
+    fetch_extent();
     __syncwarp();
     const uint16_t* ranks = p.ranks + static_cast<int64_t>(row) * kBmrSlots;
     // Chunks of kGrpChunk steps behind warp-uniform branches: all loads of a
@@ -772,11 +786,14 @@ __global__ void __launch_bounds__(32 * kRowsPerCta, 6) bmr_group_numeric_kernel(
             const int rr = rk[u] & 0x7fff;
             if (rr >= cnt) {
               bad = true;
-            } else if (rk[u] & 0x8000) {
-              st_val[rr] += h_a[st] * val[u];
             } else {
-              st_key[rr] = col[u];
-              st_val[rr] = h_a[st] * val[u];
+              // one multiply-add for first products and repeats (a branch
+              // issues two fp64 instructions per step, 16 cycles of the SM
+              // each); -0.0 keeps the sign of a first product that is zero
+              const bool repeat = (rk[u] & 0x8000) != 0;
+              const T before = repeat ? st_val[rr] : T(-0.0);
+              st_val[rr] = fma(h_a[st], val[u], before);
+              if (!repeat) st_key[rr] = col[u];
             }
           }
           __syncwarp();
