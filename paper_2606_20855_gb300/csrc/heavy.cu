@@ -209,18 +209,19 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
 // keep the fp64 pipe busy for 0.8 ms; the rest is the latency of an item's
 // other steps, which three CTAs per SM overlap (windows of 64 KB with two CTAs
 // per SM: 3.9 ms against 3.3 ms).  Columns and values are loaded kAhead rounds
-// before they are added and ranked one round before.  Short parts go to groups
-// of lanes and are added atomically.
+// before they are added and ranked one round before.  Parts of up to 96 entries
+// go to a warp each and are added atomically (R-MAT 2^16 and 2^14 squared: 3.46
+// and 0.405 ms in all; groups of 16 lanes for up to 64 entries 3.51 and 0.429; a
+// warp for up to 256 entries 3.53 and 0.421).
 constexpr int kNumThreads = 256;
 constexpr int kNumCacheA = kNumThreads;       // stored A entries handled at a time
 constexpr int kNumPer = 2;                    // entries per thread and round
 constexpr int kNumPiece = kNumThreads * kNumPer;
 constexpr int kNumDesc = 128;                 // rounds described at a time
 constexpr int kNumWords = kRcdWords / kNumThreads;  // bitmap words per thread
-constexpr int kNumShort = 64;
-constexpr int kNumLanes = 16;  // lanes of a group, four entries each
+constexpr int kNumShort = 96;   // a warp each, three entries per lane
 constexpr int kAhead = 3;
-static_assert(kNumLanes * 4 >= kNumShort, "a short part takes one round of loads");
+static_assert(kNumShort % 32 == 0, "whole entries per lane");
 static_assert(kNumWords == 8, "two 16-byte words of the bitmap per thread");
 
 // One round: entries [b, b + n) of B, times a stored A entry (cached entry j).
@@ -472,21 +473,23 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
         __syncthreads();
       }
       // 4b. short parts
-      for (int j = warp * (32 / kNumLanes) + lane / kNumLanes; j < n; j += kWarps * (32 / kNumLanes)) {
+      constexpr int kPerLane = kNumShort / 32;
+#pragma unroll 2
+      for (int j = warp; j < n; j += kWarps) {
         const int len = s.len[j];
         if (len > kNumShort) continue;
         const T a = s.a[j];
         const long long b0 = s.b0[j];
-        int c[4];
-        T bv[4];
+        int c[kPerLane];
+        T bv[kPerLane];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int t = lane % kNumLanes + u * kNumLanes;
+        for (int u = 0; u < kPerLane; ++u) {
+          const int t = lane + u * 32;
           c[u] = t < len ? p.B.colidx[b0 + t] : -1;
           bv[u] = t < len ? p.B.vals[b0 + t] : T(0);
         }
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < kPerLane; ++u) {
           if (c[u] >= 0) {
             const int q = rank_of(c[u]);
             if (q < kWidth) {

@@ -282,7 +282,7 @@ def test_dense_rows_windows_and_rounds(dtype):
     """Dense heavy rows at the edges of their output windows (49,152 bytes of
     values: one entry less than a window, exactly one, one more, exactly two)
     and of the parts of B rows inside a window: around the short-part limit
-    (64), around one and two rounds (512, 1024), more rounds than are
+    (96), around one and two rounds (512, 1024), more rounds than are
     described at a time (128), and 255, 256 and 257 stored entries (256 are
     cached at a time; the symbolic pass caches 1024)."""
     rng = np.random.default_rng(37)
@@ -291,7 +291,7 @@ def test_dense_rows_windows_and_rounds(dtype):
     perm = rng.permutation(n)
     blocks = [perm[:window - 1], perm[:window], perm[:window + 1], perm[:2 * window]]
     rows = {i: c.tolist() for i, c in enumerate(blocks)}
-    lens = [1, 63, 64, 65, 511, 512, 513, 1023, 1024, 1025, 3000]
+    lens = [1, 32, 33, 95, 96, 97, 511, 512, 513, 1023, 1024, 1025, 3000]
     first_len = len(rows)
     for L in lens:
         rows[len(rows)] = rng.choice(n, size=L, replace=False).tolist()
