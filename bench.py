@@ -237,8 +237,8 @@ def numeric_kernels(info: dict) -> str:
     """Which numeric kernels a plan launches (from ws_spgemm_plan_info)."""
     names = []
     for key, kern in (("direct_rows", "direct_rows_kernel"), ("bitmap_rows", "bmr_numeric/bitmap_rows_kernel"),
-                      ("hash_rows", "hash_rows_kernel"), ("sorted_rows", "sort_rows_kernel"),
-                      ("rcd_rows", "rcd_numeric_kernel"), ("wb_rows", "wb_kernel"), ("dense_rows", "dense_rows_kernel")):
+                      ("hash_rows", "hash_rows_kernel"), ("rcd_rows", "rcd_numeric_kernel"), ("wb_rows", "wb_kernel"),
+                      ("dense_rows", "dense_rows_kernel")):
         if info.get(key):
             names.append(kern)
     return ", ".join(names) or "none"
@@ -475,7 +475,7 @@ def run_spmspv(args, world, rank, local, pg) -> None:
                    "parallelism": f"replicas x{world}" if world > 1 else "single GPU"},
         "phases_ms": {"step_min": round(min(step_ms), 4), "step_median": round(statistics.median(step_ms), 4)},
         "roofline": dict(roofline_obj(algo, statistics.mean(step_ms) / 1e3, peaks, None),
-                         kernel="whole product (offsets, scan, scatter, tile counts, scan, write; read-back included)"),
+                         kernel="whole product (clear and offsets, scan, scatter, tile counts, write; read-back included)"),
         "gpu_launches": int(launches * args.steps),
         "clocks": clk, "e2e": e2e, "cpu_baseline": base,
     }
@@ -715,7 +715,7 @@ def measure(args, name, A, B, steps, warmup, e2e_steps, cpu_s, world, rank, loca
                                                      "read once, C.rowptr written)"),
                              "numeric": dict(roofline_obj(algo_bytes, statistics.mean(num_ms) / 1e3, peaks,
                                                           traffic["numeric"]),
-                                             kernel="numeric pass: " + ("ew_merge_kernel" if ew else
+                                             kernel="numeric pass: " + ("ew_tile_kernel" if ew else
                                                                             numeric_kernels(info))),
                          }),
         "gpu_launches": int(launches_per_step * steps),

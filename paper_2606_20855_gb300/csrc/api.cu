@@ -7,7 +7,7 @@
 //   3. dense     expand dense-window rows into column slices, count (2 launches)
 //   4. hash      count distinct columns per hash bin                (1 launch per non-empty bin)
 //   5. scan      counts -> C.rowptr                                 (1 or 2 launches)
-//   -- read nnz(C) and the status word back (one small copy + stream sync)
+//   -- nnz(C) and the status word reach the host (written by the scan, stream sync)
 // Numeric pass (ws_spgemm_numeric): one launch per non-empty class, no sync.
 #include <cstdarg>
 #include <cstddef>
@@ -289,6 +289,7 @@ struct Plan {
   long long* rcd_items = nullptr;
   uint32_t* rcd_bits = nullptr;
   int rcd_words = 0;
+  int64_t rcd_batch = 0;  // dense heavy rows that rcd_items and rcd_bits have room for
   // submatrix plan (kPlanSub): the block the symbolic pass counted
   int64_t sub_r0 = 0, sub_r1 = 0, sub_c0 = 0, sub_c1 = 0;
   HostSummary* host_sum = nullptr;  // pinned
@@ -530,16 +531,69 @@ uint16_t* hash_ranks_of(const Plan* pl, int b) {
   return static_cast<uint16_t*>(pl->hranks.ptr) + off;
 }
 
+// Most memory that ranks or bitmaps of rows may take between the two passes.
+// They spare the numeric pass a repetition of the symbolic one, but the caller
+// still has to find room for C.  4 GiB holds the ranks of 2^31 products, or
+// the bitmaps of 524,288 rows of 65,536 columns.
+constexpr size_t kMaxKeptBytes = size_t{4} << 30;
+
 // Room for the ranks of the hash rows.  They are an aid, not a need: if the
 // memory is not to be had the numeric pass works them out again.
 void reserve_hash_ranks(Plan* pl, cudaStream_t s) {
   size_t n = 0;
   for (int b = 0; b < kNumHashBins; ++b) n += static_cast<size_t>(pl->seg_count[kSegHash0 + b]) << (kMinHashLog + b);
-  pl->hash_ranked = n > 0 && pl->hranks.reserve(n * sizeof(uint16_t), s) == WS_OK;
+  pl->hash_ranked = n > 0 && n * sizeof(uint16_t) <= kMaxKeptBytes && pl->hranks.reserve(n * sizeof(uint16_t), s) == WS_OK;
   if (n > 0 && !pl->hash_ranked) {
     cudaGetLastError();  // the failed allocation is not an error of this call
     g_last_error.clear();
   }
+}
+
+// Room for the bitmaps and numeric items of the dense heavy rows: of all of
+// them, or else of as many as can be had.  The rows are then taken in batches,
+// and the numeric pass makes the bitmaps again.
+template <typename T>
+ws_status_t carve_rcd(Plan* pl, int64_t ncols, cudaStream_t s) {
+  constexpr int64_t kMinBatch = 1024;
+  const int64_t nr = pl->seg_count[kSegRcd];
+  pl->rcd_words = static_cast<int>(align_up(((ncols < kMaxBitmapSpan ? ncols : kMaxBitmapSpan) + 31) / 32, 4));
+  const int64_t most = static_cast<int64_t>(kMaxKeptBytes / (static_cast<size_t>(pl->rcd_words) * 4));
+  const size_t o_items = align_up(4 * kRcdCounters, 256);
+  for (int64_t n = nr < most ? nr : most;; n = n / 2 < kMinBatch ? kMinBatch : n / 2) {
+    const size_t o_bits = align_up(o_items + 8 * static_cast<size_t>(n) * rcd_slices<T>(), 256);
+    ws_status_t st = pl->rcd.reserve(o_bits + static_cast<size_t>(n) * pl->rcd_words * 4, s);
+    if (st == WS_OK) {
+      char* b = static_cast<char*>(pl->rcd.ptr);
+      pl->rcd_ctr = reinterpret_cast<int32_t*>(b);
+      pl->rcd_items = reinterpret_cast<long long*>(b + o_items);
+      pl->rcd_bits = reinterpret_cast<uint32_t*>(b + o_bits);
+      pl->rcd_batch = n;
+      return WS_OK;
+    }
+    if (st != WS_ERR_ALLOC || n <= kMinBatch) return st;
+    cudaGetLastError();  // the failed allocation is not an error of this call
+    g_last_error.clear();
+  }
+}
+
+// A pass over the dense heavy rows, on stream s.
+template <typename T>
+ws_status_t run_rcd(Plan* pl, RowPlan<T> p, bool numeric, int sms, cudaStream_t s, int* launches) {
+  const int64_t begin = pl->seg_offset[kSegRcd], nr = pl->seg_count[kSegRcd];
+  const bool whole = pl->rcd_batch >= nr;
+  for (int64_t r = 0; r < nr; r += pl->rcd_batch) {
+    p.seg_begin = begin + r;
+    p.seg_len = nr - r < pl->rcd_batch ? nr - r : pl->rcd_batch;
+    if (!numeric || !whole) {
+      p.rcd_again = numeric;
+      WS_CUDA(cudaMemsetAsync(pl->rcd_ctr, 0, kRcdCounters * sizeof(int32_t), s), "cudaMemsetAsync(rcd counters)");
+      launch_rcd<T>(p, false, sms, s, launches);
+    } else {
+      WS_CUDA(cudaMemsetAsync(pl->rcd_ctr + kRcdNextItem, 0, sizeof(int32_t), s), "cudaMemsetAsync(rcd work counter)");
+    }
+    if (numeric) launch_rcd<T>(p, true, sms, s, launches);
+  }
+  return WS_OK;
 }
 
 // Row kernels of a pass (the symbolic pass has none for direct and planned rows).
@@ -572,17 +626,8 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     if (st != WS_OK) return st;
   }
   if (pl->seg_count[kSegRcd] > 0) {
-    const int64_t nr = pl->seg_count[kSegRcd];
-    const size_t o_items = align_up(4 * kRcdCounters, 256);
-    const size_t o_bits = align_up(o_items + 8 * static_cast<size_t>(nr) * rcd_slices<T>(), 256);
-    pl->rcd_words = static_cast<int>(align_up(((B->ncols < kMaxBitmapSpan ? B->ncols : kMaxBitmapSpan) + 31) / 32, 4));
-    st = pl->rcd.reserve(o_bits + static_cast<size_t>(nr) * pl->rcd_words * 4, s);
+    st = carve_rcd<T>(pl, B->ncols, s);
     if (st != WS_OK) return st;
-    char* b = static_cast<char*>(pl->rcd.ptr);
-    pl->rcd_ctr = reinterpret_cast<int32_t*>(b);
-    pl->rcd_items = reinterpret_cast<long long*>(b + o_items);
-    pl->rcd_bits = reinterpret_cast<uint32_t*>(b + o_bits);
-    WS_CUDA(cudaMemsetAsync(pl->rcd_ctr, 0, kRcdCounters * sizeof(int32_t), s), "cudaMemsetAsync(rcd counters)");
   }
   reserve_hash_ranks(pl, s);
   p = make_rowplan<T>(A, B, C, pl);
@@ -592,7 +637,10 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     p.seg_len = pl->seg_count[g];
     return p.seg_len > 0;
   };
-  if (segment(kSegRcd)) launch_rcd<T>(p, false, sms, fork.next(), &pl->sym_launches);
+  if (segment(kSegRcd)) {
+    st = run_rcd<T>(pl, p, false, sms, fork.next(), &pl->sym_launches);
+    if (st != WS_OK) return st;
+  }
   if (segment(kSegWb)) launch_wb<T>(p, false, sms, fork.next(), &pl->sym_launches);
   if (segment(kSegDense)) {
     const cudaStream_t q = fork.next();
@@ -705,15 +753,16 @@ ws_status_t numeric_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan
   const int sms = num_sms_of(C->device);
   pl->num_launches = 0;
   RowPlan<T> p = make_rowplan<T>(A, B, C, pl);
-  if (pl->seg_count[kSegRcd] > 0)
-    WS_CUDA(cudaMemsetAsync(pl->rcd_ctr + kRcdNextItem, 0, sizeof(int32_t), s), "cudaMemsetAsync(rcd work counter)");
   Fork fork(s, C->device, bin_launches(pl, true));
   auto segment = [&](int g) {
     p.seg_begin = pl->seg_offset[g];
     p.seg_len = pl->seg_count[g];
     return p.seg_len > 0;
   };
-  if (segment(kSegRcd)) launch_rcd<T>(p, true, sms, fork.next(), &pl->num_launches);
+  if (segment(kSegRcd)) {
+    const ws_status_t st = run_rcd<T>(pl, p, true, sms, fork.next(), &pl->num_launches);
+    if (st != WS_OK) return st;
+  }
   if (segment(kSegWb)) launch_wb<T>(p, true, sms, fork.next(), &pl->num_launches);
   if (segment(kSegDense)) launch_dense<T>(p, pl->dense_slices, true, sms, fork.next(), &pl->num_launches);
   if (segment(kSegBmrWide)) {

@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
     if (threadIdx.x == 0) {
       const int total = static_cast<int>(sums & 0xffffffffll);
       const bool big = (sums >> 32) > kRcdBigProducts;
-      p.c_rowptr[row + 1] = total;
+      if (!p.rcd_again) p.c_rowptr[row + 1] = total;
       const int nw = (total + kWidth - 1) / kWidth;
       const long long cap = static_cast<long long>(p.seg_len) * kS;
       if (big) {

@@ -175,6 +175,7 @@ struct RowPlan {
   int rcd_words;               // a multiple of 4, enough for min(columns of B, kMaxBitmapSpan)
   long long* rcd_items;        // their numeric work items (row * rcd_slices<T>() + window): rows with many products
                                // from the front, the others from the back of seg_len * rcd_slices<T>() places
+  bool rcd_again;              // their bitmaps and items are wanted once more, the counts stand
   int32_t* rcd_ctr;            // counters kRcdBigItems .. kRcdNextItem
   DevSummary* sum;
   int* status;         // error flags (pinned host memory)

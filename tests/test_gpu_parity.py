@@ -372,6 +372,57 @@ def test_hash_rows_bin_edges(dtype, run_limit):
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+def test_dense_rows_without_room_for_bitmaps():
+    """With almost all device memory taken the bitmaps of the dense heavy rows
+    do not fit: the rows are taken in batches, and the numeric pass makes the
+    bitmaps again (more launches, the same C).  (A process of its own: an
+    earlier test's freed scratch would serve.)"""
+    import subprocess
+    import sys
+    code = """
+import numpy as np, torch
+from tests._gpu import assert_matches_oracle
+from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+from synth import HostCSR
+rng = np.random.default_rng(39)
+k, n, m = 1400, 1 << 16, 12001  # 98 MB of bitmaps, an odd last batch
+lens = rng.integers(0, 140, size=k)
+brp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+bci = np.concatenate([np.sort(rng.choice(n, size=x, replace=False)) for x in lens]).astype(np.int32)
+B = HostCSR(k, n, brp, bci, 2 * rng.random(bci.size) - 1)
+aci = np.sort(rng.random((m, k)).argsort(axis=1)[:, :100], axis=1).astype(np.int32).ravel()
+A = HostCSR(m, k, np.arange(m + 1, dtype=np.int64) * 100, aci, 2 * rng.random(aci.size) - 1)
+dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+def product(hog):
+    op = SpGEMM(dA, dB)
+    held = []
+    if hog:
+        size = 1 << 30
+        while size >= 1 << 24:  # leave less than 56 MB
+            if torch.cuda.mem_get_info()[0] - size > 40 << 20:
+                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            else:
+                size >>= 1
+    op.symbolic()
+    del held
+    torch.cuda.empty_cache()
+    C = op.numeric()
+    op.wait()
+    return op, C.to_host()
+op2, (rp2, ci2, v2) = product(False)  # kept: its scratch stays taken
+op1, (rp1, ci1, v1) = product(True)
+i1, i2 = op1.plan_info(), op2.plan_info()
+assert i1["rcd_rows"] == i2["rcd_rows"] > 11900
+assert i1["numeric_launches"] > i2["numeric_launches"]
+assert np.array_equal(rp1, rp2) and np.array_equal(ci1, ci2)
+assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.concatenate([np.arange(0, m, 101), [m - 1]]))
+"""
+    import os
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-2000:]
+
+
 def test_hash_rows_without_room_for_ranks():
     """With almost all device memory taken the symbolic pass cannot keep the
     ranks of the hash rows and the numeric pass works them out: the same C.
