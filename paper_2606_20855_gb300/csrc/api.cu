@@ -276,6 +276,7 @@ struct Plan {
   DevBuf sv;      // sparse matrix - sparse vector product (in A^T's handle): accumulator, byte-map, offsets
   DevBuf hranks;  // hash rows: uint16 ranks of their products, one block per bin
   DevBuf rcd;     // dense heavy rows: work counters, numeric items, the rows' bitmaps
+  DevBuf wb;      // wide-bitmap rows: work counters, numeric items, the rows' bitmaps
   int kind = kPlanNone;  // which symbolic pass filled this plan
   // elementwise plan (kPlanEwise)
   int ew_op = 0;
@@ -289,6 +290,11 @@ struct Plan {
   long long* rcd_items = nullptr;
   uint32_t* rcd_bits = nullptr;
   int rcd_words = 0;
+  int32_t* wb_ctr = nullptr;
+  long long* wb_items = nullptr;
+  uint32_t* wb_bits = nullptr;
+  int wb_words = 0;
+  int64_t wb_cap = 0;
   int64_t rcd_batch = 0;  // dense heavy rows that rcd_items and rcd_bits have room for
   // submatrix plan (kPlanSub): the block the symbolic pass counted
   int64_t sub_r0 = 0, sub_r1 = 0, sub_c0 = 0, sub_c1 = 0;
@@ -328,7 +334,7 @@ struct Plan {
 
   size_t scratch_bytes() const {
     size_t n = 0;
-    for (const DevBuf* b : {&rows, &slices, &ranks, &ew, &sv, &hranks, &rcd}) n += b->bytes;
+    for (const DevBuf* b : {&rows, &slices, &ranks, &ew, &sv, &hranks, &rcd, &wb}) n += b->bytes;
     return n;
   }
   // Back to a new plan that owns the same scratch and pinned block.
@@ -341,6 +347,7 @@ struct Plan {
     fresh.sv = sv;
     fresh.hranks = hranks;
     fresh.rcd = rcd;
+    fresh.wb = wb;
     fresh.host_sum = host_sum;
     fresh.slot = slot;
     fresh.clean_buf = clean_buf;  // points into this object, whose address stays
@@ -477,6 +484,11 @@ RowPlan<T> make_rowplan(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan*
   p.rcd_items = pl->rcd_items;
   p.rcd_bits = pl->rcd_bits;
   p.rcd_words = pl->rcd_words;
+  p.wb_ctr = pl->wb_ctr;
+  p.wb_items = pl->wb_items;
+  p.wb_bits = pl->wb_bits;
+  p.wb_words = pl->wb_words;
+  p.wb_cap = pl->wb_cap;
   p.sum = pl->dsum;
   p.status = status_word(pl);
   p.log2_group = pl->log2_group;
@@ -576,6 +588,30 @@ ws_status_t carve_rcd(Plan* pl, int64_t ncols, cudaStream_t s) {
   }
 }
 
+// Room for the numeric items of the wide-bitmap rows and, if it can be had,
+// for their bitmaps.
+ws_status_t carve_wb(Plan* pl, int64_t ncols, cudaStream_t s) {
+  const int64_t nr = pl->seg_count[kSegWb];
+  pl->wb_words = static_cast<int>(align_up(((ncols < kWbMaxSpan ? ncols : kWbMaxSpan) + 31) / 32, 4));
+  pl->wb_cap = nr + pl->products / kWbPart;
+  const size_t o_items = align_up(4 * kWbCounters, 256);
+  const size_t o_bits = align_up(o_items + 8 * static_cast<size_t>(pl->wb_cap), 256);
+  const size_t bits = static_cast<size_t>(nr) * pl->wb_words * 4;
+  bool kept = bits <= kMaxKeptBytes && pl->wb.reserve(o_bits + bits, s) == WS_OK;
+  if (!kept) {
+    cudaGetLastError();  // the failed allocation is not an error of this call
+    g_last_error.clear();
+    ws_status_t st = pl->wb.reserve(o_bits, s);
+    if (st != WS_OK) return st;
+  }
+  char* b = static_cast<char*>(pl->wb.ptr);
+  pl->wb_ctr = reinterpret_cast<int32_t*>(b);
+  pl->wb_items = reinterpret_cast<long long*>(b + o_items);
+  pl->wb_bits = kept ? reinterpret_cast<uint32_t*>(b + o_bits) : nullptr;
+  WS_CUDA(cudaMemsetAsync(pl->wb_ctr, 0, kWbCounters * sizeof(int32_t), s), "cudaMemsetAsync(wide row counters)");
+  return WS_OK;
+}
+
 // A pass over the dense heavy rows, on stream s.
 template <typename T>
 ws_status_t run_rcd(Plan* pl, RowPlan<T> p, bool numeric, int sms, cudaStream_t s, int* launches) {
@@ -627,6 +663,10 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
   }
   if (pl->seg_count[kSegRcd] > 0) {
     st = carve_rcd<T>(pl, B->ncols, s);
+    if (st != WS_OK) return st;
+  }
+  if (pl->seg_count[kSegWb] > 0) {
+    st = carve_wb(pl, B->ncols, s);
     if (st != WS_OK) return st;
   }
   reserve_hash_ranks(pl, s);
@@ -753,6 +793,8 @@ ws_status_t numeric_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan
   const int sms = num_sms_of(C->device);
   pl->num_launches = 0;
   RowPlan<T> p = make_rowplan<T>(A, B, C, pl);
+  if (pl->seg_count[kSegWb] > 0)
+    WS_CUDA(cudaMemsetAsync(pl->wb_ctr + kWbNextItem, 0, sizeof(int32_t), s), "cudaMemsetAsync(wide row counter)");
   Fork fork(s, C->device, bin_launches(pl, true));
   auto segment = [&](int g) {
     p.seg_begin = pl->seg_offset[g];
@@ -1009,7 +1051,7 @@ void release_outer(Plan* pl, cudaStream_t s) {
 void release_plan_async(Plan* pl, cudaStream_t s) {
   if (!pl) return;
   release_outer(pl, s);
-  DevBuf* bufs[] = {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd};
+  DevBuf* bufs[] = {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd, &pl->wb};
   for (DevBuf* b : bufs) {
     if (b->ptr) cudaFreeAsync(b->ptr, s);
     b->ptr = nullptr;
@@ -1517,7 +1559,7 @@ ws_status_t ws_csr_destroy(ws_csr_t h) {
     if (pl->scratch_bytes() > 0 || pl->outer) idle = cudaDeviceSynchronize() == cudaSuccess;
     release_outer(pl, nullptr);
     if (!idle || !keep_plan(pl)) {
-      for (DevBuf* b : {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd}) b->release();
+      for (DevBuf* b : {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd, &pl->wb}) b->release();
       release_host_sum(pl->host_sum);
       delete pl;
     }

@@ -19,11 +19,13 @@
 //
 // Wide rows (kClsWb): column range up to 2^20 columns.  A bitmap over the
 // whole range (one bit per column) is the workspace:
-//   symbolic: atomicOr every product column, count the bits that were 0.
-//   numeric:  set the bits, rank the bitmap in 128-bit chunks, write C's
-//             column indices in order straight from the bitmap, zero C's
-//             values, and let every product add its value at the rank of its
-//             column in C (global atomic add; the row's segment is private).
+//   symbolic: atomicOr every product column, count the bits that were 0; the
+//             bitmap stays in the plan if there is room.
+//   numeric:  read the bitmap back (or set the bits again), rank it in 128-bit
+//             chunks, write C's column indices in order straight from it, zero
+//             C's values, and let every product add its value at the rank of its
+//             column in C (global atomic add).  The products of a row of more
+//             than kWbPart are cut into parts, an item each.
 #include <climits>
 #include <cstddef>
 
@@ -511,141 +513,211 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
 
 // ----------------------------------------------------------------- wide rows
 
-template <typename T, bool NUMERIC>
-__global__ void __launch_bounds__(kWbThreads, 1) wb_kernel(const RowPlan<T> p) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  uint32_t* bm = reinterpret_cast<uint32_t*>(smem_raw);          // kWbMaxSpan / 32 words
-  uint4* bm4 = reinterpret_cast<uint4*>(smem_raw);
-  uint32_t* pre = bm + kWbMaxSpan / 32;                           // one prefix per 128-bit chunk
-  __shared__ long long s_scan[32];
+// Measured on R-MAT 2^20 (edge factor 8, fp64) times rows of 4 entries, 1,048
+// such rows of 12,500 products on average and 93,000 at most: symbolic 95 us,
+// numeric 186 us and 7 us for the zeroes.  A CTA per row that also set the bits
+// again in the numeric pass, one thread writing the columns of 8 consecutive
+// chunks, took 87 and 361 us, bound by its longest row.  Storing the bitmaps
+// (137 MB) costs the symbolic pass 8 us.  Bound by the latency of a round's
+// three dependent loads.
+
+// Calls f(column, value of B, value of A) for the products of the stored A
+// entries [ra, re).  A group of lanes takes kWbBatch entries per round, so
+// their row-pointer loads and then their columns and values are in flight
+// together (a hub row has tens of thousands of entries).
+template <typename T, bool VALUES, typename F>
+__device__ __forceinline__ void wb_products(const RowPlan<T>& p, int64_t ra, int64_t re, F&& f) {
   const int lg = p.log2_group;
   const int gsize = 1 << lg;
   const int grp = threadIdx.x >> lg;
   const int gl = threadIdx.x & (gsize - 1);
   const int ngrp = kWbThreads >> lg;
+  for (int64_t pa0 = ra + grp; pa0 < re; pa0 += static_cast<int64_t>(kWbBatch) * ngrp) {
+    int64_t qb[kWbBatch];
+    int len[kWbBatch], most = 0;
+    T av[kWbBatch];
+#pragma unroll
+    for (int u = 0; u < kWbBatch; ++u) {
+      const int64_t pa = pa0 + static_cast<int64_t>(u) * ngrp;
+      qb[u] = 0;
+      len[u] = 0;
+      av[u] = T(0);
+      if (pa < re) {
+        const int k = p.A.colidx[pa];
+        if constexpr (VALUES) av[u] = p.A.vals[pa];
+        qb[u] = p.B.rowptr[k];
+        len[u] = static_cast<int>(p.B.rowptr[k + 1] - qb[u]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kWbBatch; ++u) most = max(most, len[u]);
+    for (int t = gl; t < most; t += gsize) {
+      int c[kWbBatch];
+      T bv[kWbBatch];
+#pragma unroll
+      for (int u = 0; u < kWbBatch; ++u) {
+        c[u] = t < len[u] ? p.B.colidx[qb[u] + t] : -1;
+        bv[u] = VALUES && t < len[u] ? p.B.vals[qb[u] + t] : T(0);
+      }
+#pragma unroll
+      for (int u = 0; u < kWbBatch; ++u) {
+        if (c[u] >= 0) f(c[u], bv[u], av[u]);
+      }
+    }
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kWbThreads, 1) wb_symbolic_kernel(const RowPlan<T> p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* bm = reinterpret_cast<uint32_t*>(smem_raw);  // kWbMaxSpan / 32 words
+  uint4* bm4 = reinterpret_cast<uint4*>(smem_raw);
+  __shared__ long long s_scan[32];
+  constexpr int kShift = 24;
+  static_assert(kWbMaxSpan < 1 << kShift, "a row's entries fit below its products");
   for (int i = threadIdx.x; i < kWbMaxSpan / 128; i += kWbThreads) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   for (int64_t r = blockIdx.x; r < p.seg_len; r += gridDim.x) {
     const int32_t row = p.perm[p.seg_begin + r];
     const int lo = p.lo[row];
-    const int span = p.hi[row] - lo + 1;
-    const int nchunks = (span + 127) >> 7;
-    const int64_t ra = p.A.rowptr[row], re = p.A.rowptr[row + 1];
-    int64_t cbase = 0, cend = 0;
-    if constexpr (NUMERIC) {
-      cbase = p.c_rowptr[row];
-      cend = p.c_rowptr[row + 1];
-      for (int64_t i = cbase + threadIdx.x; i < cend; i += kWbThreads) p.c_vals[i] = T(0);
+    const int nchunks = (p.hi[row] - lo + 128) >> 7;
+    long long sums = 0;  // entries in the low bits, products above them
+    wb_products<T, false>(p, p.A.rowptr[row], p.A.rowptr[row + 1], [&](int c, T, T) {
+      const uint32_t off = static_cast<uint32_t>(c - lo);
+      const uint32_t bit = 1u << (off & 31u);
+      sums += (1ll << kShift) + ((atomicOr(bm + (off >> 5), bit) & bit) == 0u);
+    });
+    __syncthreads();
+    long long total;
+    block_exclusive_scan(sums, s_scan, &total);
+    if (threadIdx.x == 0) {
+      p.c_rowptr[row + 1] = total & ((1ll << kShift) - 1);
+      const long long products = total >> kShift;
+      const int parts = !p.wb_bits ? 1 : static_cast<int>(min((products + kWbPart - 1) / kWbPart, static_cast<long long>(kWbMaxParts)));
+      const int at = atomicAdd(&p.wb_ctr[parts > 1 ? kWbBigItems : kWbItems], parts);
+      for (int q = 0; q < parts; ++q) {
+        p.wb_items[parts > 1 ? at + q : p.wb_cap - 1 - at - q] = r << 32 | static_cast<long long>(q) << 16 | parts;
+      }
     }
-    // Set the bit of every product column.  A group takes kWbBatch stored A
-    // entries per round, so their row-pointer and column loads are in flight
-    // together (a hub row has tens of thousands of entries).
-    long long fresh = 0;
-    for (int64_t pa0 = ra + grp; pa0 < re; pa0 += static_cast<int64_t>(kWbBatch) * ngrp) {
-      int64_t qb[kWbBatch], qe[kWbBatch];
-#pragma unroll
-      for (int u = 0; u < kWbBatch; ++u) {
-        const int64_t pa = pa0 + static_cast<int64_t>(u) * ngrp;
-        qb[u] = 0;
-        qe[u] = 0;
-        if (pa < re) {
-          const int k = p.A.colidx[pa];
-          qb[u] = p.B.rowptr[k];
-          qe[u] = p.B.rowptr[k + 1];
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kWbBatch; ++u) {
-        for (int64_t q = qb[u] + gl; q < qe[u]; q += gsize) {
-          const uint32_t off = static_cast<uint32_t>(p.B.colidx[q] - lo);
-          const uint32_t bit = 1u << (off & 31u);
-          if constexpr (NUMERIC) {
-            atomicOr(bm + (off >> 5), bit);
-          } else {
-            fresh += (atomicOr(bm + (off >> 5), bit) & bit) == 0u;
-          }
-        }
-      }
+    uint4* bits = reinterpret_cast<uint4*>(p.wb_bits ? p.wb_bits + r * p.wb_words : nullptr);
+    for (int i = threadIdx.x; i < nchunks; i += kWbThreads) {
+      if (bits) bits[i] = bm4[i];
+      bm4[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
-    if constexpr (!NUMERIC) {
-      long long total;
-      block_exclusive_scan(fresh, s_scan, &total);
-      if (threadIdx.x == 0) p.c_rowptr[row + 1] = total;
-      for (int i = threadIdx.x; i < nchunks; i += kWbThreads) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
+// Zeroes the values of the rows that several items add to.
+template <typename T>
+__global__ void __launch_bounds__(256) wb_zero_kernel(const RowPlan<T> p) {
+  const int nbig = p.wb_ctr[kWbBigItems];
+  for (int it = blockIdx.x; it < nbig; it += gridDim.x) {
+    const long long item = p.wb_items[it];
+    const int32_t row = p.perm[p.seg_begin + (item >> 32)];
+    const long long q = item >> 16 & 0xffff, parts = item & 0xffff;
+    const int64_t c0 = p.c_rowptr[row], n = p.c_rowptr[row + 1] - c0;
+    for (int64_t i = n * q / parts + threadIdx.x; i < n * (q + 1) / parts; i += 256) p.c_vals[c0 + i] = T(0);
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kWbThreads, 1) wb_numeric_kernel(const RowPlan<T> p) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  uint32_t* bm = reinterpret_cast<uint32_t*>(smem_raw);          // kWbMaxSpan / 32 words
+  uint4* bm4 = reinterpret_cast<uint4*>(smem_raw);
+  uint32_t* pre = bm + kWbMaxSpan / 32;                           // one prefix per 128-bit chunk
+  __shared__ long long s_scan[32];
+  __shared__ int s_item;
+  const int lane = static_cast<int>(threadIdx.x) & 31, warp = static_cast<int>(threadIdx.x) >> 5;
+  const int nbig = p.wb_ctr[kWbBigItems], nitems = nbig + p.wb_ctr[kWbItems];
+  bool bad = false;
+  for (int guard = 0; guard <= nitems; ++guard) {
+    __syncthreads();  // the previous item is done with the shared state
+    if (threadIdx.x == 0) s_item = atomicAdd(&p.wb_ctr[kWbNextItem], 1);
+    __syncthreads();
+    const int it = s_item;
+    if (it >= nitems) break;
+    const long long item = it < nbig ? p.wb_items[it] : p.wb_items[p.wb_cap - 1 - (it - nbig)];
+    const int64_t r = item >> 32, part = item >> 16 & 0xffff, parts = item & 0xffff;
+    const int32_t row = p.perm[p.seg_begin + r];
+    const int lo = p.lo[row];
+    const int nchunks = (p.hi[row] - lo + 128) >> 7;
+    const int64_t ra = p.A.rowptr[row], na = p.A.rowptr[row + 1] - ra;
+    const int64_t cbase = p.c_rowptr[row], cend = p.c_rowptr[row + 1];
+    if (parts == 1) {
+      for (int64_t i = cbase + threadIdx.x; i < cend; i += kWbThreads) p.c_vals[i] = T(0);
+    }
+    // 1. the row's bitmap: from the plan, or made again
+    const uint4* bits = reinterpret_cast<const uint4*>(p.wb_bits ? p.wb_bits + r * p.wb_words : nullptr);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < nchunks; i += kWbThreads) bm4[i] = bits ? bits[i] : make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    if (!bits) {
+      wb_products<T, false>(p, ra, ra + na, [&](int c, T, T) {
+        const uint32_t off = static_cast<uint32_t>(c - lo);
+        atomicOr(bm + (off >> 5), 1u << (off & 31u));
+      });
       __syncthreads();
-    } else {
-      // Rank the chunks: thread t owns a run of consecutive chunks.
-      const int per = (nchunks + kWbThreads - 1) / kWbThreads;
-      const int my0 = threadIdx.x * per;
-      const int my1 = min(my0 + per, nchunks);
-      long long mine = 0;
-      for (int i = my0; i < my1; ++i) {
+    }
+    // 2. the chunks' ranks.  A warp owns consecutive chunks, 32 at a time.
+    const int per = (nchunks + kWbThreads - 1) / kWbThreads;
+    const int first = warp * per * 32 + lane;
+    int mine = 0;
+    for (int j = 0; j < per; ++j) {
+      const int i = first + j * 32;
+      if (i < nchunks) {
         const uint4 v = bm4[i];
         mine += __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
       }
-      long long total;
-      long long run = block_exclusive_scan(mine, s_scan, &total);
-      bool bad = total != cend - cbase;
-      // Write the column indices in order and keep each chunk's prefix.
-      for (int i = my0; i < my1; ++i) {
-        pre[i] = static_cast<uint32_t>(run);
-        const uint4 v = bm4[i];
+    }
+    long long total;
+    long long run = block_exclusive_scan(static_cast<long long>(mine), s_scan, &total);
+    run = __shfl_sync(0xffffffffu, run, 0);  // entries before the warp's chunks
+    bad |= total != cend - cbase;
+    // The part's share of the columns is written on the way.
+    const int e0 = static_cast<int>(nchunks * part / parts), e1 = static_cast<int>(nchunks * (part + 1) / parts);
+    for (int j = 0; j < per; ++j) {
+      const int i = first + j * 32;
+      const uint4 v = i < nchunks ? bm4[i] : make_uint4(0u, 0u, 0u, 0u);
+      const int n = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+      int upto = n;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, upto, d);
+        if (lane >= d) upto += x;
+      }
+      int64_t pos = cbase + run + upto - n;
+      if (i < nchunks) pre[i] = static_cast<uint32_t>(pos - cbase);
+      if (i >= e0 && i < e1) {
         const uint32_t wv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          uint32_t x = wv[q];
-          while (x) {
-            const int b = __ffs(x) - 1;
-            x &= x - 1u;
-            const int64_t pos = cbase + run;
-            if (pos < cend) p.c_colidx[pos] = lo + (i << 7) + (q << 5) + b;
-            ++run;
+          for (uint32_t x = wv[q]; x; x &= x - 1u, ++pos) {
+            if (pos < cend) p.c_colidx[pos] = lo + (i << 7) + (q << 5) + __ffs(x) - 1;
           }
         }
       }
-      __syncthreads();  // prefixes and the zeroed values are visible to the CTA
-      for (int64_t pa0 = ra + grp; pa0 < re; pa0 += static_cast<int64_t>(kWbBatch) * ngrp) {
-        int64_t qb[kWbBatch], qe[kWbBatch];
-        T avs[kWbBatch];
-#pragma unroll
-        for (int u = 0; u < kWbBatch; ++u) {
-          const int64_t pa = pa0 + static_cast<int64_t>(u) * ngrp;
-          qb[u] = 0;
-          qe[u] = 0;
-          avs[u] = T(0);
-          if (pa < re) {
-            const int k = p.A.colidx[pa];
-            avs[u] = p.A.vals[pa];
-            qb[u] = p.B.rowptr[k];
-            qe[u] = p.B.rowptr[k + 1];
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kWbBatch; ++u) {
-        const T av = avs[u];
-        for (int64_t q = qb[u] + gl; q < qe[u]; q += gsize) {
-          const uint32_t off = static_cast<uint32_t>(p.B.colidx[q] - lo);
-          const uint32_t i = off >> 7;
-          const uint4 v = bm4[i];
-          const uint32_t wq = (off >> 5) & 3u;
-          const uint32_t wd = wq == 0 ? v.x : wq == 1 ? v.y : wq == 2 ? v.z : v.w;
-          const int64_t pos = cbase + pre[i] + (wq > 0 ? __popc(v.x) : 0) + (wq > 1 ? __popc(v.y) : 0) +
-                              (wq > 2 ? __popc(v.z) : 0) + __popc(wd & ((1u << (off & 31u)) - 1u));
-          if (pos < cend) {
-            atomicAdd(p.c_vals + pos, av * p.B.vals[q]);
-          } else {
-            bad = true;
-          }
-        }
-        }
-      }
-      if (bad) atomicOr(p.status, kErrCount);
-      __syncthreads();
-      for (int i = threadIdx.x; i < nchunks; i += kWbThreads) bm4[i] = make_uint4(0u, 0u, 0u, 0u);
-      __syncthreads();
+      run += __shfl_sync(0xffffffffu, upto, 31);
     }
+    __syncthreads();  // prefixes and the zeroed values are visible to the CTA
+    // 3. the part's products
+    wb_products<T, true>(p, ra + na * part / parts, ra + na * (part + 1) / parts, [&](int c, T b, T a) {
+      const uint32_t off = static_cast<uint32_t>(c - lo);
+      const uint32_t i = off >> 7;
+      const uint4 v = bm4[i];
+      const uint32_t wq = (off >> 5) & 3u;
+      const uint32_t wd = wq == 0 ? v.x : wq == 1 ? v.y : wq == 2 ? v.z : v.w;
+      const int64_t pos = cbase + pre[i] + (wq > 0 ? __popc(v.x) : 0) + (wq > 1 ? __popc(v.y) : 0) +
+                          (wq > 2 ? __popc(v.z) : 0) + __popc(wd & ((1u << (off & 31u)) - 1u));
+      if (pos < cend) {
+        atomicAdd(p.c_vals + pos, a * b);
+      } else {
+        bad = true;
+      }
+    });
   }
+  if (bad) atomicOr(p.status, kErrCount);
 }
 
 template <typename K>
@@ -684,12 +756,23 @@ void launch_rcd(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, 
 
 template <typename T>
 void launch_wb(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, int* launches) {
-  const size_t smem = kWbMaxSpan / 8 + (kWbMaxSpan / 128) * 4;
-  auto kern = numeric ? wb_kernel<T, true> : wb_kernel<T, false>;
-  static int per_sm[2] = {0, 0};
-  if (per_sm[numeric] == 0) per_sm[numeric] = occupancy(kern, kWbThreads, smem);
-  kern<<<grid_of(p.seg_len, num_sms, per_sm[numeric]), kWbThreads, smem, s>>>(p);
-  *launches += 1;
+  if (!numeric) {
+    const size_t smem = kWbMaxSpan / 8;
+    static int per_sm = 0;
+    if (per_sm == 0) per_sm = occupancy(wb_symbolic_kernel<T>, kWbThreads, smem);
+    wb_symbolic_kernel<T><<<grid_of(p.seg_len, num_sms, per_sm), kWbThreads, smem, s>>>(p);
+    *launches += 1;
+  } else {
+    const size_t smem = kWbMaxSpan / 8 + (kWbMaxSpan / 128) * 4;
+    static int per_sm = 0;
+    if (per_sm == 0) per_sm = occupancy(wb_numeric_kernel<T>, kWbThreads, smem);
+    if (p.wb_bits) {
+      wb_zero_kernel<T><<<grid_of(p.wb_cap, num_sms, 8), 256, 0, s>>>(p);
+      *launches += 1;
+    }
+    wb_numeric_kernel<T><<<grid_of(p.wb_cap, num_sms, per_sm), kWbThreads, smem, s>>>(p);
+    *launches += 1;
+  }
 }
 
 template void launch_rcd<float>(const RowPlan<float>&, bool, int, cudaStream_t, int*);

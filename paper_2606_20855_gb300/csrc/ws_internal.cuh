@@ -81,6 +81,10 @@ constexpr int kRcdDefaultMaxA = 8192;     // default limit used by the classific
 constexpr int kRcdWidthBytes = 49152;     // value window of one item of a dense heavy row
 // Counters of the dense heavy rows: items of rows with many products, other
 // items, next row of the symbolic pass, next item of the numeric pass.
+// Wide-bitmap rows: products per numeric item, most items of a row, counters.
+constexpr int kWbPart = 16384;
+constexpr int kWbMaxParts = 1024;
+constexpr int kWbBigItems = 0, kWbItems = 1, kWbNextItem = 2, kWbCounters = 3;
 constexpr int kRcdBigItems = 0, kRcdItems = 1, kRcdNextRow = 2, kRcdNextItem = 3, kRcdCounters = 4;
 // Value windows of a dense heavy row at most (it has at most kMaxBitmapSpan entries).
 template <typename T>
@@ -177,6 +181,11 @@ struct RowPlan {
                                // from the front, the others from the back of seg_len * rcd_slices<T>() places
   bool rcd_again;              // their bitmaps and items are wanted once more, the counts stand
   int32_t* rcd_ctr;            // counters kRcdBigItems .. kRcdNextItem
+  uint32_t* wb_bits;           // wide-bitmap rows: the row's bitmap, wb_words words per row (nullptr: no room)
+  int wb_words;                // a multiple of 4, enough for min(columns of B, kWbMaxSpan)
+  long long* wb_items;         // numeric items (row << 32 | part << 16 | parts of the row): rows of several parts
+  long long wb_cap;            // from the front, the others from the back of wb_cap places
+  int32_t* wb_ctr;             // counters kWbBigItems .. kWbNextItem
   DevSummary* sum;
   int* status;         // error flags (pinned host memory)
   int64_t seg_begin;   // first position in perm of the segment a kernel processes

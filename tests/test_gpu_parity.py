@@ -581,6 +581,75 @@ def test_single_dense_row_and_wide_output():
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+@pytest.mark.parametrize("dtype", [np.float32, np.float64])
+def test_wide_rows_in_parts(dtype):
+    """Wide-bitmap rows around the 16,384 products of a numeric item: one, two
+    and four items, and a hub row of short and long B rows."""
+    rng = np.random.default_rng(40)
+    k, n = 9000, 1 << 20
+    rows = {i: np.unique(rng.integers(0, n, size=8)).tolist() for i in range(k - 40)}
+    for i in range(k - 40, k):
+        rows[i] = np.unique(rng.integers(0, n, size=700)).tolist()
+    rows[0] = [0, 1, 2, 3, 4, 5, 6, n - 1]
+    B = _csr(k, n, rows, dtype=dtype)
+    B.vals = (2 * rng.random(B.nnz) - 1).astype(dtype)
+    eight = np.flatnonzero(np.diff(B.rowptr[:k - 39]) == 8)
+    arows = {i: [0] + eight[1:na].tolist() for i, na in enumerate((2047, 2048, 2049, 4096, 4097, 8193))}
+    arows[6] = list(range(k - 1500, k))
+    A = _csr(7, k, arows, dtype=dtype)
+    A.vals = (2 * rng.random(A.nnz) - 1).astype(dtype)
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["wb_rows"] == 7
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
+def test_wide_rows_without_room_for_bitmaps():
+    """With almost all device memory taken the bitmaps of the wide rows are not
+    kept and the numeric pass makes them again: the same C.  (A process of its
+    own: an earlier test's freed scratch would serve.)"""
+    import subprocess
+    import sys
+    code = """
+import numpy as np, torch
+from tests._gpu import assert_matches_oracle
+from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+from synth import HostCSR, uniform_csr
+rng = np.random.default_rng(41)
+B = uniform_csr(5000, 1 << 20, 20, rng)
+aci = np.sort(rng.random((601, 5000)).argsort(axis=1)[:, :900], axis=1).astype(np.int32).ravel()
+A = HostCSR(601, 5000, np.arange(602, dtype=np.int64) * 900, aci, 2 * rng.random(aci.size) - 1)  # 79 MB of bitmaps
+dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+def product(hog):
+    op = SpGEMM(dA, dB)
+    held = []
+    if hog:
+        size = 1 << 30
+        while size >= 1 << 24:  # leave less than 56 MB
+            if torch.cuda.mem_get_info()[0] - size > 40 << 20:
+                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            else:
+                size >>= 1
+    op.symbolic()
+    del held
+    torch.cuda.empty_cache()
+    C = op.numeric()
+    op.wait()
+    return op, C.to_host()
+op2, (rp2, ci2, v2) = product(False)  # kept: its scratch stays taken
+op1, (rp1, ci1, v1) = product(True)
+i1, i2 = op1.plan_info(), op2.plan_info()
+assert i1["wb_rows"] == i2["wb_rows"] == 601
+assert i1["numeric_launches"] < i2["numeric_launches"]  # no launch to zero the values
+assert np.array_equal(rp1, rp2) and np.array_equal(ci1, ci2)
+assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.arange(0, 601, 10))
+assert_matches_oracle(A, B, rp2, ci2, v2, rows=np.arange(0, 601, 10))
+"""
+    import os
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-2000:]
+
+
 def test_cancellation_keeps_structural_zero():
     A = _csr(1, 2, {0: [0, 1]}, vals=[1.0, -1.0])
     B = _csr(2, 3, {0: [0, 2], 1: [0, 1]}, vals=[2.0, 5.0, 2.0, 3.0])
