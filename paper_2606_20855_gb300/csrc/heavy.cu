@@ -37,7 +37,7 @@ namespace {
 
 constexpr int kRcdThreads = 512;
 constexpr int kWbThreads = 1024;  // one CTA per SM (its 128 KB bitmap), so 32 warps hide the gathers
-constexpr int kWbBatch = 4;  // stored A entries a lane group has in flight in the wide-bitmap kernel
+constexpr int kWbBatch = 4;  // stored A entries a lane group has in flight in the wide-bitmap numeric pass
 
 // ---------------------------------------------------------------- dense rows
 
@@ -514,30 +514,30 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
 // ----------------------------------------------------------------- wide rows
 
 // Measured on R-MAT 2^20 (edge factor 8, fp64) times rows of 4 entries, 1,048
-// such rows of 12,500 products on average and 93,000 at most: symbolic 95 us,
+// such rows of 12,500 products on average and 93,000 at most: symbolic 86 us,
 // numeric 186 us and 7 us for the zeroes.  A CTA per row that also set the bits
 // again in the numeric pass, one thread writing the columns of 8 consecutive
-// chunks, took 87 and 361 us, bound by its longest row.  Storing the bitmaps
-// (137 MB) costs the symbolic pass 8 us.  Bound by the latency of a round's
-// three dependent loads.
+// chunks, took 87 and 361 us, bound by its longest row.  Bound by the latency
+// of a round's three dependent loads: with four instead of eight entries in
+// flight the symbolic pass, which also stores 137 MB of bitmaps, takes 95 us.
 
 // Calls f(column, value of B, value of A) for the products of the stored A
-// entries [ra, re).  A group of lanes takes kWbBatch entries per round, so
+// entries [ra, re).  A group of lanes takes BATCH entries per round, so
 // their row-pointer loads and then their columns and values are in flight
 // together (a hub row has tens of thousands of entries).
-template <typename T, bool VALUES, typename F>
+template <typename T, bool VALUES, int BATCH, typename F>
 __device__ __forceinline__ void wb_products(const RowPlan<T>& p, int64_t ra, int64_t re, F&& f) {
   const int lg = p.log2_group;
   const int gsize = 1 << lg;
   const int grp = threadIdx.x >> lg;
   const int gl = threadIdx.x & (gsize - 1);
   const int ngrp = kWbThreads >> lg;
-  for (int64_t pa0 = ra + grp; pa0 < re; pa0 += static_cast<int64_t>(kWbBatch) * ngrp) {
-    int64_t qb[kWbBatch];
-    int len[kWbBatch], most = 0;
-    T av[kWbBatch];
+  for (int64_t pa0 = ra + grp; pa0 < re; pa0 += static_cast<int64_t>(BATCH) * ngrp) {
+    int64_t qb[BATCH];
+    int len[BATCH], most = 0;
+    T av[BATCH];
 #pragma unroll
-    for (int u = 0; u < kWbBatch; ++u) {
+    for (int u = 0; u < BATCH; ++u) {
       const int64_t pa = pa0 + static_cast<int64_t>(u) * ngrp;
       qb[u] = 0;
       len[u] = 0;
@@ -550,17 +550,17 @@ __device__ __forceinline__ void wb_products(const RowPlan<T>& p, int64_t ra, int
       }
     }
 #pragma unroll
-    for (int u = 0; u < kWbBatch; ++u) most = max(most, len[u]);
+    for (int u = 0; u < BATCH; ++u) most = max(most, len[u]);
     for (int t = gl; t < most; t += gsize) {
-      int c[kWbBatch];
-      T bv[kWbBatch];
+      int c[BATCH];
+      T bv[BATCH];
 #pragma unroll
-      for (int u = 0; u < kWbBatch; ++u) {
+      for (int u = 0; u < BATCH; ++u) {
         c[u] = t < len[u] ? p.B.colidx[qb[u] + t] : -1;
         bv[u] = VALUES && t < len[u] ? p.B.vals[qb[u] + t] : T(0);
       }
 #pragma unroll
-      for (int u = 0; u < kWbBatch; ++u) {
+      for (int u = 0; u < BATCH; ++u) {
         if (c[u] >= 0) f(c[u], bv[u], av[u]);
       }
     }
@@ -582,7 +582,7 @@ __global__ void __launch_bounds__(kWbThreads, 1) wb_symbolic_kernel(const RowPla
     const int lo = p.lo[row];
     const int nchunks = (p.hi[row] - lo + 128) >> 7;
     long long sums = 0;  // entries in the low bits, products above them
-    wb_products<T, false>(p, p.A.rowptr[row], p.A.rowptr[row + 1], [&](int c, T, T) {
+    wb_products<T, false, 2 * kWbBatch>(p, p.A.rowptr[row], p.A.rowptr[row + 1], [&](int c, T, T) {
       const uint32_t off = static_cast<uint32_t>(c - lo);
       const uint32_t bit = 1u << (off & 31u);
       sums += (1ll << kShift) + ((atomicOr(bm + (off >> 5), bit) & bit) == 0u);
@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(kWbThreads, 1) wb_numeric_kernel(const RowPlan
     for (int i = threadIdx.x; i < nchunks; i += kWbThreads) bm4[i] = bits ? bits[i] : make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     if (!bits) {
-      wb_products<T, false>(p, ra, ra + na, [&](int c, T, T) {
+      wb_products<T, false, 2 * kWbBatch>(p, ra, ra + na, [&](int c, T, T) {
         const uint32_t off = static_cast<uint32_t>(c - lo);
         atomicOr(bm + (off >> 5), 1u << (off & 31u));
       });
@@ -702,7 +702,7 @@ __global__ void __launch_bounds__(kWbThreads, 1) wb_numeric_kernel(const RowPlan
     }
     __syncthreads();  // prefixes and the zeroed values are visible to the CTA
     // 3. the part's products
-    wb_products<T, true>(p, ra + na * part / parts, ra + na * (part + 1) / parts, [&](int c, T b, T a) {
+    wb_products<T, true, kWbBatch>(p, ra + na * part / parts, ra + na * (part + 1) / parts, [&](int c, T b, T a) {
       const uint32_t off = static_cast<uint32_t>(c - lo);
       const uint32_t i = off >> 7;
       const uint4 v = bm4[i];
