@@ -520,6 +520,8 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
 // chunks, took 87 and 361 us, bound by its longest row.  Bound by the latency
 // of a round's three dependent loads: with four instead of eight entries in
 // flight the symbolic pass, which also stores 137 MB of bitmaps, takes 95 us.
+// 20 rows of 8 entries times rows of 30,000 take 0.69 ms in all; with one load
+// of each of eight B rows in flight at any length they took 1.28.
 
 // Calls f(column, value of B, value of A) for the products of the stored A
 // entries [ra, re).  A group of lanes takes BATCH entries per round, so
@@ -551,6 +553,32 @@ __device__ __forceinline__ void wb_products(const RowPlan<T>& p, int64_t ra, int
     }
 #pragma unroll
     for (int u = 0; u < BATCH; ++u) most = max(most, len[u]);
+    if (most > 4 * gsize) {  // long B rows: one at a time, kWbBatch steps in flight
+#pragma unroll 1
+      for (int u = 0; u < BATCH; ++u) {
+        const int64_t pa = pa0 + static_cast<int64_t>(u) * ngrp;
+        if (pa >= re) break;
+        const int k = p.A.colidx[pa];
+        const T a = VALUES ? p.A.vals[pa] : T(0);
+        const int64_t b0 = p.B.rowptr[k];
+        const int n = static_cast<int>(p.B.rowptr[k + 1] - b0);
+        for (int t = gl; t < n; t += kWbBatch * gsize) {
+          int c[kWbBatch];
+          T bv[kWbBatch];
+#pragma unroll
+          for (int v = 0; v < kWbBatch; ++v) {
+            const int i = t + v * gsize;
+            c[v] = i < n ? p.B.colidx[b0 + i] : -1;
+            bv[v] = VALUES && i < n ? p.B.vals[b0 + i] : T(0);
+          }
+#pragma unroll
+          for (int v = 0; v < kWbBatch; ++v) {
+            if (c[v] >= 0) f(c[v], bv[v], a);
+          }
+        }
+      }
+      continue;
+    }
     for (int t = gl; t < most; t += gsize) {
       int c[BATCH];
       T bv[BATCH];
