@@ -337,8 +337,10 @@ struct Plan {
     for (const DevBuf* b : {&rows, &slices, &ranks, &ew, &sv, &hranks, &rcd, &wb}) n += b->bytes;
     return n;
   }
-  // Back to a new plan that owns the same scratch and pinned block.
+  // Back to a new plan that owns the same scratch and pinned block, whose
+  // status words start clear like those of a new one.
   void recycle() {
+    host_sum->slot[0] = host_sum->slot[1] = 0;
     Plan fresh;
     fresh.rows = rows;
     fresh.slices = slices;

@@ -1,0 +1,71 @@
+// Checks of the library's host code on a fake CUDA runtime: checks <name>.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+
+#include "fake_launchers.cuh"
+#include "ws_spgemm.h"
+
+namespace {
+
+#define CHECK(cond)                                                              \
+  do {                                                                           \
+    if (!(cond)) {                                                               \
+      std::printf("%s:%d: %s (%s)\n", __func__, __LINE__, #cond, ws_last_error()); \
+      std::exit(1);                                                              \
+    }                                                                            \
+  } while (0)
+
+// An m x n handle with `nnz` stored entries, whose arrays nothing reads.
+ws_csr_t matrix(int64_t m, int64_t n, int64_t nnz) {
+  ws_csr_t h = nullptr;
+  auto* rowptr = static_cast<int64_t*>(std::calloc(static_cast<size_t>(m + 1), 8));
+  CHECK(ws_csr_create(&h, m, n, nnz, rowptr, static_cast<int32_t*>(std::calloc(static_cast<size_t>(nnz + 1), 4)),
+                      std::calloc(static_cast<size_t>(nnz + 1), 8), WS_F64, 0, nullptr) == WS_OK);
+  return h;
+}
+
+ws_status_t failing_spmspv(ws_csr_t At) {
+  int32_t idx[8] = {};
+  double val[8] = {};
+  int64_t n = 0;
+  fake::launch_status = wsk::kErrCount;
+  const ws_status_t st = ws_spmspv(At, 1, idx, val, idx, val, &n, nullptr);
+  fake::launch_status = 0;
+  return st;
+}
+
+// A device error of a destroyed handle does not come up in another caller's
+// operation that takes over its plan.
+void error_stays_with_its_handle() {
+  ws_csr_t A = matrix(8, 8, 8), B = matrix(8, 8, 8), C = matrix(8, 8, 0), X = matrix(8, 8, 8);
+  int64_t nnz = 0;
+  CHECK(ws_spgemm_outer_symbolic(A, B, C, 3, &nnz, nullptr) == WS_OK);
+  CHECK(failing_spmspv(X) == WS_ERR_DEVICE);
+  CHECK(ws_csr_destroy(X) == WS_OK);
+  CHECK(ws_spgemm_outer_symbolic(A, B, C, 3, &nnz, nullptr) == WS_OK);
+}
+
+struct {
+  const char* name;
+  void (*run)();
+} const kChecks[] = {
+    {"error_stays_with_its_handle", error_stays_with_its_handle},
+};
+
+}  // namespace
+
+int main(int argc, char** argv) {
+  if (argc < 2) {
+    for (const auto& c : kChecks) std::puts(c.name);
+    return 0;
+  }
+  for (const auto& c : kChecks) {
+    if (std::strcmp(c.name, argv[1]) == 0) {
+      c.run();
+      return 0;
+    }
+  }
+  std::puts("no such check");
+  return 2;
+}

@@ -14,7 +14,7 @@ import pytest
 import torch
 
 from paper_2606_20855_gb300 import _abi
-from paper_2606_20855_gb300.spgemm import DeviceCSR, spgemm_outer, submatrix
+from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMMOuter, SpMSpV, spgemm_outer, submatrix
 from synth import HostCSR, laplacian_2d, random_csr, rmat_pattern, uniform_csr
 from tests._gpu import assert_matches_oracle
 from tests._helpers import check_csr_invariants, dense
@@ -126,3 +126,21 @@ def test_outer_repeated_on_one_handle_and_errors():
         op.parts = 0
         with pytest.raises(_abi.WsError, match="WS_ERR_INVALID_ARG"):
             op.symbolic()
+
+
+def test_after_another_handles_error():
+    """A handle that reported a device error is destroyed and its plan serves the next operations: they succeed."""
+    rng = np.random.default_rng(11)
+    A, B = uniform_csr(60, 50, 4, rng), uniform_csr(50, 40, 4, rng)
+    dA, dB = DeviceCSR.from_host(A, DEV), DeviceCSR.from_host(B, DEV)
+    with SpGEMMOuter(dA, dB, parts=3) as op:
+        op.symbolic()
+        op.numeric()
+        op.wait()
+        with SpMSpV(DeviceCSR.from_host(random_csr(20, 30, 0.2, rng, np.float64, "sym"), DEV)) as bad:
+            with pytest.raises(_abi.WsError, match="WS_ERR_DEVICE"):
+                bad(torch.tensor([25], dtype=torch.int32, device=DEV), torch.ones(1, dtype=torch.float64, device=DEV))
+        op.symbolic()
+        C = op.numeric()
+        op.wait()
+        assert_matches_oracle(A, B, *C.to_host())
