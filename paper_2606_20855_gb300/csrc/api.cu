@@ -60,6 +60,27 @@ ws_status_t cuda_fail(cudaError_t e, const char* what) {
 
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+// Makes `device` the current device for its own lifetime.
+class DeviceGuard {
+ public:
+  explicit DeviceGuard(int device) {
+    if (cudaGetDevice(&before_) != cudaSuccess) return;
+    ok_ = before_ == device || cudaSetDevice(device) == cudaSuccess;
+    changed_ = ok_ && before_ != device;
+    if (!ok_) cudaGetLastError();
+  }
+  DeviceGuard(const DeviceGuard&) = delete;
+  DeviceGuard& operator=(const DeviceGuard&) = delete;
+  ~DeviceGuard() {
+    if (changed_) cudaSetDevice(before_);
+  }
+  bool ok() const { return ok_; }
+
+ private:
+  int before_ = 0;
+  bool ok_ = false, changed_ = false;
+};
+
 // Grow-only stream-ordered device buffer.
 struct DevBuf {
   void* ptr = nullptr;
@@ -1557,8 +1578,9 @@ ws_status_t ws_spgemm_wait(ws_csr_t C, ws_stream_t stream) {
 ws_status_t ws_csr_destroy(ws_csr_t h) {
   if (!h) return WS_OK;
   if (Plan* pl = h->plan) {
-    bool idle = true;
-    if (pl->scratch_bytes() > 0 || pl->outer) idle = cudaDeviceSynchronize() == cudaSuccess;
+    const DeviceGuard guard(h->device);  // the scratch is that device's, whichever is current
+    bool idle = guard.ok();
+    if (pl->scratch_bytes() > 0 || pl->outer) idle = cudaDeviceSynchronize() == cudaSuccess && idle;
     release_outer(pl, nullptr);
     if (!idle || !keep_plan(pl)) {
       for (DevBuf* b : {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd, &pl->wb}) b->release();

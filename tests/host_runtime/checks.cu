@@ -2,6 +2,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <vector>
 
 #include "fake_launchers.cuh"
 #include "ws_spgemm.h"
@@ -46,11 +47,26 @@ void error_stays_with_its_handle() {
   CHECK(ws_spgemm_outer_symbolic(A, B, C, 3, &nnz, nullptr) == WS_OK);
 }
 
+// A handle destroyed while another device is current waits for its own device
+// before its scratch goes to the next handle, and leaves the current device.
+void destroy_waits_for_the_handles_device() {
+  fake::device = 1;
+  ws_csr_t X = matrix(8, 8, 8);
+  int64_t nnz = 0;
+  ws_csr_t S = matrix(8, 8, 0);
+  CHECK(ws_csr_submatrix_symbolic(X, 0, 8, 0, 8, S, &nnz, nullptr) == WS_OK);
+  fake::device = 0;
+  CHECK(ws_csr_destroy(S) == WS_OK);
+  CHECK(fake::synced_devices == std::vector<int>{1});
+  CHECK(fake::device == 0);
+}
+
 struct {
   const char* name;
   void (*run)();
 } const kChecks[] = {
     {"error_stays_with_its_handle", error_stays_with_its_handle},
+    {"destroy_waits_for_the_handles_device", destroy_waits_for_the_handles_device},
 };
 
 }  // namespace
