@@ -196,7 +196,8 @@ SideStreams* acquire_side(int device) {
   SideStreams* x = new (std::nothrow) SideStreams;
   if (!x) return nullptr;
   x->device = device;
-  bool ok = cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
+  const DeviceGuard guard(device);
+  bool ok = guard.ok() && cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < SideStreams::kStreams && ok; ++i) {
     ok = cudaStreamCreateWithFlags(&x->st[i], cudaStreamNonBlocking) == cudaSuccess &&
          cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) == cudaSuccess;

@@ -61,12 +61,28 @@ void destroy_waits_for_the_handles_device() {
   CHECK(fake::device == 0);
 }
 
+// Side streams and their events are made on the device of the operation.
+void side_streams_belong_to_the_handles_device() {
+  fake::device = 1;
+  ws_csr_t A = matrix(1 << 17, 1 << 17, 64), B = matrix(1 << 17, 1 << 17, 64), C = matrix(1 << 17, 1 << 17, 0);
+  fake::device = 0;
+  for (int b = 0; b < 4; ++b) fake::summary.seg_count[wsk::kSegHash0 + b] = 1;
+  int64_t nnz = 0;
+  CUstream_st stream{1, 0};
+  CHECK(ws_spgemm_symbolic(A, B, C, &nnz, &stream) == WS_OK);
+  CHECK(!fake::streams.empty() && !fake::events.empty());
+  for (const CUstream_st* s : fake::streams) CHECK(s->device == 1);
+  for (const CUevent_st* e : fake::events) CHECK(e->device == 1);
+  CHECK(fake::device == 0);
+}
+
 struct {
   const char* name;
   void (*run)();
 } const kChecks[] = {
     {"error_stays_with_its_handle", error_stays_with_its_handle},
     {"destroy_waits_for_the_handles_device", destroy_waits_for_the_handles_device},
+    {"side_streams_belong_to_the_handles_device", side_streams_belong_to_the_handles_device},
 };
 
 }  // namespace
