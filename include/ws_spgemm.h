@@ -109,7 +109,11 @@ ws_status_t ws_csr_create(ws_csr_t* out, int64_t nrows, int64_t ncols, int64_t n
  * (host pointer).  C must be an output handle of shape A.nrows x B.ncols and
  * the same dtype.  Work is queued on `stream`; the call returns after the
  * stream has reached the end of the pass (it synchronises `stream`), because
- * the caller needs nnz(C) to allocate C's arrays.  The row plan (row classes,
+ * the caller needs nnz(C) to allocate C's arrays.  Independent row kernels of
+ * a pass may run side by side on streams of the library that have the
+ * priority of `stream`; they start after what `stream` holds and end before
+ * what is queued on it later.  While `stream` is being captured everything
+ * stays on it.  The row plan (row classes,
  * per-row workspaces) is kept in C's handle for ws_spgemm_numeric.
  * Device scratch is allocated stream-ordered on `stream` and cached in C's
  * handle across calls.  The first call on a device sets the release
@@ -129,7 +133,8 @@ ws_status_t ws_spgemm_symbolic(ws_csr_t A, ws_csr_t B, ws_csr_t C, int64_t* nnz_
  *   c_colidx  device int32[nnz(C)] written with C's column indices
  *   c_vals    device value array [nnz(C)] of C's dtype
  * Requires a completed ws_spgemm_symbolic for the same A, B and C (and A, B
- * unchanged since).  Asynchronous: work is queued on `stream` and the call
+ * unchanged since).  Asynchronous: work is queued on `stream` (row kernels
+ * side by side, as in the symbolic pass) and the call
  * returns without waiting; device-side failures are reported by
  * ws_spgemm_wait.  The two arrays are recorded in C's handle.
  * Passage: Sec. 5.1 (Gustavson's loop: w[j] += A[i,k] * B[k,j] in a per-row

@@ -160,12 +160,13 @@ void keep_pool_memory(int dev) {
 
 // Side streams for the independent row kernels of one pass: the classes of
 // rows touch different rows of C, so their kernels may overlap, and a class of
-// few long rows then does not leave the GPU to one CTA per row.  Sets are
-// checked out for the duration of one call, recycled across handles and
+// few long rows then does not leave the GPU to one CTA per row.  They have the
+// priority of the caller's stream.  Sets are checked out for the duration of one call, recycled across handles and
 // threads, and at most kMaxSets are kept.
 struct SideStreams {
   static constexpr int kStreams = 3;
   int device = 0;
+  int priority = 0;
   cudaStream_t st[kStreams] = {};
   cudaEvent_t fork = nullptr, join[kStreams] = {};
 };
@@ -182,11 +183,11 @@ void destroy_side(SideStreams* x) {
   delete x;
 }
 
-SideStreams* acquire_side(int device) {
+SideStreams* acquire_side(int device, int priority) {
   {
     std::lock_guard<std::mutex> lock(g_side_mutex);
     for (size_t i = 0; i < g_side_free.size(); ++i) {
-      if (g_side_free[i]->device == device) {
+      if (g_side_free[i]->device == device && g_side_free[i]->priority == priority) {
         SideStreams* x = g_side_free[i];
         g_side_free.erase(g_side_free.begin() + static_cast<std::ptrdiff_t>(i));
         return x;
@@ -196,10 +197,11 @@ SideStreams* acquire_side(int device) {
   SideStreams* x = new (std::nothrow) SideStreams;
   if (!x) return nullptr;
   x->device = device;
+  x->priority = priority;
   const DeviceGuard guard(device);
   bool ok = guard.ok() && cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < SideStreams::kStreams && ok; ++i) {
-    ok = cudaStreamCreateWithFlags(&x->st[i], cudaStreamNonBlocking) == cudaSuccess &&
+    ok = cudaStreamCreateWithPriority(&x->st[i], cudaStreamNonBlocking, priority) == cudaSuccess &&
          cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) == cudaSuccess;
   }
   if (!ok) {
@@ -240,7 +242,12 @@ class Fork {
       cudaGetLastError();
       return;
     }
-    side_ = acquire_side(device);
+    int priority = 0;
+    if (cudaStreamGetPriority(main, &priority) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    side_ = acquire_side(device, priority);
     if (side_ && cudaEventRecord(side_->fork, main_) != cudaSuccess) {
       cudaGetLastError();
       release_side(side_);

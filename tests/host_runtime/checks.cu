@@ -76,6 +76,35 @@ void side_streams_belong_to_the_handles_device() {
   CHECK(fake::device == 0);
 }
 
+// A product with a row in each of `kinds` hash bins, through both passes, on `stream`.
+void hash_product(int kinds, cudaStream_t stream) {
+  const int64_t m = 1 << 17;  // above 65,536 columns: no planning pass
+  ws_csr_t A = matrix(m, m, 64), B = matrix(m, m, 64), C = matrix(m, m, 0);
+  fake::summary = wsk::DevSummary{};
+  for (int b = 0; b < kinds; ++b) fake::summary.seg_count[wsk::kSegHash0 + b] = 1;
+  fake::summary.nnz = 64;
+  fake::row_kernels.clear();
+  int64_t nnz = 0;
+  CHECK(ws_spgemm_symbolic(A, B, C, &nnz, stream) == WS_OK);
+  CHECK(ws_spgemm_numeric(A, B, C, static_cast<int32_t*>(std::malloc(64 * 4)), std::malloc(64 * 8), stream) == WS_OK);
+  CHECK(fake::row_kernels.size() == 2u * static_cast<unsigned>(kinds));
+}
+
+// Every row kernel runs at the priority of the caller's stream.
+void side_streams_keep_the_callers_priority() {
+  CUstream_st plain{0, 0}, high{0, -5};
+  for (CUstream_st* s : {&plain, &high, &plain, &high}) {
+    hash_product(4, s);
+    int others = 0;
+    for (cudaStream_t q : fake::row_kernels) {
+      CHECK(q->priority == s->priority);
+      others += q != s;
+    }
+    CHECK(others > 0);
+  }
+  CHECK(fake::streams.size() == 6);  // a set for each priority, used again
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -83,6 +112,7 @@ struct {
     {"error_stays_with_its_handle", error_stays_with_its_handle},
     {"destroy_waits_for_the_handles_device", destroy_waits_for_the_handles_device},
     {"side_streams_belong_to_the_handles_device", side_streams_belong_to_the_handles_device},
+    {"side_streams_keep_the_callers_priority", side_streams_keep_the_callers_priority},
 };
 
 }  // namespace

@@ -42,6 +42,11 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
   fake::streams.push_back(*s = new CUstream_st{fake::device, 0});
   return cudaSuccess;
 }
+cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned, int priority) {
+  fake::streams.push_back(*s = new CUstream_st{fake::device, priority});
+  return cudaSuccess;
+}
+cudaError_t cudaStreamGetPriority(cudaStream_t s, int* priority) { *priority = s ? s->priority : 0; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) { *c = cudaStreamCaptureStatusNone; return cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
