@@ -112,7 +112,8 @@ ws_status_t ws_csr_create(ws_csr_t* out, int64_t nrows, int64_t ncols, int64_t n
  * the caller needs nnz(C) to allocate C's arrays.  Independent row kernels of
  * a pass may run side by side on streams of the library that have the
  * priority of `stream`; they start after what `stream` holds and end before
- * what is queued on it later.  While `stream` is being captured everything
+ * what is queued on it later.  While `stream` is being captured,
+ * and if it is confined to a part of the GPU (a green context), everything
  * stays on it.  The row plan (row classes,
  * per-row workspaces) is kept in C's handle for ws_spgemm_numeric.
  * Device scratch is allocated stream-ordered on `stream` and cached in C's

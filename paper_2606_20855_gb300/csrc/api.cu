@@ -9,6 +9,8 @@
 //   5. scan      counts -> C.rowptr                                 (1 or 2 launches)
 //   -- nnz(C) and the status word reach the host (written by the scan, stream sync)
 // Numeric pass (ws_spgemm_numeric): one launch per non-empty class, no sync.
+#include <cuda.h>
+
 #include <cstdarg>
 #include <cstddef>
 #include <cstdio>
@@ -158,6 +160,34 @@ void keep_pool_memory(int dev) {
   done[dev] = true;
 }
 
+// A driver function by name (nullptr if the driver has none of that name).
+template <typename F>
+F driver_function(const char* name, unsigned version) {
+  void* f = nullptr;
+  cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+  if (cudaGetDriverEntryPointByVersion(name, &f, version, cudaEnableDefault, &found) != cudaSuccess ||
+      found != cudaDriverEntryPointSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return reinterpret_cast<F>(f);
+}
+
+// The number of the current context, and whether `s` is confined to a part of
+// the GPU (a stream of a green context).  False if the driver cannot tell.
+bool stream_place(cudaStream_t s, unsigned long long* context, bool* confined) {
+  static const auto get_current = driver_function<CUresult(CUDAAPI*)(CUcontext*)>("cuCtxGetCurrent", 4000);
+  static const auto get_id = driver_function<CUresult(CUDAAPI*)(CUcontext, unsigned long long*)>("cuCtxGetId", 12000);
+  static const auto get_green = driver_function<CUresult(CUDAAPI*)(CUstream, CUgreenCtx*)>("cuStreamGetGreenCtx", 12040);
+  CUcontext ctx = nullptr;
+  CUgreenCtx green = nullptr;
+  if (!get_current || !get_id || !get_green || get_current(&ctx) != CUDA_SUCCESS || !ctx ||
+      get_id(ctx, context) != CUDA_SUCCESS || get_green(s, &green) != CUDA_SUCCESS)
+    return false;
+  *confined = green != nullptr;
+  return true;
+}
+
 // Side streams for the independent row kernels of one pass: the classes of
 // rows touch different rows of C, so their kernels may overlap, and a class of
 // few long rows then does not leave the GPU to one CTA per row.  They have the
@@ -167,6 +197,7 @@ struct SideStreams {
   static constexpr int kStreams = 3;
   int device = 0;
   int priority = 0;
+  unsigned long long context = 0;  // streams serve the context they were made in only
   cudaStream_t st[kStreams] = {};
   cudaEvent_t fork = nullptr, join[kStreams] = {};
 };
@@ -183,12 +214,12 @@ void destroy_side(SideStreams* x) {
   delete x;
 }
 
-SideStreams* acquire_side(int device, int priority) {
+SideStreams* acquire_side(int device, int priority, unsigned long long context) {
   {
     std::lock_guard<std::mutex> lock(g_side_mutex);
     for (size_t i = 0; i < g_side_free.size(); ++i) {
-      if (g_side_free[i]->device == device && g_side_free[i]->priority == priority) {
-        SideStreams* x = g_side_free[i];
+      SideStreams* x = g_side_free[i];
+      if (x->device == device && x->priority == priority && x->context == context) {
         g_side_free.erase(g_side_free.begin() + static_cast<std::ptrdiff_t>(i));
         return x;
       }
@@ -198,8 +229,8 @@ SideStreams* acquire_side(int device, int priority) {
   if (!x) return nullptr;
   x->device = device;
   x->priority = priority;
-  const DeviceGuard guard(device);
-  bool ok = guard.ok() && cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
+  x->context = context;
+  bool ok = cudaEventCreateWithFlags(&x->fork, cudaEventDisableTiming) == cudaSuccess;
   for (int i = 0; i < SideStreams::kStreams && ok; ++i) {
     ok = cudaStreamCreateWithPriority(&x->st[i], cudaStreamNonBlocking, priority) == cudaSuccess &&
          cudaEventCreateWithFlags(&x->join[i], cudaEventDisableTiming) == cudaSuccess;
@@ -230,24 +261,30 @@ void release_side(SideStreams* x) {
 // of side streams, everything ordered after what the caller's stream holds;
 // join() orders the caller's stream after all of them, so outside the call
 // the work looks as if it had been queued on that stream alone.  Fewer than
-// kMinKernels launches, and streams that are being captured (a recycled stream
-// must not stay in a capture), use the caller's stream only.
+// kMinKernels launches, streams that are being captured (a recycled stream
+// must not stay in a capture) and streams confined to a part of the GPU use the
+// caller's stream only.
 class Fork {
  public:
   static constexpr int kMinKernels = 3;
   Fork(cudaStream_t main, int device, int kernels) : main_(main) {
     if (kernels < kMinKernels) return;
+    const DeviceGuard guard(device);
+    if (!guard.ok()) return;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(main, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
       cudaGetLastError();
       return;
     }
+    unsigned long long context = 0;
+    bool confined = false;
+    if (!stream_place(main, &context, &confined) || confined) return;
     int priority = 0;
     if (cudaStreamGetPriority(main, &priority) != cudaSuccess) {
       cudaGetLastError();
       return;
     }
-    side_ = acquire_side(device, priority);
+    side_ = acquire_side(device, priority, context);
     if (side_ && cudaEventRecord(side_->fork, main_) != cudaSuccess) {
       cudaGetLastError();
       release_side(side_);

@@ -105,6 +105,21 @@ void side_streams_keep_the_callers_priority() {
   CHECK(fake::streams.size() == 6);  // a set for each priority, used again
 }
 
+// A stream confined to a part of the GPU keeps all row kernels; side streams
+// made in one context are not used in another.
+void side_streams_stay_where_the_caller_is() {
+  CUstream_st confined{0, 0, true}, plain{0, 0};
+  hash_product(4, &confined);
+  for (cudaStream_t q : fake::row_kernels) CHECK(q == &confined);
+  CHECK(fake::streams.empty());
+  for (unsigned long long context : {1, 2, 1}) {
+    fake::context = context;
+    hash_product(4, &plain);
+    for (cudaStream_t q : fake::row_kernels) CHECK(q == &plain || q->context == context);
+  }
+  CHECK(fake::streams.size() == 6);  // a set for each context, used again
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -113,6 +128,7 @@ struct {
     {"destroy_waits_for_the_handles_device", destroy_waits_for_the_handles_device},
     {"side_streams_belong_to_the_handles_device", side_streams_belong_to_the_handles_device},
     {"side_streams_keep_the_callers_priority", side_streams_keep_the_callers_priority},
+    {"side_streams_stay_where_the_caller_is", side_streams_stay_where_the_caller_is},
 };
 
 }  // namespace

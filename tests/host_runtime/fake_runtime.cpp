@@ -39,11 +39,11 @@ cudaError_t cudaMallocHost(void** p, size_t n) { *p = std::calloc(1, n); return 
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { std::memset(p, v, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { std::memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
-  fake::streams.push_back(*s = new CUstream_st{fake::device, 0});
+  fake::streams.push_back(*s = new CUstream_st{fake::device, 0, false, fake::context});
   return cudaSuccess;
 }
 cudaError_t cudaStreamCreateWithPriority(cudaStream_t* s, unsigned, int priority) {
-  fake::streams.push_back(*s = new CUstream_st{fake::device, priority});
+  fake::streams.push_back(*s = new CUstream_st{fake::device, priority, false, fake::context});
   return cudaSuccess;
 }
 cudaError_t cudaStreamGetPriority(cudaStream_t s, int* priority) { *priority = s ? s->priority : 0; return cudaSuccess; }
@@ -56,6 +56,22 @@ cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) {
 }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+// the driver
+static CUresult current_context(CUcontext* c) { *c = reinterpret_cast<CUcontext>(&fake::context); return CUDA_SUCCESS; }
+static CUresult context_id(CUcontext c, unsigned long long* id) { *id = *reinterpret_cast<unsigned long long*>(c); return CUDA_SUCCESS; }
+static CUresult green_context(CUstream s, CUgreenCtx* g) {
+  *g = s && s->confined ? reinterpret_cast<CUgreenCtx>(s) : nullptr;
+  return CUDA_SUCCESS;
+}
+cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** f, unsigned, unsigned long long,
+                                             cudaDriverEntryPointQueryResult* found) {
+  *f = std::strcmp(name, "cuCtxGetCurrent") == 0       ? reinterpret_cast<void*>(current_context)
+       : std::strcmp(name, "cuCtxGetId") == 0          ? reinterpret_cast<void*>(context_id)
+       : std::strcmp(name, "cuStreamGetGreenCtx") == 0 ? reinterpret_cast<void*>(green_context)
+                                                       : nullptr;
+  *found = *f ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
+  return cudaSuccess;
+}
 // nvcc's registration of (no) kernels
 void** __cudaRegisterFatBinary(void*) { return nullptr; }
 void __cudaRegisterFatBinaryEnd(void**) {}

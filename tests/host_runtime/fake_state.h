@@ -1,5 +1,6 @@
 // State of the fake CUDA runtime (fake_runtime.cpp) that checks look at.
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime_api.h>
 
 #include <map>
@@ -8,6 +9,8 @@
 // A stream of the fake runtime.
 struct CUstream_st {
   int device = 0, priority = 0;
+  bool confined = false;  // belongs to a green context
+  unsigned long long context = 0;
 };
 struct CUevent_st {
   int device = 0;
@@ -16,6 +19,7 @@ struct CUevent_st {
 namespace fake {
 
 inline int device = 0;                        // current device
+inline unsigned long long context = 1;        // number of the current context
 inline std::map<void*, size_t> live;          // device memory
 inline size_t bytes = 0, peak = 0;            // in use now, and at most
 inline long long fail_in = -1;                // the allocation with this number from now on fails (-1: none)
