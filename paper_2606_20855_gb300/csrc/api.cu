@@ -1116,15 +1116,22 @@ void release_outer(Plan* pl, cudaStream_t s) {
   pl->outer = nullptr;
 }
 
-void release_plan_async(Plan* pl, cudaStream_t s) {
-  if (!pl) return;
-  release_outer(pl, s);
+// The same, but the plan (its status words) stays: what is queued on s still
+// uses the scratch, nothing after it does.
+void release_scratch_async(Plan* pl, cudaStream_t s) {
   DevBuf* bufs[] = {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd, &pl->wb};
   for (DevBuf* b : bufs) {
     if (b->ptr) cudaFreeAsync(b->ptr, s);
     b->ptr = nullptr;
     b->bytes = 0;
   }
+  pl->ready = false;
+}
+
+void release_plan_async(Plan* pl, cudaStream_t s) {
+  if (!pl) return;
+  release_outer(pl, s);
+  release_scratch_async(pl, s);
   release_host_sum(pl->host_sum);
   delete pl;
 }
@@ -1252,6 +1259,7 @@ ws_status_t outer_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
     if ((st = owned_entries(cp, nnz_p, s)) != WS_OK) break;
     if ((st = numeric_impl<T>(&ab->h, &bp, &cp->h, cp->h.plan, s)) != WS_OK) break;
     launches += cp->h.plan->sym_launches + cp->h.plan->num_launches;
+    release_scratch_async(cp->h.plan, s);  // the next block's pass takes it
   }
   // every extraction has completed (each block's structure pass synchronised)
   if (st == WS_OK) st = plan_status(ab->h.plan);

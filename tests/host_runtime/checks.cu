@@ -120,6 +120,21 @@ void side_streams_stay_where_the_caller_is() {
   CHECK(fake::streams.size() == 6);  // a set for each context, used again
 }
 
+// The outer product's blocks use the same scratch one after another.
+void outer_blocks_share_scratch() {
+  const int64_t m = 1 << 17;
+  ws_csr_t A = matrix(m, m, 64), B = matrix(m, m, 64), C = matrix(m, m, 0);
+  const size_t rows = 20000, ranks = rows * 2 * wsk::kMaxHashProducts;
+  fake::summary.seg_count[wsk::kSegHash0 + wsk::kNumHashBins - 1] = rows;
+  fake::summary.nnz = 64;
+  int64_t nnz = 0;
+  CHECK(ws_spgemm_outer_symbolic(A, B, C, 8, &nnz, nullptr) == WS_OK);
+  CHECK(fake::peak > ranks && fake::peak < 2 * ranks);
+  CHECK(fake::bytes < ranks / 2);  // none of it waits for the numeric call
+  CHECK(ws_spgemm_outer_numeric(A, B, C, static_cast<int32_t*>(std::malloc(64 * 4)), std::malloc(64 * 8), nullptr) == WS_OK);
+  CHECK(ws_spgemm_wait(C, nullptr) == WS_OK);
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -129,6 +144,7 @@ struct {
     {"side_streams_belong_to_the_handles_device", side_streams_belong_to_the_handles_device},
     {"side_streams_keep_the_callers_priority", side_streams_keep_the_callers_priority},
     {"side_streams_stay_where_the_caller_is", side_streams_stay_where_the_caller_is},
+    {"outer_blocks_share_scratch", outer_blocks_share_scratch},
 };
 
 }  // namespace
