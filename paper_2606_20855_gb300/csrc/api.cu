@@ -1209,6 +1209,9 @@ ws_status_t outer_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
   void* ex_mem = nullptr;  // the extraction's summary and scan partials
   ws_status_t st = WS_OK;
   auto cleanup = [&]() {
+    // Queued kernels may still write to the status words that the plans give
+    // back to the pool here.
+    if (cudaStreamSynchronize(s) != cudaSuccess) cudaGetLastError();
     for (Owned* o : partial) release_owned(o, s);
     release_owned(ab, s);
     if (ex_mem) cudaFreeAsync(ex_mem, s);

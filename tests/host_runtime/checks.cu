@@ -135,6 +135,23 @@ void outer_blocks_share_scratch() {
   CHECK(ws_spgemm_wait(C, nullptr) == WS_OK);
 }
 
+// When a block of the outer product finds no memory, the status words of the
+// blocks before it are given back after the kernels that may write to them.
+void failed_outer_product_waits_for_its_kernels() {
+  const int64_t m = 1 << 17;
+  ws_csr_t A = matrix(m, m, 64), B = matrix(m, m, 64), C = matrix(m, m, 0);
+  fake::summary.seg_count[wsk::kSegHash0] = 1;
+  fake::summary.nnz = 64;
+  int64_t nnz = 0;
+  int failed = 0;
+  for (int k = 0; k < 40; ++k) {  // some allocations the call can do without
+    fake::fail_in = k;
+    failed += ws_spgemm_outer_symbolic(A, B, C, 5, &nnz, nullptr) == WS_ERR_ALLOC;
+    CHECK(fake::pending.empty());
+  }
+  CHECK(failed > 20);
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -145,6 +162,7 @@ struct {
     {"side_streams_keep_the_callers_priority", side_streams_keep_the_callers_priority},
     {"side_streams_stay_where_the_caller_is", side_streams_stay_where_the_caller_is},
     {"outer_blocks_share_scratch", outer_blocks_share_scratch},
+    {"failed_outer_product_waits_for_its_kernels", failed_outer_product_waits_for_its_kernels},
 };
 
 }  // namespace

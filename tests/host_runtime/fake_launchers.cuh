@@ -40,7 +40,10 @@ void launch_scatter(const RowPlan<T>&, int64_t, const int64_t*, int, cudaStream_
 template <typename T>
 void launch_dense_slices(const RowPlan<T>&, int32_t*, int32_t*, int32_t*, int, cudaStream_t, int*) {}
 template <typename T>
-void launch_hash(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
+void launch_hash(const RowPlan<T>& p, int, bool, int, cudaStream_t s, int*) {
+  fake::row_kernels.push_back(s);
+  fake::pending[p.status] = s;
+}
 template <typename T>
 void launch_bmr(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
 template <typename T>

@@ -3,6 +3,7 @@
 // where they were made, a record of the synchronisations.
 #include <cstdlib>
 #include <cstring>
+#include <iterator>
 
 #include "fake_state.h"
 
@@ -15,7 +16,10 @@ cudaError_t cudaMemPoolSetAttribute(cudaMemPool_t, cudaMemPoolAttr, void*) { ret
 cudaError_t cudaGetLastError() { return cudaSuccess; }
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "error"; }
 cudaError_t cudaDeviceSynchronize() { fake::synced_devices.push_back(fake::device); return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t s) { fake::synced.push_back(s); return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  for (auto it = fake::pending.begin(); it != fake::pending.end();) it = it->second == s ? fake::pending.erase(it) : std::next(it);
+  return cudaSuccess;
+}
 cudaError_t cudaMallocAsync(void** p, size_t n, cudaStream_t) {
   if (fake::fail_in == 0) {
     fake::fail_in = -1;

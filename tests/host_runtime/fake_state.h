@@ -24,7 +24,7 @@ inline std::map<void*, size_t> live;          // device memory
 inline size_t bytes = 0, peak = 0;            // in use now, and at most
 inline long long fail_in = -1;                // the allocation with this number from now on fails (-1: none)
 inline std::vector<int> synced_devices;       // device of every cudaDeviceSynchronize
-inline std::vector<cudaStream_t> synced;      // stream of every cudaStreamSynchronize
+inline std::map<int*, cudaStream_t> pending;  // status words that queued hash kernels may write to, and their stream
 inline std::vector<CUstream_st*> streams;     // streams created by the library
 inline std::vector<CUevent_st*> events;
 
