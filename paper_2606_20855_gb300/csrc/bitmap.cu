@@ -176,7 +176,7 @@ __global__ void __launch_bounds__(32 * WPR * RPC, 1024 / (32 * WPR * RPC))
 #define WS_BITMAP_VISIT(c_, v_)                                                                   \
   do {                                                                                          \
     const uint32_t off_ = static_cast<uint32_t>((c_) - lo);                                     \
-    const uint32_t w_ = off_ >> 5;                                                              \
+    const uint32_t w_ = (off_ >> 5) & ((1u << LOGW) - 1u); /* inside, even for a changed input */ \
     const uint32_t bit_ = 1u << (off_ & 31u);                                                   \
     if (phase == 0) {                                                                           \
       if constexpr (NUMERIC) {                                                                  \

@@ -86,7 +86,9 @@ struct RcdSymbolic {
   RcdParts e;
 };
 
-template <typename T>
+// AGAIN: the numeric pass makes the bitmaps once more; a column outside the
+// row's range (the input changed since) is left out and reported.
+template <typename T, bool AGAIN>
 __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowPlan<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RcdSymbolic& s = *reinterpret_cast<RcdSymbolic*>(smem_raw);
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint4* flags4 = reinterpret_cast<uint4*>(s.flags);
   for (int i = threadIdx.x; i < kMaxBitmapSpan / 16; i += kRcdThreads) flags4[i] = make_uint4(0u, 0u, 0u, 0u);
+  bool bad = false;
   for (int64_t guard = 0; guard <= p.seg_len; ++guard) {
     if (threadIdx.x == 0) s_row = atomicAdd(&p.rcd_ctr[kRcdNextRow], 1);
     __syncthreads();
@@ -109,6 +112,18 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
     const int lo = p.lo[row];
     const int span = p.hi[row] - lo + 1;
     const int64_t ra = p.A.rowptr[row], re = p.A.rowptr[row + 1];
+    auto flag = [&](int c) {
+      if constexpr (AGAIN) {
+        uint32_t off;
+        if (column_place(c, lo, span, &off)) {
+          s.flags[off] = 1;
+        } else {
+          bad |= c >= 0;
+        }
+      } else {
+        if (c >= 0) s.flags[c - lo] = 1;
+      }
+    };
     long long products = 0;
     for (int64_t e0 = ra; e0 < re; e0 += kRcdCacheA) {
       const int n = static_cast<int>(min(static_cast<int64_t>(kRcdCacheA), re - e0));
@@ -142,9 +157,7 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
 #pragma unroll
         for (int u = 0; u < kSymPiece / 32; ++u) c[u] = t0 + u * 32 < end ? cols[t0 + u * 32] : -1;
 #pragma unroll
-        for (int u = 0; u < kSymPiece / 32; ++u) {
-          if (c[u] >= 0) s.flags[c[u] - lo] = 1;
-        }
+        for (int u = 0; u < kSymPiece / 32; ++u) flag(c[u]);
       }
       for (int j = warp * (32 / kSymLanes) + lane / kSymLanes; j < n; j += kWarps * (32 / kSymLanes)) {
         const int len = e.len[j];
@@ -154,9 +167,7 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
 #pragma unroll
         for (int u = 0; u < 4; ++u) c[u] = lane % kSymLanes + u * kSymLanes < len ? cols[lane % kSymLanes + u * kSymLanes] : -1;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (c[u] >= 0) s.flags[c[u] - lo] = 1;
-        }
+        for (int u = 0; u < 4; ++u) flag(c[u]);
       }
       __syncthreads();
     }
@@ -181,7 +192,7 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
     if (threadIdx.x == 0) {
       const int total = static_cast<int>(sums & 0xffffffffll);
       const bool big = (sums >> 32) > kRcdBigProducts;
-      if (!p.rcd_again) p.c_rowptr[row + 1] = total;
+      if (!AGAIN) p.c_rowptr[row + 1] = total;
       const int nw = (total + kWidth - 1) / kWidth;
       const long long cap = static_cast<long long>(p.seg_len) * kS;
       if (big) {
@@ -193,6 +204,7 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
       }
     }
   }
+  if (AGAIN && bad) atomicOr(p.status, kErrCount);
 }
 
 // Numeric pass: one item (row, window of kWidth output ranks) per CTA at a
@@ -683,8 +695,12 @@ __global__ void __launch_bounds__(kWbThreads, 1) wb_numeric_kernel(const RowPlan
     __syncthreads();
     if (!bits) {
       wb_products<T, false, 2 * kWbBatch>(p, ra, ra + na, [&](int c, T, T) {
-        const uint32_t off = static_cast<uint32_t>(c - lo);
-        atomicOr(bm + (off >> 5), 1u << (off & 31u));
+        uint32_t off;
+        if (column_place(c, lo, nchunks << 7, &off)) {
+          atomicOr(bm + (off >> 5), 1u << (off & 31u));
+        } else {
+          bad = true;
+        }
       });
       __syncthreads();
     }
@@ -731,7 +747,11 @@ __global__ void __launch_bounds__(kWbThreads, 1) wb_numeric_kernel(const RowPlan
     __syncthreads();  // prefixes and the zeroed values are visible to the CTA
     // 3. the part's products
     wb_products<T, true, kWbBatch>(p, ra + na * part / parts, ra + na * (part + 1) / parts, [&](int c, T b, T a) {
-      const uint32_t off = static_cast<uint32_t>(c - lo);
+      uint32_t off;
+      if (!column_place(c, lo, nchunks << 7, &off)) {
+        bad = true;
+        return;
+      }
       const uint32_t i = off >> 7;
       const uint4 v = bm4[i];
       const uint32_t wq = (off >> 5) & 3u;
@@ -770,9 +790,10 @@ template <typename T>
 void launch_rcd(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, int* launches) {
   if (!numeric) {
     const size_t smem = sizeof(RcdSymbolic);
-    static int per_sm = 0;
-    if (per_sm == 0) per_sm = occupancy(rcd_symbolic_kernel<T>, kRcdThreads, smem);
-    rcd_symbolic_kernel<T><<<grid_of(p.seg_len, num_sms, per_sm), kRcdThreads, smem, s>>>(p);
+    auto kern = p.rcd_again ? rcd_symbolic_kernel<T, true> : rcd_symbolic_kernel<T, false>;
+    static int per_sm[2] = {0, 0};
+    if (per_sm[p.rcd_again] == 0) per_sm[p.rcd_again] = occupancy(kern, kRcdThreads, smem);
+    kern<<<grid_of(p.seg_len, num_sms, per_sm[p.rcd_again]), kRcdThreads, smem, s>>>(p);
   } else {
     const size_t smem = sizeof(RcdNumeric<T>);
     static int per_sm = 0;

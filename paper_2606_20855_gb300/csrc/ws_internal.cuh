@@ -148,6 +148,14 @@ __device__ __forceinline__ void publish_summary(DevSummary* sum, DevSummary* hos
   }
 }
 
+// Whether column c lies in a workspace that covers the `span` columns from lo
+// on, and its offset there.  A numeric pass asks before it touches a workspace
+// laid out for the columns that the symbolic pass saw; a negative c is outside.
+__host__ __device__ __forceinline__ bool column_place(int c, int lo, int span, uint32_t* off) {
+  *off = static_cast<uint32_t>(c) - static_cast<uint32_t>(lo);
+  return *off < static_cast<uint32_t>(span);
+}
+
 // Read-only view of an input CSR matrix.
 template <typename T>
 struct CsrView {

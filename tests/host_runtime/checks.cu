@@ -1,4 +1,5 @@
 // Checks of the library's host code on a fake CUDA runtime: checks <name>.
+#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -152,6 +153,23 @@ void failed_outer_product_waits_for_its_kernels() {
   CHECK(failed > 20);
 }
 
+// A column has a place in a row's workspace only inside the row's range.
+void columns_outside_have_no_place() {
+  const int lows[] = {0, 1, 65535, 1 << 20, INT_MAX - (1 << 20)}, spans[] = {1, 31, 128, 65536, 1 << 20};
+  for (int lo : lows) {
+    for (int span : spans) {
+      const long long end = static_cast<long long>(lo) + span;
+      for (long long c : {-1ll, 0ll, lo - 1ll, static_cast<long long>(lo), end - 1, end, end + 1, static_cast<long long>(INT_MAX)}) {
+        if (c > INT_MAX) continue;
+        uint32_t off = 0;
+        const bool in = wsk::column_place(static_cast<int>(c), lo, span, &off);
+        CHECK(in == (c >= lo && c < end));
+        CHECK(!in || off == c - lo);
+      }
+    }
+  }
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -162,6 +180,7 @@ struct {
     {"side_streams_keep_the_callers_priority", side_streams_keep_the_callers_priority},
     {"side_streams_stay_where_the_caller_is", side_streams_stay_where_the_caller_is},
     {"outer_blocks_share_scratch", outer_blocks_share_scratch},
+    {"columns_outside_have_no_place", columns_outside_have_no_place},
     {"failed_outer_product_waits_for_its_kernels", failed_outer_product_waits_for_its_kernels},
 };
 

@@ -9,6 +9,7 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2606_20855_gb300 import _abi
 from synth import HostCSR, random_csr, rmat_pattern, uniform_csr
 from tests._gpu import assert_matches_oracle, run_gpu, tuning
 from tests._helpers import TOL
@@ -648,6 +649,43 @@ assert_matches_oracle(A, B, rp2, ci2, v2, rows=np.arange(0, 601, 10))
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0, res.stderr[-2000:]
+
+
+def _changed_columns_case(kind):
+    """(A, B, other columns of B that are valid but leave the range of the rows of A*B)."""
+    rng = np.random.default_rng(52)
+    if kind == "bitmap":  # 20 entries of 20 over 400 columns: crowded rows; a shift would keep the counts
+        A, B, ncols = uniform_csr(200, 300, 20, rng), uniform_csr(300, 400, 20, rng), 70_000
+        other = rng.permutation(ncols)[B.colidx]
+    else:  # "wide": 5000 products over 100,000 columns
+        A, B, ncols = uniform_csr(40, 3000, 250, rng), uniform_csr(3000, 100_000, 20, rng), 1 << 21
+        other = B.colidx + 1_500_000
+    return A, HostCSR(B.nrows, ncols, B.rowptr, B.colidx, B.vals), other.astype(np.int32)
+
+
+def _check_changed_columns(kind, rows_key):
+    from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+    A, B, other = _changed_columns_case(kind)
+    dB = DeviceCSR.from_host(B)
+    with SpGEMM(DeviceCSR.from_host(A), dB) as op:
+        op.symbolic()
+        assert op.plan_info()[rows_key] == A.nrows
+        dB.colidx.copy_(torch.from_numpy(other))
+        op.numeric()
+        with pytest.raises(_abi.WsError, match="WS_ERR_DEVICE"):
+            op.wait()
+        dB.colidx.copy_(torch.from_numpy(B.colidx))
+        op.symbolic()
+        C = op.numeric()
+        op.wait()
+        assert_matches_oracle(A, B, *C.to_host(), rows=np.arange(0, A.nrows, 7))
+
+
+@pytest.mark.parametrize("kind,rows_key", [("bitmap", "bitmap_rows"), ("wide", "wb_rows")])
+def test_columns_changed_between_the_passes(kind, rows_key):
+    """Columns that leave a row's range after the symbolic pass touch nothing outside its workspace; the error is
+    reported and the handle stays usable."""
+    _check_changed_columns(kind, rows_key)
 
 
 def test_cancellation_keeps_structural_zero():
