@@ -23,37 +23,134 @@ __device__ __forceinline__ int ceil_log2_ll(long long x) {  // x >= 1
   return x <= 1 ? 0 : 64 - __clzll(x - 1);
 }
 
-// Class of a row from its stored-entry count, product count and column range.
+// Class of a row from its stored-entry count, product count, column range and
+// the shape of its B rows.
 // Regular rows (at most kBmrMaxA entries whose B rows fit one lane group) with
 // a range that fits a bitmap not much larger than their products (at most 8
 // words per product plus 64) take the register bitmap bins (the bitmap bins
 // if those are disabled).  The other rows of at most hash_max products take the
 // hash bins unless
 // - their products crowd a range of less than kCrowded columns per product:
-//   most products repeat a column there, and the hash buckets fill up; or
+//   most products repeat a column there, and the hash buckets fill up;
 // - one of their B rows is longer than kShortB: such rows (hub rows of a
-//   power-law matrix) tend to be dense at one end, which fills some buckets.
-// Those take the bitmap bins, and the dense rows above them.  Measured (100,000
-// rows, fp32, bitmap bins against hash bins): rows of 0-48 entries and B rows of
-// 0-24 over 1000 to 32,000 columns 0.97-1.69 against 0.69-0.72 ms; 20 entries
-// of 6 over 4000 columns 0.42 against 0.31, 24 of 12 0.62 against 0.72; 60 of
-// 60 inside 800 columns 5.3 against 10.4, 40 of 20 inside 80 0.65 against 1.45;
-// R-MAT 2^16 squared without the second exception 3.6 against 4.5.
+//   power-law matrix) tend to be dense at one end, which fills some buckets;
+// - the row has more than 16 entries and its B rows have lumps (three of four
+//   of the first kLooks of more than three columns): runs of neighbouring
+//   columns, as of a box stencil or of blocks, fill a bucket each; or
+// - a bitmap is cheaper although the columns spread: above kLargeHash products
+//   of B rows of kLongB columns and more (the windows of the dense rows), and in
+//   the bin of kSmallTo products and 16,384 columns when the B rows are of about the
+//   same length, so that the lane groups are full (that hash bin holds as much
+//   as twice the products for the same time).
+// Those take the bitmap bins, and the dense rows above them.  Measured (24
+// million products, fp32, bitmap or dense rows against hash bins, ms): rows of
+// 0-40 entries and B rows of 0-20 over 16,000 columns 0.86 against 0.59; 40 of 20
+// 0.81 against 0.57, 24 of 12 0.48 against 0.63, 42 of 12 0.47 against 0.53 (over
+// 32,000 columns 24 of 12 0.68 against 0.60); 60 of 60 over 16,000 0.41 against
+// 0.57, 150 of 16 0.49 against 0.65, 300 of 10 0.67 against 0.65; 60 of 60 over 250
+// 0.32 against 1.26.  27-point stencil of 64^3 squared 3.9 against 16.4, 9-point
+// stencil of 3 x 3 blocks on 128^2 0.91 against 3.4.  R-MAT 2^16 squared with and
+// without the second exception 3.5 and 4.3.
 // Rows with more products go to the dense rows (range up to 65,536 columns), the
 // 8192-entry bitmap bin, the wide bitmap (range up to 2^20) and finally the
 // column-sliced dense window.
 constexpr long long kCrowded = 2;
 constexpr int kShortB = 64;
+constexpr int kLooks = 8;
+constexpr long long kLargeHash = 2048, kLongB = 16;
+constexpr long long kSmallFrom = bitmap_cap(0), kSmallTo = bitmap_cap(1), kSmallSpan = 32ll << bitmap_log_words(1);
+constexpr int kBatch = 4;  // stored A entries of a long row that a thread has in flight
 
-__device__ __forceinline__ uint8_t classify(long long nnza, long long ub, int lo, int hi, int maxlen,
-                                            const AnalyzeParams& ap) {
+// What a row's class depends on, gathered over its stored A entries.
+struct RowShape {
+  long long ub = 0;  // products
+  int lo = INT_MAX, hi = -1, maxlen = 0;
+  int looked = 0, lumps = 0;  // B rows whose columns were looked at, and those of them with lumps
+
+  // B row [bs, be).
+  __device__ __forceinline__ void add(const int32_t* colidx, int64_t bs, int64_t be) {
+    if (be > bs) {
+      ub += be - bs;
+      maxlen = max(maxlen, static_cast<int>(min(be - bs, static_cast<int64_t>(INT_MAX))));
+      lo = min(lo, colidx[bs]);
+      hi = max(hi, colidx[be - 1]);
+    }
+  }
+  // The B rows of the stored A entries q0, q0 + step, ... before e, BATCH at a
+  // time, so that each of the three dependent loads is in flight for all of
+  // them.  A B row of an entry before look_end has lumps if its first three
+  // columns lie within a quarter of its average distance between two columns
+  // (one of 38 rows of columns drawn at random does).
+  template <typename T, int BATCH>
+  __device__ __forceinline__ void gather(const RowPlan<T>& p, int64_t q0, int64_t e, int step, int64_t look_end) {
+    for (; q0 < e; q0 += static_cast<int64_t>(BATCH) * step) {
+      int64_t bs[BATCH], be[BATCH];
+      int k[BATCH], first[BATCH], last[BATCH], third = 0;
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        const int64_t q = q0 + static_cast<int64_t>(u) * step;
+        k[u] = q < e ? p.A.colidx[q] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        bs[u] = k[u] >= 0 ? p.B.rowptr[k[u]] : 0;
+        be[u] = k[u] >= 0 ? p.B.rowptr[k[u] + 1] : 0;
+      }
+      const bool look = q0 < look_end && be[0] - bs[0] > 3;
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        first[u] = be[u] > bs[u] ? p.B.colidx[bs[u]] : INT_MAX;
+        last[u] = be[u] > bs[u] ? p.B.colidx[be[u] - 1] : -1;
+      }
+      if (look) third = p.B.colidx[bs[0] + 2];
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        const int64_t n = be[u] - bs[u];
+        ub += n;
+        maxlen = max(maxlen, static_cast<int>(min(n, static_cast<int64_t>(INT_MAX))));
+        lo = min(lo, first[u]);
+        hi = max(hi, last[u]);
+      }
+      looked += look;
+      lumps += look && 4 * (static_cast<int64_t>(third) - first[0]) * (be[0] - bs[0] - 1) <= static_cast<int64_t>(last[0]) - first[0];
+    }
+  }
+  __device__ __forceinline__ bool lumpy() const { return looked > 0 && 4 * lumps >= 3 * looked; }
+
+  __device__ __forceinline__ void merge(const RowShape& o) {
+    ub += o.ub;
+    lo = min(lo, o.lo);
+    hi = max(hi, o.hi);
+    maxlen = max(maxlen, o.maxlen);
+    looked += o.looked;
+    lumps += o.lumps;
+  }
+  // Over the lanes of a warp.
+  __device__ __forceinline__ void warp_merge() {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ub += __shfl_xor_sync(0xffffffffu, ub, o);
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    maxlen = __reduce_max_sync(0xffffffffu, maxlen);
+    const int both = __reduce_add_sync(0xffffffffu, looked << 16 | lumps);
+    looked = both >> 16;
+    lumps = both & 0xffff;
+  }
+};
+
+__device__ __forceinline__ uint8_t classify(long long nnza, const RowShape& r, const AnalyzeParams& ap) {
+  const long long ub = r.ub;
+  const int lo = r.lo, hi = r.hi, maxlen = r.maxlen;
   if (ub == 0) return kClsEmpty;
   if (nnza == 1) return kClsDirect;
   const long long span = static_cast<long long>(hi) - lo + 1;
   const long long est = ub < span ? ub : span;  // entries of the row are at most this
   const bool bitmap_ok = span <= ap.bitmap_span && ((span + 31) >> 5) <= 8 * ub + 64;
   const bool regular = nnza <= kBmrMaxA && maxlen <= ap.group;
-  const bool hashed = ub <= ap.hash_max && (!bitmap_ok || (!regular && maxlen <= kShortB && span >= kCrowded * ub));
+  const bool spread = span >= kCrowded * ub && maxlen <= kShortB && !r.lumpy();
+  const bool bitmap_cheaper = (ub > kLargeHash && ub >= kLongB * nnza) ||
+                              (ub > kSmallFrom && ub <= kSmallTo && span <= kSmallSpan && 4 * ub >= 3 * nnza * maxlen);
+  const bool hashed = ub <= ap.hash_max && (!bitmap_ok || (!regular && spread && !bitmap_cheaper));
   if (bitmap_ok && !hashed) {
     if (regular && nnza <= ap.bmr_max_a) {
 #pragma unroll
@@ -94,17 +191,17 @@ __device__ __forceinline__ int segment_of(uint8_t cls) {
 // already) and returns the class.
 template <typename T>
 __device__ __forceinline__ uint8_t store_row(const RowPlan<T>& p, const AnalyzeParams& ap, int64_t i, long long nnza,
-                                             long long ub, int lo, int hi, int maxlen, long long* s_slices) {
-  const uint8_t c = classify(nnza, ub, lo, hi, maxlen, ap);
+                                             const RowShape& r, long long* s_slices) {
+  const uint8_t c = classify(nnza, r, ap);
   p.cls[i] = c;
   // Direct rows know their count already; the others start at 0 and are
   // filled by the hash / dense-window symbolic kernels.
-  p.c_rowptr[i + 1] = (c == kClsDirect) ? ub : 0;
+  p.c_rowptr[i + 1] = (c == kClsDirect) ? r.ub : 0;
   if (c != kClsEmpty) {
-    p.lo[i] = lo;
-    p.hi[i] = hi;
+    p.lo[i] = r.lo;
+    p.hi[i] = r.hi;
     if (c == kClsDense) {
-      const long long span = static_cast<long long>(hi) - lo + 1;
+      const long long span = static_cast<long long>(r.hi) - r.lo + 1;
       atomicAdd(reinterpret_cast<unsigned long long*>(s_slices),
                 static_cast<unsigned long long>((span + ap.dense_width - 1) / ap.dense_width));
     }
@@ -116,15 +213,15 @@ __device__ __forceinline__ uint8_t store_row(const RowPlan<T>& p, const AnalyzeP
 // to the CTA's counters.
 template <typename T>
 __device__ __forceinline__ void record_row(const RowPlan<T>& p, const AnalyzeParams& ap, int64_t i, long long nnza,
-                                           long long ub, int lo, int hi, int maxlen, int* s_seg, long long* s_prod,
-                                           long long* s_slices, int* s_empty) {
-  const uint8_t c = store_row(p, ap, i, nnza, ub, lo, hi, maxlen, s_slices);
+                                           const RowShape& r, int* s_seg, long long* s_prod, long long* s_slices,
+                                           int* s_empty) {
+  const uint8_t c = store_row(p, ap, i, nnza, r, s_slices);
   if (c == kClsEmpty) {
     atomicAdd(s_empty, 1);
   } else {
     atomicAdd(&s_seg[segment_of(c)], 1);
   }
-  atomicAdd(reinterpret_cast<unsigned long long*>(s_prod), static_cast<unsigned long long>(ub));
+  atomicAdd(reinterpret_cast<unsigned long long*>(s_prod), static_cast<unsigned long long>(r.ub));
 }
 
 template <typename T>
@@ -180,22 +277,15 @@ __global__ void __launch_bounds__(256) analyze_kernel(const RowPlan<T> p, const 
           long_rows[ap.m - 1 - atomicAdd(&p.sum->n_long, 1)] = static_cast<int32_t>(i);
         }
       } else {
-        long long ub = 0;
-        int lo = INT_MAX, hi = -1, maxlen = 0;
+        RowShape r;
 #pragma unroll 4
         for (int64_t q = s; q < e; ++q) {
           const int k = p.A.colidx[q];
-          const int64_t bs = p.B.rowptr[k], be = p.B.rowptr[k + 1];
-          if (be > bs) {
-            ub += be - bs;
-            maxlen = max(maxlen, static_cast<int>(min(be - bs, static_cast<int64_t>(INT_MAX))));
-            lo = min(lo, p.B.colidx[bs]);
-            hi = max(hi, p.B.colidx[be - 1]);
-          }
+          r.add(p.B.colidx, p.B.rowptr[k], p.B.rowptr[k + 1]);
         }
-        const uint8_t c = store_row(p, ap, i, e - s, ub, lo, hi, maxlen, &s_slices);
+        const uint8_t c = store_row(p, ap, i, e - s, r, &s_slices);
         seg = c == kClsEmpty ? -1 : segment_of(c);
-        prod += static_cast<unsigned long long>(ub);
+        prod += static_cast<unsigned long long>(r.ub);
       }
     }
     const unsigned peers = __match_any_sync(0xffffffffu, seg);
@@ -217,13 +307,14 @@ __global__ void __launch_bounds__(256) analyze_kernel(const RowPlan<T> p, const 
 // Rows queued by analyze_kernel.  First one CTA per long row (a power-law
 // row can hold tens of thousands of entries, and its three dependent loads
 // per entry are a latency chain), then one warp per row of long_threshold + 1
-// .. kMidRowMax entries (the lanes stride over the entries, eight in flight
-// each, and warp reductions give the product count and the column range).
-// For a long row:
-// threads stride over the row's stored entries, eight in flight each, and
-// the CTA reduces the product count and column range.
+// .. kMidRowMax entries (the lanes stride over the entries, kBatch in flight
+// each, and warp reductions give the row's shape).  For a long row the threads
+// stride over the row's stored entries, kBatch in flight each, and the CTA
+// reduces its shape.  Five CTAs per SM with four entries in flight: 57 registers
+// (four CTAs) cost rows of 17-24 entries 1%; an unrolled loop over conditional loads
+// took 15 us more on R-MAT 2^20 than these batches.
 template <typename T>
-__global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, const AnalyzeParams ap,
+__global__ void __launch_bounds__(256, 5) analyze_long_kernel(const RowPlan<T> p, const AnalyzeParams ap,
                                                            const int32_t* long_rows, DevSummary* host) {
   const int nlong = *reinterpret_cast<volatile int*>(&p.sum->n_long);
   const int nmid = *reinterpret_cast<volatile int*>(&p.sum->n_mid);
@@ -235,8 +326,7 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
   __shared__ int s_seg[kNumSegs];
   __shared__ long long s_prod, s_slices;
   __shared__ int s_empty;
-  __shared__ long long s_ub[8];
-  __shared__ int s_lo[8], s_hi[8], s_maxlen[8];
+  __shared__ RowShape s_shape[8];
   if (threadIdx.x < kNumSegs) s_seg[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     s_prod = 0;
@@ -248,70 +338,30 @@ __global__ void __launch_bounds__(256) analyze_long_kernel(const RowPlan<T> p, c
   for (int64_t w = blockIdx.x; w < nlong; w += gridDim.x) {
     const int64_t i = long_rows[ap.m - 1 - w];  // long rows fill the list from the back
     const int64_t s = p.A.rowptr[i], e = p.A.rowptr[i + 1];
-    long long ub = 0;
-    int lo = INT_MAX, hi = -1, maxlen = 0;
-#pragma unroll 8
-    for (int64_t q = s + threadIdx.x; q < e; q += blockDim.x) {
-      const int k = p.A.colidx[q];
-      const int64_t bs = p.B.rowptr[k], be = p.B.rowptr[k + 1];
-      if (be > bs) {
-        ub += be - bs;
-        maxlen = max(maxlen, static_cast<int>(min(be - bs, static_cast<int64_t>(INT_MAX))));
-        lo = min(lo, p.B.colidx[bs]);
-        hi = max(hi, p.B.colidx[be - 1]);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ub += __shfl_xor_sync(0xffffffffu, ub, o);
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      maxlen = max(maxlen, __shfl_xor_sync(0xffffffffu, maxlen, o));
-    }
-    if (lane == 0) {
-      s_ub[warp] = ub;
-      s_lo[warp] = lo;
-      s_hi[warp] = hi;
-      s_maxlen[warp] = maxlen;
-    }
+    RowShape r;
+    r.gather<T, kBatch>(p, s + threadIdx.x, e, blockDim.x, s + kLooks);
+    r.warp_merge();
+    if (lane == 0) s_shape[warp] = r;
     __syncthreads();
     if (threadIdx.x == 0) {
-      for (int w2 = 1; w2 < static_cast<int>(blockDim.x >> 5); ++w2) {
-        ub += s_ub[w2];
-        lo = min(lo, s_lo[w2]);
-        hi = max(hi, s_hi[w2]);
-        maxlen = max(maxlen, s_maxlen[w2]);
-      }
-      record_row(p, ap, i, e - s, ub, lo, hi, maxlen, s_seg, &s_prod, &s_slices, &s_empty);
+      for (int w2 = 1; w2 < static_cast<int>(blockDim.x >> 5); ++w2) r.merge(s_shape[w2]);
+      record_row(p, ap, i, e - s, r, s_seg, &s_prod, &s_slices, &s_empty);
     }
-    __syncthreads();  // s_ub/s_lo/s_hi are reused by the next row
+    __syncthreads();  // s_shape is reused by the next row
   }
   const int64_t gw = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
   for (int64_t w = gw; w < nmid; w += nw) {
     const int64_t i = long_rows[w];
     const int64_t s = p.A.rowptr[i], e = p.A.rowptr[i + 1];
-    long long ub = 0;
-    int lo = INT_MAX, hi = -1, maxlen = 0;
-#pragma unroll 8
-    for (int64_t q = s + lane; q < e; q += 32) {
-      const int k = p.A.colidx[q];
-      const int64_t bs = p.B.rowptr[k], be = p.B.rowptr[k + 1];
-      if (be > bs) {
-        ub += be - bs;
-        maxlen = max(maxlen, static_cast<int>(min(be - bs, static_cast<int64_t>(INT_MAX))));
-        lo = min(lo, p.B.colidx[bs]);
-        hi = max(hi, p.B.colidx[be - 1]);
-      }
+    RowShape r;
+    if (e - s <= 32) {
+      r.gather<T, 1>(p, s + lane, e, 32, s + kLooks);
+    } else {
+      r.gather<T, kBatch>(p, s + lane, e, 32, s + kLooks);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ub += __shfl_xor_sync(0xffffffffu, ub, o);
-      lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-      hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-      maxlen = max(maxlen, __shfl_xor_sync(0xffffffffu, maxlen, o));
-    }
-    if (lane == 0) record_row(p, ap, i, e - s, ub, lo, hi, maxlen, s_seg, &s_prod, &s_slices, &s_empty);
+    r.warp_merge();
+    if (lane == 0) record_row(p, ap, i, e - s, r, s_seg, &s_prod, &s_slices, &s_empty);
   }
   __syncthreads();
   flush_counts(p, s_seg, &s_prod, &s_slices, &s_empty);

@@ -651,6 +651,49 @@ assert_matches_oracle(A, B, rp2, ci2, v2, rows=np.arange(0, 601, 10))
     assert res.returncode == 0, res.stderr[-2000:]
 
 
+def _box_stencil(dims, dof, rng, dtype):
+    """All neighbours of a grid point in a box of three per dimension, dof x dof blocks."""
+    at = np.arange(np.prod(dims)).reshape(dims)
+    pad = np.full([d + 2 for d in dims], -1)
+    pad[tuple(slice(1, -1) for _ in dims)] = at
+    near = np.stack([pad[tuple(slice(o, o + d) for o, d in zip(off, dims))].ravel()
+                     for off in np.ndindex(*[3] * len(dims))], axis=1)
+    cols = np.where(near[:, :, None] < 0, -1, near[:, :, None] * dof + np.arange(dof)).reshape(near.shape[0], -1)
+    cols = np.repeat(cols, dof, axis=0)
+    lens = (cols >= 0).sum(axis=1)
+    rowptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    vals = (2 * rng.random(rowptr[-1]) - 1).astype(dtype)
+    return HostCSR(cols.shape[0], cols.shape[0], rowptr, cols[cols >= 0].astype(np.int32), vals)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("dims,dof", [((5, 40, 40), 1), ((7, 90), 3)])
+def test_rows_of_neighbouring_columns_take_bitmaps(dims, dof, dtype):
+    """Box stencils: wide rows whose columns come in runs would fill a hash bucket with every run."""
+    A = _box_stencil(dims, dof, np.random.default_rng(61), dtype)
+    rowptr, colidx, vals, info = run_gpu(A, A)
+    assert info["hash_rows"] <= 0.02 * A.nrows  # some rows at the edges of the grid
+    assert_matches_oracle(A, A, rowptr, colidx, vals, rows=np.arange(0, A.nrows, 5))
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("ra,rb,n,rows_key", [
+    (24, 12, 4000, "bitmap_rows"), (42, 12, 16_000, "bitmap_rows"),  # 288 and 504 products of B rows of one length
+    (43, 12, 16_000, "hash_rows"), (24, 12, 60_000, "hash_rows"),    # more products, wider than 16,384 columns
+    (21, 12, 4000, "hash_rows"), (40, 40, 30_000, "hash_rows"),
+    (60, 40, 16_000, "rcd_rows"), (150, 16, 16_000, "rcd_rows"),     # 2400 products of long B rows
+    (160, 15, 16_000, "hash_rows"),                                  # and of shorter ones
+])
+def test_route_of_spread_rows(ra, rb, n, rows_key, dtype):
+    rng = np.random.default_rng(ra * rb)
+    A, B = uniform_csr(120, 2000, ra, rng), uniform_csr(2000, n, rb, rng)
+    A = HostCSR(A.nrows, A.ncols, A.rowptr, A.colidx, A.vals.astype(dtype))
+    B = HostCSR(B.nrows, B.ncols, B.rowptr, B.colidx, B.vals.astype(dtype))
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info[rows_key] >= 0.9 * A.nrows  # a few rows cover a narrower range
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
 def _changed_columns_case(kind):
     """(A, B, other columns of B that are valid but leave the range of the rows of A*B)."""
     rng = np.random.default_rng(52)
