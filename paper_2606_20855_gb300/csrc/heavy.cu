@@ -227,6 +227,12 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
 // go to a warp each and are added atomically (R-MAT 2^16 and 2^14 squared: 3.46
 // and 0.405 ms in all; groups of 16 lanes for up to 64 entries 3.51 and 0.429; a
 // warp for up to 256 entries 3.53 and 0.421).
+// Parts of up to 16 entries take four lanes each: hub rows over short B rows
+// are bound by the latency of the parts in flight, and a warp per part had the
+// fewest (4000 rows of 2000 entries times rows of 3 over 4000 columns, fp32: 1.31
+// ms in all with a warp, 0.69 with four lanes, 0.75 with eight; of 8 over
+// 60,000 1.28, 0.76 and 0.80; of 16 over 30,000 0.52, 0.40 and 0.39; the column
+// slices before the windows 0.93, 1.17 and 0.67).
 constexpr int kNumThreads = 256;
 constexpr int kNumCacheA = kNumThreads;       // stored A entries handled at a time
 constexpr int kNumPer = 2;                    // entries per thread and round
@@ -234,6 +240,8 @@ constexpr int kNumPiece = kNumThreads * kNumPer;
 constexpr int kNumDesc = 128;                 // rounds described at a time
 constexpr int kNumWords = kRcdWords / kNumThreads;  // bitmap words per thread
 constexpr int kNumShort = 96;   // a warp each, three entries per lane
+constexpr int kNumTiny = 16;    // a group of kNumTinyLanes lanes each
+constexpr int kNumTinyLanes = 4;
 constexpr int kAhead = 3;
 static_assert(kNumShort % 32 == 0, "whole entries per lane");
 static_assert(kNumWords == 8, "two 16-byte words of the bitmap per thread");
@@ -390,6 +398,15 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
       const uint32_t at = rk.y + __popc(rk.x & ((1u << (off & 31u)) - 1u));
       return at < static_cast<uint32_t>(kWidth) ? static_cast<int>(at) : kWidth;
     };
+    auto add = [&](int c, T x) {  // one product (none if c < 0)
+      if (c < 0) return;
+      const int q = rank_of(c);
+      if (q < kWidth) {
+        atomicAdd(s.win + q, x);
+      } else {
+        bad = true;
+      }
+    };
     const int64_t ra = p.A.rowptr[row], re = p.A.rowptr[row + 1];
     for (int64_t e0 = ra; e0 < re; e0 += kNumCacheA) {
       const int n = static_cast<int>(min(static_cast<int64_t>(kNumCacheA), re - e0));
@@ -486,12 +503,32 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
         }
         __syncthreads();
       }
-      // 4b. short parts
+      // 4b. the shortest parts
+      constexpr int kTinyPer = kNumTiny / kNumTinyLanes;
+      const int tl = lane % kNumTinyLanes;
+#pragma unroll 2
+      for (int j = tid / kNumTinyLanes; j < n; j += kNumThreads / kNumTinyLanes) {
+        const int len = s.len[j];
+        if (len > kNumTiny) continue;
+        const T a = s.a[j];
+        const long long b0 = s.b0[j];
+        int c[kTinyPer];
+        T bv[kTinyPer];
+#pragma unroll
+        for (int u = 0; u < kTinyPer; ++u) {
+          const int t = tl + u * kNumTinyLanes;
+          c[u] = t < len ? p.B.colidx[b0 + t] : -1;
+          bv[u] = t < len ? p.B.vals[b0 + t] : T(0);
+        }
+#pragma unroll
+        for (int u = 0; u < kTinyPer; ++u) add(c[u], a * bv[u]);
+      }
+      // 4c. short parts
       constexpr int kPerLane = kNumShort / 32;
 #pragma unroll 2
       for (int j = warp; j < n; j += kWarps) {
         const int len = s.len[j];
-        if (len > kNumShort) continue;
+        if (len > kNumShort || len <= kNumTiny) continue;
         const T a = s.a[j];
         const long long b0 = s.b0[j];
         int c[kPerLane];
@@ -503,16 +540,7 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
           bv[u] = t < len ? p.B.vals[b0 + t] : T(0);
         }
 #pragma unroll
-        for (int u = 0; u < kPerLane; ++u) {
-          if (c[u] >= 0) {
-            const int q = rank_of(c[u]);
-            if (q < kWidth) {
-              atomicAdd(s.win + q, a * bv[u]);
-            } else {
-              bad = true;
-            }
-          }
-        }
+        for (int u = 0; u < kPerLane; ++u) add(c[u], a * bv[u]);
       }
       __syncthreads();
     }

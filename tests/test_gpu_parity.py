@@ -694,6 +694,23 @@ def test_route_of_spread_rows(ra, rb, n, rows_key, dtype):
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("ncols", [500, 40_000])
+def test_dense_rows_of_short_b_rows(ncols, dtype):
+    """Dense heavy rows over B rows of 0 to 99 entries: every length around the lane groups of the numeric pass, in
+    one window and in several."""
+    rng = np.random.default_rng(62)
+    k = 2600
+    rows = {i: rng.choice(ncols, size=min(i % 20 if i % 5 else i % 100, ncols), replace=False) for i in range(k)}
+    B = _csr(k, ncols, rows, dtype=dtype)
+    B.vals = (2 * rng.random(B.nnz) - 1).astype(dtype)
+    A = _csr(12, k, {i: rng.choice(k, size=(600, 257, 256, 2000)[i % 4], replace=False) for i in range(12)}, dtype=dtype)
+    A.vals = (2 * rng.random(A.nnz) - 1).astype(dtype)
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["rcd_rows"] >= 6
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
 def _changed_columns_case(kind):
     """(A, B, other columns of B that are valid but leave the range of the rows of A*B)."""
     rng = np.random.default_rng(52)
