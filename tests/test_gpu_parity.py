@@ -695,7 +695,7 @@ def test_route_of_spread_rows(ra, rb, n, rows_key, dtype):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
-@pytest.mark.parametrize("ncols", [500, 40_000])
+@pytest.mark.parametrize("ncols", [1100, 40_000])
 def test_dense_rows_of_short_b_rows(ncols, dtype):
     """Dense heavy rows over B rows of 0 to 99 entries: every length around the lane groups of the numeric pass, in
     one window and in several."""
