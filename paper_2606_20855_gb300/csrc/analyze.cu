@@ -191,7 +191,7 @@ __device__ __forceinline__ int segment_of(uint8_t cls) {
 // already) and returns the class.
 template <typename T>
 __device__ __forceinline__ uint8_t store_row(const RowPlan<T>& p, const AnalyzeParams& ap, int64_t i, long long nnza,
-                                             const RowShape& r, long long* s_slices) {
+                                             const RowShape& r, long long* s_slices, long long* s_wb) {
   const uint8_t c = classify(nnza, r, ap);
   p.cls[i] = c;
   // Direct rows know their count already; the others start at 0 and are
@@ -205,6 +205,7 @@ __device__ __forceinline__ uint8_t store_row(const RowPlan<T>& p, const AnalyzeP
       atomicAdd(reinterpret_cast<unsigned long long*>(s_slices),
                 static_cast<unsigned long long>((span + ap.dense_width - 1) / ap.dense_width));
     }
+    if (c == kClsWb) atomicAdd(reinterpret_cast<unsigned long long*>(s_wb), static_cast<unsigned long long>(r.ub));
   }
   return c;
 }
@@ -214,8 +215,8 @@ __device__ __forceinline__ uint8_t store_row(const RowPlan<T>& p, const AnalyzeP
 template <typename T>
 __device__ __forceinline__ void record_row(const RowPlan<T>& p, const AnalyzeParams& ap, int64_t i, long long nnza,
                                            const RowShape& r, int* s_seg, long long* s_prod, long long* s_slices,
-                                           int* s_empty) {
-  const uint8_t c = store_row(p, ap, i, nnza, r, s_slices);
+                                           long long* s_wb, int* s_empty) {
+  const uint8_t c = store_row(p, ap, i, nnza, r, s_slices, s_wb);
   if (c == kClsEmpty) {
     atomicAdd(s_empty, 1);
   } else {
@@ -226,13 +227,14 @@ __device__ __forceinline__ void record_row(const RowPlan<T>& p, const AnalyzePar
 
 template <typename T>
 __device__ __forceinline__ void flush_counts(const RowPlan<T>& p, int* s_seg, long long* s_prod,
-                                             long long* s_slices, int* s_empty) {
+                                             long long* s_slices, long long* s_wb, int* s_empty) {
   if (threadIdx.x < kNumSegs && s_seg[threadIdx.x]) atomicAdd(&p.sum->seg_count[threadIdx.x], s_seg[threadIdx.x]);
   if (threadIdx.x == 0) {
     if (*s_prod) atomicAdd(reinterpret_cast<unsigned long long*>(&p.sum->products),
                            static_cast<unsigned long long>(*s_prod));
     if (*s_slices) atomicAdd(reinterpret_cast<unsigned long long*>(&p.sum->dense_slices),
                              static_cast<unsigned long long>(*s_slices));
+    if (*s_wb) atomicAdd(reinterpret_cast<unsigned long long*>(&p.sum->wb_products), static_cast<unsigned long long>(*s_wb));
     if (*s_empty) atomicAdd(&p.sum->n_empty, *s_empty);
   }
 }
@@ -248,12 +250,13 @@ template <typename T>
 __global__ void __launch_bounds__(256) analyze_kernel(const RowPlan<T> p, const AnalyzeParams ap,
                                                       int32_t* long_rows, const int32_t* rows) {
   __shared__ int s_seg[kNumSegs];
-  __shared__ long long s_prod, s_slices;
+  __shared__ long long s_prod, s_slices, s_wb;
   __shared__ int s_empty;
   if (threadIdx.x < kNumSegs) s_seg[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     s_prod = 0;
     s_slices = 0;
+    s_wb = 0;
     s_empty = 0;
   }
   __syncthreads();
@@ -283,7 +286,7 @@ __global__ void __launch_bounds__(256) analyze_kernel(const RowPlan<T> p, const 
           const int k = p.A.colidx[q];
           r.add(p.B.colidx, p.B.rowptr[k], p.B.rowptr[k + 1]);
         }
-        const uint8_t c = store_row(p, ap, i, e - s, r, &s_slices);
+        const uint8_t c = store_row(p, ap, i, e - s, r, &s_slices, &s_wb);
         seg = c == kClsEmpty ? -1 : segment_of(c);
         prod += static_cast<unsigned long long>(r.ub);
       }
@@ -301,7 +304,7 @@ __global__ void __launch_bounds__(256) analyze_kernel(const RowPlan<T> p, const 
   for (int o = 16; o > 0; o >>= 1) prod += __shfl_xor_sync(0xffffffffu, prod, o);
   if (lane == 0 && prod) atomicAdd(reinterpret_cast<unsigned long long*>(&s_prod), prod);
   __syncthreads();
-  flush_counts(p, s_seg, &s_prod, &s_slices, &s_empty);
+  flush_counts(p, s_seg, &s_prod, &s_slices, &s_wb, &s_empty);
 }
 
 // Rows queued by analyze_kernel.  First one CTA per long row (a power-law
@@ -324,13 +327,14 @@ __global__ void __launch_bounds__(256, 5) analyze_long_kernel(const RowPlan<T> p
   }
   __shared__ int s_last;
   __shared__ int s_seg[kNumSegs];
-  __shared__ long long s_prod, s_slices;
+  __shared__ long long s_prod, s_slices, s_wb;
   __shared__ int s_empty;
   __shared__ RowShape s_shape[8];
   if (threadIdx.x < kNumSegs) s_seg[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     s_prod = 0;
     s_slices = 0;
+    s_wb = 0;
     s_empty = 0;
   }
   __syncthreads();
@@ -345,7 +349,7 @@ __global__ void __launch_bounds__(256, 5) analyze_long_kernel(const RowPlan<T> p
     __syncthreads();
     if (threadIdx.x == 0) {
       for (int w2 = 1; w2 < static_cast<int>(blockDim.x >> 5); ++w2) r.merge(s_shape[w2]);
-      record_row(p, ap, i, e - s, r, s_seg, &s_prod, &s_slices, &s_empty);
+      record_row(p, ap, i, e - s, r, s_seg, &s_prod, &s_slices, &s_wb, &s_empty);
     }
     __syncthreads();  // s_shape is reused by the next row
   }
@@ -361,10 +365,10 @@ __global__ void __launch_bounds__(256, 5) analyze_long_kernel(const RowPlan<T> p
       r.gather<T, kBatch>(p, s + lane, e, 32, s + kLooks);
     }
     r.warp_merge();
-    if (lane == 0) record_row(p, ap, i, e - s, r, s_seg, &s_prod, &s_slices, &s_empty);
+    if (lane == 0) record_row(p, ap, i, e - s, r, s_seg, &s_prod, &s_slices, &s_wb, &s_empty);
   }
   __syncthreads();
-  flush_counts(p, s_seg, &s_prod, &s_slices, &s_empty);
+  flush_counts(p, s_seg, &s_prod, &s_slices, &s_wb, &s_empty);
   if (host) {  // the last CTA to get here copies the summary for the host
     __threadfence();
     __syncthreads();

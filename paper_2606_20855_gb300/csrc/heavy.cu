@@ -661,7 +661,8 @@ __global__ void __launch_bounds__(kWbThreads, 1) wb_symbolic_kernel(const RowPla
     if (threadIdx.x == 0) {
       p.c_rowptr[row + 1] = total & ((1ll << kShift) - 1);
       const long long products = total >> kShift;
-      const int parts = !p.wb_bits ? 1 : static_cast<int>(min((products + kWbPart - 1) / kWbPart, static_cast<long long>(kWbMaxParts)));
+      const long long most = min(static_cast<long long>(kWbMaxParts), static_cast<long long>(p.A.rowptr[row + 1] - p.A.rowptr[row]));
+      const int parts = !p.wb_bits ? 1 : static_cast<int>(min((products + p.wb_part - 1) / p.wb_part, most));
       const int at = atomicAdd(&p.wb_ctr[parts > 1 ? kWbBigItems : kWbItems], parts);
       for (int q = 0; q < parts; ++q) {
         p.wb_items[parts > 1 ? at + q : p.wb_cap - 1 - at - q] = r << 32 | static_cast<long long>(q) << 16 | parts;

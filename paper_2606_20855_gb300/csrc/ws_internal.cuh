@@ -82,7 +82,7 @@ constexpr int kRcdWidthBytes = 49152;     // value window of one item of a dense
 // Counters of the dense heavy rows: items of rows with many products, other
 // items, next row of the symbolic pass, next item of the numeric pass.
 // Wide-bitmap rows: products per numeric item, most items of a row, counters.
-constexpr int kWbPart = 16384;
+constexpr int kWbPart = 16384;  // at least
 constexpr int kWbMaxParts = 1024;
 constexpr int kWbBigItems = 0, kWbItems = 1, kWbNextItem = 2, kWbCounters = 3;
 constexpr int kRcdBigItems = 0, kRcdItems = 1, kRcdNextRow = 2, kRcdNextItem = 3, kRcdCounters = 4;
@@ -116,6 +116,7 @@ struct DevSummary {
   long long nnz;       // nnz(C), written by the scan
   long long products;  // sum of ub_i
   long long dense_slices;
+  long long wb_products;  // products of the wide-bitmap rows
   long long slice_cursor;
   int status;   // validation only; the passes use the status word of their plan
   int n_done;   // CTAs of analyze_long_kernel that have added their counts
@@ -194,6 +195,7 @@ struct RowPlan {
   long long* wb_items;         // numeric items (row << 32 | part << 16 | parts of the row): rows of several parts
   long long wb_cap;            // from the front, the others from the back of wb_cap places
   int32_t* wb_ctr;             // counters kWbBigItems .. kWbNextItem
+  int64_t wb_part;             // products per numeric item
   DevSummary* sum;
   int* status;         // error flags (pinned host memory)
   int64_t seg_begin;   // first position in perm of the segment a kernel processes

@@ -170,6 +170,25 @@ void columns_outside_have_no_place() {
   }
 }
 
+// Wide rows share few large items when there are many of them (the fake GPU
+// has 4 SMs).
+void wide_rows_are_cut_as_far_as_the_gpu_needs() {
+  const int64_t m = 1 << 17;
+  const struct {
+    int rows;
+    int64_t products, part;
+  } cases[] = {{1, 5000, 16384}, {7, 7 * 18000, 16384}, {8, 8 * 18000, 32768}, {100, 100 * 18000, 100 * 18000 / 16}};
+  for (const auto& c : cases) {
+    ws_csr_t A = matrix(m, m, 64), B = matrix(m, m, 64), C = matrix(m, m, 0);
+    fake::summary = wsk::DevSummary{};
+    fake::summary.seg_count[wsk::kSegWb] = c.rows;
+    fake::summary.products = fake::summary.wb_products = c.products;
+    int64_t nnz = 0;
+    CHECK(ws_spgemm_symbolic(A, B, C, &nnz, nullptr) == WS_OK);
+    CHECK(fake::wb_part == c.part);
+  }
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -180,6 +199,7 @@ struct {
     {"side_streams_keep_the_callers_priority", side_streams_keep_the_callers_priority},
     {"side_streams_stay_where_the_caller_is", side_streams_stay_where_the_caller_is},
     {"outer_blocks_share_scratch", outer_blocks_share_scratch},
+    {"wide_rows_are_cut_as_far_as_the_gpu_needs", wide_rows_are_cut_as_far_as_the_gpu_needs},
     {"columns_outside_have_no_place", columns_outside_have_no_place},
     {"failed_outer_product_waits_for_its_kernels", failed_outer_product_waits_for_its_kernels},
 };

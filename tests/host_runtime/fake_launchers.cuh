@@ -9,6 +9,7 @@
 namespace fake {
 
 inline wsk::DevSummary summary{};             // what a pass hands to the host
+inline int64_t wb_part = 0;  // products per item that the wide rows' kernels were given
 inline int launch_status = 0;                 // error flags that SpMSpV's kernels find
 inline std::vector<cudaStream_t> row_kernels; // stream of every row kernel launched
 
@@ -51,7 +52,10 @@ void launch_bitmap(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) { fa
 template <typename T>
 void launch_rcd(const RowPlan<T>&, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
 template <typename T>
-void launch_wb(const RowPlan<T>&, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
+void launch_wb(const RowPlan<T>& p, bool, int, cudaStream_t s, int*) {
+  fake::row_kernels.push_back(s);
+  fake::wb_part = p.wb_part;
+}
 template <typename T>
 void launch_dense(const RowPlan<T>&, int64_t, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
 template <typename T>

@@ -604,6 +604,23 @@ def test_wide_rows_in_parts(dtype):
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+def _drawn_csr(m, n, r, rng):
+    """r distinct columns per row, for any r <= n."""
+    cols = np.concatenate([np.sort(rng.choice(n, size=r, replace=False)) for _ in range(m)]).astype(np.int32)
+    return HostCSR(m, n, np.arange(m + 1, dtype=np.int64) * r, cols, 2 * rng.random(cols.size) - 1)
+
+
+@pytest.mark.parametrize("rows,entries,length", [(310, 900, 40), (5, 3, 20_000), (2, 2, 9000)])
+def test_wide_rows_in_parts(rows, entries, length):
+    """Many wide rows of 36,000 products (larger parts), and rows of more parts by products than stored entries."""
+    rng = np.random.default_rng(63)
+    A = _drawn_csr(rows, 3000 if length < 100 else 8, entries, rng)
+    B = _drawn_csr(A.ncols, 1 << 20, length, rng)
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["wb_rows"] == rows
+    assert_matches_oracle(A, B, rowptr, colidx, vals, rows=np.arange(0, rows, 1 if rows < 10 else 31))
+
+
 def test_wide_rows_without_room_for_bitmaps():
     """With almost all device memory taken the bitmaps of the wide rows are not
     kept and the numeric pass makes them again: the same C.  (A process of its
