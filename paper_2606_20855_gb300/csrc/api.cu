@@ -710,11 +710,36 @@ ws_status_t run_rcd(Plan* pl, RowPlan<T> p, bool numeric, int sms, cudaStream_t 
   return WS_OK;
 }
 
-// Row kernels of a pass (the symbolic pass has none for direct and planned rows).
+// Segments whose kernels run by themselves, ahead of the side streams: the
+// bitmap bin of 512 entries over 65,536 columns when its rows fill the GPU
+// several times over.  Its CTAs take most of an SM's shared memory, and next
+// to CTAs that want the memory as L1 cache both run at a fraction of their
+// occupancy.  Rows of 0-10 entries times rows of 0-80 over 32,000 columns (24
+// million products, fp32): 0.70 ms, 0.97 overlapped, 0.77 without side streams.
+// Other bins gained nothing or lost by it (rows of 0-80 entries times rows of 0-40
+// over 1000 columns, in the bin of 1024 entries: 1.04 against 0.99), and with few
+// rows the overlap is worth more (R-MAT 2^14: 0.58 without, 0.40 with).
+constexpr int64_t kAloneRows = 16384;
+bool runs_alone(const Plan* pl, int g) { return g == kSegBitmap0 + 2 && pl->seg_count[g] > kAloneRows; }
+
+// Row kernels of a pass next to them (the symbolic pass has none for direct
+// and planned rows).
 int bin_launches(const Plan* pl, bool numeric) {
   int n = 0;
-  for (int g = 0; g < kNumSegs; ++g) n += pl->seg_count[g] > 0 && (numeric || (g != kSegDirect && g != kSegBmrWide));
+  for (int g = 0; g < kNumSegs; ++g)
+    n += pl->seg_count[g] > 0 && (numeric || (g != kSegDirect && g != kSegBmrWide)) && !runs_alone(pl, g);
   return n;
+}
+
+template <typename T>
+void launch_alone(const Plan* pl, RowPlan<T> p, bool numeric, int sms, cudaStream_t s, int* launches) {
+  for (int b = 0; b < kNumBitmapBins; ++b) {
+    const int g = kSegBitmap0 + b;
+    if (!runs_alone(pl, g)) continue;
+    p.seg_begin = pl->seg_offset[g];
+    p.seg_len = pl->seg_count[g];
+    launch_bitmap<T>(p, b, numeric, sms, s, launches);
+  }
 }
 
 // Second half of the symbolic pass when some rows were not ranked by the
@@ -749,6 +774,7 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
   }
   reserve_hash_ranks(pl, s);
   p = make_rowplan<T>(A, B, C, pl);
+  launch_alone<T>(pl, p, false, sms, s, &pl->sym_launches);
   Fork fork(s, C->device, bin_launches(pl, false));
   auto segment = [&](int g) {
     p.seg_begin = pl->seg_offset[g];
@@ -770,7 +796,7 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     if (segment(kSegHash0 + b)) launch_hash<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
   }
   for (int b = kNumBitmapBins - 1; b >= 0; --b) {
-    if (segment(kSegBitmap0 + b)) launch_bitmap<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
+    if (segment(kSegBitmap0 + b) && !runs_alone(pl, kSegBitmap0 + b)) launch_bitmap<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
   }
   for (int b = kNumBmrBins - 1; b >= 0; --b) {
     if (segment(kSegBmr0 + b)) launch_bmr<T>(p, b, false, sms, fork.next(), &pl->sym_launches);
@@ -874,6 +900,7 @@ ws_status_t numeric_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan
   RowPlan<T> p = make_rowplan<T>(A, B, C, pl);
   if (pl->seg_count[kSegWb] > 0)
     WS_CUDA(cudaMemsetAsync(pl->wb_ctr + kWbNextItem, 0, sizeof(int32_t), s), "cudaMemsetAsync(wide row counter)");
+  launch_alone<T>(pl, p, true, sms, s, &pl->num_launches);
   Fork fork(s, C->device, bin_launches(pl, true));
   auto segment = [&](int g) {
     p.seg_begin = pl->seg_offset[g];
@@ -896,7 +923,7 @@ ws_status_t numeric_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan
     if (segment(kSegHash0 + b)) launch_hash<T>(p, b, true, sms, fork.next(), &pl->num_launches);
   }
   for (int b = kNumBitmapBins - 1; b >= 0; --b) {
-    if (segment(kSegBitmap0 + b)) launch_bitmap<T>(p, b, true, sms, fork.next(), &pl->num_launches);
+    if (segment(kSegBitmap0 + b) && !runs_alone(pl, kSegBitmap0 + b)) launch_bitmap<T>(p, b, true, sms, fork.next(), &pl->num_launches);
   }
   for (int b = kNumBmrBins - 1; b >= 0; --b) {
     if (segment(kSegBmr0 + b)) launch_bmr<T>(p, b, true, sms, fork.next(), &pl->num_launches);

@@ -189,6 +189,29 @@ void wide_rows_are_cut_as_far_as_the_gpu_needs() {
   }
 }
 
+// The bitmap bin of 65,536 columns is ahead of the side streams if it has rows
+// enough, and shares them otherwise.
+void many_wide_bitmap_rows_run_by_themselves() {
+  const int64_t m = 1 << 17;
+  CUstream_st stream{0, 0};
+  for (int rows : {16384, 16385}) {
+    ws_csr_t A = matrix(m, m, 64), B = matrix(m, m, 64), C = matrix(m, m, 0);
+    fake::summary = wsk::DevSummary{};
+    fake::summary.seg_count[wsk::kSegBitmap0 + 2] = rows;
+    for (int b = 0; b < 4; ++b) fake::summary.seg_count[wsk::kSegHash0 + b] = 1;
+    fake::summary.nnz = 64;
+    int64_t nnz = 0;
+    fake::row_kernels.clear();
+    fake::bitmap_after.clear();
+    CHECK(ws_spgemm_symbolic(A, B, C, &nnz, &stream) == WS_OK);
+    CHECK(ws_spgemm_numeric(A, B, C, static_cast<int32_t*>(std::malloc(64 * 4)), std::malloc(64 * 8), &stream) == WS_OK);
+    CHECK(fake::row_kernels.size() == 10u && fake::bitmap_after.size() == 2u);
+    // kernels queued before it, the same in both passes
+    CHECK(fake::bitmap_after[0] == (rows > 16384 ? 0u : 4u) && fake::bitmap_after[1] == fake::bitmap_after[0] + 5u);
+    if (rows > 16384) CHECK(fake::row_kernels[0] == &stream && fake::row_kernels[5] == &stream);
+  }
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -200,6 +223,7 @@ struct {
     {"side_streams_stay_where_the_caller_is", side_streams_stay_where_the_caller_is},
     {"outer_blocks_share_scratch", outer_blocks_share_scratch},
     {"wide_rows_are_cut_as_far_as_the_gpu_needs", wide_rows_are_cut_as_far_as_the_gpu_needs},
+    {"many_wide_bitmap_rows_run_by_themselves", many_wide_bitmap_rows_run_by_themselves},
     {"columns_outside_have_no_place", columns_outside_have_no_place},
     {"failed_outer_product_waits_for_its_kernels", failed_outer_product_waits_for_its_kernels},
 };

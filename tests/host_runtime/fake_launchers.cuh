@@ -9,6 +9,7 @@
 namespace fake {
 
 inline wsk::DevSummary summary{};             // what a pass hands to the host
+inline std::vector<size_t> bitmap_after;      // row kernels queued before every bitmap kernel
 inline int64_t wb_part = 0;  // products per item that the wide rows' kernels were given
 inline int launch_status = 0;                 // error flags that SpMSpV's kernels find
 inline std::vector<cudaStream_t> row_kernels; // stream of every row kernel launched
@@ -48,7 +49,10 @@ void launch_hash(const RowPlan<T>& p, int, bool, int, cudaStream_t s, int*) {
 template <typename T>
 void launch_bmr(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
 template <typename T>
-void launch_bitmap(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
+void launch_bitmap(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) {
+  fake::bitmap_after.push_back(fake::row_kernels.size());
+  fake::row_kernels.push_back(s);
+}
 template <typename T>
 void launch_rcd(const RowPlan<T>&, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
 template <typename T>
