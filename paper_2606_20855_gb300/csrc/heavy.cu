@@ -398,20 +398,25 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
       const uint32_t at = rk.y + __popc(rk.x & ((1u << (off & 31u)) - 1u));
       return at < static_cast<uint32_t>(kWidth) ? static_cast<int>(at) : kWidth;
     };
-    auto add = [&](int c, T x) {  // one product (none if c < 0)
-      if (c < 0) return;
-      const int q = rank_of(c);
-      if (q < kWidth) {
-        atomicAdd(s.win + q, x);
-      } else {
-        bad = true;
+    // One product, none if c < 0.  Only a warp with a product multiplies: an
+    // fp64 multiplication of empty slots cost parts of 39 entries 8%.
+    auto add = [&](int c, T a, T b) {
+      if (c >= 0) {
+        const int q = rank_of(c);
+        if (q < kWidth) {
+          atomicAdd(s.win + q, a * b);
+        } else {
+          bad = true;
+        }
       }
     };
     const int64_t ra = p.A.rowptr[row], re = p.A.rowptr[row + 1];
     for (int64_t e0 = ra; e0 < re; e0 += kNumCacheA) {
       const int n = static_cast<int>(min(static_cast<int64_t>(kNumCacheA), re - e0));
       // 3. the part of every entry's B row inside the window's columns, and the
-      // rounds of the long parts
+      // rounds of the long parts (with the number of shortest parts above them)
+      constexpr int kTinyShift = 20;
+      static_assert(static_cast<long long>(kNumCacheA) * kMaxBitmapSpan / kNumPiece < 1 << kTinyShift, "all rounds fit below");
       int rounds = 0;
       if (tid < n) {
         const int k = p.A.colidx[e0 + tid];
@@ -421,10 +426,14 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
         if (!whole) part_bounds(p.B.colidx + b0, end, c0, c1, &start, &end);
         s.b0[tid] = b0 + start;
         s.len[tid] = end - start;
-        rounds = end - start > kNumShort ? (end - start + kNumPiece - 1) / kNumPiece : 0;
+        rounds = end - start > kNumShort  ? (end - start + kNumPiece - 1) / kNumPiece
+                 : end - start > kNumTiny ? 0
+                                          : 1 << kTinyShift;
       }
       int nrounds;
-      s.first[tid] = block_exclusive_scan(rounds, s_scan, &nrounds);
+      s.first[tid] = block_exclusive_scan(rounds, s_scan, &nrounds) & ((1 << kTinyShift) - 1);
+      const int ntiny = nrounds >> kTinyShift;
+      nrounds &= (1 << kTinyShift) - 1;
       __syncthreads();
       // 4a. long parts, round by round
       for (int p0 = 0; p0 < nrounds; p0 += kNumDesc) {
@@ -507,7 +516,7 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
       constexpr int kTinyPer = kNumTiny / kNumTinyLanes;
       const int tl = lane % kNumTinyLanes;
 #pragma unroll 2
-      for (int j = tid / kNumTinyLanes; j < n; j += kNumThreads / kNumTinyLanes) {
+      for (int j = tid / kNumTinyLanes; ntiny > 0 && j < n; j += kNumThreads / kNumTinyLanes) {
         const int len = s.len[j];
         if (len > kNumTiny) continue;
         const T a = s.a[j];
@@ -521,7 +530,7 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
           bv[u] = t < len ? p.B.vals[b0 + t] : T(0);
         }
 #pragma unroll
-        for (int u = 0; u < kTinyPer; ++u) add(c[u], a * bv[u]);
+        for (int u = 0; u < kTinyPer; ++u) add(c[u], a, bv[u]);
       }
       // 4c. short parts
       constexpr int kPerLane = kNumShort / 32;
@@ -540,7 +549,7 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
           bv[u] = t < len ? p.B.vals[b0 + t] : T(0);
         }
 #pragma unroll
-        for (int u = 0; u < kPerLane; ++u) add(c[u], a * bv[u]);
+        for (int u = 0; u < kPerLane; ++u) add(c[u], a, bv[u]);
       }
       __syncthreads();
     }
