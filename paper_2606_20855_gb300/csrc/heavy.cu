@@ -96,8 +96,6 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
   __shared__ int s_scan[32];
   __shared__ long long s_sums[32];
   __shared__ int s_row;
-  constexpr int kS = rcd_slices<T>();
-  constexpr int kWidth = kRcdWidthBytes / static_cast<int>(sizeof(T));
   constexpr int kWarps = kRcdThreads / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   uint4* flags4 = reinterpret_cast<uint4*>(s.flags);
@@ -193,21 +191,21 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
       const int total = static_cast<int>(sums & 0xffffffffll);
       const bool big = (sums >> 32) > kRcdBigProducts;
       if (!AGAIN) p.c_rowptr[row + 1] = total;
-      const int nw = (total + kWidth - 1) / kWidth;
-      const long long cap = static_cast<long long>(p.seg_len) * kS;
+      const int nw = (total + p.rcd_width - 1) / p.rcd_width;
+      const long long cap = static_cast<long long>(p.seg_len) * p.rcd_slices;
       if (big) {
         const int at = atomicAdd(&p.rcd_ctr[kRcdBigItems], nw);
-        for (int w = 0; w < nw; ++w) p.rcd_items[at + w] = static_cast<long long>(r) * kS + w;
+        for (int w = 0; w < nw; ++w) p.rcd_items[at + w] = static_cast<long long>(r) * p.rcd_slices + w;
       } else {
         const int at = atomicAdd(&p.rcd_ctr[kRcdItems], nw);
-        for (int w = 0; w < nw; ++w) p.rcd_items[cap - 1 - at - w] = static_cast<long long>(r) * kS + w;
+        for (int w = 0; w < nw; ++w) p.rcd_items[cap - 1 - at - w] = static_cast<long long>(r) * p.rcd_slices + w;
       }
     }
   }
   if (AGAIN && bad) atomicOr(p.status, kErrCount);
 }
 
-// Numeric pass: one item (row, window of kWidth output ranks) per CTA at a
+// Numeric pass: one item (row, window of p.rcd_width output ranks) per CTA at a
 // time, the items of rows with many products first.
 //
 // A B row part of more than kNumShort entries is taken by the whole CTA, in
@@ -306,14 +304,13 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using S = RcdNumeric<T>;
   S& s = *reinterpret_cast<S*>(smem_raw);
-  constexpr int kS = rcd_slices<T>();
-  constexpr int kWidth = S::kWidth;
+  constexpr int kWidth = S::kWidth;  // p.rcd_width is at most this
   constexpr int kWarps = kNumThreads / 32;
   __shared__ int s_scan[32];
   __shared__ int s_item, s_c0, s_c1;
   const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
   const int nbig = p.rcd_ctr[kRcdBigItems], nitems = nbig + p.rcd_ctr[kRcdItems];
-  const long long cap = static_cast<long long>(p.seg_len) * kS;
+  const long long cap = static_cast<long long>(p.seg_len) * p.rcd_slices;
   bool bad = false;
   for (int guard = 0; guard <= nitems; ++guard) {
     __syncthreads();  // the previous item is done with the shared state
@@ -322,8 +319,8 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
     const int it = s_item;
     if (it >= nitems) break;
     const long long item = it < nbig ? p.rcd_items[it] : p.rcd_items[cap - 1 - (it - nbig)];
-    const int64_t r = item / kS;
-    const int q0 = static_cast<int>(item % kS) * kWidth;  // first rank of the window
+    const int64_t r = item / p.rcd_slices;
+    const int q0 = static_cast<int>(item % p.rcd_slices) * p.rcd_width;  // first rank of the window
     const int32_t row = p.perm[p.seg_begin + r];
     const int lo = p.lo[row];
     const int64_t cbase = p.c_rowptr[row] + q0;
@@ -350,7 +347,7 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
       run += __popc(wv[q]);
     }
     if (total - q0 != want) bad = true;
-    const int in_win = min(kWidth, total - q0);  // ranks in the window, at least 1
+    const int in_win = min(p.rcd_width, total - q0);  // ranks in the window, at least 1
     const int n_out = static_cast<int>(max(0ll, min(static_cast<long long>(in_win), want)));
     __syncthreads();
     // 2. the window's columns, placed in the (still unused) window memory:
@@ -386,10 +383,10 @@ __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPl
 #pragma unroll 4
     for (int i = tid; i < n_out; i += kNumThreads) p.c_colidx[cbase + i] = cols[i];
     __syncthreads();
-    for (int i = tid; i < kWidth * static_cast<int>(sizeof(T)) / 16; i += kNumThreads)
+    for (int i = tid; i < (in_win * static_cast<int>(sizeof(T)) + 15) / 16; i += kNumThreads)
       reinterpret_cast<uint4*>(s.win)[i] = make_uint4(0u, 0u, 0u, 0u);
     const int c0 = s_c0, c1 = s_c1;
-    const bool whole = total <= kWidth;
+    const bool whole = total <= p.rcd_width;
     // Rank of column c in the window; kWidth (and an error) if it has none,
     // which only an input changed since the symbolic pass can cause.
     auto rank_of = [&](int c) {
@@ -836,7 +833,7 @@ void launch_rcd(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, 
     const size_t smem = sizeof(RcdNumeric<T>);
     static int per_sm = 0;
     if (per_sm == 0) per_sm = occupancy(rcd_numeric_kernel<T>, kNumThreads, smem);
-    rcd_numeric_kernel<T><<<grid_of(p.seg_len * rcd_slices<T>(), num_sms, per_sm), kNumThreads, smem, s>>>(p);
+    rcd_numeric_kernel<T><<<grid_of(p.seg_len * p.rcd_slices, num_sms, per_sm), kNumThreads, smem, s>>>(p);
   }
   *launches += 1;
 }

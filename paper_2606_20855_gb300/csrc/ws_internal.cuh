@@ -78,7 +78,8 @@ constexpr uint8_t kClsWb = kClsRcd + 1;         // heavy rows, wide bitmap works
 // Heavy-row limits.
 constexpr int kRcdMaxA = 8192;            // stored A entries a dense row may have (cursor slots)
 constexpr int kRcdDefaultMaxA = 8192;     // default limit used by the classification
-constexpr int kRcdWidthBytes = 49152;     // value window of one item of a dense heavy row
+constexpr int kRcdWidthBytes = 49152;     // value window of one item of a dense heavy row, at most
+constexpr int kRcdLeastWidth = 512;       // entries of a window, at least
 // Counters of the dense heavy rows: items of rows with many products, other
 // items, next row of the symbolic pass, next item of the numeric pass.
 // Wide-bitmap rows: products per numeric item, most items of a row, counters.
@@ -86,11 +87,6 @@ constexpr int kWbPart = 16384;  // at least
 constexpr int kWbMaxParts = 1024;
 constexpr int kWbBigItems = 0, kWbItems = 1, kWbNextItem = 2, kWbCounters = 3;
 constexpr int kRcdBigItems = 0, kRcdItems = 1, kRcdNextRow = 2, kRcdNextItem = 3, kRcdCounters = 4;
-// Value windows of a dense heavy row at most (it has at most kMaxBitmapSpan entries).
-template <typename T>
-constexpr int rcd_slices() {
-  return (kMaxBitmapSpan + kRcdWidthBytes / static_cast<int>(sizeof(T)) - 1) / (kRcdWidthBytes / static_cast<int>(sizeof(T)));
-}
 constexpr int kWbMaxSpan = 1 << 20;       // widest column range of a wide-bitmap row
 
 // Segments of the row permutation: direct rows, register bitmap bins, bitmap
@@ -186,8 +182,10 @@ struct RowPlan {
                                // (nullptr: the plan has no room, the numeric pass ranks again)
   uint32_t* rcd_bits;          // dense heavy rows: bitmap of the row's columns from lo on, rcd_words words per row
   int rcd_words;               // a multiple of 4, enough for min(columns of B, kMaxBitmapSpan)
-  long long* rcd_items;        // their numeric work items (row * rcd_slices<T>() + window): rows with many products
-                               // from the front, the others from the back of seg_len * rcd_slices<T>() places
+  int rcd_width;               // entries of a value window
+  int rcd_slices;              // value windows of a row at most
+  long long* rcd_items;        // their numeric work items (row * rcd_slices + window): rows with many products
+                               // from the front, the others from the back of seg_len * rcd_slices places
   bool rcd_again;              // their bitmaps and items are wanted once more, the counts stand
   int32_t* rcd_ctr;            // counters kRcdBigItems .. kRcdNextItem
   uint32_t* wb_bits;           // wide-bitmap rows: the row's bitmap, wb_words words per row (nullptr: no room)

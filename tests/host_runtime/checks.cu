@@ -212,6 +212,27 @@ void many_wide_bitmap_rows_run_by_themselves() {
   }
 }
 
+// Dense rows are cut into value windows for three CTAs per SM (of 4) if they
+// would not keep every SM busy.
+void few_dense_rows_take_small_windows() {
+  const int widest = wsk::kRcdWidthBytes / 8;
+  const struct {
+    int rows;
+    int64_t ncols;
+    int width;
+  } cases[] = {{1, 3000, 512}, {3, 3000, 1024}, {4, 3000, widest}, {1, 60000, widest}, {1, 20000, widest}, {1, 18000, 1536}};
+  for (const auto& c : cases) {
+    ws_csr_t A = matrix(100, 1 << 17, 64), B = matrix(1 << 17, c.ncols, 64), C = matrix(100, c.ncols, 0);
+    fake::summary = wsk::DevSummary{};
+    fake::summary.n_pending = 1;
+    fake::summary.seg_count[wsk::kSegRcd] = c.rows;
+    int64_t nnz = 0;
+    CHECK(ws_spgemm_symbolic(A, B, C, &nnz, nullptr) == WS_OK);
+    CHECK(fake::rcd_width == c.width);
+    CHECK(fake::rcd_slices == (c.ncols + c.width - 1) / c.width);
+  }
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -224,6 +245,7 @@ struct {
     {"outer_blocks_share_scratch", outer_blocks_share_scratch},
     {"wide_rows_are_cut_as_far_as_the_gpu_needs", wide_rows_are_cut_as_far_as_the_gpu_needs},
     {"many_wide_bitmap_rows_run_by_themselves", many_wide_bitmap_rows_run_by_themselves},
+    {"few_dense_rows_take_small_windows", few_dense_rows_take_small_windows},
     {"columns_outside_have_no_place", columns_outside_have_no_place},
     {"failed_outer_product_waits_for_its_kernels", failed_outer_product_waits_for_its_kernels},
 };

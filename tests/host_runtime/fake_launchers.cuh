@@ -10,6 +10,7 @@ namespace fake {
 
 inline wsk::DevSummary summary{};             // what a pass hands to the host
 inline std::vector<size_t> bitmap_after;      // row kernels queued before every bitmap kernel
+inline int rcd_width = 0, rcd_slices = 0;     // value windows of the dense rows
 inline int64_t wb_part = 0;  // products per item that the wide rows' kernels were given
 inline int launch_status = 0;                 // error flags that SpMSpV's kernels find
 inline std::vector<cudaStream_t> row_kernels; // stream of every row kernel launched
@@ -54,7 +55,11 @@ void launch_bitmap(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) {
   fake::row_kernels.push_back(s);
 }
 template <typename T>
-void launch_rcd(const RowPlan<T>&, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
+void launch_rcd(const RowPlan<T>& p, bool, int, cudaStream_t s, int*) {
+  fake::row_kernels.push_back(s);
+  fake::rcd_width = p.rcd_width;
+  fake::rcd_slices = p.rcd_slices;
+}
 template <typename T>
 void launch_wb(const RowPlan<T>& p, bool, int, cudaStream_t s, int*) {
   fake::row_kernels.push_back(s);

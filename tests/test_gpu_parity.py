@@ -668,6 +668,19 @@ assert_matches_oracle(A, B, rp2, ci2, v2, rows=np.arange(0, 601, 10))
     assert res.returncode == 0, res.stderr[-2000:]
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("rows,ncols", [(1, 1100), (3, 1536), (2, 1537), (40, 3000), (7, 30_000)])
+def test_few_dense_rows_in_small_windows(rows, ncols, dtype):
+    """Too few dense heavy rows for the GPU: windows of 512 entries and more, full and ragged ones."""
+    rng = np.random.default_rng(64)
+    B = _drawn_csr(400, ncols, min(900, ncols), rng)
+    A = _drawn_csr(rows, 400, 130, rng)
+    A, B = (HostCSR(x.nrows, x.ncols, x.rowptr, x.colidx, x.vals.astype(dtype)) for x in (A, B))
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["rcd_rows"] == rows
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
 def _box_stencil(dims, dof, rng, dtype):
     """All neighbours of a grid point in a box of three per dimension, dof x dof blocks."""
     at = np.arange(np.prod(dims)).reshape(dims)
