@@ -183,6 +183,7 @@ struct RowPlan {
   uint32_t* rcd_bits;          // dense heavy rows: bitmap of the row's columns from lo on, rcd_words words per row
   int rcd_words;               // a multiple of 4, enough for min(columns of B, kMaxBitmapSpan)
   int rcd_width;               // entries of a value window
+  bool rcd_direct;             // a window covers all columns of B
   int rcd_slices;              // value windows of a row at most
   long long* rcd_items;        // their numeric work items (row * rcd_slices + window): rows with many products
                                // from the front, the others from the back of seg_len * rcd_slices places

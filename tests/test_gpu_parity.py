@@ -669,6 +669,24 @@ assert_matches_oracle(A, B, rp2, ci2, v2, rows=np.arange(0, 601, 10))
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("ncols", [1100, 6144, 6145, 12_288, 12_289])
+def test_dense_rows_around_the_window(ncols, dtype):
+    """Enough dense heavy rows for whole windows, B as wide as a window has places (6,144 in float64, 12,288 in
+    float32) and one column wider; rows over all columns and over the last ones only."""
+    rng = np.random.default_rng(65)
+    whole, last = _drawn_csr(60, ncols, 400, rng), _drawn_csr(60, 1030, 400, rng)
+    B = HostCSR(120, ncols, np.arange(121, dtype=np.int64) * 400,
+                np.concatenate([whole.colidx, last.colidx + (ncols - 1030)]).astype(np.int32),
+                np.concatenate([whole.vals, last.vals]).astype(dtype))
+    rows = [np.sort(rng.choice(60, size=25, replace=False)) + 60 * (i % 2) for i in range(200)]
+    A = HostCSR(200, 120, np.arange(201, dtype=np.int64) * 25, np.concatenate(rows).astype(np.int32),
+                (2 * rng.random(5000) - 1).astype(dtype))
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["rcd_rows"] >= 100
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("rows,ncols", [(1, 1100), (3, 1536), (2, 1537), (40, 3000), (7, 30_000)])
 def test_few_dense_rows_in_small_windows(rows, ncols, dtype):
     """Too few dense heavy rows for the GPU: windows of 512 entries and more, full and ragged ones."""
