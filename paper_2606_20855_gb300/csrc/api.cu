@@ -557,6 +557,7 @@ RowPlan<T> make_rowplan(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan*
   p.rcd_words = pl->rcd_words;
   p.rcd_width = pl->rcd_width;
   p.rcd_direct = B->ncols <= pl->rcd_width;
+  p.rcd_long_b = B->nnz / 512 > B->nrows;
   p.rcd_slices = pl->rcd_slices;
   p.wb_ctr = pl->wb_ctr;
   p.wb_items = pl->wb_items;

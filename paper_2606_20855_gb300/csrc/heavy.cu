@@ -209,7 +209,7 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
 // time, the items of rows with many products first.
 //
 // A B row part of more than kNumShort entries is taken by the whole CTA, in
-// rounds of kNumPiece entries: its columns are distinct, so the window is
+// rounds of kNumThreads * PER entries: its columns are distinct, so the window is
 // updated with a load, one multiply-add and a store, and a barrier separates
 // it from the next part.  Shared-memory fp64 adds by compare-and-swap were
 // what bound this pass: this GPU issues an fp64 instruction over about 16
@@ -233,8 +233,6 @@ __global__ void __launch_bounds__(kRcdThreads, 2) rcd_symbolic_kernel(const RowP
 // slices before the windows 0.93, 1.17 and 0.67).
 constexpr int kNumThreads = 256;
 constexpr int kNumCacheA = kNumThreads;       // stored A entries handled at a time
-constexpr int kNumPer = 2;                    // entries per thread and round
-constexpr int kNumPiece = kNumThreads * kNumPer;
 constexpr int kNumDesc = 128;                 // rounds described at a time
 constexpr int kNumWords = kRcdWords / kNumThreads;  // bitmap words per thread
 constexpr int kNumShort = 96;   // a warp each, three entries per lane
@@ -304,12 +302,19 @@ __device__ __forceinline__ void part_bounds(const int32_t* cols, int n, int c0, 
 // no look-up of its rank (2000 rows of 280 entries times rows of 280 over 2000
 // columns: 0.61 against 0.72 ms in fp32, 0.70 against 0.87 in fp64; the column
 // slices before the windows 0.66 and 1.25).
-template <typename T, bool DIRECT>
+// PER: entries per thread and round.  Direct fp32 rounds are so short that B rows
+// of more than 512 entries on average take 1024 at a time (2000 rows of 590
+// entries times rows of 590 over 2000 columns 1.89 ms with two per thread, 1.62
+// with four; fp64 2.27 and 2.11, but 5.00 and 5.10 with rows of 1000, and rows of
+// 280 entries 0.61 and 0.75 in fp32).
+template <typename T, bool DIRECT, int PER>
 __global__ void __launch_bounds__(kNumThreads, 3) rcd_numeric_kernel(const RowPlan<T> p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   using S = RcdNumeric<T>;
   S& s = *reinterpret_cast<S*>(smem_raw);
   constexpr int kWidth = S::kWidth;  // p.rcd_width is at most this
+  constexpr int kNumPer = PER;       // entries per thread and round
+  constexpr int kNumPiece = kNumThreads * kNumPer;
   constexpr int kWarps = kNumThreads / 32;
   __shared__ int s_scan[32];
   __shared__ int s_item, s_c0, s_c1;
@@ -841,10 +846,14 @@ void launch_rcd(const RowPlan<T>& p, bool numeric, int num_sms, cudaStream_t s, 
     kern<<<grid_of(p.seg_len, num_sms, per_sm[p.rcd_again]), kRcdThreads, smem, s>>>(p);
   } else {
     const size_t smem = sizeof(RcdNumeric<T>);
-    static int per_sm[2] = {0, 0};
-    auto kern = p.rcd_direct ? rcd_numeric_kernel<T, true> : rcd_numeric_kernel<T, false>;
-    if (per_sm[p.rcd_direct] == 0) per_sm[p.rcd_direct] = occupancy(kern, kNumThreads, smem);
-    kern<<<grid_of(p.seg_len * p.rcd_slices, num_sms, per_sm[p.rcd_direct]), kNumThreads, smem, s>>>(p);
+    static int per_sm[3] = {0, 0, 0};
+    const int v = !p.rcd_direct ? 0 : sizeof(T) == 4 && p.rcd_long_b ? 2 : 1;
+    auto kern = v == 0 ? rcd_numeric_kernel<T, false, 2> : rcd_numeric_kernel<T, true, 2>;
+    if constexpr (sizeof(T) == 4) {
+      if (v == 2) kern = rcd_numeric_kernel<T, true, 4>;
+    }
+    if (per_sm[v] == 0) per_sm[v] = occupancy(kern, kNumThreads, smem);
+    kern<<<grid_of(p.seg_len * p.rcd_slices, num_sms, per_sm[v]), kNumThreads, smem, s>>>(p);
   }
   *launches += 1;
 }

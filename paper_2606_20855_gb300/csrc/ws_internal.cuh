@@ -184,6 +184,7 @@ struct RowPlan {
   int rcd_words;               // a multiple of 4, enough for min(columns of B, kMaxBitmapSpan)
   int rcd_width;               // entries of a value window
   bool rcd_direct;             // a window covers all columns of B
+  bool rcd_long_b;             // B's rows have more than 512 entries on average
   int rcd_slices;              // value windows of a row at most
   long long* rcd_items;        // their numeric work items (row * rcd_slices + window): rows with many products
                                // from the front, the others from the back of seg_len * rcd_slices places

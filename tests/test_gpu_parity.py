@@ -687,6 +687,22 @@ def test_dense_rows_around_the_window(ncols, dtype):
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("length", [513, 1024, 1025, 2049])
+def test_dense_rows_of_long_b_rows(length, dtype):
+    """Rounds of 1024 entries (float32) and of 512 at their edges, with short B rows among the long ones."""
+    rng = np.random.default_rng(66)
+    long_rows, short = _drawn_csr(80, 3000, length, rng), _drawn_csr(20, 3000, 40, rng)
+    B = HostCSR(100, 3000, np.concatenate([long_rows.rowptr, long_rows.rowptr[-1] + short.rowptr[1:]]),
+                np.concatenate([long_rows.colidx, short.colidx]),
+                np.concatenate([long_rows.vals, short.vals]).astype(dtype))
+    A = _drawn_csr(180, 100, 30, rng)
+    A = HostCSR(A.nrows, A.ncols, A.rowptr, A.colidx, A.vals.astype(dtype))
+    rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["rcd_rows"] == A.nrows
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
+@pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("rows,ncols", [(1, 1100), (3, 1536), (2, 1537), (40, 3000), (7, 30_000)])
 def test_few_dense_rows_in_small_windows(rows, ncols, dtype):
     """Too few dense heavy rows for the GPU: windows of 512 entries and more, full and ragged ones."""
