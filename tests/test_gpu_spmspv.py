@@ -115,6 +115,32 @@ def test_index_out_of_range_is_reported():
         check(A, xi, xv, op)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+@pytest.mark.parametrize("m", [1 << 23, (1 << 23) + 1, 9_000_000])
+def test_long_results(m, dtype):
+    """y around 2,048 compaction tiles of 4,096 positions (more of them are counted by a scan): hit at its first and
+    last positions, in a stretch, and scattered."""
+    rng = np.random.default_rng(m % 97)
+    n = 30
+    rows = [np.unique(np.concatenate([[0, m - 1 - j % 3], np.arange(40_000 * j, 40_000 * j + 300),
+                                      rng.integers(0, m, size=2000)])) for j in range(n)]
+    At = HostCSR(n, m, np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64),
+                 np.concatenate(rows).astype(np.int32), rng.uniform(0.5, 1.0, sum(r.size for r in rows)).astype(dtype))
+    xi, xv = sparse_vector(n, 0.6, rng, dtype, "sym")
+    dev = torch.device("cuda:0")
+    with SpMSpV(DeviceCSR.from_host(At, dev)) as op:
+        yi, yv = op(torch.from_numpy(xi).to(dev), torch.from_numpy(xv).to(dev))
+        yi, yv = yi.cpu().numpy(), yv.cpu().numpy()
+    hit = np.concatenate([rows[j] for j in xi])
+    prod = np.concatenate([At.vals[At.rowptr[j]:At.rowptr[j + 1]].astype(np.float64) * v for j, v in zip(xi, xv)])
+    ref_idx, where = np.unique(hit, return_inverse=True)
+    ref, mass = np.zeros(ref_idx.size), np.zeros(ref_idx.size)
+    np.add.at(ref, where, prod)
+    np.add.at(mass, where, np.abs(prod))
+    np.testing.assert_array_equal(yi, ref_idx)
+    assert value_error(yv, ref, mass) <= TOL[np.dtype(dtype)]
+
+
 @pytest.mark.slow
 def test_full_size_workload():
     A, xi, xv = spmspv_workload("spmspv_rmat20")
