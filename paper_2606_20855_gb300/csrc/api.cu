@@ -88,6 +88,7 @@ struct DevBuf {
   void* ptr = nullptr;
   size_t bytes = 0;
   uint64_t gen = 0;  // changes with every allocation (0: none yet)
+  static size_t allocated(size_t need) { return need + need / 8; }
   ws_status_t reserve(size_t need, cudaStream_t s) {
     if (need <= bytes) return WS_OK;
     if (ptr) {
@@ -96,7 +97,7 @@ struct DevBuf {
       bytes = 0;
       if (e != cudaSuccess) return cuda_fail(e, "cudaFreeAsync");
     }
-    size_t want = need + need / 8;
+    const size_t want = allocated(need);
     cudaError_t e = cudaMallocAsync(&ptr, want, s);
     if (e != cudaSuccess) {
       ptr = nullptr;
@@ -621,8 +622,9 @@ uint16_t* hash_ranks_of(const Plan* pl, int b) {
 
 // Most memory that ranks or bitmaps of rows may take between the two passes.
 // They spare the numeric pass a repetition of the symbolic one, but the caller
-// still has to find room for C.  4 GiB holds the ranks of 2^31 products, or
-// the bitmaps of 524,288 rows of 65,536 columns.
+// still has to find room for C.  Each of the three (hash ranks, bitmaps of the
+// dense and of the wide rows) takes 4 GiB at most: the ranks of 466,000 rows of
+// 4096 products, or the bitmaps of 466,000 rows of 65,536 columns.
 constexpr size_t kMaxKeptBytes = size_t{4} << 30;
 
 // Room for the ranks of the hash rows.  They are an aid, not a need: if the
@@ -630,7 +632,7 @@ constexpr size_t kMaxKeptBytes = size_t{4} << 30;
 void reserve_hash_ranks(Plan* pl, cudaStream_t s) {
   size_t n = 0;
   for (int b = 0; b < kNumHashBins; ++b) n += static_cast<size_t>(pl->seg_count[kSegHash0 + b]) << (kMinHashLog + b);
-  pl->hash_ranked = n > 0 && n * sizeof(uint16_t) <= kMaxKeptBytes && pl->hranks.reserve(n * sizeof(uint16_t), s) == WS_OK;
+  pl->hash_ranked = n > 0 && DevBuf::allocated(n * sizeof(uint16_t)) <= kMaxKeptBytes && pl->hranks.reserve(n * sizeof(uint16_t), s) == WS_OK;
   if (n > 0 && !pl->hash_ranked) {
     cudaGetLastError();  // the failed allocation is not an error of this call
     g_last_error.clear();
@@ -655,7 +657,8 @@ ws_status_t carve_rcd(Plan* pl, int64_t ncols, int sms, cudaStream_t s) {
   pl->rcd_width = static_cast<int>(width < kWidest ? width : kWidest);
   pl->rcd_slices = static_cast<int>((span + pl->rcd_width - 1) / pl->rcd_width);
   pl->rcd_words = static_cast<int>(align_up((span + 31) / 32, 4));
-  const int64_t most = static_cast<int64_t>(kMaxKeptBytes / (static_cast<size_t>(pl->rcd_words) * 4));
+  const size_t row_bytes = static_cast<size_t>(pl->rcd_words) * 4;
+  const int64_t fit = static_cast<int64_t>(kMaxKeptBytes / DevBuf::allocated(row_bytes)), most = fit > kMinBatch ? fit : kMinBatch;
   const size_t o_items = align_up(4 * kRcdCounters, 256);
   for (int64_t n = nr < most ? nr : most;; n = n / 2 < kMinBatch ? kMinBatch : n / 2) {
     const size_t o_bits = align_up(o_items + 8 * static_cast<size_t>(n) * pl->rcd_slices, 256);
@@ -690,7 +693,7 @@ ws_status_t carve_wb(Plan* pl, int64_t ncols, int sms, cudaStream_t s) {
   const size_t o_items = align_up(4 * kWbCounters, 256);
   const size_t o_bits = align_up(o_items + 8 * static_cast<size_t>(pl->wb_cap), 256);
   const size_t bits = static_cast<size_t>(nr) * pl->wb_words * 4;
-  bool kept = bits <= kMaxKeptBytes && pl->wb.reserve(o_bits + bits, s) == WS_OK;
+  bool kept = DevBuf::allocated(bits) <= kMaxKeptBytes && pl->wb.reserve(o_bits + bits, s) == WS_OK;
   if (!kept) {
     cudaGetLastError();  // the failed allocation is not an error of this call
     g_last_error.clear();

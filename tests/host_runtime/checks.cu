@@ -233,6 +233,27 @@ void few_dense_rows_take_small_windows() {
   }
 }
 
+// Ranks and bitmaps kept between the passes take at most 4 GiB of each kind, as
+// allocated, and a little more with the items and the rows' arrays.
+void kept_scratch_is_bounded() {
+  const struct {
+    int seg;
+    int64_t ncols, rows;
+  } cases[] = {{wsk::kSegHash0 + wsk::kNumHashBins - 1, 1 << 17, 500000}, {wsk::kSegRcd, 60000, 560000}, {wsk::kSegWb, 1 << 21, 32000}};
+  for (const auto& c : cases) {
+    ws_csr_t A = matrix(c.rows, 1 << 17, 64), B = matrix(1 << 17, c.ncols, 64), C = matrix(c.rows, c.ncols, 0);
+    fake::summary = wsk::DevSummary{};
+    fake::summary.n_pending = 1;
+    fake::summary.seg_count[c.seg] = static_cast<int>(c.rows);
+    fake::peak = fake::bytes;
+    const size_t before = fake::bytes;
+    int64_t nnz = 0;
+    CHECK(ws_spgemm_symbolic(A, B, C, &nnz, nullptr) == WS_OK);
+    CHECK(fake::peak - before < (size_t{4} << 30) + 100 * static_cast<size_t>(c.rows) + (size_t{64} << 20));
+    CHECK(ws_csr_destroy(C) == WS_OK);
+  }
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -246,6 +267,7 @@ struct {
     {"wide_rows_are_cut_as_far_as_the_gpu_needs", wide_rows_are_cut_as_far_as_the_gpu_needs},
     {"many_wide_bitmap_rows_run_by_themselves", many_wide_bitmap_rows_run_by_themselves},
     {"few_dense_rows_take_small_windows", few_dense_rows_take_small_windows},
+    {"kept_scratch_is_bounded", kept_scratch_is_bounded},
     {"columns_outside_have_no_place", columns_outside_have_no_place},
     {"failed_outer_product_waits_for_its_kernels", failed_outer_product_waits_for_its_kernels},
 };
