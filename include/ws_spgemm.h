@@ -319,6 +319,10 @@ ws_status_t ws_spgemm_plan_info(ws_csr_t C, int64_t* info, int n);
  *   key 8 (-1, 0, 1, 2, 4, 8, 16, 32 or 64; default -1) and key 9 ([2,
  *          1048576]; default 64): accepted, without effect (the elementwise
  *          operations once had several paths; they have one)
+ *   key 10: most bytes that the ranks of hash rows, the bitmaps of dense heavy
+ *          rows and those of wide heavy rows may each take between the passes
+ *          (default and maximum 2^32; beyond it the numeric pass works them
+ *          out again, dense heavy rows in batches of at least 1024)
  * Returns WS_ERR_INVALID_ARG for an unknown key or out-of-range value.
  */
 ws_status_t ws_set_tuning(int key, int64_t value);

@@ -626,13 +626,14 @@ uint16_t* hash_ranks_of(const Plan* pl, int b) {
 // dense and of the wide rows) takes 4 GiB at most: the ranks of 466,000 rows of
 // 4096 products, or the bitmaps of 466,000 rows of 65,536 columns.
 constexpr size_t kMaxKeptBytes = size_t{4} << 30;
+size_t g_kept_bytes = kMaxKeptBytes;  // ws_set_tuning can lower it
 
 // Room for the ranks of the hash rows.  They are an aid, not a need: if the
 // memory is not to be had the numeric pass works them out again.
 void reserve_hash_ranks(Plan* pl, cudaStream_t s) {
   size_t n = 0;
   for (int b = 0; b < kNumHashBins; ++b) n += static_cast<size_t>(pl->seg_count[kSegHash0 + b]) << (kMinHashLog + b);
-  pl->hash_ranked = n > 0 && DevBuf::allocated(n * sizeof(uint16_t)) <= kMaxKeptBytes && pl->hranks.reserve(n * sizeof(uint16_t), s) == WS_OK;
+  pl->hash_ranked = n > 0 && DevBuf::allocated(n * sizeof(uint16_t)) <= g_kept_bytes && pl->hranks.reserve(n * sizeof(uint16_t), s) == WS_OK;
   if (n > 0 && !pl->hash_ranked) {
     cudaGetLastError();  // the failed allocation is not an error of this call
     g_last_error.clear();
@@ -658,7 +659,7 @@ ws_status_t carve_rcd(Plan* pl, int64_t ncols, int sms, cudaStream_t s) {
   pl->rcd_slices = static_cast<int>((span + pl->rcd_width - 1) / pl->rcd_width);
   pl->rcd_words = static_cast<int>(align_up((span + 31) / 32, 4));
   const size_t row_bytes = static_cast<size_t>(pl->rcd_words) * 4;
-  const int64_t fit = static_cast<int64_t>(kMaxKeptBytes / DevBuf::allocated(row_bytes)), most = fit > kMinBatch ? fit : kMinBatch;
+  const int64_t fit = static_cast<int64_t>(g_kept_bytes / DevBuf::allocated(row_bytes)), most = fit > kMinBatch ? fit : kMinBatch;
   const size_t o_items = align_up(4 * kRcdCounters, 256);
   for (int64_t n = nr < most ? nr : most;; n = n / 2 < kMinBatch ? kMinBatch : n / 2) {
     const size_t o_bits = align_up(o_items + 8 * static_cast<size_t>(n) * pl->rcd_slices, 256);
@@ -693,7 +694,7 @@ ws_status_t carve_wb(Plan* pl, int64_t ncols, int sms, cudaStream_t s) {
   const size_t o_items = align_up(4 * kWbCounters, 256);
   const size_t o_bits = align_up(o_items + 8 * static_cast<size_t>(pl->wb_cap), 256);
   const size_t bits = static_cast<size_t>(nr) * pl->wb_words * 4;
-  bool kept = DevBuf::allocated(bits) <= kMaxKeptBytes && pl->wb.reserve(o_bits + bits, s) == WS_OK;
+  bool kept = DevBuf::allocated(bits) <= g_kept_bytes && pl->wb.reserve(o_bits + bits, s) == WS_OK;
   if (!kept) {
     cudaGetLastError();  // the failed allocation is not an error of this call
     g_last_error.clear();
@@ -1792,6 +1793,10 @@ ws_status_t ws_set_tuning(int key, int64_t value) {
       return WS_OK;
     case 9:  // likewise
       if (value < 2 || value > (int64_t{1} << 20)) return fail(WS_ERR_INVALID_ARG, "elementwise chunk length out of range");
+      return WS_OK;
+    case 10:
+      if (value < 0 || value > static_cast<int64_t>(kMaxKeptBytes)) return fail(WS_ERR_INVALID_ARG, "kept bytes out of range");
+      g_kept_bytes = static_cast<size_t>(value);
       return WS_OK;
   }
   return fail(WS_ERR_INVALID_ARG, "unknown tuning key %d", key);

@@ -373,6 +373,16 @@ def test_hash_rows_bin_edges(dtype, run_limit):
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+@pytest.mark.parametrize("dtype", DTYPES)
+def test_hash_rows_without_kept_ranks(dtype):
+    """The numeric pass works the ranks of every hash bin out itself."""
+    A, B = _hash_edge_case(dtype)
+    with tuning(kept_bytes=0):
+        rowptr, colidx, vals, info = run_gpu(A, B)
+    assert info["hash_rows"] == A.nrows
+    assert_matches_oracle(A, B, rowptr, colidx, vals)
+
+
 def test_dense_rows_without_room_for_bitmaps():
     """With almost all device memory taken the bitmaps of the dense heavy rows
     do not fit: the rows are taken in batches, and the numeric pass makes the
@@ -781,8 +791,11 @@ def _changed_columns_case(kind):
     if kind == "bitmap":  # 20 entries of 20 over 400 columns: crowded rows; a shift would keep the counts
         A, B, ncols = uniform_csr(200, 300, 20, rng), uniform_csr(300, 400, 20, rng), 70_000
         other = rng.permutation(ncols)[B.colidx]
+    elif kind == "dense":  # 5000 products over 30,000 columns, rows for three batches
+        A, B, ncols = _drawn_csr(2100, 3000, 250, rng), uniform_csr(3000, 30_000, 20, rng), 200_000
+        other = B.colidx + 150_000
     else:  # "wide": 5000 products over 100,000 columns
-        A, B, ncols = uniform_csr(40, 3000, 250, rng), uniform_csr(3000, 100_000, 20, rng), 1 << 21
+        A, B, ncols = _drawn_csr(40, 3000, 250, rng), uniform_csr(3000, 100_000, 20, rng), 1 << 21
         other = B.colidx + 1_500_000
     return A, HostCSR(B.nrows, ncols, B.rowptr, B.colidx, B.vals), other.astype(np.int32)
 
@@ -803,6 +816,12 @@ def _check_changed_columns(kind, rows_key):
         C = op.numeric()
         op.wait()
         assert_matches_oracle(A, B, *C.to_host(), rows=np.arange(0, A.nrows, 7))
+
+
+@pytest.mark.parametrize("kind,rows_key", [("wide", "wb_rows"), ("dense", "rcd_rows")])
+def test_columns_changed_before_bitmaps_are_made_again(kind, rows_key):
+    with tuning(kept_bytes=0):
+        _check_changed_columns(kind, rows_key)
 
 
 @pytest.mark.parametrize("kind,rows_key", [("bitmap", "bitmap_rows"), ("wide", "wb_rows")])
