@@ -254,6 +254,18 @@ void kept_scratch_is_bounded() {
   }
 }
 
+// Buckets of more than 63 products are sorted, whatever limit is asked for.
+void bucket_limit_is_what_the_kernel_can_hold() {
+  hash_product(1, nullptr);
+  CHECK(fake::run_limit == 63);
+  for (int64_t limit : {4096, 64, 63, 62, 1}) {
+    CHECK(ws_set_tuning(2, limit) == WS_OK);
+    hash_product(1, nullptr);
+    CHECK(fake::run_limit == (limit < 63 ? limit : 63));
+  }
+  CHECK(ws_set_tuning(2, 4097) == WS_ERR_INVALID_ARG);
+}
+
 struct {
   const char* name;
   void (*run)();
@@ -268,6 +280,7 @@ struct {
     {"many_wide_bitmap_rows_run_by_themselves", many_wide_bitmap_rows_run_by_themselves},
     {"few_dense_rows_take_small_windows", few_dense_rows_take_small_windows},
     {"kept_scratch_is_bounded", kept_scratch_is_bounded},
+    {"bucket_limit_is_what_the_kernel_can_hold", bucket_limit_is_what_the_kernel_can_hold},
     {"columns_outside_have_no_place", columns_outside_have_no_place},
     {"failed_outer_product_waits_for_its_kernels", failed_outer_product_waits_for_its_kernels},
 };

@@ -10,6 +10,7 @@ namespace fake {
 
 inline wsk::DevSummary summary{};             // what a pass hands to the host
 inline std::vector<size_t> bitmap_after;      // row kernels queued before every bitmap kernel
+inline int run_limit = 0;                    // products of a hash bucket that are compared
 inline int rcd_width = 0, rcd_slices = 0;     // value windows of the dense rows
 inline int64_t wb_part = 0;  // products per item that the wide rows' kernels were given
 inline int launch_status = 0;                 // error flags that SpMSpV's kernels find
@@ -46,6 +47,7 @@ template <typename T>
 void launch_hash(const RowPlan<T>& p, int, bool, int, cudaStream_t s, int*) {
   fake::row_kernels.push_back(s);
   fake::pending[p.status] = s;
+  fake::run_limit = p.run_limit;
 }
 template <typename T>
 void launch_bmr(const RowPlan<T>&, int, bool, int, cudaStream_t s, int*) { fake::row_kernels.push_back(s); }
