@@ -303,9 +303,9 @@ ws_status_t ws_spgemm_plan_info(ws_csr_t C, int64_t* info, int n);
  *   key 1: largest product count of a row that uses the shared-memory hash
  *          path (default 4096; smaller values send more rows to the
  *          dense-window path, 0 sends every multi-entry row there)
- *   key 2: most products a bucket of a hash row may hold (default 64; a row
+ *   key 2: most products a bucket of a hash row may hold (default 63; a row
  *          with a fuller bucket is sorted; smaller values send more rows
- *          there)
+ *          there, larger ones, up to 4096, act as 63)
  *   key 3: dense-window slice width in columns (default 8192 for double,
  *          16384 for float; must be a multiple of 1024, 0 = default)
  *   key 4: widest column range of a row that uses the bitmap path

@@ -35,7 +35,7 @@ int64_t g_bitmap_span = kMaxBitmapSpan;
 int g_bmr_max_a = kBmrMaxA;
 int g_rcd_max_a = kRcdDefaultMaxA;
 int64_t g_wb_span = kWbMaxSpan;
-int g_run_limit = 64;
+int g_run_limit = kMaxHashBucket;
 int g_dense_width = 0;  // 0 = default per value type
 constexpr int kLongRowThreshold = 16;  // rows with more stored entries are analysed by a warp or a CTA
 
@@ -396,7 +396,7 @@ struct Plan {
   int log2_group = 5;
   bool all_planned = false;  // the planning pass took every row: its segment is rows 0..m-1 in order
   int dense_width = 0;
-  int run_limit = 64;
+  int run_limit = kMaxHashBucket;
   bool hash_ranked = false;  // hranks holds the hash rows' ranks
   int sym_launches = 0, num_launches = 0;
   struct OuterState* outer = nullptr;  // outer-product SpGEMM between its two passes
@@ -1764,7 +1764,7 @@ ws_status_t ws_set_tuning(int key, int64_t value) {
       return WS_OK;
     case 2:
       if (value < 1 || value > 4096) return fail(WS_ERR_INVALID_ARG, "run limit out of range");
-      g_run_limit = static_cast<int>(value);
+      g_run_limit = value < kMaxHashBucket ? static_cast<int>(value) : kMaxHashBucket;
       return WS_OK;
     case 3:
       if (value != 0 && (value < 1024 || value > 16384 || value % 1024 != 0))

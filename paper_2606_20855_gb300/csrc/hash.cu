@@ -46,7 +46,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kDupBit = 0x8000;
-constexpr int kMaxBucket = 63;  // most products of a bucket that are compared with one another
 
 // Shape of a bin: rows of at most kCap products, a team of W warps, kS
 // products per thread.
@@ -269,7 +268,7 @@ __device__ __forceinline__ int rank_row(const int (&col)[Bin<LOGC, W>::kS], int 
 #pragma unroll
       for (int w = 0; w < W; ++w) most = max(most, scratch[w]);
     }
-    if (most <= run_limit && most <= kMaxBucket) {
+    if (most <= run_limit) {  // at most kMaxHashBucket
 #pragma unroll
       for (int j = 0; j < kOwn; ++j) cnt[t * kOwn + j] = own[j] + (ex | (ex << 16));
       if (t == 0) base[kCap] = static_cast<uint16_t>(ub);

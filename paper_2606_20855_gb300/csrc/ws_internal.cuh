@@ -25,6 +25,7 @@ namespace wsk {
 
 constexpr int kNumHashBins = 8;
 constexpr int kMinHashLog = 5;  // bin b holds rows of at most 1 << (kMinHashLog + b) products
+constexpr int kMaxHashBucket = 63;  // most products of a hash bucket that are compared with one another (6 bits)
 constexpr int kMaxHashProducts = 32 << (kNumHashBins - 1);  // 4096
 
 // Bitmap bins: bitmap of 1 << log_words 32-bit words (the row's column range
