@@ -246,8 +246,12 @@ __global__ void __launch_bounds__(kSvThreads) sv_tile_count_kernel(const uint8_t
 // cnt[t]: thread k takes the 16 positions from 16 k on, so a tile costs one
 // round of loads (rounds of 32 positions per warp were a chain of sixteen: 15
 // us for 2^20 positions).
-template <typename T>
-__global__ void __launch_bounds__(kSvThreads) sv_write_kernel(const SpmspvPlan<T> p, bool scanned) {
+// SCANNED: the tiles' offsets are in cnt.  There are thousands of tiles then, so
+// the values are not fetched ahead of the scan, which leaves registers for
+// twice the CTAs (2^24 positions, fp64: 43 us with the values fetched ahead, 11
+// without).
+template <typename T, bool SCANNED>
+__global__ void __launch_bounds__(kSvThreads, SCANNED ? 6 : 3) sv_write_kernel(const SpmspvPlan<T> p) {
   __shared__ int scratch[32];
   __shared__ long long sums[32];
   const int64_t tiles = (p.m + kSvTile - 1) / kSvTile;
@@ -261,13 +265,16 @@ __global__ void __launch_bounds__(kSvThreads) sv_write_kernel(const SpmspvPlan<T
       const uint32_t m = __vcmpne4(word[h], 0u) & 0x01010101u;
       set |= ((m * 0x01020408u) >> 24 & 15u) << (4 * h);  // byte k of the word to bit k
     }
-    T acc[16];
+    T acc[SCANNED ? 1 : 16];
+    auto value = [&](int b) { return p.acc[i0 + b] + T(0); };  // + 0: no -0.0 from the start value
+    if constexpr (!SCANNED) {
 #pragma unroll
-    for (int b = 0; b < 16; ++b) acc[b] = (set >> b) & 1u ? p.acc[i0 + b] + T(0) : T(0);  // + 0: no -0.0 from the start value
+      for (int b = 0; b < 16; ++b) acc[b] = (set >> b) & 1u ? value(b) : T(0);
+    }
     int total;
     const int before = block_exclusive_scan(__popc(set), scratch, &total);
     long long base = 0;  // marked positions of the tiles before
-    if (scanned) {
+    if constexpr (SCANNED) {
       base = p.cnt[t];
     } else {
       long long x = 0;
@@ -282,7 +289,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_write_kernel(const SpmspvPlan<T
         const long long at = base + before + k;
         if (at < p.cap && i0 + b < p.m) {
           p.y_idx[at] = static_cast<int32_t>(i0 + b);
-          p.y_vals[at] = acc[b];
+          p.y_vals[at] = SCANNED ? value(b) : acc[SCANNED ? 0 : b];
         } else {
           bad = true;
         }
@@ -290,7 +297,7 @@ __global__ void __launch_bounds__(kSvThreads) sv_write_kernel(const SpmspvPlan<T
       }
     }
     if (threadIdx.x == 0) {
-      if (total != p.cnt[t + 1] - (scanned ? base : 0)) bad = true;
+      if (total != p.cnt[t + 1] - (SCANNED ? base : 0)) bad = true;
       if (t == tiles - 1) *const_cast<volatile long long*>(&p.host->nnz) = base + total;
     }
     if (bad) atomicOr(p.status, kErrCount);
@@ -323,7 +330,7 @@ void launch_spmspv(const SpmspvPlan<T>& p, int num_sms, cudaStream_t s, int* lau
   const bool scanned = tiles > kDirectTiles;
   sv_tile_count_kernel<<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p.mark, p.m, p.cnt);
   if (scanned) launch_scan(p.cnt, tiles, p.partials, p.sum, s, launches);
-  sv_write_kernel<T><<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p, scanned);
+  (scanned ? sv_write_kernel<T, true> : sv_write_kernel<T, false>)<<<grid_for(tiles, 1, num_sms, 8), kSvThreads, 0, s>>>(p);
   *launches += 3;
 }
 
