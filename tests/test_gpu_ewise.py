@@ -4,7 +4,7 @@ the CPU oracle, through the C ABI.
 Structure (rowptr, colidx) must be bit-exact; values within 1e-12 (float64)
 or 1e-5 (float32) of |A[i,j]| + |B[i,j]| (SpAdd) or |A[i,j] B[i,j]|
 (Hadamard): one rounding in the value type against the float64 oracle.
-Cases: random shapes, every lane-group size, rows cut into many chunks with
+Cases: random shapes, rows of many lengths, rows cut into many tiles with
 equal columns on both sides of the cuts, empty operands and shapes, cancelled
 sums, the full-size R-MAT inputs (B a relabelled copy of A, and B = A), and
 the error paths.
@@ -53,39 +53,41 @@ def check(A, B, op, validate=False):
     return info
 
 
-# lanes per chunk: 1 (one thread per chunk), 2 (one lane per chunk of a
-# warp-staged tile of 32 chunks), 0 (lane groups of 4..32 sized from the mean
-# row length) and 64 (a warp per 64-position chunk ranking every entry by
-# binary search)
-LANES = [1, 2, 0, 64]
-
-
-@pytest.mark.parametrize("lanes", LANES)
 @pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("dtype", DTYPES)
 @pytest.mark.parametrize("seed", range(10))
-def test_random_shapes(seed, dtype, op, lanes):
+def test_random_shapes(seed, dtype, op):
     rng = np.random.default_rng(900 + seed)
     m, n = (int(x) for x in rng.integers(1, 500, size=2))
     A = random_csr(m, n, float(rng.choice([0.005, 0.03, 0.2])), rng, dtype, "sym", empty_rows=0.1)
     B = random_csr(m, n, float(rng.choice([0.005, 0.03, 0.2])), rng, dtype, "sym", empty_rows=0.1)
-    with tuning(ewise_lanes=lanes):
-        check(A, B, op, validate=True)
+    check(A, B, op, validate=True)
 
 
-@pytest.mark.parametrize("lanes", LANES)
 @pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("per_row", [2, 6, 12, 40, 200])
-def test_every_group_size(per_row, op, lanes):
-    # mean merged row lengths 4 .. 400 select 4, 8, 16 and 32 lanes per chunk
-    # (lanes 0), or cut rows into 1..7 chunks of 64 (lanes 1); 30,011 rows
-    # give many CTAs and a ragged last one
+def test_row_lengths(per_row, op):
+    # mean merged row lengths 4 .. 400: 400 to 5 rows per tile; 30,011 rows give
+    # many tiles and a ragged last one
     rng = np.random.default_rng(per_row)
     n = max(64, per_row * per_row // 2)  # rejection sampling of distinct columns needs n >> per_row^2 / 2
     A = uniform_csr(30_011, n, per_row, rng, np.float64, "sym")
     B = uniform_csr(30_011, n, per_row, rng, np.float64, "sym")
-    with tuning(ewise_lanes=lanes):
-        check(A, B, op)
+    check(A, B, op)
+
+
+def test_tuning_without_effect():
+    """The two keys of the paths that are gone are accepted and change nothing."""
+    rng = np.random.default_rng(5)
+    A = random_csr(300, 200, 0.1, rng, np.float64, "sym")
+    B = random_csr(300, 200, 0.1, rng, np.float64, "sym")
+    want = run_ewise(A, B, "add")
+    for lanes, chunk in ((1, 2), (2, 7), (0, 64), (32, 64), (64, 1 << 20)):
+        with tuning(ewise_lanes=lanes, ewise_chunk=chunk):
+            got = run_ewise(A, B, "add")
+        for x, y in zip(want[:3], got[:3]):
+            np.testing.assert_array_equal(x, y)
+        assert got[3] == want[3]
 
 
 def _long_rows(m, n, lens, rng, overlap):
@@ -105,19 +107,15 @@ def _long_rows(m, n, lens, rng, overlap):
     return build(ra), build(rb)
 
 
-@pytest.mark.parametrize("lanes,chunk", [(1, 64), (1, 2), (1, 7), (2, 16), (2, 2), (2, 7), (0, 64), (32, 64),
-                                         (64, 64), (-1, 64)])
 @pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("overlap", [0.0, 0.5, 1.0])
-def test_long_rows_many_chunks(overlap, op, lanes, chunk):
-    # rows of up to 20,000 entries per operand are cut into hundreds of chunks
-    # (tens of thousands with chunks of 2); with overlap 1.0 every column is an
-    # equal pair, so pairs meet every cut
+def test_long_rows_many_tiles(overlap, op):
+    # rows of up to 20,000 entries per operand are cut into twenty tiles; with
+    # overlap 1.0 every column is an equal pair, so pairs meet every cut
     rng = np.random.default_rng(31)
     lens = [20_000, 1, 0, 5_000, 777, 3, 12_345, 64, 65, 0]
     A, B = _long_rows(len(lens), 40_000, lens, rng, overlap)
-    with tuning(ewise_lanes=lanes, ewise_chunk=chunk):
-        check(A, B, op)
+    check(A, B, op)
 
 
 @pytest.mark.parametrize("op", OPS)
@@ -185,20 +183,18 @@ def test_cancelled_sums_are_kept():
 
 
 @pytest.mark.slow
-@pytest.mark.parametrize("lanes", [None, 1, 64])
 @pytest.mark.parametrize("op", OPS)
 @pytest.mark.parametrize("name", list(EWISE_WORKLOADS))
-def test_full_size_workloads(name, op, lanes):
+def test_full_size_workloads(name, op):
     A, B = ewise_workload(name)
     dA = DeviceCSR.from_host(A, "cuda:0")
     dB = dA if B is A else DeviceCSR.from_host(B, "cuda:0")
-    with tuning(**({} if lanes is None else {"ewise_lanes": lanes})):
-        with Ewise(dA, dB, op) as e:
-            e.symbolic()
-            C = e.numeric()
-            e.wait()
-            device_invariants(C)
-            rowptr, colidx, vals = C.to_host()
+    with Ewise(dA, dB, op) as e:
+        e.symbolic()
+        C = e.numeric()
+        e.wait()
+        device_invariants(C)
+        rowptr, colidx, vals = C.to_host()
     ref = oracle_ewise(A, B, op)
     np.testing.assert_array_equal(rowptr, ref.rowptr)
     np.testing.assert_array_equal(colidx, ref.colidx)
