@@ -148,11 +148,11 @@ def test_full_size_workload():
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
-@pytest.mark.parametrize("m", [1, 15, 4095, 4096, 4097, 70_000])
+@pytest.mark.parametrize("m", [1, 15, 2047, 2048, 2049, 4095, 4096, 4097, 70_000])
 def test_signed_zeros_and_tiny_products(dtype, m):
     """Positions whose products are -0.0, +0.0, subnormal of either sign or
     cancel exactly stay in y's pattern, for lengths around the compaction tile
-    (4096) and the positions summed in shared memory (1024), more than once on
+    (4096) and the positions summed in shared memory (2048), more than once on
     one handle; y holds no -0.0."""
     rng = np.random.default_rng(m)
     tiny = np.finfo(dtype).tiny
