@@ -7,9 +7,12 @@ device.  For them the library keeps the scan's scratch in a fixed array.
 
 Checks:
 - the result equals numpy's cumulative sum of the host counts (a check that
-  shares nothing with the library's scan), at sizes that take the one-launch
-  path, the three-launch path with a ragged tail, the multi-round scan of the
-  tile sums (more than 1024 tiles) and exactly the 16,777,216-row limit;
+  shares nothing with the library's scan), at the sizes around the one-launch
+  path (4096 rows) and on the two-launch path, where every tile of 4096 rows
+  adds up the tile sums before it: with a ragged tail, and with 4096 tiles at
+  exactly the 16,777,216-row limit;
+- above that limit the regular passes scan the tile sums in a launch of their
+  own: the row pointer of a product of 16,777,217 and more rows;
 - it equals the row pointer that the regular symbolic pass
   (ws_spgemm_symbolic) writes for the same product, on two calls in a row
   with different sizes (the second call must not see the first call's
@@ -37,7 +40,7 @@ def _scan(rp, m):
     torch.cuda.synchronize()
 
 
-@pytest.mark.parametrize("m", [1, 16_384, 16_385, 300_001, 4_194_305, MAX_ROWS])
+@pytest.mark.parametrize("m", [1, 4096, 4097, 16_384, 16_385, 300_001, 4_194_305, MAX_ROWS])
 def test_static_scan_matches_numpy_cumsum(m):
     rng = np.random.default_rng(m)
     counts = rng.integers(0, 1000, size=m, dtype=np.int64)
@@ -70,6 +73,32 @@ def test_static_scan_matches_symbolic_rowptr_twice():
         rp[0] = 123_456_789          # ignored on entry, must become 0
         _scan(rp, m)
         assert torch.equal(rp, ref)
+
+
+@pytest.mark.parametrize("m", [MAX_ROWS + 1, MAX_ROWS + 4097])
+def test_rowptr_of_more_rows_than_direct_tile_sums(m):
+    from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+    rng = np.random.default_rng(m % 101)
+    filled = np.unique(np.concatenate([[0, 4095, 4096, MAX_ROWS - 1, MAX_ROWS, m - 1], rng.integers(0, m, size=50_000)]))
+    lens = np.zeros(m, dtype=np.int64)
+    lens[filled] = 1 + filled % 3
+    rowptr = np.concatenate([[0], np.cumsum(lens)])
+    cols = np.concatenate([np.arange(k) * 20 + 7 for k in lens[filled]])  # B rows 7, 27, 47: no common columns
+    dev = torch.device("cuda:0")
+    A = DeviceCSR(m, 60, torch.from_numpy(rowptr).to(dev), torch.from_numpy(cols.astype(np.int32)).to(dev),
+                  torch.ones(cols.size, dtype=torch.float64, device=dev))
+    b_lens = np.arange(60, dtype=np.int64)
+    b_rowptr = np.concatenate([[0], np.cumsum(b_lens)])
+    b_cols = np.concatenate([np.arange(k) + 100 * i for i, k in enumerate(b_lens)])
+    B = DeviceCSR(60, 100_000, torch.from_numpy(b_rowptr).to(dev), torch.from_numpy(b_cols.astype(np.int32)).to(dev),
+                  torch.ones(b_cols.size, dtype=torch.float64, device=dev))
+    want = np.zeros(m + 1, dtype=np.int64)
+    np.add.at(want, np.repeat(filled, lens[filled]) + 1, b_lens[cols])
+    np.cumsum(want, out=want)
+    with SpGEMM(A, B) as op:
+        for _ in range(2):  # the second pass starts from the summary that the first one cleared
+            assert op.symbolic() == want[-1]
+            np.testing.assert_array_equal(op.c_rowptr.cpu().numpy(), want)
 
 
 def test_static_scan_zero_rows_and_refusal():
