@@ -5,6 +5,10 @@ error 1e-12 (float64) or 1e-5 (float32) of the summation-order bound.
 """
 from __future__ import annotations
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -383,17 +387,52 @@ def test_hash_rows_without_kept_ranks(dtype):
     assert_matches_oracle(A, B, rowptr, colidx, vals)
 
 
+# A product twice in a process of its own (an earlier test's freed scratch would
+# serve): op2 with all the room it wants, then op1 whose symbolic pass finds less
+# than 56 MB of device memory left.  `setup` makes A and B, `check` looks at the
+# operations and at C as (rp, ci, v) of both.
+_SHORT_OF_MEMORY = """
+import numpy as np, torch
+from tests._gpu import assert_matches_oracle
+from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+%s
+dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+def product(short):
+    op = SpGEMM(dA, dB)
+    held = []
+    if short:
+        size = 1 << 30
+        while size >= 1 << 24:
+            if torch.cuda.mem_get_info()[0] - size > 40 << 20:
+                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
+            else:
+                size >>= 1
+    op.symbolic()
+    del held
+    torch.cuda.empty_cache()
+    C = op.numeric()
+    op.wait()
+    return op, C.to_host()
+op2, (rp2, ci2, v2) = product(False)  # its scratch stays taken
+op1, (rp1, ci1, v1) = product(True)
+assert np.array_equal(rp1, rp2) and np.array_equal(ci1, ci2)
+%s
+"""
+
+
+def _run_short_of_memory(setup, check):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    res = subprocess.run([sys.executable, "-c", _SHORT_OF_MEMORY % (setup, check)], cwd=root, capture_output=True,
+                         text=True, timeout=300)
+    assert res.returncode == 0, res.stderr[-2000:]
+
+
 def test_dense_rows_without_room_for_bitmaps():
     """With almost all device memory taken the bitmaps of the dense heavy rows
     do not fit: the rows are taken in batches, and the numeric pass makes the
     bitmaps again (more launches, the same C).  (A process of its own: an
     earlier test's freed scratch would serve.)"""
-    import subprocess
-    import sys
-    code = """
-import numpy as np, torch
-from tests._gpu import assert_matches_oracle
-from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+    _run_short_of_memory("""
 from synth import HostCSR
 rng = np.random.default_rng(39)
 k, n, m = 1400, 1 << 16, 12001  # 98 MB of bitmaps, an odd last batch
@@ -403,81 +442,30 @@ bci = np.concatenate([np.sort(rng.choice(n, size=x, replace=False)) for x in len
 B = HostCSR(k, n, brp, bci, 2 * rng.random(bci.size) - 1)
 aci = np.sort(rng.random((m, k)).argsort(axis=1)[:, :100], axis=1).astype(np.int32).ravel()
 A = HostCSR(m, k, np.arange(m + 1, dtype=np.int64) * 100, aci, 2 * rng.random(aci.size) - 1)
-dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
-def product(hog):
-    op = SpGEMM(dA, dB)
-    held = []
-    if hog:
-        size = 1 << 30
-        while size >= 1 << 24:  # leave less than 56 MB
-            if torch.cuda.mem_get_info()[0] - size > 40 << 20:
-                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
-            else:
-                size >>= 1
-    op.symbolic()
-    del held
-    torch.cuda.empty_cache()
-    C = op.numeric()
-    op.wait()
-    return op, C.to_host()
-op2, (rp2, ci2, v2) = product(False)  # kept: its scratch stays taken
-op1, (rp1, ci1, v1) = product(True)
+""", """
 i1, i2 = op1.plan_info(), op2.plan_info()
 assert i1["rcd_rows"] == i2["rcd_rows"] > 11900
 assert i1["numeric_launches"] > i2["numeric_launches"]
-assert np.array_equal(rp1, rp2) and np.array_equal(ci1, ci2)
 assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.concatenate([np.arange(0, m, 101), [m - 1]]))
-"""
-    import os
-    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
-    assert res.returncode == 0, res.stderr[-2000:]
+""")
 
 
 def test_hash_rows_without_room_for_ranks():
     """With almost all device memory taken the symbolic pass cannot keep the
     ranks of the hash rows and the numeric pass works them out: the same C.
     (A process of its own: an earlier test's freed scratch would serve.)"""
-    import subprocess
-    import sys
-    code = """
-import numpy as np, torch
+    _run_short_of_memory("""
 from tests.test_gpu_parity import _hash_edge_case
-from tests._gpu import assert_matches_oracle
-from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
 from synth import HostCSR
 A, B = _hash_edge_case(np.float64)
 reps = 400  # 100 rows, 400 times: the ranks take about 88 MB
 rp = np.concatenate([[0], np.cumsum(np.tile(np.diff(A.rowptr), reps))]).astype(np.int64)
 A = HostCSR(A.nrows * reps, A.ncols, rp, np.tile(A.colidx, reps), np.tile(A.vals, reps))
-dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
-def product(hog):
-    op = SpGEMM(dA, dB)
-    held = []
-    if hog:
-        size = 1 << 30
-        while size >= 1 << 24:  # leave less than 48 MB
-            if torch.cuda.mem_get_info()[0] - size > 40 << 20:
-                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
-            else:
-                size >>= 1
-    op.symbolic()
-    del held
-    torch.cuda.empty_cache()
-    C = op.numeric()
-    op.wait()
-    return op, C.to_host()
-op2, (rp2, ci2, v2) = product(False)  # kept: its scratch stays taken
-op1, (rp1, ci1, v1) = product(True)
+""", """
 assert op1.plan_info()["hash_rows"] == A.nrows
-assert np.array_equal(rp1, rp2) and np.array_equal(ci1, ci2)
 assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.arange(100))
 assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.arange(A.nrows - 100, A.nrows))
-"""
-    import os
-    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
-    assert res.returncode == 0, res.stderr[-2000:]
+""")
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
@@ -635,47 +623,19 @@ def test_wide_rows_without_room_for_bitmaps():
     """With almost all device memory taken the bitmaps of the wide rows are not
     kept and the numeric pass makes them again: the same C.  (A process of its
     own: an earlier test's freed scratch would serve.)"""
-    import subprocess
-    import sys
-    code = """
-import numpy as np, torch
-from tests._gpu import assert_matches_oracle
-from paper_2606_20855_gb300.spgemm import DeviceCSR, SpGEMM
+    _run_short_of_memory("""
 from synth import HostCSR, uniform_csr
 rng = np.random.default_rng(41)
 B = uniform_csr(5000, 1 << 20, 20, rng)
 aci = np.sort(rng.random((601, 5000)).argsort(axis=1)[:, :900], axis=1).astype(np.int32).ravel()
 A = HostCSR(601, 5000, np.arange(602, dtype=np.int64) * 900, aci, 2 * rng.random(aci.size) - 1)  # 79 MB of bitmaps
-dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
-def product(hog):
-    op = SpGEMM(dA, dB)
-    held = []
-    if hog:
-        size = 1 << 30
-        while size >= 1 << 24:  # leave less than 56 MB
-            if torch.cuda.mem_get_info()[0] - size > 40 << 20:
-                held.append(torch.empty(size, dtype=torch.uint8, device="cuda"))
-            else:
-                size >>= 1
-    op.symbolic()
-    del held
-    torch.cuda.empty_cache()
-    C = op.numeric()
-    op.wait()
-    return op, C.to_host()
-op2, (rp2, ci2, v2) = product(False)  # kept: its scratch stays taken
-op1, (rp1, ci1, v1) = product(True)
+""", """
 i1, i2 = op1.plan_info(), op2.plan_info()
 assert i1["wb_rows"] == i2["wb_rows"] == 601
 assert i1["numeric_launches"] < i2["numeric_launches"]  # no launch to zero the values
-assert np.array_equal(rp1, rp2) and np.array_equal(ci1, ci2)
 assert_matches_oracle(A, B, rp1, ci1, v1, rows=np.arange(0, 601, 10))
 assert_matches_oracle(A, B, rp2, ci2, v2, rows=np.arange(0, 601, 10))
-"""
-    import os
-    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-    res = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
-    assert res.returncode == 0, res.stderr[-2000:]
+""")
 
 
 @pytest.mark.parametrize("dtype", DTYPES)
