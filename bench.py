@@ -236,9 +236,10 @@ def roofline_obj(nbytes: int, seconds: float, peaks: dict, traffic) -> dict:
 def numeric_kernels(info: dict) -> str:
     """Which numeric kernels a plan launches (from ws_spgemm_plan_info)."""
     names = []
-    for key, kern in (("direct_rows", "direct_rows_kernel"), ("bitmap_rows", "bmr_numeric/bitmap_rows_kernel"),
-                      ("hash_rows", "hash_rows_kernel"), ("rcd_rows", "rcd_numeric_kernel"), ("wb_rows", "wb_kernel"),
-                      ("dense_rows", "dense_rows_kernel")):
+    for key, kern in (("direct_rows", "direct_rows_kernel"),
+                      ("bitmap_rows", "bmr_numeric_kernel/bmr_group_numeric_kernel/bitmap_rows_kernel"),
+                      ("hash_rows", "hash_rows_kernel"), ("rcd_rows", "rcd_numeric_kernel"),
+                      ("wb_rows", "wb_zero_kernel/wb_numeric_kernel"), ("dense_rows", "dense_rows_kernel")):
         if info.get(key):
             names.append(kern)
     return ", ".join(names) or "none"

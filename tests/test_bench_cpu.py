@@ -105,3 +105,16 @@ def test_traffic_records_follow_the_kernel_source(tmp_path, monkeypatch):
     assert bench.recorded_traffic("other", "k_kernel") is None
     src.write_text("// kernel v2\n")  # the kernel changed after the capture
     assert bench.recorded_traffic("w", "k_kernel") is None
+
+
+def test_named_kernels_exist():
+    """The kernels that the bench names for a plan are kernels of the library."""
+    import glob
+    import re
+    sys.path.insert(0, ROOT)
+    import bench
+
+    keys = ("direct_rows", "bitmap_rows", "hash_rows", "rcd_rows", "wb_rows", "dense_rows")
+    source = "".join(open(f).read() for f in glob.glob(os.path.join(ROOT, "paper_2606_20855_gb300", "csrc", "*.cu")))
+    for name in re.split("[,/ ]+", bench.numeric_kernels({k: 1 for k in keys})):
+        assert re.search(rf"__global__[^;{{]*\b{name}\(", source), name
