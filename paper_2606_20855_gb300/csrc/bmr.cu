@@ -75,38 +75,6 @@ __device__ __forceinline__ uint32_t rank_pack(int lo_rank, int hi_rank) {
   return static_cast<uint32_t>(lo_rank & 0xffff) | (static_cast<uint32_t>(hi_rank & 0xffff) << 16);
 }
 
-// Loads the row's products into registers: lane j < na first loads stored A
-// entry j (its B row start, length and value), then every lane loads its
-// elements of the B rows of its group.
-template <typename T, int G, bool NUMERIC, int kSteps>
-__device__ __forceinline__ void load_products(const RowPlan<T>& p, int64_t ra, int na, int lane, int* col, T* val) {
-  constexpr int kGroups = 32 / G;
-  const int grp = lane / G, gl = lane % G;
-  long long my_b0 = 0;
-  int my_len = 0;
-  T my_a = T(0);
-  if (lane < na) {
-    const int k = p.A.colidx[ra + lane];
-    my_b0 = p.B.rowptr[k];
-    my_len = static_cast<int>(p.B.rowptr[k + 1] - my_b0);
-    if constexpr (NUMERIC) my_a = p.A.vals[ra + lane];
-  }
-#pragma unroll
-  for (int s = 0; s < kSteps; ++s) {
-    const int j = s * kGroups + grp;
-    const long long b0 = __shfl_sync(kFull, my_b0, j & 31);
-    const int len = __shfl_sync(kFull, my_len, j & 31);
-    T a = T(0);
-    if constexpr (NUMERIC) a = __shfl_sync(kFull, my_a, j & 31);
-    col[s] = -1;
-    val[s] = T(0);
-    if (j < na && gl < len) {
-      col[s] = p.B.colidx[b0 + gl];
-      if constexpr (NUMERIC) val[s] = a * p.B.vals[b0 + gl];
-    }
-  }
-}
-
 template <class S, int kSteps>
 __device__ __forceinline__ void clear_bits(uint32_t* bm, const int* col, int lo) {
 #pragma unroll
