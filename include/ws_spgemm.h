@@ -263,10 +263,11 @@ ws_status_t ws_spgemm_wait(ws_csr_t C, ws_stream_t stream);
 
 /*
  * ws_csr_destroy -- releases the handle and the scratch it owns (never the
- * borrowed arrays).  NULL-safe.  Synchronises the device if the handle owns
- * scratch, so pending work that uses it completes first; device scratch goes
- * back to the stream-ordered pool and the pinned host summary to a
- * process-wide free list.
+ * borrowed arrays).  NULL-safe.  Synchronises the handle's device (whichever
+ * is current) if the handle owns scratch, so pending work that uses it completes
+ * first.  Scratch of up to 32 MiB is kept for the next handles of the device, of
+ * up to eight handles in the process; other device scratch goes back to the
+ * stream-ordered pool and the pinned host summary to a process-wide free list.
  * Passage: the end of the lifecycle of Sec. 4 ("Building on Finch"): once C is
  * frozen, the workspaces the passes declared are no longer needed.  The
  * paper has no explicit release call; this one frees the library's share.
@@ -288,7 +289,8 @@ ws_status_t ws_csr_nnz(ws_csr_t handle, int64_t* nnz_out);
 /*
  * ws_spgemm_plan_info -- counts from the last symbolic pass of C, for
  * diagnostics and tests: info[0] empty rows, info[1] single-entry (direct
- * copy) rows, info[2] hash rows, info[3] hash rows ranked by a sort, info[4] dense-window rows, info[5] dense-window slices,
+ * copy) rows, info[2] hash rows, info[3] hash rows ranked by a sort,
+ * info[4] dense-window rows, info[5] dense-window slices,
  * info[6] total products (sum over rows of the product count),
  * info[7] number of kernel launches queued by the last symbolic pass,
  * info[8] number queued by the last numeric pass, info[9] bitmap rows,

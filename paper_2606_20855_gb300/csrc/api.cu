@@ -1,14 +1,20 @@
 // C ABI of the SpGEMM library (declared in include/ws_spgemm.h).
 //
-// Symbolic pass (ws_spgemm_symbolic), all on the caller's stream:
-//   1. analyze   per-row product count, column range, class       (2 launches)
-//   -- the class counts reach the host (written by the last kernel, stream sync)
+// Symbolic pass (ws_spgemm_symbolic):
+//   1. plan      regular rows counted in the first read of A, where
+//                columns and averages allow                         (1 launch and a scan)
+//      analyze   per-row product count, column range, class         (2 launches)
+//   -- the class counts reach the host (written by the last kernel, stream sync);
+//      if the planning pass took every row, this is the end
 //   2. scatter   group rows by class                                (1 launch)
-//   3. dense     expand dense-window rows into column slices, count (2 launches)
-//   4. hash      count distinct columns per hash bin                (1 launch per non-empty bin)
-//   5. scan      counts -> C.rowptr                                 (1 or 2 launches)
+//   3. rows      count the distinct columns, per class and bin      (1 launch each, 2 for dense windows)
+//   4. scan      counts -> C.rowptr                                 (1, 2 or 3 launches)
 //   -- nnz(C) and the status word reach the host (written by the scan, stream sync)
-// Numeric pass (ws_spgemm_numeric): one launch per non-empty class, no sync.
+// Numeric pass (ws_spgemm_numeric), no sync: one launch per non-empty class and
+// bin; one more that zeroes the wide rows cut into parts; dense heavy rows without
+// room for all bitmaps go in batches of two.
+// The row kernels of both passes are spread over the caller's stream and up to
+// three side streams (class Fork), everything else stays on the caller's stream.
 #include <cuda.h>
 
 #include <cstdarg>

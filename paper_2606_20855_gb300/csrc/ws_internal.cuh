@@ -8,14 +8,21 @@
 //   direct        exactly one stored A[i,k]      -> C[i,:] = A[i,k] * B[k,:]
 //   bitmap bin b  column range of the row at most 32 << log_words(b) columns and
 //                 min(ub_i, range) <= cap(b)     -> bitmap + rank workspace
+//   register      at most 16 stored A entries whose B rows fit a lane group
+//   bitmap bin b                                 -> bitmap ranked by one warp, ranks kept
 //   hash bin b    ub_i <= 32 << b (b = 0..7)     -> products in registers, ranked through
 //                                                  32 << b monotone-hash buckets
-//   dense window  ub_i above the hash limit      -> column slices of the row, each a
+//   dense heavy   range up to 65,536 columns     -> flag bytes and a kept bitmap, then windows
+//                                                  of consecutive output entries
+//   wide heavy    range up to 2^20 columns       -> kept bitmap, then parts of the row's
+//                                                  products added to C
+//   dense window  rows above the others' limits  -> column slices of the row, each a
 //                                                  dense bitmap + value workspace
-// Each class is a different realisation of the per-row workspace w of
-// Gustavson's algorithm (Sec. 5.1); every row is written by exactly one
-// thread team (or, for dense-window rows, each column slice by one team),
-// so C's segments are disjoint (the shard pattern, Sec. 4).
+// (analyze.cu says which rows take which).  Each class is a different
+// realisation of the per-row workspace w of Gustavson's algorithm (Sec. 5.1).
+// Every row, or window or slice of a row, is written by exactly one thread team,
+// so C's segments are disjoint (the shard pattern, Sec. 4); only the parts of a
+// wide heavy row add to the same segment (the atomic level).
 #pragma once
 
 #include <cstdint>
@@ -73,22 +80,23 @@ constexpr uint8_t kClsBitmap0 = kClsBmr0 + kNumBmrBins;    // .. + kNumBitmapBin
 constexpr uint8_t kClsHash0 = kClsBitmap0 + kNumBitmapBins;  // .. + kNumHashBins - 1
 constexpr uint8_t kClsDense = kClsHash0 + kNumHashBins;
 constexpr uint8_t kClsBmrWide = kClsDense + 1;  // register bitmap rows counted by the planning pass
-constexpr uint8_t kClsRcd = kClsBmrWide + 1;    // heavy rows, dense column-slice workspace, CTA per row
-constexpr uint8_t kClsWb = kClsRcd + 1;         // heavy rows, wide bitmap workspace, CTA per row
+constexpr uint8_t kClsRcd = kClsBmrWide + 1;    // dense heavy rows
+constexpr uint8_t kClsWb = kClsRcd + 1;         // wide heavy rows (wide bitmap)
 
-// Heavy-row limits.
-constexpr int kRcdMaxA = 8192;            // stored A entries a dense row may have (cursor slots)
+// Dense heavy rows.
+constexpr int kRcdMaxA = 8192;            // stored A entries a row may have
 constexpr int kRcdDefaultMaxA = 8192;     // default limit used by the classification
-constexpr int kRcdWidthBytes = 49152;     // value window of one item of a dense heavy row, at most
+constexpr int kRcdWidthBytes = 49152;     // value window of a numeric item, at most
 constexpr int kRcdLeastWidth = 512;       // entries of a window, at least
-// Counters of the dense heavy rows: items of rows with many products, other
-// items, next row of the symbolic pass, next item of the numeric pass.
-// Wide-bitmap rows: products per numeric item, most items of a row, counters.
-constexpr int kWbPart = 16384;  // at least
-constexpr int kWbMaxParts = 1024;
-constexpr int kWbBigItems = 0, kWbItems = 1, kWbNextItem = 2, kWbCounters = 3;
+// Counters: items of rows with many products, other items, next row of the
+// symbolic pass, next item of the numeric pass.
 constexpr int kRcdBigItems = 0, kRcdItems = 1, kRcdNextRow = 2, kRcdNextItem = 3, kRcdCounters = 4;
-constexpr int kWbMaxSpan = 1 << 20;       // widest column range of a wide-bitmap row
+// Wide heavy rows.
+constexpr int kWbMaxSpan = 1 << 20;       // widest column range
+constexpr int kWbPart = 16384;            // products of a numeric item, at least
+constexpr int kWbMaxParts = 1024;         // items of a row, at most
+// Counters: items of rows of several items, other items, next item of the numeric pass.
+constexpr int kWbBigItems = 0, kWbItems = 1, kWbNextItem = 2, kWbCounters = 3;
 
 // Segments of the row permutation: direct rows, register bitmap bins, bitmap
 // bins, hash bins, dense-window rows.
@@ -281,7 +289,7 @@ struct AnalyzeParams {
   int64_t wb_span;     // widest column range of a wide-bitmap heavy row (0: none)
   int dense_width;
   int long_threshold;
-  int64_t nnz;         // stored entries of A, at most
+  int64_t nnz;         // stored entries of A; an estimate, which sizes a grid only
 };
 // rows == nullptr: every row of A; otherwise the first sum->n_pending entries of rows.
 // host != nullptr: the summary is copied there at the end.
