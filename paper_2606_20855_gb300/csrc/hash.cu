@@ -268,7 +268,7 @@ __device__ __forceinline__ int rank_row(const int (&col)[Bin<LOGC, W>::kS], int 
 #pragma unroll
       for (int w = 0; w < W; ++w) most = max(most, scratch[w]);
     }
-    if (most <= run_limit) {  // at most kMaxHashBucket
+    if (most <= run_limit && most <= kMaxHashBucket) {  // the second test is for the compiler: the loops below are short
 #pragma unroll
       for (int j = 0; j < kOwn; ++j) cnt[t * kOwn + j] = own[j] + (ex | (ex << 16));
       if (t == 0) base[kCap] = static_cast<uint16_t>(ub);
