@@ -35,8 +35,10 @@ __device__ __forceinline__ int ceil_log2_ll(long long x) {  // x >= 1
 // - one of their B rows is longer than kShortB: such rows (hub rows of a
 //   power-law matrix) tend to be dense at one end, which fills some buckets;
 // - the row has more than 16 entries and its B rows have lumps (three of four
-//   of the first kLooks of more than three columns): runs of neighbouring
-//   columns, as of a box stencil or of blocks, fill a bucket each; or
+//   of those of more than three columns among the first kLooks, at least
+//   kLeastLooks): runs of neighbouring columns, as of a box stencil or of blocks,
+//   fill a bucket each (with one look as the least, 26 of 128,000 rows of
+//   scattered columns went to bins of their own, whose launches cost 20 us); or
 // - a bitmap is cheaper although the columns spread: above kLargeHash products
 //   of B rows of kLongB columns and more (the windows of the dense rows), and in
 //   the bin of kSmallTo products and 16,384 columns when the B rows are of about the
@@ -56,7 +58,7 @@ __device__ __forceinline__ int ceil_log2_ll(long long x) {  // x >= 1
 // column-sliced dense window.
 constexpr long long kCrowded = 2;
 constexpr int kShortB = 64;
-constexpr int kLooks = 8;
+constexpr int kLooks = 8, kLeastLooks = 5;
 constexpr long long kLargeHash = 2048, kLongB = 16;
 constexpr long long kSmallFrom = bitmap_cap(0), kSmallTo = bitmap_cap(1), kSmallSpan = 32ll << bitmap_log_words(1);
 constexpr int kBatch = 4;  // stored A entries of a long row that a thread has in flight
@@ -115,7 +117,7 @@ struct RowShape {
       lumps += look && 4 * (static_cast<int64_t>(third) - first[0]) * (be[0] - bs[0] - 1) <= static_cast<int64_t>(last[0]) - first[0];
     }
   }
-  __device__ __forceinline__ bool lumpy() const { return looked > 0 && 4 * lumps >= 3 * looked; }
+  __device__ __forceinline__ bool lumpy() const { return looked >= kLeastLooks && 4 * lumps >= 3 * looked; }
 
   __device__ __forceinline__ void merge(const RowShape& o) {
     ub += o.ub;
