@@ -24,6 +24,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "ws_internal.cuh"
@@ -1179,22 +1180,32 @@ void release_outer(Plan* pl, cudaStream_t s) {
   pl->outer = nullptr;
 }
 
-// The same, but the plan (its status words) stays: what is queued on s still
-// uses the scratch, nothing after it does.
-void release_scratch_async(Plan* pl, cudaStream_t s) {
+// The scratch of `from`, whose last pass is queued on a stream, for passes of
+// `to` on the same stream (and the scratch of `to`, if it has some, for `from`).
+// So the blocks of an outer product use the scratch of one.  Freeing it after
+// every block instead left the stream-ordered pool with other free ranges than
+// the next partial product and merge ask for, and a product of 65,539 rows
+// of 16 entries times rows of 32 in four blocks took 2.71 instead of 2.06 ms.
+void hand_over_scratch(Plan* from, Plan* to) {
+  DevBuf* a[] = {&from->rows, &from->slices, &from->ranks, &from->ew, &from->sv, &from->hranks, &from->rcd, &from->wb};
+  DevBuf* b[] = {&to->rows, &to->slices, &to->ranks, &to->ew, &to->sv, &to->hranks, &to->rcd, &to->wb};
+  for (size_t i = 0; i < sizeof(a) / sizeof(a[0]); ++i) std::swap(*a[i], *b[i]);
+  // a summary block that the last pass left cleared goes with its buffer
+  to->clean_buf = from->clean_buf == &from->rows ? &to->rows : nullptr;
+  to->clean_gen = from->clean_gen;
+  from->clean_buf = nullptr;
+  from->ready = false;
+}
+
+void release_plan_async(Plan* pl, cudaStream_t s) {
+  if (!pl) return;
+  release_outer(pl, s);
   DevBuf* bufs[] = {&pl->rows, &pl->slices, &pl->ranks, &pl->ew, &pl->sv, &pl->hranks, &pl->rcd, &pl->wb};
   for (DevBuf* b : bufs) {
     if (b->ptr) cudaFreeAsync(b->ptr, s);
     b->ptr = nullptr;
     b->bytes = 0;
   }
-  pl->ready = false;
-}
-
-void release_plan_async(Plan* pl, cudaStream_t s) {
-  if (!pl) return;
-  release_outer(pl, s);
-  release_scratch_async(pl, s);
   release_host_sum(pl->host_sum);
   delete pl;
 }
@@ -1319,13 +1330,13 @@ ws_status_t outer_symbolic_impl(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* 
     Owned* cp = nullptr;
     if ((st = new_owned(m, n, A->dtype, C->device, s, &cp)) != WS_OK) break;
     partial.push_back(cp);
+    if (partial.size() > 1) hand_over_scratch(partial[partial.size() - 2]->h.plan, cp->h.plan);
     int64_t nnz_p = 0;
     if ((st = symbolic_impl<T>(&ab->h, &bp, &cp->h, cp->h.plan, s, &nnz_p)) != WS_OK) break;
     cp->h.nnz = nnz_p;
     if ((st = owned_entries(cp, nnz_p, s)) != WS_OK) break;
     if ((st = numeric_impl<T>(&ab->h, &bp, &cp->h, cp->h.plan, s)) != WS_OK) break;
     launches += cp->h.plan->sym_launches + cp->h.plan->num_launches;
-    release_scratch_async(cp->h.plan, s);  // the next block's pass takes it
   }
   // every extraction has completed (each block's structure pass synchronised)
   if (st == WS_OK) st = plan_status(ab->h.plan);
