@@ -42,8 +42,9 @@ __device__ __forceinline__ int ceil_log2_ll(long long x) {  // x >= 1
 // - a bitmap is cheaper although the columns spread: above kLargeHash products
 //   of B rows of kLongB columns and more (the windows of the dense rows), and in
 //   the bin of kSmallTo products and 16,384 columns when the B rows are of about the
-//   same length, so that the lane groups are full (that hash bin holds as much
-//   as twice the products for the same time).
+//   same length, of kSmallB columns and more, so that the lane groups are full
+//   (that hash bin holds as much as twice the products for the same time; a few
+//   rows of 150 entries and B rows of 2 took 10 us more in a bitmap).
 // Those take the bitmap bins, and the dense rows above them.  Measured (24
 // million products, fp32, bitmap or dense rows against hash bins, ms): rows of
 // 0-40 entries and B rows of 0-20 over 16,000 columns 0.86 against 0.59; 40 of 20
@@ -60,7 +61,7 @@ constexpr long long kCrowded = 2;
 constexpr int kShortB = 64;
 constexpr int kLooks = 8, kLeastLooks = 5;
 constexpr long long kLargeHash = 2048, kLongB = 16;
-constexpr long long kSmallFrom = bitmap_cap(0), kSmallTo = bitmap_cap(1), kSmallSpan = 32ll << bitmap_log_words(1);
+constexpr long long kSmallB = 8, kSmallFrom = bitmap_cap(0), kSmallTo = bitmap_cap(1), kSmallSpan = 32ll << bitmap_log_words(1);
 constexpr int kBatch = 4;  // stored A entries of a long row that a thread has in flight
 
 // What a row's class depends on, gathered over its stored A entries.
@@ -151,7 +152,8 @@ __device__ __forceinline__ uint8_t classify(long long nnza, const RowShape& r, c
   const bool regular = nnza <= kBmrMaxA && maxlen <= ap.group;
   const bool spread = span >= kCrowded * ub && maxlen <= kShortB && !r.lumpy();
   const bool bitmap_cheaper = (ub > kLargeHash && ub >= kLongB * nnza) ||
-                              (ub > kSmallFrom && ub <= kSmallTo && span <= kSmallSpan && 4 * ub >= 3 * nnza * maxlen);
+                              (ub > kSmallFrom && ub <= kSmallTo && span <= kSmallSpan && ub >= kSmallB * nnza &&
+                               4 * ub >= 3 * nnza * maxlen);
   const bool hashed = ub <= ap.hash_max && (!bitmap_ok || (!regular && spread && !bitmap_cheaper));
   if (bitmap_ok && !hashed) {
     if (regular && nnza <= ap.bmr_max_a) {

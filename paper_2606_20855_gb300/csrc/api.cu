@@ -564,7 +564,7 @@ RowPlan<T> make_rowplan(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan*
   p.rcd_bits = pl->rcd_bits;
   p.rcd_words = pl->rcd_words;
   p.rcd_width = pl->rcd_width;
-  p.rcd_direct = B->ncols <= pl->rcd_width;
+  p.rcd_direct = B->ncols <= pl->rcd_width && B->nnz / kRcdLongB > B->nrows;
   p.rcd_long_b = B->nnz / 512 > B->nrows;
   p.rcd_slices = pl->rcd_slices;
   p.wb_ctr = pl->wb_ctr;
@@ -650,18 +650,19 @@ void reserve_hash_ranks(Plan* pl, cudaStream_t s) {
 // Room for the bitmaps and numeric items of the dense heavy rows: of all of
 // them, or else of as many as can be had.  The rows are then taken in batches,
 // and the numeric pass makes the bitmaps again.  The value windows are as large
-// as shared memory allows, unless there would be fewer than one per SM: an item
-// is one CTA's work, and three fit an SM.  30 rows of 2000 entries times rows of
+// as shared memory allows, unless B's rows are long and there would be fewer
+// windows than one per SM: an item is one CTA's work, and three fit an SM.  (Every
+// item walks all stored entries of its row, so short B rows gain nothing: XX.)  30 rows of 2000 entries times rows of
 // 1460 over 3000 columns: 0.83 ms (fp64) and 0.76 (fp32), 1.98 and 1.58 with a window
 // each; 300 rows of 500 entries times rows of 460, two windows a row instead of
 // one: 0.52 and 0.46 against 0.35 and 0.27.
 template <typename T>
-ws_status_t carve_rcd(Plan* pl, int64_t ncols, int sms, cudaStream_t s) {
+ws_status_t carve_rcd(Plan* pl, int64_t ncols, bool long_b, int sms, cudaStream_t s) {
   constexpr int64_t kMinBatch = 1024;
   constexpr int64_t kWidest = kRcdWidthBytes / sizeof(T);
   const int64_t nr = pl->seg_count[kSegRcd], span = ncols < kMaxBitmapSpan ? ncols : kMaxBitmapSpan;
   int64_t width = kWidest;
-  if (nr * ((span + kWidest - 1) / kWidest) < sms) width = align_up(static_cast<size_t>(span * nr / (3 * sms) + 1), kRcdLeastWidth);
+  if (long_b && nr * ((span + kWidest - 1) / kWidest) < sms) width = align_up(static_cast<size_t>(span * nr / (3 * sms) + 1), kRcdLeastWidth);
   pl->rcd_width = static_cast<int>(width < kWidest ? width : kWidest);
   pl->rcd_slices = static_cast<int>((span + pl->rcd_width - 1) / pl->rcd_width);
   pl->rcd_words = static_cast<int>(align_up((span + 31) / 32, 4));
@@ -791,7 +792,7 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     if (st != WS_OK) return st;
   }
   if (pl->seg_count[kSegRcd] > 0) {
-    st = carve_rcd<T>(pl, B->ncols, sms, s);
+    st = carve_rcd<T>(pl, B->ncols, B->nnz / kRcdLongB > B->nrows, sms, s);
     if (st != WS_OK) return st;
   }
   if (pl->seg_count[kSegWb] > 0) {

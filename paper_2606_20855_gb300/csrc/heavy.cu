@@ -235,7 +235,7 @@ constexpr int kNumThreads = 256;
 constexpr int kNumCacheA = kNumThreads;       // stored A entries handled at a time
 constexpr int kNumDesc = 128;                 // rounds described at a time
 constexpr int kNumWords = kRcdWords / kNumThreads;  // bitmap words per thread
-constexpr int kNumShort = 96;   // a warp each, three entries per lane
+constexpr int kNumShort = kRcdLongB;  // a warp each, three entries per lane
 constexpr int kNumTiny = 16;    // a group of kNumTinyLanes lanes each
 constexpr int kNumTinyLanes = 4;
 constexpr int kAhead = 3;

@@ -88,6 +88,7 @@ constexpr int kRcdMaxA = 8192;            // stored A entries a row may have
 constexpr int kRcdDefaultMaxA = 8192;     // default limit used by the classification
 constexpr int kRcdWidthBytes = 49152;     // value window of a numeric item, at most
 constexpr int kRcdLeastWidth = 512;       // entries of a window, at least
+constexpr int kRcdLongB = 96;             // longest part of a B row that a warp takes; B is long above it on average
 // Counters: items of rows with many products, other items, next row of the
 // symbolic pass, next item of the numeric pass.
 constexpr int kRcdBigItems = 0, kRcdItems = 1, kRcdNextRow = 2, kRcdNextItem = 3, kRcdCounters = 4;
@@ -192,7 +193,7 @@ struct RowPlan {
   uint32_t* rcd_bits;          // dense heavy rows: bitmap of the row's columns from lo on, rcd_words words per row
   int rcd_words;               // a multiple of 4, enough for min(columns of B, kMaxBitmapSpan)
   int rcd_width;               // entries of a value window
-  bool rcd_direct;             // a window covers all columns of B
+  bool rcd_direct;             // a window covers all columns of B, whose rows are long on average
   bool rcd_long_b;             // B's rows have more than 512 entries on average
   int rcd_slices;              // value windows of a row at most
   long long* rcd_items;        // their numeric work items (row * rcd_slices + window): rows with many products
