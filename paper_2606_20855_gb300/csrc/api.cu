@@ -564,8 +564,8 @@ RowPlan<T> make_rowplan(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Plan*
   p.rcd_bits = pl->rcd_bits;
   p.rcd_words = pl->rcd_words;
   p.rcd_width = pl->rcd_width;
-  p.rcd_direct = B->ncols <= pl->rcd_width && B->nnz / kRcdLongB > B->nrows;
-  p.rcd_long_b = B->nnz / 512 > B->nrows;
+  p.rcd_direct = B->ncols <= pl->rcd_width && B->nnz > kRcdLongB * B->nrows;
+  p.rcd_long_b = B->nnz > 512 * B->nrows;
   p.rcd_slices = pl->rcd_slices;
   p.wb_ctr = pl->wb_ctr;
   p.wb_items = pl->wb_items;
@@ -651,8 +651,11 @@ void reserve_hash_ranks(Plan* pl, cudaStream_t s) {
 // them, or else of as many as can be had.  The rows are then taken in batches,
 // and the numeric pass makes the bitmaps again.  The value windows are as large
 // as shared memory allows, unless B's rows are long and there would be fewer
-// windows than one per SM: an item is one CTA's work, and three fit an SM.  (Every
-// item walks all stored entries of its row, so short B rows gain nothing: XX.)  30 rows of 2000 entries times rows of
+// windows than one per SM: an item is one CTA's work, and three fit an SM.  Every
+// item walks all stored entries of its row, so short B rows gain from it only
+// where rows are very few (fp32: 100 rows of 2800 entries times rows of 90 over 12,000
+// columns 0.39 whole and 0.46 split, 40 of 6600 times rows of 10 over 5000 0.26
+// and 0.28, 10 of 6600 times rows of 60 over 30,000 0.68 and 0.48).  30 rows of 2000 entries times rows of
 // 1460 over 3000 columns: 0.83 ms (fp64) and 0.76 (fp32), 1.98 and 1.58 with a window
 // each; 300 rows of 500 entries times rows of 460, two windows a row instead of
 // one: 0.52 and 0.46 against 0.35 and 0.27.
@@ -792,7 +795,7 @@ ws_status_t symbolic_bins(const ws_csr_s* A, const ws_csr_s* B, ws_csr_s* C, Pla
     if (st != WS_OK) return st;
   }
   if (pl->seg_count[kSegRcd] > 0) {
-    st = carve_rcd<T>(pl, B->ncols, B->nnz / kRcdLongB > B->nrows, sms, s);
+    st = carve_rcd<T>(pl, B->ncols, B->nnz > kRcdLongB * B->nrows, sms, s);
     if (st != WS_OK) return st;
   }
   if (pl->seg_count[kSegWb] > 0) {

@@ -213,16 +213,17 @@ void many_wide_bitmap_rows_run_by_themselves() {
 }
 
 // Dense rows are cut into value windows for three CTAs per SM (of 4) if they
-// would not keep every SM busy.
+// would not keep every SM busy and B's rows have more than 96 entries on average.
 void few_dense_rows_take_small_windows() {
   const int widest = wsk::kRcdWidthBytes / 8;
   const struct {
     int rows;
-    int64_t ncols;
+    int64_t ncols, b_row;
     int width;
-  } cases[] = {{1, 3000, 512}, {3, 3000, 1024}, {4, 3000, widest}, {1, 60000, widest}, {1, 20000, widest}, {1, 18000, 1536}};
+  } cases[] = {{1, 3000, 97, 512},      {3, 3000, 97, 1024},     {4, 3000, 97, widest}, {1, 60000, 97, widest},
+               {1, 20000, 97, widest}, {1, 18000, 97, 1536}, {1, 3000, 96, widest}};
   for (const auto& c : cases) {
-    ws_csr_t A = matrix(100, 1 << 17, 64), B = matrix(1 << 17, c.ncols, 64), C = matrix(100, c.ncols, 0);
+    ws_csr_t A = matrix(100, 1 << 10, 64), B = matrix(1 << 10, c.ncols, c.b_row << 10), C = matrix(100, c.ncols, 0);
     fake::summary = wsk::DevSummary{};
     fake::summary.n_pending = 1;
     fake::summary.seg_count[wsk::kSegRcd] = c.rows;
