@@ -32,7 +32,13 @@ namespace wsk {
 
 constexpr int kNumHashBins = 8;
 constexpr int kMinHashLog = 5;  // bin b holds rows of at most 1 << (kMinHashLog + b) products
-constexpr int kMaxHashBucket = 63;  // most products of a hash bucket that are compared with one another (6 bits)
+// Most products of a hash bucket that are compared with one another: what the 6 bits
+// of its counter hold; fuller buckets sort the row.  Lower limits of 48, 32 and 16
+// measured against 63: 27-point stencil over a range wider than 65,536 columns,
+// squared, 17.5, 17.3 and 17.3 ms against 26.6; R-MAT 2^17 (edge factor 8) squared
+// 19.24, 19.47 and 19.86 against 19.40; R-MAT 2^20 (edge factor 2) squared 56.2, 56.6
+// and 56.7 against 56.0.
+constexpr int kMaxHashBucket = 63;
 constexpr int kMaxHashProducts = 32 << (kNumHashBins - 1);  // 4096
 
 // Bitmap bins: bitmap of 1 << log_words 32-bit words (the row's column range
